@@ -236,11 +236,11 @@ const char *syn_last_cuda_error(void);
  * call syn_op_linear_reset after the contents of w changed or w was freed (a new matrix may land at
  * the old address).  K a multiple of 64 is not required (TMA zero-fills the tail) but K*2 bytes must
  * be a multiple of 16; N arbitrary.  Blocks until the result is there.
- * syn_op_linear_as runs the same product under the schedule the step uses for the projection with
- * epilogue `schedule_as` (0 plain, 1 qkv, 2 residual, 3 SwiGLU, 4 lm_head; see syn_gemm_plan_host), so
+ * syn_op_linear_as runs the same product under the schedule that the one-CTA and CTA-pair kernels use for the
+ * projection with epilogue `schedule_as` (0 plain, 1 qkv, 2 residual, 3 SwiGLU, 4 lm_head; see syn_gemm_plan_host), so
  * that every schedule can be checked against a plain matrix product; 5 and 6 take the CTA-pair kernel
  * with items of 512 and of 256 features whatever the shape, 7 and 8 the same as residual projections
- * (K shared between clusters where the shape allows it).
+ * (K shared between clusters where the shape allows it), 9 the thin kernel of the batches of few tokens.
  * Errors: SYN_E_INVALID_ARG, SYN_E_CUDA, SYN_E_DEVICE_TIMEOUT. */
 int syn_op_linear(const void *x, const void *w, float *y, int32_t T, int32_t N, int32_t K, void *cuda_stream);
 int syn_op_linear_as(const void *x, const void *w, float *y, int32_t T, int32_t N, int32_t K, int32_t schedule_as,
@@ -325,6 +325,13 @@ int syn_gemm_work_host(int32_t T, int32_t N, int32_t K, int32_t n_sm, int32_t ep
 int syn_gemm2_plan_host(int32_t T, int32_t N, int32_t K, int32_t n_sm, int32_t epilogue, int32_t force, int32_t *out);
 int syn_gemm2_work_host(int32_t T, int32_t N, int32_t K, int32_t n_sm, int32_t epilogue, int32_t force, int32_t cluster,
                         int32_t i, int32_t *out);
+
+/* The launch shape of a projection on the thin kernel, which serves batches of few tokens: out[SYN_THIN_PLAN_FIELDS] =
+ * {1 when the projection with this epilogue takes it, 128-feature tiles, token tiles, tokens per tile, k-blocks of 64, CTAs
+ * (a cluster) that share a tile's K range: part s covers the k-blocks [s nkb / S, (s + 1) nkb / S), operand stages,
+ * bytes of the operand ring that the exchange and the epilogue leave unused}.  Errors: SYN_E_INVALID_ARG. */
+#define SYN_THIN_PLAN_FIELDS 8
+int syn_thin_plan_host(int32_t T, int32_t N, int32_t K, int32_t n_sm, int32_t epilogue, int32_t *out);
 
 /* Sampling-based verification (paper Sec. 4.2, "Compression before transmission": for
  * verification the LLM needs the drafts and the SLM's distributions, of which the device sends

@@ -62,7 +62,8 @@ EXPORTS = ["syn_model_load", "syn_model_free", "syn_kv_alloc", "syn_kv_free", "s
            "syn_debug_set_attention",
            "syn_op_attention", "syn_op_attention_static",
            "syn_set_profile", "syn_get_profile", "syn_verify_batch_sampled", "syn_op_sample_verify",
-           "syn_gemm_plan_host", "syn_gemm_work_host", "syn_gemm2_plan_host", "syn_gemm2_work_host"]
+           "syn_gemm_plan_host", "syn_gemm_work_host", "syn_gemm2_plan_host", "syn_gemm2_work_host",
+           "syn_thin_plan_host"]
 SCHED_EXPORTS = ["syn_sched_create", "syn_sched_free", "syn_sched_add_request", "syn_sched_add_verify", "syn_sched_finish",
                  "syn_sched_peek", "syn_sched_commit", "syn_sched_step", "syn_sched_get_stats"]
 
@@ -499,8 +500,9 @@ GEMM_PLAN_FIELDS = ("n_pairs", "n_tt", "TN", "num_kb", "n_cta", "pair_mode", "sp
 GEMM_WORK_FIELDS = ("pair", "tt", "mt_lo", "mt_hi", "kb0", "kb1", "split", "role", "rtile", "hpart")
 GEMM_EPILOGUES = {"plain": 0, "qkv": 1, "resid": 2, "swiglu": 3, "lmhead": 4}
 # syn_op_linear_as only: the CTA-pair kernel with 512-feature (quad) or 256-feature (duo) items, as a
-# plain projection or as a residual projection (K shared between clusters where the shape allows it)
-LINEAR_SCHEDULES = dict(GEMM_EPILOGUES, pair_quad=5, pair_duo=6, pair_quad_resid=7, pair_duo_resid=8)
+# plain projection or as a residual projection (K shared between clusters where the shape allows it), and the
+# thin kernel of the batches of few tokens
+LINEAR_SCHEDULES = dict(GEMM_EPILOGUES, pair_quad=5, pair_duo=6, pair_quad_resid=7, pair_duo_resid=8, thin=9)
 
 
 def gemm_plan_host(T: int, N: int, K: int, epilogue: str, n_sm: int = 148) -> Dict[str, int]:
@@ -545,6 +547,17 @@ def gemm2_work_host(T: int, N: int, K: int, epilogue: str, cluster: int, i: int,
     if r < 0:
         _check(r, "syn_gemm2_work_host")
     return dict(zip(GEMM2_WORK_FIELDS, out)) if r == 1 else None
+
+
+THIN_PLAN_FIELDS = ("takes_it", "n_tiles", "n_tt", "TN", "num_kb", "splits", "n_stages", "ring_left")
+
+
+def thin_plan_host(T: int, N: int, K: int, epilogue: str = "plain", n_sm: int = 148) -> Dict[str, int]:
+    """syn_thin_plan_host: the launch shape of one projection on the thin kernel, without a device."""
+    out = (C.c_int32 * len(THIN_PLAN_FIELDS))()
+    _check(load_library().syn_thin_plan_host(C.c_int32(T), C.c_int32(N), C.c_int32(K), C.c_int32(n_sm),
+                                             C.c_int32(GEMM_EPILOGUES[epilogue]), out), "syn_thin_plan_host")
+    return dict(zip(THIN_PLAN_FIELDS, out))
 
 
 def syn_op_linear(x: torch.Tensor, w: torch.Tensor, stream=None, schedule_as: str = "plain",

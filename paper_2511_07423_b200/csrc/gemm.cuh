@@ -115,13 +115,58 @@ constexpr int EPI_SCR_FLOATS = EPI_COLS * EPI_SCR_STRIDE;   // per epilogue warp
 
 __device__ __forceinline__ uint2 pack4_op(float a, float b, float c, float d) { return make_uint2(pack_op(a, b), pack_op(c, d)); }
 
+// What an epilogue reads besides the accumulators: the residual rows and the gains (EPI_RESID) or the RoPE rows and KV
+// slots (EPI_QKV).  Loaded on its own so that a caller can have it in flight while it waits for the accumulators.
 template <int MODE>
-__device__ __forceinline__ void epi_unit(const EpiParams& p, const float (&a)[EPI_COLS], float* scr, int m0, int t0, int ncols,
-                                         int quarter, int lane) {
+struct EpiOperand {
+    float4 v[MODE == EPI_QKV ? 8 : (MODE == EPI_RESID ? 4 : 1)];
+    uint2 gain;
+    int slot;
+};
+
+template <int MODE>
+__device__ __forceinline__ void epi_load_rope(const EpiParams& p, EpiOperand<MODE>& o, int t0, int ncols, int quarter, int lane) {
+    const int tq = lane >> 3, c0 = (lane & 7) * 4;
+    const int half = p.hd >> 1, dim = 16 * (quarter & ((half >> 4) - 1)) + (c0 & 15);   // lower dim of the pair
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)(t0 + tq + 4 * i) * half + dim);   // 4 x (cos, sin)
+        const bool tv = tq + 4 * i < ncols;
+        o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)] = tv ? __ldg(cs) : make_float4(1.f, 0.f, 1.f, 0.f);
+        o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)] = tv ? __ldg(cs + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
+    }
+}
+
+template <int MODE>
+__device__ __forceinline__ void epi_load(const EpiParams& p, EpiOperand<MODE>& o, int m0, int t0, int ncols, int quarter, int lane) {
+    const int tq = lane >> 3, c0 = (lane & 7) * 4;
+    if (MODE == EPI_RESID) {
+        const int f = m0 + quarter * 32 + c0;
+        o.gain = __ldg(reinterpret_cast<const uint2*>(p.gain + f));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            o.v[i & (MODE == EPI_RESID ? 3 : 0)] = tq + 4 * i < ncols ? *reinterpret_cast<const float4*>(p.x + (size_t)(t0 + tq + 4 * i) * p.d + f)
+                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (MODE == EPI_QKV) {
+        const int which = m0 < p.q_dim ? 0 : (m0 < p.q_dim + p.kv_dim ? 1 : 2);
+        // KV slot (page * 16 + row) of token lane & 15, handed round by shuffles
+        o.slot = (which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0;
+        if (which < 2) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane);
+    }
+}
+
+// The chunk into the warp's scratch, one feature per lane ...
+__device__ __forceinline__ void epi_stage(const float (&a)[EPI_COLS], float* scr, int lane) {
     __syncwarp();   // the previous chunk's rows have been read
 #pragma unroll
     for (int j = 0; j < EPI_COLS; ++j) scr[j * EPI_SCR_STRIDE + lane] = a[j];
     __syncwarp();
+}
+
+// ... and out of it row by row.  LOADED: the operands are in `o` already; otherwise they are loaded where they are used.
+template <int MODE, bool LOADED>
+__device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float* scr, int m0, int t0, int ncols,
+                                         int quarter, int lane) {
     const int tq = lane >> 3, c0 = (lane & 7) * 4;   // token (+ 4 i) and first of four columns of this lane
     if (MODE == EPI_PLAIN) {
         const int f = m0 + quarter * 32 + c0;
@@ -143,20 +188,16 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, const float (&a)[EP
     } else if (MODE == EPI_RESID) {
         // x += D; operand of the next projection bf16(x * gain); sum of x^2 over this warp's 32 features
         const int f = m0 + quarter * 32 + c0;
-        const uint2 gb = __ldg(reinterpret_cast<const uint2*>(p.gain + f));
-        const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&gb.x);
-        const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&gb.y);
-        float4 xv[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            xv[i] = tq + 4 * i < ncols ? *reinterpret_cast<const float4*>(p.x + (size_t)(t0 + tq + 4 * i) * p.d + f)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!LOADED) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
+        const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.x);
+        const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.y);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = tq + 4 * i;
             const bool tv = t < ncols;
             const float* row = scr + t * EPI_SCR_STRIDE + c0;
-            const float4 nx = make_float4(xv[i].x + row[0], xv[i].y + row[1], xv[i].z + row[2], xv[i].w + row[3]);
+            const float4 xv = o.v[i & (MODE == EPI_RESID ? 3 : 0)];
+            const float4 nx = make_float4(xv.x + row[0], xv.y + row[1], xv.z + row[2], xv.w + row[3]);
             float ss = tv ? (nx.x * nx.x + nx.y * nx.y) + (nx.z * nx.z + nx.w * nx.w) : 0.f;
             if (tv) {
                 const size_t at = (size_t)(t0 + t) * p.d + f;
@@ -172,41 +213,34 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, const float (&a)[EP
     } else if (MODE == EPI_QKV) {
         const int which = m0 < p.q_dim ? 0 : (m0 < p.q_dim + p.kv_dim ? 1 : 2);
         const int region0 = which == 0 ? 0 : (which == 1 ? p.q_dim : p.q_dim + p.kv_dim);
-        const int half = p.hd >> 1;
+        const int half = p.hd >> 1, hd_log = p.hd == 128 ? 7 : 6;   // head_dim is 64 or 128
         const size_t page_stride = (size_t)p.n_kv_heads * 2 * 16 * p.hd;
-        // KV slot (page * 16 + row) of token lane & 15, handed round by shuffles
-        const int my_slot = (which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0;
+        const int my_slot = LOADED ? o.slot : ((which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0);
         if (which < 2) {
             // q and k tiles: columns 0..15 of the block are the dims [d0, d0 + 16) of one head, columns 16..31
             // the same dims + hd/2 (rope_tile_feature); a lane rotates its four columns with their partners
-            const int groups = half >> 4;
-            const int fhead = (m0 - region0) + (quarter / groups) * p.hd;   // first feature of the head, inside q or k
+            const int g_log = hd_log - 5;                                   // 16-dim groups of a half
+            const int fhead = (m0 - region0) + ((quarter >> g_log) << hd_log);   // first feature of the head, inside q or k
             const bool hi = c0 >= 16;
-            const int dim = 16 * (quarter % groups) + (c0 & 15);            // lower dim of the pair
-            float4 w[4][2];
+            const int dim = 16 * (quarter & ((1 << g_log) - 1)) + (c0 & 15);            // lower dim of the pair
+            if (!LOADED) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)(t0 + tq + 4 * i) * half + dim);   // 4 x (cos, sin)
-                const bool tv = tq + 4 * i < ncols;
-                w[i][0] = tv ? __ldg(cs) : make_float4(1.f, 0.f, 1.f, 0.f);
-                w[i][1] = tv ? __ldg(cs + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
+                const float4 w0 = o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)], w1 = o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)];
                 const int t = tq + 4 * i;
                 const float* mine = scr + t * EPI_SCR_STRIDE + c0;
                 const float* part = scr + t * EPI_SCR_STRIDE + (c0 ^ 16);
                 const float sg = hi ? 1.f : -1.f;   // dim i: x cos - y sin; dim i + hd/2: y cos + x sin
-                const float o0 = mine[0] * w[i][0].x + sg * part[0] * w[i][0].y;
-                const float o1 = mine[1] * w[i][0].z + sg * part[1] * w[i][0].w;
-                const float o2 = mine[2] * w[i][1].x + sg * part[2] * w[i][1].y;
-                const float o3 = mine[3] * w[i][1].z + sg * part[3] * w[i][1].w;
+                const float r0 = mine[0] * w0.x + sg * part[0] * w0.y;
+                const float r1 = mine[1] * w0.z + sg * part[1] * w0.w;
+                const float r2 = mine[2] * w1.x + sg * part[2] * w1.y;
+                const float r3 = mine[3] * w1.z + sg * part[3] * w1.w;
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
                     op16* dst;
                     if (which == 0) dst = p.q + (size_t)(t0 + t) * p.q_dim + fhead;
-                    else dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fhead / p.hd) * 2) * 16 * p.hd + (size_t)(sl & 15) * p.hd;
-                    *reinterpret_cast<uint2*>(dst + dim + (hi ? half : 0)) = pack4_op(o0, o1, o2, o3);
+                    else dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fhead >> hd_log) * 2) * 16 * p.hd + (size_t)(sl & 15) * p.hd;
+                    *reinterpret_cast<uint2*>(dst + dim + (hi ? half : 0)) = pack4_op(r0, r1, r2, r3);
                 }
             }
         } else {
@@ -218,7 +252,7 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, const float (&a)[EP
                 const float* row = scr + t * EPI_SCR_STRIDE + c0;
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
-                    op16* dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fr / p.hd) * 2 + 1) * 16 * p.hd +
+                    op16* dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fr >> hd_log) * 2 + 1) * 16 * p.hd +
                                          (size_t)(sl & 15) * p.hd + (fr & (p.hd - 1));
                     *reinterpret_cast<uint2*>(dst) = pack4_op(row[0], row[1], row[2], row[3]);
                 }
@@ -278,6 +312,14 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, const float (&a)[EP
     }
 }
 
+template <int MODE>
+__device__ __forceinline__ void epi_whole(const EpiParams& p, const float (&a)[EPI_COLS], float* scr, int m0, int t0, int ncols,
+                                          int quarter, int lane) {
+    EpiOperand<MODE> o;
+    epi_stage(a, scr, lane);
+    epi_unit<MODE, false>(p, o, scr, m0, t0, ncols, quarter, lane);
+}
+
 __device__ __forceinline__ void epi_dispatch(int mode, const EpiParams& p, const uint32_t (&r)[EPI_COLS], const float* rs, float* scr,
                                              int m0, int t0, int ncols, int quarter, int lane) {
     float a[EPI_COLS];
@@ -288,11 +330,11 @@ __device__ __forceinline__ void epi_dispatch(int mode, const EpiParams& p, const
         for (int j = 0; j < EPI_COLS; ++j) a[j] *= rs[j];
     }
     switch (mode) {
-        case EPI_PLAIN: epi_unit<EPI_PLAIN>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_QKV: epi_unit<EPI_QKV>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_RESID: epi_unit<EPI_RESID>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_SWIGLU: epi_unit<EPI_SWIGLU>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        default: epi_unit<EPI_LMHEAD>(p, a, scr, m0, t0, ncols, quarter, lane); break;
+        case EPI_PLAIN: epi_whole<EPI_PLAIN>(p, a, scr, m0, t0, ncols, quarter, lane); break;
+        case EPI_QKV: epi_whole<EPI_QKV>(p, a, scr, m0, t0, ncols, quarter, lane); break;
+        case EPI_RESID: epi_whole<EPI_RESID>(p, a, scr, m0, t0, ncols, quarter, lane); break;
+        case EPI_SWIGLU: epi_whole<EPI_SWIGLU>(p, a, scr, m0, t0, ncols, quarter, lane); break;
+        default: epi_whole<EPI_LMHEAD>(p, a, scr, m0, t0, ncols, quarter, lane); break;
     }
 }
 
@@ -571,8 +613,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (elect_one()) {
-            uint32_t it = 0;
-            bool ok = true;
+            // (stage and k-block indices are carried along: a remainder costs this one thread more than its requests do)
+            int s = 0;
+            uint32_t ph = 1;   // parity of the use of stage s that the MMAs have to release; nothing to wait for in the first round
+            bool ok = true, first = true;
             GemmWork w;
             for (int i = 0; ok && gemm_work<KSPLIT>(g, cta, n_cta, i, w); ++i) {
                 const int n0 = w.tt * g.TN;
@@ -584,17 +628,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                 // whole ring are requested before waiting for the predecessor, whose output is only the
                 // token operand.
                 const int n_early = i == 0 ? min(nk, g.n_stages) : 0;
+                int kb = w.kb0 + rot;
                 for (int j = 0; j < n_early; ++j) {
-                    const int kb = w.kb0 + (j + rot) % nk;
                     uint8_t* a_s = smem + j * stage_bytes;
                     mbar_expect_tx(&full_bar[j], a_bytes + nbox * GEMM_BOX_BYTES);
                     bulk_load(a_s + w.mt_lo * GEMM_TILE_BYTES, wsrc + (size_t)kb * (2 * 128 * 64), a_bytes, &full_bar[j]);
+                    if (++kb == w.kb1) kb = w.kb0;
                 }
                 if (i == 0) pdl_wait();
-                for (int j = 0; j < nk; ++j, ++it) {
-                    const int kb = w.kb0 + (j + rot) % nk;
-                    const int s = it % g.n_stages;
-                    if (it >= (uint32_t)g.n_stages && !mbar_wait(&empty_bar[s], ((it / g.n_stages) - 1) & 1, g.status, limit)) {
+                kb = w.kb0 + rot;
+                for (int j = 0; j < nk; ++j) {
+                    if (!first && !mbar_wait(&empty_bar[s], ph, g.status, limit)) {
                         ok = false;
                         break;
                     }
@@ -606,6 +650,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     }
                     for (int b = 0; b < nbox; ++b)
                         tma_load_2d(b_s + b * GEMM_BOX_BYTES, &tmB, &full_bar[s], kb * GEMM_BK, n0 + b * GEMM_BOX_ROWS);
+                    if (++kb == w.kb1) kb = w.kb0;
+                    if (++s == g.n_stages) { s = 0; ph ^= 1; first = false; }
                 }
             }
         }
@@ -613,7 +659,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (elect_one()) {
-            uint32_t it = 0;
+            int s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             GemmWork w;
             for (int i = 0; ok && gemm_work<KSPLIT>(g, cta, n_cta, i, w); ++i) {
@@ -625,9 +672,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     tc_fence_after();
                 }
                 const int nk = w.kb1 - w.kb0;
-                for (int j = 0; j < nk; ++j, ++it) {
-                    const int s = it % g.n_stages;
-                    ok = mbar_wait(&full_bar[s], (it / g.n_stages) & 1, g.status, limit);
+                for (int j = 0; j < nk; ++j) {
+                    ok = mbar_wait(&full_bar[s], ph, g.status, limit);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t a_addr = smem_u32(smem + s * stage_bytes);
@@ -641,6 +687,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                             umma_bf16(tmem_base + mt * acc_stride, da + 2 * k, db + 2 * k, idesc, j > 0 || k > 0);
                         }
                     umma_commit(&empty_bar[s]);
+                    if (++s == g.n_stages) { s = 0; ph ^= 1; }
                 }
                 if (ok) umma_commit(accf_bar);
             }

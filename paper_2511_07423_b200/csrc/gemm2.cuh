@@ -140,8 +140,10 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     if (warp == 0) {
         // ------------------------------------------------------------ producer (one per CTA)
         if (elect_one()) {
-            uint32_t it = 0;
-            bool ok = true;
+            // (stage and k-block indices are carried along: a remainder costs this one thread more than its requests do)
+            int s = 0;
+            uint32_t ph = 1;   // parity of the use of stage s that the MMAs have to release; nothing to wait for in the first round
+            bool ok = true, first = true;
             Gemm2Work w;
             for (int i = 0; ok && gemm2_work(g, cl, n_cl, i, w); ++i) {
                 const int n0 = w.tt * g.TN;
@@ -155,17 +157,17 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 // the weights never depend on an earlier kernel: the first item's ring is requested
                 // before waiting for the predecessor, whose output is only the token operand
                 const int n_early = i == 0 ? min(nk, g.n_stages) : 0;
+                int kb = w.kb0 + rot;
                 for (int j = 0; j < n_early; ++j) {
-                    const int kb = w.kb0 + (j + rot) % nk;
                     if (rank == 0) mbar_expect_tx(&full_bar[j], 2 * my_bytes);
                     tma_load_2d_pair(smem + j * stage_bytes, &tmA, mapa_rank(smem_u32(&full_bar[j]), 0), 0,
                                      ((pair * g.num_kb + kb) * 2 + (DUO ? (int)rank : 0)) * 128);
+                    if (++kb == w.kb1) kb = w.kb0;
                 }
                 if (i == 0) pdl_wait();
-                for (int j = 0; j < nk; ++j, ++it) {
-                    const int kb = w.kb0 + (j + rot) % nk;
-                    const int s = it % g.n_stages;
-                    if (it >= (uint32_t)g.n_stages && !mbar_wait(&empty_bar[s], ((it / g.n_stages) - 1) & 1, g.status, limit)) {
+                kb = w.kb0 + rot;
+                for (int j = 0; j < nk; ++j) {
+                    if (!first && !mbar_wait(&empty_bar[s], ph, g.status, limit)) {
                         ok = false;
                         break;
                     }
@@ -178,6 +180,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     }
                     for (int b = 0; b < nbox; ++b)
                         tma_load_2d_pair(b_s + b * GEMM_BOX_BYTES, &tmB, fb, kb * GEMM_BK, n0 + (int)rank * half + b * GEMM_BOX_ROWS);
+                    if (++kb == w.kb1) kb = w.kb0;
+                    if (++s == g.n_stages) { s = 0; ph ^= 1; first = false; }
                 }
             }
         }
@@ -185,7 +189,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (rank 0 only)
         if (rank == 0 && elect_one()) {
-            uint32_t it = 0;
+            int s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             Gemm2Work w;
             for (int i = 0; ok && gemm2_work(g, cl, n_cl, i, w); ++i) {
@@ -197,9 +202,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     tc_fence_after();
                 }
                 const int nk = w.kb1 - w.kb0;
-                for (int j = 0; j < nk; ++j, ++it) {
-                    const int s = it % g.n_stages;
-                    ok = mbar_wait(&full_bar[s], (it / g.n_stages) & 1, g.status, limit);
+                for (int j = 0; j < nk; ++j) {
+                    ok = mbar_wait(&full_bar[s], ph, g.status, limit);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t a_addr = smem_u32(smem + s * stage_bytes);
@@ -218,6 +222,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                         }
                     }
                     umma_commit_pair(&empty_bar[s]);
+                    if (++s == g.n_stages) { s = 0; ph ^= 1; }
                 }
                 if (ok) umma_commit_pair(accf_bar);
             }

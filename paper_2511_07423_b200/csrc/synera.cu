@@ -16,6 +16,7 @@
 #include "attention2.cuh"
 #include "gemm.cuh"
 #include "gemm2.cuh"
+#include "gemm_thin.cuh"
 #include "sampling.cuh"
 
 using namespace syn;
@@ -67,9 +68,9 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return note_cuda(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
 }
 
-// The same for a kernel whose CTAs form clusters of two.
+// The same for a kernel whose CTAs form clusters of `cluster` neighbours.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl_pairs(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+static cudaError_t launch_pdl_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -78,7 +79,7 @@ static cudaError_t launch_pdl_pairs(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return note_cuda(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
@@ -202,6 +203,17 @@ static int make_wmaps(const void* packed, int packed_rows, int K, WMaps* out) {
     return SYN_OK;
 }
 
+// The token operand of a projection, [tokens][K] half precision, as boxes of 32 rows (the kernels of gemm.cuh and
+// gemm2.cuh) and, for the thin kernel, of 16, 32, ... THIN_MAX_TN rows: one box is a whole token tile.
+struct XMaps {
+    CUtensorMap box, thin[THIN_MAX_TN / 16];
+};
+static int make_xmaps(XMaps* out, const void* base, uint64_t rows, uint64_t K) {
+    int r = make_map_2d(&out->box, base, rows, K, K, GEMM_BOX_ROWS);
+    for (int i = 0; i < THIN_MAX_TN / 16 && !r; ++i) r = make_map_2d(&out->thin[i], base, rows, K, K, 16 * (i + 1));
+    return r;
+}
+
 struct syn_model {
     syn_model_desc desc;
     int f_pad, n_sm, gu_rows, qkv_rows, v_rows;
@@ -222,7 +234,8 @@ struct syn_model {
     unsigned long long* best = nullptr;
     int *acc_dev = nullptr, *corr_dev = nullptr;
     int b_cap = 0;
-    CUtensorMap tm_xn, tm_attn, tm_act, tm_q, tm_q4;
+    XMaps tm_xn, tm_attn, tm_act;
+    CUtensorMap tm_q, tm_q4;
     float* fix_part = nullptr;      // stored accumulators of K-split remainder tiles (one slot per SM)
     int* fix_flag = nullptr;        // their arrival / release counters, [GEMM_FLAG_INTS * n_sm], zero between launches
     float* part_o = nullptr;
@@ -323,9 +336,9 @@ static int ensure_workspace(syn_model* m, int T, int B, int n_parts) {
         CU_OK(cudaMemset(m->act, 0, (size_t)cap * m->f_pad * 2));
         m->t_cap = cap;
         int r;
-        if ((r = make_map_2d(&m->tm_xn, m->xn, cap, c.d_model, c.d_model, GEMM_BOX_ROWS))) return r;
-        if ((r = make_map_2d(&m->tm_attn, m->attn, cap, q_dim, q_dim, GEMM_BOX_ROWS))) return r;
-        if ((r = make_map_2d(&m->tm_act, m->act, cap, m->f_pad, m->f_pad, GEMM_BOX_ROWS))) return r;
+        if ((r = make_xmaps(&m->tm_xn, m->xn, cap, c.d_model))) return r;
+        if ((r = make_xmaps(&m->tm_attn, m->attn, cap, q_dim))) return r;
+        if ((r = make_xmaps(&m->tm_act, m->act, cap, m->f_pad))) return r;
         // Q tile of the attention kernel: [token][128-byte line][64]; box = min(16, 64/G) tokens x (G * hd/64) lines
         const uint32_t G = c.n_q_heads / c.n_kv_heads, halves = c.head_dim / 64;
         const uint32_t box_tokens = std::min(16u, 64u / G);
@@ -372,6 +385,29 @@ static int ensure_workspace(syn_model* m, int T, int B, int n_parts) {
         m->part_cap = cap;
     }
     return SYN_OK;
+}
+
+// Dynamic shared memory of every kernel that needs more than the default, and the same carveout for all kernels of
+// the step: an SM has to drain before it can change its carveout, which would keep neighbours apart.
+template <typename K>
+static cudaError_t kernel_smem(K kernel, int bytes) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && bytes > 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
+static cudaError_t set_kernel_attributes() {
+    const cudaError_t all[] = {
+        kernel_smem(gemm_kernel<GEMM_WAVES>, GEMM_SMEM_MAX), kernel_smem(gemm_kernel<GEMM_KSPLIT>, GEMM_SMEM_MAX),
+        kernel_smem(gemm_kernel<GEMM_RSPLIT>, GEMM_SMEM_MAX), kernel_smem(gemm2_kernel<false>, GEMM_SMEM_MAX),
+        kernel_smem(gemm2_kernel<true>, GEMM_SMEM_MAX), kernel_smem(thin_kernel<EPI_PLAIN>, THIN_SMEM_MAX),
+        kernel_smem(thin_kernel<EPI_QKV>, THIN_SMEM_MAX), kernel_smem(thin_kernel<EPI_RESID>, THIN_SMEM_MAX),
+        kernel_smem(thin_kernel<EPI_SWIGLU>, THIN_SMEM_MAX), kernel_smem(thin_kernel<EPI_LMHEAD>, THIN_SMEM_MAX),
+        kernel_smem(attn_kernel<128>, AttnSmem<128>::TOTAL), kernel_smem(attn_kernel<64>, AttnSmem<64>::TOTAL),
+        kernel_smem(attn2_kernel<128>, Attn2Smem<128>::TOTAL), kernel_smem(attn2_kernel<64>, Attn2Smem<64>::TOTAL),
+        kernel_smem(prep_kernel, 0), kernel_smem(verify_kernel, 0), kernel_smem(topk_rows_kernel, 0), kernel_smem(sample_verify_kernel, 0)};
+    for (cudaError_t e : all)
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 // ------------------------------------------------------------------------------------------ model
@@ -562,15 +598,7 @@ static int syn_model_load_impl(const syn_model_desc* desc, const syn_weights* w,
     CU_M(cudaMemcpy(m->inv_freq, inv.data(), inv.size() * 8, cudaMemcpyHostToDevice));
     CU_M(cudaMalloc(&m->status_dev, 4));
     CU_M(cudaMemset(m->status_dev, 0, 4));
-    CU_M(cudaFuncSetAttribute(gemm_kernel<GEMM_WAVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_M(cudaFuncSetAttribute(gemm_kernel<GEMM_KSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_M(cudaFuncSetAttribute(gemm_kernel<GEMM_RSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_M(cudaFuncSetAttribute(gemm2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_M(cudaFuncSetAttribute(gemm2_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_M(cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<128>::TOTAL));
-    CU_M(cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::TOTAL));
-    CU_M(cudaFuncSetAttribute(attn2_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Attn2Smem<128>::TOTAL));
-    CU_M(cudaFuncSetAttribute(attn2_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Attn2Smem<64>::TOTAL));
+    CU_M(set_kernel_attributes());
     CU_M(cudaDeviceSynchronize());
     *out = m;
     return SYN_OK;
@@ -1152,13 +1180,12 @@ static int gemm_plan(int T, int packed_rows, int K, int n_sm, int mode, bool may
 // One projection with the epilogue `ep`; `plan_mode` = the epilogue its schedule is made for (the
 // same, except in the test hook, which runs any schedule with the plain store epilogue).
 static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, int packed_rows, int K,
-                       const CUtensorMap& tmB, EpiParams ep, cudaStream_t st, float* fix_part, int* fix_flag,
-                       int plan_mode = -1) {
+                       const CUtensorMap& tmB, const EpiParams& ep, cudaStream_t st, float* fix_part, int* fix_flag,
+                       int plan_mode) {
     ProfScope prof(cls >= 0 ? prof_m : nullptr, cls, st);
     GemmParams g;
     memset(&g, 0, sizeof(g));
     int n_cta = 0;
-    if (plan_mode < 0) plan_mode = ep.mode;
     if (!fix_part || !fix_flag) return SYN_E_INVALID_ARG;
     const int pr = gemm_plan(ep.T, packed_rows, K, n_sm, plan_mode, plan_mode != EPI_RESID, g, n_cta);
     if (pr) return pr;
@@ -1234,25 +1261,92 @@ static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int for
     return kind;
 }
 
+constexpr int THIN_MAX_TOKENS = 512;
+
+// Launch shape of a projection on the thin kernel (gemm_thin.cuh): at most one CTA per SM where K is shared, so that the
+// other half of every SM is free for the next kernel; at least two k-blocks each.
+static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
+    memset(&g, 0, sizeof(g));
+    g.num_kb = (K + 63) / 64;
+    g.n_tiles = (packed_rows + 127) / 128;
+    g.n_tt = (T + THIN_MAX_TN - 1) / THIN_MAX_TN;
+    g.TN = ((T + g.n_tt - 1) / g.n_tt + 15) / 16 * 16;
+    g.n_tt = (T + g.TN - 1) / g.TN;
+    g.splits = std::max(1, std::min(std::min(THIN_MAX_SPLITS, n_sm / (g.n_tiles * g.n_tt)), g.num_kb / 2));
+    const int recv = g.splits > 1 ? thin_recv_bytes(g.TN, g.splits) : 0;
+    g.recv_own = recv > 0 && recv <= THIN_RECV_OWN_MAX;
+    g.n_stages = thin_stages(g.TN, g.recv_own ? recv : 0);
+}
+
+// Whether a projection takes the thin kernel.  Measured against the other kernels, event times of a class in us, other >
+// thin, at 8 layers and fewer of the three model widths:
+//   one token tile (128 tokens and fewer): 1B shape o 20.8 > 14.3 and down 26.8 > 18.5 at 40 tokens, 8B shape qkv 27.4 > 20.9,
+//   o 28.2 > 16.9, gate/up 55.2 > 48.2 (128 tokens), 32B shape o 31.0 > 20.5; not a projection with so many tiles that the
+//   launch is many rounds of CTAs (lm_head of the 8B shape 182 < 188 at 80 tokens), unless the tokens are very few (173 > 170 at 40);
+//   several token tiles read the weights once each, which only pays while every CTA has little work: 1B shape at 256 tokens
+//   qkv 31.1 > 20.9 (16 k-blocks a CTA), gate/up 29.1 > 28.1 (32), down 36.9 > 25.0 (32), 8B shape o 35.1 > 27.0 (32); but
+//   8B shape qkv 31.1 < 36.3 (176 tokens, 64 k-blocks), down 46 < 54 (112), 1B gate/up 35 < 41 at 320 tokens (384 CTAs).
+static bool thin_takes(int T, int packed_rows, int K, int n_sm, int mode) {
+    if (T > THIN_MAX_TOKENS) return false;
+    ThinParams g;
+    thin_plan(T, packed_rows, K, n_sm, g);
+    const int ctas = g.n_tiles * g.n_tt * g.splits, nk = (g.num_kb + g.splits - 1) / g.splits;
+    if (g.n_tt == 1) return T <= 64 || ctas <= 3 * n_sm;
+    return mode == EPI_RESID ? ctas <= n_sm && nk <= 64 : ctas <= 2 * n_sm && nk <= 32;
+}
+
+static int thin_smem(const ThinParams& g) {
+    return thin_fixed_smem(g.TN) + g.n_stages * thin_stage_bytes(g.TN) + (g.recv_own ? thin_recv_bytes(g.TN, g.splits) : 0);
+}
+
+template <int MODE>
+static cudaError_t launch_thin_mode(const ThinParams& g, const XMaps& xm, const EpiParams& ep, cudaStream_t st) {
+    return launch_pdl_clusters(thin_kernel<MODE>, dim3(g.n_tiles * g.n_tt * g.splits), dim3(THIN_THREADS), thin_smem(g), st, g.splits,
+                               xm.thin[g.TN / 16 - 1], g, ep);
+}
+
+static int launch_thin(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, int packed_rows, int K, const XMaps& xm,
+                       const EpiParams& ep, cudaStream_t st) {
+    ProfScope prof(cls >= 0 ? prof_m : nullptr, cls, st);
+    ThinParams g;
+    thin_plan(ep.T, packed_rows, K, n_sm, g);
+    g.w = w_packed; g.status = status; g.spin_limit = g_spin_limit;
+    cudaError_t e;
+    switch (ep.mode) {
+        case EPI_QKV: e = launch_thin_mode<EPI_QKV>(g, xm, ep, st); break;
+        case EPI_RESID: e = launch_thin_mode<EPI_RESID>(g, xm, ep, st); break;
+        case EPI_SWIGLU: e = launch_thin_mode<EPI_SWIGLU>(g, xm, ep, st); break;
+        case EPI_LMHEAD: e = launch_thin_mode<EPI_LMHEAD>(g, xm, ep, st); break;
+        default: e = launch_thin_mode<EPI_PLAIN>(g, xm, ep, st); break;
+    }
+    return e == cudaSuccess ? SYN_OK : SYN_E_CUDA;
+}
+
+// What a caller may ask of launch_proj instead of the kernel the shape calls for (test hook).
+enum { PROJ_AUTO = 0, PROJ_QUAD = PAIR_QUAD, PROJ_DUO = PAIR_DUO, PROJ_THIN, PROJ_NOT_THIN };
+
 // One projection with the epilogue `ep` on whichever kernel its shape calls for.  `plan_mode` = the
-// epilogue the schedule is made for (the same, except in the test hook); `force_pair`: test hook.
+// epilogue the schedule is made for (the same, except in the test hook); `force`: test hook.
 static int launch_proj(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, const WMaps* wm, int packed_rows,
-                       int K, const CUtensorMap& tmB, EpiParams ep, cudaStream_t st, float* fix_part, int* fix_flag,
-                       int plan_mode = -1, int force_pair = PAIR_NONE) {
+                       int K, const XMaps& xm, const EpiParams& ep, cudaStream_t st, float* fix_part, int* fix_flag,
+                       int plan_mode = -1, int force = PROJ_AUTO) {
     if (plan_mode < 0) plan_mode = ep.mode;
+    if (force == PROJ_THIN || (force == PROJ_AUTO && g_schedule != 1 && thin_takes(ep.T, packed_rows, K, n_sm, plan_mode)))
+        return launch_thin(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm, ep, st);
+    const int force_pair = force == PROJ_QUAD || force == PROJ_DUO ? force : PAIR_NONE;
     Gemm2Params g2;
     int n_cl = 0;
     const int kind = (wm && (g_schedule != 1 || force_pair != PAIR_NONE)) ? gemm2_plan(ep.T, packed_rows, K, n_sm, plan_mode, force_pair, g2, n_cl)
                                                                             : PAIR_NONE;
-    if (kind == PAIR_NONE) return launch_gemm(prof_m, cls, n_sm, status, w_packed, packed_rows, K, tmB, ep, st, fix_part, fix_flag, plan_mode);
+    if (kind == PAIR_NONE) return launch_gemm(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm.box, ep, st, fix_part, fix_flag, plan_mode);
     if (!fix_part || !fix_flag) return SYN_E_INVALID_ARG;
     ProfScope prof(cls >= 0 ? prof_m : nullptr, cls, st);
     g2.status = status; g2.spin_limit = g_spin_limit;
     g2.fix_part = fix_part; g2.fix_flag = fix_flag;
     const bool duo = kind == PAIR_DUO;
     const int smem = gemm_fixed_smem(g2.TN) + g2.n_stages * gemm2_stage_bytes(g2.TN, duo);
-    const cudaError_t le = duo ? launch_pdl_pairs(gemm2_kernel<true>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, wm->duo, tmB, g2, ep)
-                               : launch_pdl_pairs(gemm2_kernel<false>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, wm->quad, tmB, g2, ep);
+    const cudaError_t le = duo ? launch_pdl_clusters(gemm2_kernel<true>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->duo, xm.box, g2, ep)
+                               : launch_pdl_clusters(gemm2_kernel<false>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->quad, xm.box, g2, ep);
     return le == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
@@ -1660,11 +1754,7 @@ static int linear_ctx_init() {
     CU_OK(cudaGetDeviceProperties(&prop, dev));
     if (prop.major != 10) return SYN_E_ARCH;
     g_lin.n_sm = prop.multiProcessorCount;
-    CU_OK(cudaFuncSetAttribute(gemm_kernel<GEMM_WAVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_OK(cudaFuncSetAttribute(gemm_kernel<GEMM_KSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_OK(cudaFuncSetAttribute(gemm_kernel<GEMM_RSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_OK(cudaFuncSetAttribute(gemm2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
-    CU_OK(cudaFuncSetAttribute(gemm2_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX));
+    CU_OK(set_kernel_attributes());
     CU_OK(cudaMalloc(&g_lin.fix_part, (size_t)g_lin.n_sm * GEMM_FIX_SLOT_BYTES));
     CU_OK(cudaMalloc(&g_lin.fix_flag, (size_t)GEMM_FLAG_INTS * g_lin.n_sm * 4));
     CU_OK(cudaMemset(g_lin.fix_flag, 0, (size_t)GEMM_FLAG_INTS * g_lin.n_sm * 4));
@@ -1684,7 +1774,7 @@ extern "C" int syn_op_linear_reset(void) {
 
 extern "C" int syn_op_linear_as(const void* x, const void* w, float* y, int32_t T, int32_t N, int32_t K, int32_t schedule_as,
                                 void* cuda_stream) {
-    if (!x || !w || !y || T <= 0 || N <= 0 || K <= 0 || K % 8 != 0 || schedule_as < EPI_PLAIN || schedule_as > EPI_LMHEAD + 4)
+    if (!x || !w || !y || T <= 0 || N <= 0 || K <= 0 || K % 8 != 0 || schedule_as < EPI_PLAIN || schedule_as > EPI_LMHEAD + 5)
         return SYN_E_INVALID_ARG;
     int r = load_driver_entry();
     if (r) return r;
@@ -1703,16 +1793,16 @@ extern "C" int syn_op_linear_as(const void* x, const void* w, float* y, int32_t 
         g_lin.packed_src = w; g_lin.packed_n = N; g_lin.packed_k = K;
         if ((r = make_wmaps(g_lin.packed, n_mt * 128, K, &g_lin.wm))) return r;
     }
-    CUtensorMap tmB;
-    if ((r = make_map_2d(&tmB, x, T, K, K, GEMM_BOX_ROWS))) return r;
+    XMaps xm;
+    if ((r = make_xmaps(&xm, x, T, K))) return r;
     EpiParams e;
     memset(&e, 0, sizeof(e));
     e.mode = EPI_PLAIN; e.T = T; e.N = N; e.y = y; e.ldy = N;
-    // 0..4: the schedule the step would take for that epilogue; 5, 6: CTA pairs with QUAD / DUO items; 7, 8: the
-    // same as residual projections (K shared between clusters where the shape allows it)
-    const int force = schedule_as <= EPI_LMHEAD ? PAIR_NONE : (schedule_as == 5 || schedule_as == 7 ? PAIR_QUAD : PAIR_DUO);
-    const int plan_mode = schedule_as <= EPI_LMHEAD ? schedule_as : (schedule_as >= 7 ? EPI_RESID : EPI_PLAIN);
-    r = launch_proj(nullptr, -1, g_lin.n_sm, g_lin.status, g_lin.packed, &g_lin.wm, (N + 127) / 128 * 128, K, tmB, e, st, g_lin.fix_part,
+    // 0..4: the one-CTA or CTA-pair schedule for that epilogue; 5, 6: CTA pairs with QUAD / DUO items; 7, 8: the same as
+    // residual projections (K shared between clusters where the shape allows it); 9: the thin kernel
+    const int force = schedule_as <= EPI_LMHEAD ? PROJ_NOT_THIN : (schedule_as == 9 ? PROJ_THIN : (schedule_as == 5 || schedule_as == 7 ? PROJ_QUAD : PROJ_DUO));
+    const int plan_mode = schedule_as <= EPI_LMHEAD ? schedule_as : (schedule_as == 7 || schedule_as == 8 ? EPI_RESID : EPI_PLAIN);
+    r = launch_proj(nullptr, -1, g_lin.n_sm, g_lin.status, g_lin.packed, &g_lin.wm, (N + 127) / 128 * 128, K, xm, e, st, g_lin.fix_part,
                     g_lin.fix_flag, plan_mode, force);
     if (r) return r;
     CU_OK(cudaStreamSynchronize(st));
@@ -1976,6 +2066,16 @@ extern "C" int syn_gemm2_work_host(int32_t T, int32_t N, int32_t K, int32_t n_sm
     const int v[SYN_GEMM2_WORK_FIELDS] = {w.grp, w.tt, w.kb0, w.kb1, w.tile, w.split, w.nsplit, w.first_cl, w.counter};
     memcpy(out, v, sizeof(v));
     return 1;
+}
+
+extern "C" int syn_thin_plan_host(int32_t T, int32_t N, int32_t K, int32_t n_sm, int32_t epilogue, int32_t* out) {
+    if (T <= 0 || N <= 0 || K <= 0 || n_sm <= 0 || n_sm > 65535 || epilogue < EPI_PLAIN || epilogue > EPI_LMHEAD || !out) return SYN_E_INVALID_ARG;
+    ThinParams g;
+    thin_plan(T, (N + 127) / 128 * 128, K, n_sm, g);
+    const int v[SYN_THIN_PLAN_FIELDS] = {thin_takes(T, (N + 127) / 128 * 128, K, n_sm, epilogue) ? 1 : 0, g.n_tiles, g.n_tt, g.TN, g.num_kb, g.splits, g.n_stages,
+                                         g.n_stages * thin_stage_bytes(g.TN) - (g.splits > 1 && !g.recv_own ? thin_recv_bytes(g.TN, g.splits) : 0) - THIN_SCR_BYTES};
+    memcpy(out, v, sizeof(v));
+    return SYN_OK;
 }
 
 extern "C" const char* syn_last_cuda_error(void) { return g_last_cuda_error; }
