@@ -110,8 +110,8 @@ void syn_kv_free(syn_kv *kv);
  * positions pos0 .. pos0+n_pos-1, e.g. a prefix computed on another server.  k, v: DEVICE bf16
  * [n_pos][n_kv_heads][head_dim] (the pool itself holds half precision: import converts, exactly for
  * magnitudes in [2^-17, 65504], export rounds back to bf16); page_table: HOST int32, at least ceil((pos0+n_pos)/page_size)
- * entries.  Blocking: the call allocates a small device buffer for the slot list, synchronises
- * `cuda_stream` and returns when the copy is done.
+ * entries.  Blocking: the call synchronises `cuda_stream` and returns when the copy is done; it allocates
+ * nothing.
  * syn_kv_export is the inverse (reads the same positions into k, v).
  * Errors: SYN_E_INVALID_ARG, SYN_E_PAGE_OOB, SYN_E_CUDA. */
 int syn_kv_import(syn_kv *kv, uint32_t layer, const int32_t *page_table, int32_t pos0, int32_t n_pos,

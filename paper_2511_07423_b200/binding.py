@@ -104,8 +104,9 @@ def _i32(t) -> torch.Tensor:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> C.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is None:   # with the index given, torch does not look for it among the visible devices (4 us of a 10 us call)
+        stream = torch.cuda.current_stream(torch.cuda.current_device())
+    return C.c_void_p(stream.cuda_stream)
 
 
 class Model:

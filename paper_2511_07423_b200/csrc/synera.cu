@@ -133,22 +133,64 @@ __global__ void verify_kernel(const unsigned long long* __restrict__ best, const
     correction[i] = (int)(0xFFFFFFFFu - (uint32_t)(best[b + u - 1 + a] & 0xFFFFFFFFull));
 }
 
-// Copy K/V of logical positions between a dense bf16 [n_pos][Hkv][hd] buffer and the paged pool (half precision).
-__global__ void kv_copy_kernel(op16* pool_layer, const int* __restrict__ slots, bf16* k, bf16* v, int n_kv_heads, int hd,
-                               int page_size, int to_pool) {
-    const int i = blockIdx.x;
-    const int s = slots[i], page = s / page_size, row = s % page_size;
-    for (int e = threadIdx.x; e < n_kv_heads * hd; e += blockDim.x) {
-        const int h = e / hd, dd = e % hd;
-        const size_t ok = ((((size_t)page * n_kv_heads + h) * 2 + 0) * page_size + row) * hd + dd;
-        const size_t ov = ok + (size_t)page_size * hd;
-        const size_t oi = (size_t)i * n_kv_heads * hd + e;
+// Copy K/V of logical positions between a dense bf16 [n_pos][Hkv][hd] buffer and the paged pool (half precision).  The
+// page ids travel as a launch parameter, so that a transfer is one launch: no device buffer, no copy, no memory that
+// callers on several streams or threads would share.  A thread moves VEC elements of K and of V (8: 16 bytes each
+// way) of KV_COPY_POS positions, all loads before the first store.  A blocking call of 2 600 positions of the 8B shape
+// (10.6 MB each way) takes 20 us, of 100 positions 16: launch and synchronisation bound it (59 us when the slots went
+// through a device buffer of the call's own; 1 or 4 positions a thread measured the same).
+constexpr int KV_COPY_POS = 2;
+template <int CAP>
+struct KvPages {
+    int id[CAP];   // pages of the positions [16 * first page, ...)
+};
+template <int CAP, int VEC>
+__global__ void __launch_bounds__(256)
+kv_copy_kernel(op16* pool_layer, const __grid_constant__ KvPages<CAP> pages, int pos0, int n_pos, bf16* k, bf16* v, int kv_dim, int hd_log,
+               int to_pool) {
+    const int per_pos = kv_dim / VEC;   // threads of a position
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i0 = t / per_pos * KV_COPY_POS, e = (t % per_pos) * VEC;
+    if (i0 >= n_pos) return;
+    struct alignas(2 * VEC) Src { bf16 x[VEC]; };
+    struct alignas(2 * VEC) Dst { op16 x[VEC]; };
+    Src sk[KV_COPY_POS], sv[KV_COPY_POS];
+    Dst dk[KV_COPY_POS], dv[KV_COPY_POS];
+    const int hd = 1 << hd_log, head = e >> hd_log;
+    op16* at[KV_COPY_POS];
+#pragma unroll
+    for (int i = 0; i < KV_COPY_POS; ++i) {
+        const int ii = min(i0 + i, n_pos - 1), row = (pos0 & 15) + ii;
+        at[i] = pool_layer + ((size_t)pages.id[row >> 4] * kv_dim * 2 + (size_t)head * 2 * hd) * 16 + (size_t)(row & 15) * hd + (e & (hd - 1));
+        const size_t oi = (size_t)ii * kv_dim + e;
         if (to_pool) {
-            pool_layer[ok] = to_op(__bfloat162float(k[oi]));
-            pool_layer[ov] = to_op(__bfloat162float(v[oi]));
+            sk[i] = *reinterpret_cast<const Src*>(k + oi);
+            sv[i] = *reinterpret_cast<const Src*>(v + oi);
         } else {
-            k[oi] = __float2bfloat16(__half2float(pool_layer[ok]));
-            v[oi] = __float2bfloat16(__half2float(pool_layer[ov]));
+            dk[i] = *reinterpret_cast<const Dst*>(at[i]);
+            dv[i] = *reinterpret_cast<const Dst*>(at[i] + 16 * hd);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < KV_COPY_POS; ++i) {
+        if (i0 + i >= n_pos) break;
+        const size_t oi = (size_t)(i0 + i) * kv_dim + e;
+        if (to_pool) {
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) {
+                dk[i].x[c] = to_op(__bfloat162float(sk[i].x[c]));
+                dv[i].x[c] = to_op(__bfloat162float(sv[i].x[c]));
+            }
+            *reinterpret_cast<Dst*>(at[i]) = dk[i];
+            *reinterpret_cast<Dst*>(at[i] + 16 * hd) = dv[i];
+        } else {
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) {
+                sk[i].x[c] = __float2bfloat16(__half2float(dk[i].x[c]));
+                sv[i].x[c] = __float2bfloat16(__half2float(dv[i].x[c]));
+            }
+            *reinterpret_cast<Src*>(k + oi) = sk[i];
+            *reinterpret_cast<Src*>(v + oi) = sv[i];
         }
     }
 }
@@ -666,31 +708,47 @@ extern "C" int syn_kv_alloc(syn_model* m, uint32_t n_pages, uint32_t page_size, 
     return SYN_OK;
 }
 
+constexpr int KV_COPY_PAGES_SMALL = 192, KV_COPY_PAGES = 960;   // page ids a launch carries (parameters of 0.8 and 3.8 KB)
+
+template <int CAP, int VEC>
+static int kv_copy_launch(syn_kv* kv, uint32_t layer, const int32_t* pages, int n_pages, int pos0, int n_pos, bf16* k, bf16* v,
+                          cudaStream_t st, int to_pool) {
+    const syn_model_desc& c = kv->model->desc;
+    KvPages<CAP> pg;
+    memcpy(pg.id, pages, (size_t)n_pages * 4);
+    const int kv_dim = (int)(c.n_kv_heads * c.head_dim);
+    const int64_t threads = (int64_t)((n_pos + KV_COPY_POS - 1) / KV_COPY_POS) * (kv_dim / VEC);
+    kv_copy_kernel<CAP, VEC><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(kv->pool + kv->layer_elems * layer, pg, pos0, n_pos, k, v, kv_dim,
+                                                                                 c.head_dim == 128 ? 7 : 6, to_pool);
+    return launch_ok() ? SYN_OK : SYN_E_CUDA;
+}
+
 static int kv_copy(syn_kv* kv, uint32_t layer, const int32_t* page_table, int32_t pos0, int32_t n_pos, void* k, void* v,
                    void* stream, int to_pool) {
     if (!kv || !page_table || !k || !v || pos0 < 0 || n_pos <= 0 || layer >= kv->model->desc.n_layers)
         return SYN_E_INVALID_ARG;
-    const int P = (int)kv->page_size;
-    std::vector<int> slots(n_pos);
-    for (int i = 0; i < n_pos; ++i) {
-        const int p = pos0 + i, page = page_table[p / P];
-        if (page < 0 || (uint32_t)page >= kv->n_pages) return SYN_E_PAGE_OOB;
-        slots[i] = page * P + p % P;
-    }
-    int* d_slots = nullptr;
-    CU_OK(cudaMalloc(&d_slots, (size_t)n_pos * 4));
+    const int P = (int)kv->page_size, first = pos0 / P, last = (int)(((int64_t)pos0 + n_pos - 1) / P);
+    for (int i = first; i <= last; ++i)
+        if (page_table[i] < 0 || (uint32_t)page_table[i] >= kv->n_pages) return SYN_E_PAGE_OOB;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemcpyAsync(d_slots, slots.data(), (size_t)n_pos * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) {
-        const syn_model_desc& c = kv->model->desc;
-        kv_copy_kernel<<<n_pos, 128, 0, st>>>(kv->pool + kv->layer_elems * layer, d_slots, (bf16*)k, (bf16*)v,
-                                              c.n_kv_heads, c.head_dim, P, to_pool);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // launches of at most KV_COPY_PAGES pages; short transfers carry the smaller parameter
+    const size_t kv_dim = (size_t)kv->model->desc.n_kv_heads * kv->model->desc.head_dim;
+    for (int64_t done = 0; done < n_pos;) {
+        const int at = (int)(pos0 + done), p0 = at / P;
+        const int n = (int)std::min<int64_t>(n_pos - done, (int64_t)KV_COPY_PAGES * P - at % P);
+        const int n_pg = (at % P + n + P - 1) / P;
+        bf16 *kk = (bf16*)k + (size_t)done * kv_dim, *vv = (bf16*)v + (size_t)done * kv_dim;
+        const bool vec = (((uintptr_t)kk | (uintptr_t)vv) & 15) == 0;
+        const int r = n_pg <= KV_COPY_PAGES_SMALL
+                          ? (vec ? kv_copy_launch<KV_COPY_PAGES_SMALL, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
+                                 : kv_copy_launch<KV_COPY_PAGES_SMALL, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool))
+                          : (vec ? kv_copy_launch<KV_COPY_PAGES, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
+                                 : kv_copy_launch<KV_COPY_PAGES, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool));
+        if (r) return r;
+        done += n;
     }
-    cudaFree(d_slots);
-    return e == cudaSuccess ? SYN_OK : SYN_E_CUDA;
+    CU_OK(cudaStreamSynchronize(st));
+    return SYN_OK;
 }
 
 static int syn_kv_import_impl(syn_kv* kv, uint32_t layer, const int32_t* page_table, int32_t pos0, int32_t n_pos,
