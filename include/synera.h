@@ -260,7 +260,8 @@ int syn_op_linear_reset(void);
  * syn_debug_set_attention: which attention kernel the plans made AFTERWARDS are laid out for (a plan
  * keeps its kernel): 0 (default) the cheaper of the two for the batch by the planner's cost model, 1 the
  * warp-level-MMA kernel (row tiles of 64), 2 the tcgen05 kernel (row tiles of 128: a whole chunk of up to
- * 128 / G tokens is one work item per kv head).  Process-wide. */
+ * 128 / G tokens is one work item per kv head), 3 the warp-level-MMA kernel in CTAs of half an SM (row tiles of
+ * 64; few requests).  Process-wide. */
 int syn_debug_set_spin_limit(int64_t cycles);
 int syn_debug_linear_counter(int32_t index, int32_t value);
 int syn_debug_set_schedule(int32_t which);

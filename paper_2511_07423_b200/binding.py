@@ -592,7 +592,7 @@ def debug_set_schedule(which: int) -> None:
 
 
 def debug_set_attention(which: int) -> None:
-    """syn_debug_set_attention: 0 default, 1 warp-level-MMA kernel, 2 tcgen05 kernel; applies to plans made afterwards."""
+    """syn_debug_set_attention: 0 default, 1 warp-level-MMA kernel, 2 tcgen05 kernel, 3 half-SM kernel; applies to plans made afterwards."""
     _check(load_library().syn_debug_set_attention(C.c_int32(which)), "syn_debug_set_attention")
 
 

@@ -31,7 +31,8 @@ struct AttnItem {
     int q_pos0;     // position of the item's first query token (ctx + j0): row j sees keys <= q_pos0 + j
     int part;       // -1: sole item of its rows -> writes the output; else index of its partial
     int grp;        // merge group of a partial item (index into AttnParams::groups), else -1
-    int pad0, pad1, pad2;
+    int kv_safe;    // no chunk of the batch writes this request's keys before this position (multiple of 16)
+    int pad1, pad2;
 };
 
 // Row group whose keys were split over several items.
@@ -50,6 +51,7 @@ struct AttnParams {
     int row_cap;                // rows of an item's tile: 64 (128 in the tensor-memory kernel); row stride of the partials
     int layer_block0;           // 2 * layer * n_pages * Hkv: first (K|V) block of this layer in the pool map
     float scale_log2;           // log2(e) / sqrt(hd)
+    const op16* q;              // [T][q_dim] rotated queries (the thin kernel reads them itself, the others through a tensor map)
     op16* out;                  // [T][q_dim]
     float* part_o;              // [n_parts][row_cap][hd]
     float2* part_ml;            // [n_parts][row_cap] (max in log2 units, sum)

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "attention2.cuh"
+#include "attention_thin.cuh"
 #include "gemm.cuh"
 #include "gemm2.cuh"
 #include "gemm_thin.cuh"
@@ -29,8 +30,8 @@ constexpr int GEMM_MAX_SPLITS = 8;   // most CTAs that share one pair tile's K r
 static long long g_spin_limit = SYN_SPIN_LIMIT_CYCLES;
 // 0: every projection takes the kernel its shape calls for; 1: the one-CTA kernel always (syn_debug_set_schedule).
 static int g_schedule = 0;
-// Attention kernel: 0 = whichever the planner's cost model makes cheaper for the batch, 1 = warp-level MMAs
-// (64-row tiles), 2 = tcgen05 (128-row tiles).
+// Attention kernel: 0 = whichever the planner makes cheaper for the batch, 1 = warp-level MMAs (64-row tiles),
+// 2 = tcgen05 (128-row tiles), 3 = warp-level MMAs in CTAs of half an SM.
 static int g_attention = 0;
 
 // Name of the last CUDA error a call of this library met on this thread (for syn_last_cuda_error).
@@ -51,11 +52,11 @@ static inline bool launch_ok() { return note_cuda(cudaGetLastError()) == cudaSuc
         }                                        \
     } while (0)
 
-// Launch with programmatic stream serialization: the kernel may start while its predecessor in the
+// Launch, with `pdl` with programmatic stream serialization: the kernel may then start while its predecessor in the
 // stream still runs; every kernel of the step calls pdl_wait() before it touches anything an earlier
 // kernel produces or still reads.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+static cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, Args... args) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -64,8 +65,12 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return note_cuda(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    return launch(kernel, grid, block, smem, st, true, args...);
 }
 
 // The same for a kernel whose CTAs form clusters of `cluster` neighbours.
@@ -334,10 +339,14 @@ struct syn_kv {
     CUtensorMap tm_kv, tm_kv5;   // boxes of 32 rows (K and V of a page and head); of 16 rows (K or V) with both 64-dim halves
 };
 
+// The attention kernels a work list can be made for.
+enum { ATTN_WARP = 1, ATTN_TENSOR = 2, ATTN_THIN = 3 };
+static int attn_rows(int kind) { return kind == ATTN_TENSOR ? 128 : 64; }
+
 struct syn_plan {
     syn_step_stats stats;
     int n_req = 0, T = 0, max_pages = 0, n_items = 0, n_cta = 0, n_groups = 0, n_parts = 0;
-    int row_cap = 64;   // rows of an attention item's tile: which attention kernel the work list was made for
+    int attn = ATTN_WARP;   // which attention kernel the work list was made for
     // one device buffer and its pinned host mirror
     uint8_t *dev = nullptr, *host = nullptr;
     size_t cap = 0, used = 0;
@@ -446,6 +455,7 @@ static cudaError_t set_kernel_attributes() {
         kernel_smem(thin_kernel<EPI_SWIGLU>, THIN_SMEM_MAX), kernel_smem(thin_kernel<EPI_LMHEAD>, THIN_SMEM_MAX),
         kernel_smem(attn_kernel<128>, AttnSmem<128>::TOTAL), kernel_smem(attn_kernel<64>, AttnSmem<64>::TOTAL),
         kernel_smem(attn2_kernel<128>, Attn2Smem<128>::TOTAL), kernel_smem(attn2_kernel<64>, Attn2Smem<64>::TOTAL),
+        kernel_smem(attn_thin_kernel<128>, AttnThinSmem<128>::TOTAL), kernel_smem(attn_thin_kernel<64>, AttnThinSmem<64>::TOTAL),
         kernel_smem(prep_kernel, 0), kernel_smem(verify_kernel, 0), kernel_smem(topk_rows_kernel, 0), kernel_smem(sample_verify_kernel, 0)};
     for (cudaError_t e : all)
         if (e != cudaSuccess) return e;
@@ -773,7 +783,7 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Host-side result of planning one batch (no device involved).
 struct HostPlan {
-    int T = 0, n_cta = 0, n_parts = 0, row_cap = 64;
+    int T = 0, n_cta = 0, n_parts = 0, kind = ATTN_WARP;
     std::vector<int> pos, slot, cta_begin;
     std::vector<AttnItem> items;          // sorted by CTA
     std::vector<MergeGroup> groups;
@@ -781,10 +791,10 @@ struct HostPlan {
 };
 
 // Validate the batch, then build token positions, KV slots and the attention work list
-// (the "flatten" of paper Sec. 4.5).  Pure host code.
+// (the "flatten" of paper Sec. 4.5).  Pure host code.  thin_ctas: CTAs to plan for when the half-SM kernel is taken.
 static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_sm, int32_t n_req,
                         const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables,
-                        int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int attention, HostPlan& hp) {
+                        int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int attention, int thin_ctas, HostPlan& hp) {
     if (n_req <= 0 || !chunk_tokens || !chunk_offsets || !page_tables || !ctx_lens || max_pages <= 0 || n_sm <= 0)
         return SYN_E_INVALID_ARG;
     const int G = c.n_q_heads / c.n_kv_heads, Hkv = c.n_kv_heads;
@@ -837,43 +847,95 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
             if (std::adjacent_find(s2.begin(), s2.end()) != s2.end()) return SYN_E_PAGE_ALIAS;
         }
     }
-    // Attention work list: (request, kv head, token group, key range).  Cost of an item, in SM
-    // cycles: its 64-key stages times a per-stage time that grows with the number of 16-row query
-    // tiles (more tensor work per key byte), plus a fixed overhead per item; the figures are a
-    // least-squares fit to per-CTA durations measured on full batches.  A key range is split only
-    // when one unit alone would exceed a CTA's fair share: every split costs an fp32 partial and a
-    // merge.
-    const int n_cta_max = n_sm;
-    // Two kernels: the warp-level-MMA one (row tiles of 64: a stage costs more the more 16-row tiles the
-    // item has, and a chunk of more than 64 / G tokens is several items that each read the request's keys)
-    // and the tensor-memory one (row tiles of 128: the same time per stage whatever the number of rows,
-    // a larger fixed cost per item).  Unless one is asked for, the batch takes the cheaper by this model.
-    static const int STAGE_COST[5] = {0, 1040, 1200, 1500, 1540};
-    const int WIDE_STAGE_COST = 1450;
-    auto total_of = [&](bool w) {
-        const int tpg = w ? std::min(SYN_MAX_CHUNK, 128 / G) : std::min(16, 64 / G);
-        int64_t sum = 0;
+    // Attention work list: (request, kv head, token group, key range).  Cost of an item, in SM cycles: its blocks of
+    // 64 keys times a time per block that grows with the number of 16-row query tiles (more tensor work per key byte),
+    // plus a fixed overhead per item, plus one more if it covers only part of its unit's keys (an fp32 partial, a merge);
+    // least-squares fits to per-CTA durations measured on full batches.
+    // Three kernels.  Unless one is asked for: the tensor-memory one (row tiles of 128: the same time per block whatever
+    // the number of rows, a larger fixed cost per item; a chunk of more than 64 / G tokens is one item there and several
+    // items that each read the request's keys in the others) when it is cheaper by 3 %: it draws more power, and under the
+    // power cap a step that uses it runs its other kernels at a lower clock; at 544 tokens of the 8B shape the two are
+    // level and the step is not faster with it.  Otherwise the kernel of half-SM CTAs when there are no more units
+    // (request, token group, kv head) than SMs, so that keys have to be shared out in parts, the full-SM one else.
+    struct AttnCost { int block[5], item, part; };
+    static const AttnCost COST_WARP_128 = {{0, 1040, 1200, 1500, 1540}, 5500, 3000}, COST_WARP_64 = {{0, 765, 843, 967, 1062}, 3200, 3000},
+                          COST_TENSOR = {{0, 1450, 1450, 1450, 1450}, 8000, 4000}, COST_THIN_128 = {{0, 2300, 2400, 2600, 2900}, 3000, 4000},
+                          COST_THIN_64 = {{0, 1300, 1400, 1600, 1800}, 3000, 4000};
+    const AttnCost& cost_warp = c.head_dim == 128 ? COST_WARP_128 : COST_WARP_64;
+    auto group_of = [&](int kind) { return kind == ATTN_TENSOR ? std::min(SYN_MAX_CHUNK, 128 / G) : std::min(16, 64 / G); };
+    auto blocks_of = [](int L) { return (L + 63) / 64; };
+    auto total_of = [&](int kind, const AttnCost& ac, int64_t* units) {
+        const int tpg = group_of(kind);
+        int64_t sum = 0, n_units = 0;
         for (int i = 0; i < n_req; ++i) {
             const int n = chunk_offsets[i + 1] - chunk_offsets[i];
             for (int j0 = 0; j0 < n; j0 += tpg) {
                 const int nj = std::min(tpg, n - j0);
-                sum += ((int64_t)((ctx_lens[i] + j0 + nj + 63) / 64) * (w ? WIDE_STAGE_COST : STAGE_COST[(nj * G + 15) / 16]) + (w ? 8000 : 5500)) * Hkv;
+                sum += ((int64_t)blocks_of(ctx_lens[i] + j0 + nj) * ac.block[std::min(4, (nj * G + 15) / 16)] + ac.item) * Hkv;
+                n_units += Hkv;
             }
         }
+        if (units) *units = n_units;
         return sum;
     };
-    // (The tensor-memory kernel must win by 3 %: it draws more power, and under the power cap a step that uses it
-    // runs its other kernels at a lower clock; at 544 tokens of the 8B shape the two kernels are level and the step
-    // is not faster with it.)
-    const bool wide = attention == 2 || (attention == 0 && total_of(true) * 103 < total_of(false) * 100);
-    hp.row_cap = wide ? 128 : 64;
-    const int tok_per_group = wide ? std::min(SYN_MAX_CHUNK, 128 / G) : std::min(16, 64 / G);
-    const int ITEM_COST = wide ? 8000 : 5500, PART_COST = wide ? 4000 : 3000;
-    auto unit_cost = [&](int L, int nj) {
-        return (int64_t)((L + 63) / 64) * (wide ? WIDE_STAGE_COST : STAGE_COST[(nj * G + 15) / 16]) + ITEM_COST;
+    int64_t n_units = 0;
+    const int64_t total_warp = total_of(ATTN_WARP, cost_warp, &n_units);
+    const int kind = attention ? attention
+                               : (total_of(ATTN_TENSOR, COST_TENSOR, nullptr) * 103 < total_warp * 100 ? ATTN_TENSOR : (n_units <= n_sm ? ATTN_THIN : ATTN_WARP));
+    hp.kind = kind;
+    const AttnCost& ac = kind == ATTN_TENSOR ? COST_TENSOR : (kind == ATTN_THIN ? (c.head_dim == 128 ? COST_THIN_128 : COST_THIN_64) : cost_warp);
+    const int tok_per_group = group_of(kind);
+    const int n_cta_max = kind == ATTN_THIN ? thin_ctas : n_sm;
+    const int64_t total_cost = total_of(kind, ac, &n_units);
+    auto block_cost = [&](int nj) { return (int64_t)ac.block[std::min(4, (nj * G + 15) / 16)]; };
+    // Parts of a unit: as many as bring a part down to `limit`, each of at least min_blocks.
+    const int min_blocks = kind == ATTN_THIN ? 1 : 4, max_parts = kind == ATTN_THIN ? ATTN_THIN_MAX_PARTS : 64;
+    auto parts_of = [&](int L, int nj, int64_t limit) {
+        const int nb = blocks_of(L);
+        const int64_t bc = block_cost(nj);
+        if (nb * bc + ac.item <= limit) return 1;
+        const int64_t most = std::max<int64_t>(min_blocks, (limit - ac.item - ac.part) / bc);   // blocks of a part
+        return (int)std::min<int64_t>(std::min<int64_t>(max_parts, std::max(1, nb / min_blocks)), (nb + most - 1) / most);
     };
-    const int64_t total_cost = total_of(wide);
-    const int64_t share = std::max<int64_t>(8 * (wide ? WIDE_STAGE_COST : STAGE_COST[4]) + ITEM_COST, (total_cost + n_cta_max - 1) / n_cta_max);
+    // The limit.  Units that are many to a CTA need no parts, or only where one unit alone exceeds a CTA's fair share.  With
+    // few units to a CTA the longest parts decide: the smallest limit for which there is at most one part per CTA, if that is
+    // less than the fair share of whole units and their overheads would come to.
+    int64_t limit = std::max<int64_t>(8 * block_cost(64) + ac.item, (total_cost + n_cta_max - 1) / n_cta_max);
+    if (n_units <= n_cta_max) {
+        auto n_parts_at = [&](int64_t lim) {
+            int64_t n = 0;
+            for (int i = 0; i < n_req; ++i) {
+                const int nt = chunk_offsets[i + 1] - chunk_offsets[i];
+                for (int j0 = 0; j0 < nt; j0 += tok_per_group) {
+                    const int nj = std::min(tok_per_group, nt - j0);
+                    n += (int64_t)parts_of(ctx_lens[i] + j0 + nj, nj, lim) * Hkv;
+                }
+            }
+            return n;
+        };
+        int64_t lo = ac.item + ac.part + min_blocks * (int64_t)ac.block[1], hi = lo;
+        for (int i = 0; i < n_req; ++i) hi = std::max(hi, blocks_of(ctx_lens[i] + (chunk_offsets[i + 1] - chunk_offsets[i])) * (int64_t)ac.block[4] + ac.item);
+        while (hi - lo > 256) {   // n_parts_at falls with the limit; at `hi` nothing is cut
+            const int64_t mid = (lo + hi) / 2;
+            if (n_parts_at(mid) <= n_cta_max) hi = mid; else lo = mid;
+        }
+        limit = hi;
+    }
+    // Positions that no chunk of the batch writes, for the kernel that requests keys before the chunks' are written: up
+    // to the first page of the request that holds a written slot, of whichever request.
+    std::vector<int> safe;
+    if (kind == ATTN_THIN) {
+        std::vector<uint8_t> written(n_pages, 0);
+        for (int i = 0; i < n_req; ++i)
+            for (int k = ctx_lens[i] / P; k <= (ctx_lens[i] + (chunk_offsets[i + 1] - chunk_offsets[i]) - 1) / P; ++k)
+                written[page_tables[(size_t)i * max_pages + k]] = 1;
+        safe.resize(n_req);
+        for (int i = 0; i < n_req; ++i) {
+            int k = 0;
+            while (k < ctx_lens[i] / P && !written[page_tables[(size_t)i * max_pages + k]]) ++k;
+            safe[i] = k * P;
+        }
+    }
     std::vector<AttnItem> items;
     std::vector<int> item_cost;
     std::vector<MergeGroup>& groups = hp.groups;
@@ -883,20 +945,19 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         const int b = chunk_offsets[i], n = chunk_offsets[i + 1] - b;
         for (int j0 = 0; j0 < n; j0 += tok_per_group) {
             const int nj = std::min(tok_per_group, n - j0);
-            const int L = ctx_lens[i] + j0 + nj;
-            int np = (int)std::min<int64_t>(64, (unit_cost(L, nj) + share - 1) / share);
-            int len = ((L + np - 1) / np + 63) / 64 * 64;
-            np = (L + len - 1) / len;
+            const int L = ctx_lens[i] + j0 + nj, nb = blocks_of(L);
+            const int np = parts_of(L, nj, limit);
             for (int h = 0; h < Hkv; ++h) {
                 if (np > 1) {
                     MergeGroup g = {b + j0, nj, h, n_parts, np, 0, 0, 0};
                     groups.push_back(g);
                 }
                 for (int k = 0; k < np; ++k) {
-                    AttnItem it = {b + j0, nj, h, i, k * len, std::min(L, (k + 1) * len), ctx_lens[i] + j0,
-                                   np > 1 ? n_parts + k : -1, np > 1 ? (int)groups.size() - 1 : -1, 0, 0, 0};
+                    const int b0 = (int)((int64_t)k * nb / np), b1 = (int)((int64_t)(k + 1) * nb / np);
+                    AttnItem it = {b + j0, nj, h, i, b0 * 64, std::min(L, b1 * 64), ctx_lens[i] + j0,
+                                   np > 1 ? n_parts + k : -1, np > 1 ? (int)groups.size() - 1 : -1, kind == ATTN_THIN ? safe[i] : 0, 0, 0};
                     items.push_back(it);
-                    item_cost.push_back((int)unit_cost(it.kv_end - it.kv_begin, nj) + (np > 1 ? PART_COST : 0));
+                    item_cost.push_back((int)((b1 - b0) * block_cost(nj)) + ac.item + (np > 1 ? ac.part : 0));
                 }
                 if (np > 1) n_parts += np;
             }
@@ -1037,7 +1098,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     s.attn_flops = 4.0 * qd * c.n_layers * (double)keys_seen;
     s.attn_items = n_items; s.attn_split_items = n_parts;
     s.kernel_launches = 1 + c.n_layers * 5 + 2;
-    s.attn_rows = hp.row_cap;
+    s.attn_rows = attn_rows(kind);
     return SYN_OK;
 }
 
@@ -1048,7 +1109,7 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     if (!m || !kv || kv->model != m) return SYN_E_INVALID_ARG;
     HostPlan hp;
     int r = plan_compute(m->desc, (int)kv->page_size, kv->n_pages, m->n_sm, n_req, chunk_tokens, chunk_offsets, page_tables,
-                         max_pages, ctx_lens, n_uncached, g_attention, hp);
+                         max_pages, ctx_lens, n_uncached, g_attention, 2 * m->n_sm, hp);
     if (r) return r;
     const int T = hp.T, n_items = (int)hp.items.size(), n_cta = hp.n_cta;
     size_t off = 0;
@@ -1084,7 +1145,7 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     if (!hp.groups.empty()) memcpy(p->h<MergeGroup>(p->o_groups), hp.groups.data(), hp.groups.size() * sizeof(MergeGroup));
     p->n_req = n_req; p->T = T; p->max_pages = max_pages; p->n_items = n_items; p->n_cta = n_cta;
     p->n_groups = (int)hp.groups.size(); p->n_parts = hp.n_parts;
-    p->row_cap = hp.row_cap;
+    p->attn = hp.kind;
     p->stats = hp.stats;
     p->stats.h2d_bytes = (int64_t)off;
     p->kv = kv; p->kv_pool = kv->pool; p->kv_pages = kv->n_pages;
@@ -1103,7 +1164,7 @@ static int syn_plan_host_impl(const syn_model_desc* desc, uint32_t n_pages, uint
         return SYN_E_INVALID_ARG;
     HostPlan hp;
     int r = plan_compute(*desc, (int)page_size, n_pages, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages,
-                         ctx_lens, n_uncached, g_attention, hp);
+                         ctx_lens, n_uncached, g_attention, n_sm, hp);   // n_sm CTAs whatever the kernel
     if (r) return r;
     *n_items = (int)hp.items.size();
     *n_cta = hp.n_cta;
@@ -1418,10 +1479,11 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
     ap.n_kv_heads = c.n_kv_heads;
     ap.group = c.n_q_heads / c.n_kv_heads;
     ap.q_dim = c.n_q_heads * c.head_dim;
-    ap.row_cap = p->row_cap;
-    ap.q_box_tokens = p->row_cap == 128 ? std::min(SYN_MAX_CHUNK, 128 / ap.group) : std::min(16, 64 / ap.group);
+    ap.row_cap = attn_rows(p->attn);
+    ap.q_box_tokens = p->attn == ATTN_TENSOR ? std::min(SYN_MAX_CHUNK, 128 / ap.group) : std::min(16, 64 / ap.group);
     ap.layer_block0 = (int)(2ull * layer * kv->n_pages * c.n_kv_heads);
     ap.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)c.head_dim));
+    ap.q = m->q;
     ap.out = out;
     ap.part_o = part_o;
     ap.part_ml = part_ml;
@@ -1432,23 +1494,31 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
     ap.n_parts = p->n_parts; ap.n_groups = p->n_groups;
 }
 
+// The kernel the plan was made for; `pdl`: may start while its predecessor in the stream still runs.
+static cudaError_t attention_kernel(const syn_model* m, const syn_kv* kv, const syn_plan* p, const AttnParams& ap, const CUtensorMap& tmQ, bool pdl,
+                                    cudaStream_t st) {
+    const bool wide_head = m->desc.head_dim == 128;
+    const dim3 grid(p->n_cta);
+    switch (p->attn) {
+        case ATTN_TENSOR:
+            return wide_head ? launch(attn2_kernel<128>, grid, dim3(ATT2_THREADS), Attn2Smem<128>::TOTAL, st, pdl, m->tm_q4, kv->tm_kv5, ap)
+                             : launch(attn2_kernel<64>, grid, dim3(ATT2_THREADS), Attn2Smem<64>::TOTAL, st, pdl, m->tm_q4, kv->tm_kv5, ap);
+        case ATTN_THIN:
+            return wide_head ? launch(attn_thin_kernel<128>, grid, dim3(ATTN_THIN_THREADS), AttnThinSmem<128>::TOTAL, st, pdl, kv->tm_kv, ap)
+                             : launch(attn_thin_kernel<64>, grid, dim3(ATTN_THIN_THREADS), AttnThinSmem<64>::TOTAL, st, pdl, kv->tm_kv, ap);
+        default:
+            return wide_head ? launch(attn_kernel<128>, grid, dim3(ATT_THREADS), AttnSmem<128>::TOTAL, st, pdl, tmQ, kv->tm_kv, ap)
+                             : launch(attn_kernel<64>, grid, dim3(ATT_THREADS), AttnSmem<64>::TOTAL, st, pdl, tmQ, kv->tm_kv, ap);
+    }
+}
+
 static int launch_attention(syn_model* m, syn_kv* kv, const syn_plan* p, uint32_t layer, const CUtensorMap& tmQ,
                             op16* out, cudaStream_t st) {
-    const syn_model_desc& c = m->desc;
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, out, m->part_o, m->part_ml, m->group_count);
     {
         ProfScope prof(m, 2, st);
-        cudaError_t e;
-        if (p->row_cap == 128 && c.head_dim == 128)
-            e = launch_pdl(attn2_kernel<128>, dim3(p->n_cta), dim3(ATT2_THREADS), Attn2Smem<128>::TOTAL, st, m->tm_q4, kv->tm_kv5, ap);
-        else if (p->row_cap == 128)
-            e = launch_pdl(attn2_kernel<64>, dim3(p->n_cta), dim3(ATT2_THREADS), Attn2Smem<64>::TOTAL, st, m->tm_q4, kv->tm_kv5, ap);
-        else if (c.head_dim == 128)
-            e = launch_pdl(attn_kernel<128>, dim3(p->n_cta), dim3(ATT_THREADS), AttnSmem<128>::TOTAL, st, tmQ, kv->tm_kv, ap);
-        else
-            e = launch_pdl(attn_kernel<64>, dim3(p->n_cta), dim3(ATT_THREADS), AttnSmem<64>::TOTAL, st, tmQ, kv->tm_kv, ap);
-        if (e != cudaSuccess) return SYN_E_CUDA;
+        if (attention_kernel(m, kv, p, ap, tmQ, true, st) != cudaSuccess) return SYN_E_CUDA;
     }
     return SYN_OK;
 }
@@ -1891,7 +1961,7 @@ extern "C" int syn_debug_set_schedule(int32_t which) {
 }
 
 extern "C" int syn_debug_set_attention(int32_t which) {
-    if (which < 0 || which > 2) return SYN_E_INVALID_ARG;
+    if (which < 0 || which > 3) return SYN_E_INVALID_ARG;
     g_attention = which;
     return SYN_OK;
 }
@@ -1962,7 +2032,7 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     const syn_model_desc& c = m->desc;
     const int q_dim = c.n_q_heads * c.head_dim;
     if (p->T > m->t_cap) return SYN_E_INVALID_ARG;
-    if ((int64_t)p->n_parts * p->row_cap > (int64_t)SYN_STATIC_MAX_PARTS * 64) return SYN_E_CAPACITY;
+    if ((int64_t)p->n_parts * attn_rows(p->attn) > (int64_t)SYN_STATIC_MAX_PARTS * 64) return SYN_E_CAPACITY;
     float* part_o = nullptr;
     float2* part_ml = nullptr;
     int* group_count = nullptr;
@@ -1974,15 +2044,7 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     CU_OK(cudaMemsetAsync(group_count, 0, (size_t)SYN_STATIC_MAX_PARTS * 4, st));
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, (op16*)out, part_o, part_ml, group_count);
-    if (p->row_cap == 128 && c.head_dim == 128)
-        attn2_kernel<128><<<p->n_cta, ATT2_THREADS, Attn2Smem<128>::TOTAL, st>>>(m->tm_q4, kv->tm_kv5, ap);
-    else if (p->row_cap == 128)
-        attn2_kernel<64><<<p->n_cta, ATT2_THREADS, Attn2Smem<64>::TOTAL, st>>>(m->tm_q4, kv->tm_kv5, ap);
-    else if (c.head_dim == 128)
-        attn_kernel<128><<<p->n_cta, ATT_THREADS, AttnSmem<128>::TOTAL, st>>>(m->tm_q, kv->tm_kv, ap);
-    else
-        attn_kernel<64><<<p->n_cta, ATT_THREADS, AttnSmem<64>::TOTAL, st>>>(m->tm_q, kv->tm_kv, ap);
-    return launch_ok() ? SYN_OK : SYN_E_CUDA;
+    return attention_kernel(m, kv, p, ap, m->tm_q, false, st) == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
 // The projection schedule without a device (tests): the launch shape, and work item i of CTA `cta`.

@@ -1,0 +1,57 @@
+"""The half-SM attention kernel (batches of few requests): against the CPU oracle's attention at the geometries and edges
+of the other kernels' test, at the widths of its row tiles and its key parts, and on a batch in which one request's
+context is another request's chunk."""
+import pytest
+import torch
+
+from workloads import gen
+from workloads.configs import TINY, Workload
+
+import test_gpu_attention as base
+from harness import cpu_model, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+CASES = base.CASES + [
+    (128, 8, 2, [63, 64, 65], [1, 4, 5]),        # one, two and three 64-key blocks; 1 and 2 row tiles
+    (64, 8, 2, [4000], [9]),                     # 63 blocks over the most parts of one unit, 36 rows
+    (128, 8, 8, [900, 31, 2047], [1, 16, 2]),    # G = 1
+    (128, 8, 2, [6000], [12]),                   # parts of several blocks
+]
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv,ctx,chunk", CASES)
+def test_thin_attention_matches_oracle(hd, Hq, Hkv, ctx, chunk):
+    import paper_2511_07423_b200 as syn
+    syn.debug_set_attention(3)
+    try:
+        base._run(hd, Hq, Hkv, ctx, chunk)
+    finally:
+        syn.debug_set_attention(0)
+
+
+@pytest.mark.parametrize("hd", [128, 64])
+def test_scores_that_keep_growing(hd):
+    base.test_scores_that_keep_growing_along_the_keys(hd, 8, 2, 3)
+
+
+def test_a_context_written_by_another_request_of_the_batch():
+    """Two requests over one page table, the second one's context ending with the first one's chunk (a long run of
+    uncached tokens in one step): its keys must not be read before they are written."""
+    import paper_2511_07423_b200 as syn
+    shape, seed = TINY, 31
+    glob, layers = cpu_model(shape, seed)
+    model = syn.Model(shape, *to_cuda(glob, layers))
+    toks = gen.gen_context_tokens(Workload("w", shape, seed, 1, None, None, 0.5), 0, 70)
+    table = torch.tensor([[5, 1, 7, 2, 0]], dtype=torch.int32)
+    kv = syn.KVCache(model, 8)
+    for at, n in ((0, 32), (32, 16)):
+        kv.verify_batch(toks[at:at + n], [0, n], table, [at], [n])
+    # the pieces one after the other ...
+    kv.verify_batch(toks[48:60], [0, 12], table, [48], [12])
+    _, _, want = kv.verify_batch(toks[60:70], [0, 10], table, [60], [10], want_logits=True)
+    # ... and as two requests of one batch, over slots that hold something else before
+    for _ in range(3):
+        kv.verify_batch(toks[:22].flip(0), [0, 22], table, [48], [22])
+        _, _, got = kv.verify_batch(toks[48:70], [0, 12, 22], table.repeat(2, 1), [48, 60], [12, 10], want_logits=True)
+        assert torch.equal(got[12:], want)
