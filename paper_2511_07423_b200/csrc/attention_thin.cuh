@@ -228,49 +228,67 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
             attn_thin_bar();
             if (*last_flag) {
                 __threadfence();
-                // (Compact loops on purpose: this code runs once per launch, and what it costs is the fetching of its
-                // instructions and two round trips to L2, not arithmetic.)
+                // What this costs is the round trips to L2, on the step's critical path: a thread has fifteen float4 of
+                // the partial outputs in flight (NU places of the rows x UK parts), the first of them together with the
+                // (m, l) pairs.  (8B shape, 9 parts of 20 rows: 8.8 k cycles with two parts at a time after the pairs.)
                 const int np = min(gr.n_parts, ATTN_THIN_MAX_PARTS);
                 float2* ml_s = reinterpret_cast<float2*>(merge);   // [part][64]
-#pragma unroll 4
-                for (int i = threadIdx.x; i < np * 64; i += 128)
-                    if ((i & 63) < rows) ml_s[i] = __ldcg(&p.part_ml[(size_t)(gr.part0 + (i >> 6)) * p.row_cap + (i & 63)]);
-                attn_thin_bar();
-                if (threadIdx.x < rows) {   // weight of every part of a row, already divided by the row's sum
-                    float mx = -INFINITY, lsum = 0.f;
-                    for (int k = 0; k < np; ++k) mx = fmaxf(mx, ml_s[k * 64 + threadIdx.x].x);
-                    const float bs = mx == -INFINITY ? 0.f : mx;
-                    for (int k = 0; k < np; ++k) {
-                        float2 v = ml_s[k * 64 + threadIdx.x];
-                        v.x = ex2_approx(v.x - bs);
-                        lsum += v.y * v.x;
-                        ml_s[k * 64 + threadIdx.x].x = v.x;
+                constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5;
+                const int n_vec = rows * VR;
+                const float4* src = reinterpret_cast<const float4*>(p.part_o + (size_t)gr.part0 * p.row_cap * HD);
+                float4 v[UK][NU];
+                auto fetch = [&](int u0, int k0) {
+#pragma unroll
+                    for (int k = 0; k < UK; ++k)
+#pragma unroll
+                        for (int i = 0; i < NU; ++i)
+                            v[k][i] = __ldcg(src + (size_t)min(k0 + k, np - 1) * p.row_cap * VR + min(u0 + i * 128, n_vec - 1));
+                };
+                fetch(threadIdx.x, 0);
+                {
+                    const int row = threadIdx.x & 63;
+                    const float2* ml = p.part_ml + (size_t)gr.part0 * p.row_cap + min(row, rows - 1);
+                    for (int k0 = threadIdx.x >> 6; k0 < np; k0 += 16) {
+                        float2 t[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) t[k] = __ldcg(ml + (size_t)min(k0 + 2 * k, np - 1) * p.row_cap);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (k0 + 2 * k < np) ml_s[(k0 + 2 * k) * 64 + row] = t[k];
                     }
-                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-                    for (int k = 0; k < np; ++k) ml_s[k * 64 + threadIdx.x].x *= inv;
                 }
                 attn_thin_bar();
-                constexpr int VR = HD / 4, NU = HD == 128 ? 6 : 4;   // float4 of a row; of them a thread takes NU at a time
-                const float4* src = reinterpret_cast<const float4*>(p.part_o + (size_t)gr.part0 * p.row_cap * HD);
-                for (int u0 = threadIdx.x; u0 < rows * VR; u0 += NU * 128) {
+                if (threadIdx.x < rows) {   // weight of every part of a row, already divided by the row's sum
+                    float2* col = ml_s + threadIdx.x;
+                    float mx = -INFINITY, lsum = 0.f;
+#pragma unroll 4
+                    for (int k = 0; k < np; ++k) mx = fmaxf(mx, col[k * 64].x);
+                    const float bs = mx == -INFINITY ? 0.f : mx;
+#pragma unroll 4
+                    for (int k = 0; k < np; ++k) lsum += col[k * 64].y * ex2_approx(col[k * 64].x - bs);
+                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+#pragma unroll 4
+                    for (int k = 0; k < np; ++k) col[k * 64].x = ex2_approx(col[k * 64].x - bs) * inv;
+                }
+                attn_thin_bar();
+                for (int u0 = threadIdx.x; u0 < n_vec; u0 += NU * 128) {
                     float4 acc[NU];
 #pragma unroll
                     for (int i = 0; i < NU; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-                    for (int k = 0; k < np; ++k) {
-                        float4 v[NU];
+                    for (int k0 = 0; k0 < np; k0 += UK) {
+                        if (k0 > 0 || u0 != (int)threadIdx.x) fetch(u0, k0);
 #pragma unroll
-                        for (int i = 0; i < NU; ++i) v[i] = __ldcg(src + (size_t)k * p.row_cap * VR + min(u0 + i * 128, rows * VR - 1));
+                        for (int k = 0; k < UK; ++k)
 #pragma unroll
-                        for (int i = 0; i < NU; ++i) {
-                            const float w = ml_s[k * 64 + min(u0 + i * 128, rows * VR - 1) / VR].x;
-                            acc[i].x += v[i].x * w; acc[i].y += v[i].y * w; acc[i].z += v[i].z * w; acc[i].w += v[i].w * w;
-                        }
+                            for (int i = 0; i < NU; ++i) {
+                                const float w = k0 + k < np ? ml_s[(k0 + k) * 64 + min(u0 + i * 128, n_vec - 1) / VR].x : 0.f;
+                                acc[i].x += v[k][i].x * w; acc[i].y += v[k][i].y * w; acc[i].z += v[k][i].z * w; acc[i].w += v[k][i].w * w;
+                            }
                     }
 #pragma unroll
                     for (int i = 0; i < NU; ++i) {
                         const int u = u0 + i * 128, row = u / VR, j = row / G, gq = row - j * G;
-                        if (u < rows * VR)
+                        if (u < n_vec)
                             *reinterpret_cast<uint2*>(p.out + (size_t)(gr.q_tok + j) * p.q_dim + (gr.kvh * G + gq) * HD + 4 * (u % VR)) =
                                 make_uint2(pack_op(acc[i].x, acc[i].y), pack_op(acc[i].z, acc[i].w));
                     }
