@@ -40,7 +40,16 @@ struct MergeGroup {
     int q_tok, nj, kvh, part0, n_parts, pad0, pad1, pad2;
 };
 
+// Weights that a projection behind the attention will read: k-blocks [skip, skip + count) of every (128-feature tile, part of
+// K) of a launch of the thin projection kernel, in the order its CTAs take them.
+struct WeightsAhead {
+    const op16* w;              // packed weights; count 0: nothing to ask for
+    int num_kb, n_tiles, n_tt, splits, skip, count;
+};
+
 struct AttnParams {
+    WeightsAhead ahead[2];      // (half-SM kernel) asked of L2 by CTAs that have requested their last keys ...
+    int ahead_late;             // ... 1: and whose keys have all arrived
     const AttnItem* items;      // sorted by CTA
     const int* cta_begin;       // [n_cta + 1]
     const int* page_tables;     // [B][max_pages]

@@ -35,6 +35,9 @@ struct AttnThinSmem {
 __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
 }
+__device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(src)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void attn_thin_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 template <int HD>
@@ -110,6 +113,21 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                 }
             }
         }
+        // HBM would idle while the last parts are finished and merged: ask L2 for weights of the projections behind, where
+        // there are many keys only once this CTA's own are here (sooner, the requests delay the CTAs that are behind)
+        if (p.ahead_late)
+            for (uint32_t q = st > (uint32_t)NS ? st - NS : 0u; ok && q < st; ++q)
+                if (lane == 0) ok = mbar_wait(&empty_bar[q % NS], (q / NS) & 1, p.status);
+        if (lane == 0 && ok)
+            for (int i = 0; i < 2; ++i) {
+                const WeightsAhead& a = p.ahead[i];
+                for (int b = blockIdx.x; b < a.n_tiles * a.splits * a.count; b += gridDim.x) {
+                    const int unit = b / a.count, j = a.skip + b - unit * a.count, tile = unit / a.splits, part = unit - tile * a.splits;
+                    const int k0 = (int)((long long)part * a.num_kb / a.splits), nk = (int)((long long)(part + 1) * a.num_kb / a.splits) - k0;
+                    if (j < nk)
+                        l2_prefetch(a.w + (((size_t)(tile >> 1) * a.num_kb + k0 + (j + tile * a.n_tt % nk) % nk) * 2 + (tile & 1)) * (128 * 64), 128 * 64 * 2);
+                }
+            }
         return;
     }
 

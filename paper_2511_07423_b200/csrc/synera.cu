@@ -1484,6 +1484,8 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
     ap.layer_block0 = (int)(2ull * layer * kv->n_pages * c.n_kv_heads);
     ap.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)c.head_dim));
     ap.q = m->q;
+    memset(ap.ahead, 0, sizeof(ap.ahead));
+    ap.ahead_late = 0;
     ap.out = out;
     ap.part_o = part_o;
     ap.part_ml = part_ml;
@@ -1492,6 +1494,29 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
     ap.status = m->status_dev;
     ap.n_items = p->n_items; ap.n_req = p->n_req; ap.n_tokens = p->T; ap.n_pages = (int)kv->n_pages;
     ap.n_parts = p->n_parts; ap.n_groups = p->n_groups;
+}
+
+// Weights that the half-SM attention asks of L2 for the projections behind it, while HBM would idle: 24 MB, at most ten tiles
+// of 16 KB per CTA (more, and a CTA with few keys outlasts the merge).  Measured, us a step at 0 / 16 / 24 / 40 MB: 1B shape,
+// one request 840 / 830 / - / 883 (104 CTAs), 1B shape, two requests 878 / 870 / 863 / 844, 8B shape, eight requests
+// 4 048 / 3 956 / 3 939 / 3 922, 16 requests 2 414 / 2 400 / 2 403 / 2 440 (16 layers).  Where a layer has more than 16 MB of
+// keys a CTA waits for its own first (8B shape, eight requests, without that: 3 974).
+constexpr int64_t ATTN_AHEAD_BYTES = 24 << 20, ATTN_AHEAD_TILES = 10, ATTN_AHEAD_LATE_BYTES = 16 << 20;
+
+// What the attention may ask of L2 ahead: `budget` bytes (taken off) of a projection's weights beyond what the operand rings
+// of its CTAs hold anyway.
+static WeightsAhead weights_ahead(const op16* w, int T, int packed_rows, int K, int n_sm, int mode, int64_t& budget) {
+    WeightsAhead a;
+    memset(&a, 0, sizeof(a));
+    ThinParams g;
+    if (budget <= 0 || g_schedule == 1 || !thin_takes(T, packed_rows, K, n_sm, mode)) return a;
+    thin_plan(T, packed_rows, K, n_sm, g);
+    const int units = g.n_tiles * g.splits, nk = (g.num_kb + g.splits - 1) / g.splits;
+    a.w = w; a.num_kb = g.num_kb; a.n_tiles = g.n_tiles; a.n_tt = g.n_tt; a.splits = g.splits;
+    a.skip = std::min(g.n_stages, nk);
+    a.count = (int)std::min<int64_t>(nk - a.skip, budget / ((int64_t)units * GEMM_TILE_BYTES));
+    budget -= (int64_t)units * a.count * GEMM_TILE_BYTES;
+    return a;
 }
 
 // The kernel the plan was made for; `pdl`: may start while its predecessor in the stream still runs.
@@ -1516,6 +1541,14 @@ static int launch_attention(syn_model* m, syn_kv* kv, const syn_plan* p, uint32_
                             op16* out, cudaStream_t st) {
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, out, m->part_o, m->part_ml, m->group_count);
+    if (p->attn == ATTN_THIN) {
+        const syn_model_desc& c = m->desc;
+        const int d = c.d_model, q_dim = c.n_q_heads * c.head_dim;
+        int64_t budget = std::min(ATTN_AHEAD_BYTES, (int64_t)p->n_cta * ATTN_AHEAD_TILES * GEMM_TILE_BYTES);
+        ap.ahead_late = p->stats.kv_read_bytes / c.n_layers > ATTN_AHEAD_LATE_BYTES;
+        ap.ahead[0] = weights_ahead(m->wo[layer], p->T, d, q_dim, m->n_sm, EPI_RESID, budget);
+        ap.ahead[1] = weights_ahead(m->wgu[layer], p->T, m->gu_rows, d, m->n_sm, EPI_SWIGLU, budget);
+    }
     {
         ProfScope prof(m, 2, st);
         if (attention_kernel(m, kv, p, ap, tmQ, true, st) != cudaSuccess) return SYN_E_CUDA;
