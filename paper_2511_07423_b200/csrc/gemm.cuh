@@ -103,14 +103,14 @@ constexpr int GEMM_EPI_WARPS = 16;               // four groups of four (one war
 // Epilogue of one 16-token chunk of one warp: a[j] = D[feature of this lane][token t0 + j] (tokens
 // j >= ncols are padding), already summed and scaled.  In this orientation a lane holds ONE output
 // feature for sixteen tokens, while every output is token-major in memory, so the 32 x 16 block is
-// first turned round in a shared-memory scratch of the warp (16 rows of 33 floats: no bank conflicts
+// first turned round in a shared-memory scratch of the warp (16 rows of 36 floats: no bank conflicts
 // either way).  Afterwards the lanes walk the block row by row: eight neighbouring lanes cover the 32
 // columns of one token with four columns each, so that a warp-wide access touches whole 32-byte
 // sectors of four tokens' rows (the cost of these epilogues is the number of sectors and of memory
 // instructions they issue, not their arithmetic).
 // `m0` = first packed row of the tile, `quarter` = warp's TMEM lane quarter.
 constexpr int EPI_COLS = 16;
-constexpr int EPI_SCR_STRIDE = 33;
+constexpr int EPI_SCR_STRIDE = 36;   // floats: rows stay 16-byte aligned, so that a lane reads its four columns with one load
 constexpr int EPI_SCR_FLOATS = EPI_COLS * EPI_SCR_STRIDE;   // per epilogue warp
 
 __device__ __forceinline__ uint2 pack4_op(float a, float b, float c, float d) { return make_uint2(pack_op(a, b), pack_op(c, d)); }
@@ -163,17 +163,21 @@ __device__ __forceinline__ void epi_stage(const float (&a)[EPI_COLS], float* scr
     __syncwarp();
 }
 
-// ... and out of it row by row.  LOADED: the operands are in `o` already; otherwise they are loaded where they are used.
-template <int MODE, bool LOADED>
-__device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float* scr, int m0, int t0, int ncols,
-                                         int quarter, int lane) {
+// ... and out of it row by row; `o` holds what epi_load brought (LATE: it is loaded here, once the chunk's own registers are
+// free).  SWIGLU and LMHEAD have ways of their own (below).
+template <int MODE, bool LATE = false>
+__device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float (&a)[EPI_COLS], float* scr, int m0,
+                                         int t0, int ncols, int quarter, int lane) {
+    if (MODE != EPI_SWIGLU && (MODE != EPI_LMHEAD || p.logits)) epi_stage(a, scr, lane);
+    if (LATE) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
     const int tq = lane >> 3, c0 = (lane & 7) * 4;   // token (+ 4 i) and first of four columns of this lane
     if (MODE == EPI_PLAIN) {
         const int f = m0 + quarter * 32 + c0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = tq + 4 * i;
-            const float* row = scr + t * EPI_SCR_STRIDE + c0;
+            const float4 r4 = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
+            const float row[4] = {r4.x, r4.y, r4.z, r4.w};
             if (t < ncols) {
                 float* dst = p.y + (size_t)(t0 + t) * p.ldy + f;
                 if ((p.ldy & 3) == 0 && f + 4 <= p.N) {
@@ -188,16 +192,15 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
     } else if (MODE == EPI_RESID) {
         // x += D; operand of the next projection bf16(x * gain); sum of x^2 over this warp's 32 features
         const int f = m0 + quarter * 32 + c0;
-        if (!LOADED) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
         const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.x);
         const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.y);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = tq + 4 * i;
             const bool tv = t < ncols;
-            const float* row = scr + t * EPI_SCR_STRIDE + c0;
+            const float4 row = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
             const float4 xv = o.v[i & (MODE == EPI_RESID ? 3 : 0)];
-            const float4 nx = make_float4(xv.x + row[0], xv.y + row[1], xv.z + row[2], xv.w + row[3]);
+            const float4 nx = make_float4(xv.x + row.x, xv.y + row.y, xv.z + row.z, xv.w + row.w);
             float ss = tv ? (nx.x * nx.x + nx.y * nx.y) + (nx.z * nx.z + nx.w * nx.w) : 0.f;
             if (tv) {
                 const size_t at = (size_t)(t0 + t) * p.d + f;
@@ -215,7 +218,7 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
         const int region0 = which == 0 ? 0 : (which == 1 ? p.q_dim : p.q_dim + p.kv_dim);
         const int half = p.hd >> 1, hd_log = p.hd == 128 ? 7 : 6;   // head_dim is 64 or 128
         const size_t page_stride = (size_t)p.n_kv_heads * 2 * 16 * p.hd;
-        const int my_slot = LOADED ? o.slot : ((which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0);
+        const int my_slot = o.slot;
         if (which < 2) {
             // q and k tiles: columns 0..15 of the block are the dims [d0, d0 + 16) of one head, columns 16..31
             // the same dims + hd/2 (rope_tile_feature); a lane rotates its four columns with their partners
@@ -223,18 +226,17 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
             const int fhead = (m0 - region0) + ((quarter >> g_log) << hd_log);   // first feature of the head, inside q or k
             const bool hi = c0 >= 16;
             const int dim = 16 * (quarter & ((1 << g_log) - 1)) + (c0 & 15);            // lower dim of the pair
-            if (!LOADED) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float4 w0 = o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)], w1 = o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)];
                 const int t = tq + 4 * i;
-                const float* mine = scr + t * EPI_SCR_STRIDE + c0;
-                const float* part = scr + t * EPI_SCR_STRIDE + (c0 ^ 16);
+                const float4 mine = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
+                const float4 part = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + (c0 ^ 16));
                 const float sg = hi ? 1.f : -1.f;   // dim i: x cos - y sin; dim i + hd/2: y cos + x sin
-                const float r0 = mine[0] * w0.x + sg * part[0] * w0.y;
-                const float r1 = mine[1] * w0.z + sg * part[1] * w0.w;
-                const float r2 = mine[2] * w1.x + sg * part[2] * w1.y;
-                const float r3 = mine[3] * w1.z + sg * part[3] * w1.w;
+                const float r0 = mine.x * w0.x + sg * part.x * w0.y;
+                const float r1 = mine.y * w0.z + sg * part.y * w0.w;
+                const float r2 = mine.z * w1.x + sg * part.z * w1.y;
+                const float r3 = mine.w * w1.z + sg * part.w * w1.w;
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
                     op16* dst;
@@ -249,93 +251,100 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int t = tq + 4 * i;
-                const float* row = scr + t * EPI_SCR_STRIDE + c0;
+                const float4 row = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
                     op16* dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fr >> hd_log) * 2 + 1) * 16 * p.hd +
                                          (size_t)(sl & 15) * p.hd + (fr & (p.hd - 1));
-                    *reinterpret_cast<uint2*>(dst) = pack4_op(row[0], row[1], row[2], row[3]);
+                    *reinterpret_cast<uint2*>(dst) = pack4_op(row.x, row.y, row.z, row.w);
                 }
             }
         }
     } else if (MODE == EPI_SWIGLU) {
-        // columns 0..15 of the block hold gate features, columns 16..31 the matching up features: 16
-        // outputs per token; four neighbouring lanes cover them, eight tokens per pass
-        const int tq8 = lane >> 2, g0 = (lane & 3) * 4;
+        // Lanes 0..15 hold gate features, lanes 16..31 the matching up features.  The two exchange halves of their tokens,
+        // so that each lane has gate and up of its feature for eight tokens; the results, already half precision, go
+        // through a [16 features][16 tokens] tile (rows of 48 bytes) and come out of ldmatrix.trans with four consecutive
+        // features of a token per lane.  (Half the instructions of the fp32 transposition that the other epilogues need.)
+        const bool hi = lane & 16;
+        float h[8];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int t = tq8 + 8 * i;
-            const float* row = scr + t * EPI_SCR_STRIDE + g0;
-            float h[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) h[k] = __fdividef(row[k], 1.0f + __expf(-row[k])) * row[16 + k];
-            if (t < ncols)
-                *reinterpret_cast<uint2*>(p.act + (size_t)(t0 + t) * p.f_pad + (m0 >> 1) + 16 * quarter + g0) = pack4_op(h[0], h[1], h[2], h[3]);
+        for (int k = 0; k < 8; ++k) {
+            const float other = __shfl_xor_sync(0xFFFFFFFFu, hi ? a[k] : a[k + 8], 16);
+            const float g = hi ? other : a[k], u = hi ? a[k + 8] : other;
+            h[k] = __fdividef(g, 1.0f + __expf(-g)) * u;
         }
+        uint8_t* const tile = reinterpret_cast<uint8_t*>(scr);
+        __syncwarp();   // the previous chunk's tile has been read
+        *reinterpret_cast<uint4*>(tile + (lane & 15) * 48 + (lane >> 4) * 16) =
+            make_uint4(pack_op(h[0], h[1]), pack_op(h[2], h[3]), pack_op(h[4], h[5]), pack_op(h[6], h[7]));
+        __syncwarp();
+        // matrix j of the four: tokens 8 (j / 2) .., features 4 q + 2 (j & 1) + {0, 1} for q = 0 .. 3
+        const int i = lane & 7, j = lane >> 3;
+        uint32_t r0, r1, r2, r3;
+        ldsm_x4_t(smem_u32(tile + (4 * (i >> 1) + 2 * (j & 1) + (i & 1)) * 48 + (j >> 1) * 16), r0, r1, r2, r3);
+        const int t = lane >> 2;
+        op16* dst = p.act + (size_t)(t0 + t) * p.f_pad + (m0 >> 1) + 16 * quarter + (lane & 3) * 4;
+        if (t < ncols) *reinterpret_cast<uint2*>(dst) = make_uint2(r0, r1);
+        if (t + 8 < ncols) *reinterpret_cast<uint2*>(dst + (size_t)8 * p.f_pad) = make_uint2(r2, r3);
     } else {  // EPI_LMHEAD
-        const int f = m0 + quarter * 32 + c0;
+        // Largest logit of each token among the warp's 32 features, lowest id on ties, before any transposition: a maximum over
+        // the warp and a ballot of the lanes that have it; lane j then speaks for token j.
+        const int fl = m0 + quarter * 32;
+        const bool fv = fl + lane < p.vocab;
+        uint32_t top = 0u, who = 0u;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int t = tq + 4 * i;
-            const bool tv = t < ncols;
-            const float* row = scr + t * EPI_SCR_STRIDE + c0;
-            const float v[4] = {row[0], row[1], row[2], row[3]};
-            if (p.logits && tv) {
-                float* dst = p.logits + (size_t)(t0 + t) * p.vocab + f;
-                if ((p.vocab & 3) == 0 && f + 4 <= p.vocab) {
-                    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-                } else {
+        for (int j = 0; j < EPI_COLS; ++j) {
+            const uint32_t key = fv ? orderable_f32(a[j]) : 0u;
+            const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, key);
+            const uint32_t eq = __ballot_sync(0xFFFFFFFFu, key == mx && fv);
+            if (lane == j) { top = mx; who = eq; }
+        }
+        if (lane < ncols) {
+            if (who) atomicMax(p.best + t0 + lane, pack_argmax_key(top, fl + __ffs(who) - 1));
+            // the group's maximum of the token (0: no valid feature): a threshold source for a later top-k
+            if (p.warp_max) p.warp_max[(size_t)(t0 + lane) * p.n_warp_max + (m0 >> 5) + quarter] = top;
+        }
+        if (p.logits) {
+            const int f = fl + c0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (f + k < p.vocab) dst[k] = v[k];
+            for (int i = 0; i < 4; ++i) {
+                const int t = tq + 4 * i;
+                const float4 v = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
+                if (t < ncols) {
+                    float* dst = p.logits + (size_t)(t0 + t) * p.vocab + f;
+                    if ((p.vocab & 3) == 0 && f + 4 <= p.vocab) {
+                        *reinterpret_cast<float4*>(dst) = v;
+                    } else {
+                        if (f < p.vocab) dst[0] = v.x;
+                        if (f + 1 < p.vocab) dst[1] = v.y;
+                        if (f + 2 < p.vocab) dst[2] = v.z;
+                        if (f + 3 < p.vocab) dst[3] = v.w;
+                    }
                 }
             }
-            // largest logit of the token among this lane's features, lowest id on ties; then over the
-            // token's eight lanes (the packed key orders by logit, then by lower id)
-            unsigned long long mine = 0ull;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const unsigned long long key = f + k < p.vocab ? pack_argmax_key(orderable_f32(v[k]), f + k) : 0ull;
-                if (key > mine) mine = key;
-            }
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-                const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, mine, o);
-                if (other > mine) mine = other;
-            }
-            if (tv && (lane & 7) == 0) {
-                if (mine) atomicMax(p.best + t0 + t, mine);
-                // the group's maximum of the token (0: no valid feature): a threshold source for a later top-k
-                if (p.warp_max) p.warp_max[(size_t)(t0 + t) * p.n_warp_max + (m0 >> 5) + quarter] = (uint32_t)(mine >> 32);
-            }
         }
     }
 }
 
-template <int MODE>
-__device__ __forceinline__ void epi_whole(const EpiParams& p, const float (&a)[EPI_COLS], float* scr, int m0, int t0, int ncols,
-                                          int quarter, int lane) {
-    EpiOperand<MODE> o;
-    epi_stage(a, scr, lane);
-    epi_unit<MODE, false>(p, o, scr, m0, t0, ncols, quarter, lane);
-}
+// Whether an epilogue multiplies by the RMSNorm scale of its tokens.
+__host__ __device__ constexpr bool epi_scaled(int mode) { return mode == EPI_QKV || mode == EPI_SWIGLU || mode == EPI_LMHEAD; }
 
-__device__ __forceinline__ void epi_dispatch(int mode, const EpiParams& p, const uint32_t (&r)[EPI_COLS], const float* rs, float* scr,
-                                             int m0, int t0, int ncols, int quarter, int lane) {
+// The kernels of 576 threads have no registers to hold a chunk beside the rows it meets (loaded early, the residual rows are
+// spilled and the epilogue of a 256 x 256 tile takes 50 k cycles instead of 31 k).
+__host__ __device__ constexpr bool epi_late(int mode) { return mode == EPI_QKV || mode == EPI_RESID; }
+
+// A chunk's accumulators, summed, through the epilogue.
+template <int MODE>
+__device__ __forceinline__ void epi_chunk(const EpiParams& p, EpiOperand<MODE>& o, const uint32_t (&r)[EPI_COLS], const float* rs, float* scr,
+                                          int m0, int t0, int ncols, int quarter, int lane) {
     float a[EPI_COLS];
 #pragma unroll
-    for (int j = 0; j < EPI_COLS; ++j) a[j] = __uint_as_float(r[j]);
-    if (rs != nullptr) {
-#pragma unroll
-        for (int j = 0; j < EPI_COLS; ++j) a[j] *= rs[j];
+    for (int j = 0; j < EPI_COLS; j += 4) {
+        const float4 k = epi_scaled(MODE) ? *reinterpret_cast<const float4*>(rs + j) : make_float4(1.f, 1.f, 1.f, 1.f);
+        a[j] = __uint_as_float(r[j]); a[j + 1] = __uint_as_float(r[j + 1]); a[j + 2] = __uint_as_float(r[j + 2]); a[j + 3] = __uint_as_float(r[j + 3]);
+        if (epi_scaled(MODE)) { a[j] *= k.x; a[j + 1] *= k.y; a[j + 2] *= k.z; a[j + 3] *= k.w; }
     }
-    switch (mode) {
-        case EPI_PLAIN: epi_whole<EPI_PLAIN>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_QKV: epi_whole<EPI_QKV>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_RESID: epi_whole<EPI_RESID>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        case EPI_SWIGLU: epi_whole<EPI_SWIGLU>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-        default: epi_whole<EPI_LMHEAD>(p, a, scr, m0, t0, ncols, quarter, lane); break;
-    }
+    epi_unit<MODE, epi_late(MODE)>(p, o, a, scr, m0, t0, ncols, quarter, lane);
 }
 
 // RMSNorm scales of the tokens n0 .. n0 + n_valid - 1 from the partial sums of x^2 their source rows
@@ -565,7 +574,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  : "memory");
 }
 
-template <int VARIANT>
+template <int VARIANT, int MODE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) {
     constexpr bool KSPLIT = VARIANT == GEMM_KSPLIT;
@@ -580,7 +589,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
     uint64_t* rs_bar = acce_bar + 1;                    // RMSNorm scales of the item's tokens are in rs_s
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rs_bar + 1);
     float* rs_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + GEMM_BAR_BYTES);   // [2][rs stride]
-    float* scr_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + gemm_scr_offset(g.TN));   // [epilogue warp][16][33]
+    float* scr_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + gemm_scr_offset(g.TN));   // [epilogue warp][16][36]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_cta = gridDim.x, cta = blockIdx.x;
@@ -699,7 +708,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
         const int grp = e >> 2;               // the groups take the 16-token chunks round robin
         constexpr int NGRP = GEMM_EPI_WARPS / 4;
         const int quarter = warp & 3;         // TMEM lane quarter this warp may read
-        const bool scaled = p.ssq_in != nullptr;
+        constexpr bool scaled = epi_scaled(MODE);
         float* const scr = scr_s + e * EPI_SCR_FLOATS;
         bool ok = true;
         GemmWork w;
@@ -762,6 +771,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     for (int c = c_lo; c < c_hi; ++c) {
                         if ((nth++ & (NGRP - 1)) != grp) continue;
                         const int m0 = w.pair * 256 + mt * 128;
+                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                        EpiOperand<MODE> opnd;
+                        if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
                         uint32_t own[EPI_COLS], r[EPI_COLS];
                         tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
                         tmem_ld_wait();
@@ -788,8 +800,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                                 }
                             }
                         }
-                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                        if (m0 < p.N) epi_dispatch(p.mode, p, r, scaled ? rsi + c * EPI_COLS : nullptr, scr, m0, tc0, ncols, quarter, lane);
+                        if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
                     }
                 // the last warp of the tile's CTAs to finish reading clears the counters for the next launch
                 __syncwarp();
@@ -803,6 +814,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                 for (int ci = grp; ci < total_chunks; ci += NGRP) {
                     const int mt = w.mt_lo + ci / nchunks, c = ci % nchunks;
                     const int m0 = w.pair * 256 + mt * 128;
+                    const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                    EpiOperand<MODE> opnd;
+                    if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
                     uint32_t r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                     tmem_ld_wait();
@@ -810,8 +824,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(acce_bar);
                     }
-                    const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                    if (m0 < p.N) epi_dispatch(p.mode, p, r, scaled ? rsi + c * EPI_COLS : nullptr, scr, m0, tc0, ncols, quarter, lane);
+                    if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
                 }
                 if (grp >= total_chunks) {   // a group without any chunk still releases the accumulators
                     tc_fence_before();
@@ -883,7 +896,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     }
                 }
                 const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                if (m0 < p.N) epi_dispatch(p.mode, p, r, scaled ? rsi + c * EPI_COLS : nullptr, scr, m0, tc0, ncols, quarter, lane);
+                EpiOperand<MODE> opnd;
+                if (m0 < p.N) {
+                    if (!epi_late(MODE)) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
+                    epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
+                }
             }
             if (grp >= total_chunks) {
                 tc_fence_before();

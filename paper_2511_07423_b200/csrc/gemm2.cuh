@@ -92,7 +92,7 @@ __host__ __device__ __forceinline__ bool gemm2_work(const Gemm2Params& g, int cl
     return true;
 }
 
-template <bool DUO>
+template <bool DUO, int MODE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Gemm2Params g, EpiParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -106,7 +106,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     uint64_t* rs_bar = acce_bar + 1;                    // own: RMSNorm scales of the item's tokens are in rs_s
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rs_bar + 1);
     float* rs_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + GEMM_BAR_BYTES);   // [2][rs stride]
-    float* scr_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + gemm_scr_offset(g.TN));   // [epilogue warp][16][33]
+    float* scr_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + gemm_scr_offset(g.TN));   // [epilogue warp][16][36]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
@@ -234,7 +234,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         const int grp = e >> 2;               // the groups take the 16-token chunks round robin
         constexpr int NGRP = GEMM_EPI_WARPS / 4;
         const int quarter = warp & 3;         // TMEM lane quarter this warp may read
-        const bool scaled = p.ssq_in != nullptr;
+        constexpr bool scaled = epi_scaled(MODE);
         const uint32_t acce_c = mapa_rank(smem_u32(acce_bar), 0);
         float* const scr = scr_s + e * EPI_SCR_FLOATS;
         bool ok = true;
@@ -305,6 +305,9 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     for (int c = c_lo; c < c_hi; ++c) {
                         if ((nth++ & (NGRP - 1)) != grp) continue;
                         const int m0 = row0 + mt * 128;
+                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                        EpiOperand<MODE> opnd;
+                        if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
                         uint32_t own[EPI_COLS], r[EPI_COLS];
                         tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
                         if (DUO) {
@@ -339,8 +342,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                                 }
                             }
                         }
-                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                        if (m0 < p.N) epi_dispatch(p.mode, p, r, scaled ? rsi + c * EPI_COLS : nullptr, scr, m0, tc0, ncols, quarter, lane);
+                        if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
                     }
                 __syncwarp();
                 if (lane == 0 && atomicAdd(g.fix_flag + 2 * g.n_sm + cnt, 1) == S * GEMM_EPI_WARPS - 1) {
@@ -352,6 +354,9 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             for (int ci = grp; ci < total_chunks; ci += NGRP) {
                 const int mt = ci / nchunks, c = ci % nchunks;
                 const int m0 = row0 + mt * 128;
+                const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                EpiOperand<MODE> opnd;
+                if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
                 uint32_t r[EPI_COLS];
                 tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                 if (DUO) {
@@ -367,8 +372,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     tc_fence_before();
                     if (lane == 0) mbar_arrive_cluster(acce_c);
                 }
-                const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                if (m0 < p.N) epi_dispatch(p.mode, p, r, scaled ? rsi + c * EPI_COLS : nullptr, scr, m0, tc0, ncols, quarter, lane);
+                if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
             }
             if (grp >= total_chunks) {   // a group without any chunk still releases the accumulators
                 tc_fence_before();

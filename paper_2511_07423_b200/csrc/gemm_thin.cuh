@@ -224,7 +224,7 @@ thin_kernel(const __grid_constant__ CUtensorMap tmB, ThinParams g, EpiParams p) 
         // ------------------------------------------------------------ epilogue
         const int e = warp - 2, grp = e >> 2;   // two groups take the 16-token chunks in turn
         const int quarter = warp & 3;           // TMEM lane quarter this warp may read
-        constexpr bool scaled = MODE == EPI_QKV || MODE == EPI_SWIGLU || MODE == EPI_LMHEAD;
+        constexpr bool scaled = epi_scaled(MODE);
         float* const scr = reinterpret_cast<float*>(smem + g.n_stages * stage_bytes - THIN_SCR_BYTES) + e * EPI_SCR_FLOATS;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const int m0 = tile * 128;
@@ -303,9 +303,8 @@ thin_kernel(const __grid_constant__ CUtensorMap tmB, ThinParams g, EpiParams p) 
                 for (int v = 0; v < EPI_COLS; ++v) a[v] *= rs_s[c * EPI_COLS + v];
             }
             const int tc = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-            epi_stage(a, scr, lane);
             if (c != c_first) epi_load<MODE>(p, opnd, m0, tc, ncols, quarter, lane);
-            epi_unit<MODE, true>(p, opnd, scr, m0, tc, ncols, quarter, lane);
+            epi_unit<MODE>(p, opnd, a, scr, m0, tc, ncols, quarter, lane);
         }
     }
     if (S > 1) cluster_wait();   // nobody leaves while another part may still send to it

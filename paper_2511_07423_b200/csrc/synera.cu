@@ -446,13 +446,18 @@ static cudaError_t kernel_smem(K kernel, int bytes) {
     if (e == cudaSuccess && bytes > 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
+template <int MODE>
+static cudaError_t projection_smem() {   // the projection kernels with one epilogue
+    const cudaError_t all[] = {kernel_smem(gemm_kernel<GEMM_WAVES, MODE>, GEMM_SMEM_MAX), kernel_smem(gemm_kernel<GEMM_KSPLIT, MODE>, GEMM_SMEM_MAX),
+                               kernel_smem(gemm_kernel<GEMM_RSPLIT, MODE>, GEMM_SMEM_MAX), kernel_smem(gemm2_kernel<false, MODE>, GEMM_SMEM_MAX),
+                               kernel_smem(gemm2_kernel<true, MODE>, GEMM_SMEM_MAX), kernel_smem(thin_kernel<MODE>, THIN_SMEM_MAX)};
+    for (cudaError_t e : all)
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
+}
 static cudaError_t set_kernel_attributes() {
     const cudaError_t all[] = {
-        kernel_smem(gemm_kernel<GEMM_WAVES>, GEMM_SMEM_MAX), kernel_smem(gemm_kernel<GEMM_KSPLIT>, GEMM_SMEM_MAX),
-        kernel_smem(gemm_kernel<GEMM_RSPLIT>, GEMM_SMEM_MAX), kernel_smem(gemm2_kernel<false>, GEMM_SMEM_MAX),
-        kernel_smem(gemm2_kernel<true>, GEMM_SMEM_MAX), kernel_smem(thin_kernel<EPI_PLAIN>, THIN_SMEM_MAX),
-        kernel_smem(thin_kernel<EPI_QKV>, THIN_SMEM_MAX), kernel_smem(thin_kernel<EPI_RESID>, THIN_SMEM_MAX),
-        kernel_smem(thin_kernel<EPI_SWIGLU>, THIN_SMEM_MAX), kernel_smem(thin_kernel<EPI_LMHEAD>, THIN_SMEM_MAX),
+        projection_smem<EPI_PLAIN>(), projection_smem<EPI_QKV>(), projection_smem<EPI_RESID>(), projection_smem<EPI_SWIGLU>(), projection_smem<EPI_LMHEAD>(),
         kernel_smem(attn_kernel<128>, AttnSmem<128>::TOTAL), kernel_smem(attn_kernel<64>, AttnSmem<64>::TOTAL),
         kernel_smem(attn2_kernel<128>, Attn2Smem<128>::TOTAL), kernel_smem(attn2_kernel<64>, Attn2Smem<64>::TOTAL),
         kernel_smem(attn_thin_kernel<128>, AttnThinSmem<128>::TOTAL), kernel_smem(attn_thin_kernel<64>, AttnThinSmem<64>::TOTAL),
@@ -1296,6 +1301,16 @@ static int gemm_plan(int T, int packed_rows, int K, int n_sm, int mode, bool may
     return SYN_OK;
 }
 
+// The instance of a projection kernel for the epilogue `mode`.
+#define EPI_SWITCH(mode, call)                                           \
+    switch (mode) {                                                      \
+        case EPI_QKV: { constexpr int MODE = EPI_QKV; call; break; }       \
+        case EPI_RESID: { constexpr int MODE = EPI_RESID; call; break; }   \
+        case EPI_SWIGLU: { constexpr int MODE = EPI_SWIGLU; call; break; } \
+        case EPI_LMHEAD: { constexpr int MODE = EPI_LMHEAD; call; break; } \
+        default: { constexpr int MODE = EPI_PLAIN; call; break; }          \
+    }
+
 // One projection with the epilogue `ep`; `plan_mode` = the epilogue its schedule is made for (the
 // same, except in the test hook, which runs any schedule with the plain store epilogue).
 static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, int packed_rows, int K,
@@ -1314,9 +1329,9 @@ static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const 
     g.spin_limit = g_spin_limit;
     const int smem = gemm_fixed_smem(g.TN) + g.n_stages * gemm_stage_bytes(g.TN);
     cudaError_t le;
-    if (g.splits > 1) le = launch_pdl(gemm_kernel<GEMM_RSPLIT>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep);
-    else if (g.ksplit > 1) le = launch_pdl(gemm_kernel<GEMM_KSPLIT>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep);
-    else le = launch_pdl(gemm_kernel<GEMM_WAVES>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep);
+    EPI_SWITCH(ep.mode, le = g.splits > 1 ? launch_pdl(gemm_kernel<GEMM_RSPLIT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep)
+                        : g.ksplit > 1 ? launch_pdl(gemm_kernel<GEMM_KSPLIT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep)
+                                       : launch_pdl(gemm_kernel<GEMM_WAVES, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep));
     return le == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
@@ -1431,13 +1446,7 @@ static int launch_thin(syn_model* prof_m, int cls, int n_sm, int* status, const 
     thin_plan(ep.T, packed_rows, K, n_sm, g);
     g.w = w_packed; g.status = status; g.spin_limit = g_spin_limit;
     cudaError_t e;
-    switch (ep.mode) {
-        case EPI_QKV: e = launch_thin_mode<EPI_QKV>(g, xm, ep, st); break;
-        case EPI_RESID: e = launch_thin_mode<EPI_RESID>(g, xm, ep, st); break;
-        case EPI_SWIGLU: e = launch_thin_mode<EPI_SWIGLU>(g, xm, ep, st); break;
-        case EPI_LMHEAD: e = launch_thin_mode<EPI_LMHEAD>(g, xm, ep, st); break;
-        default: e = launch_thin_mode<EPI_PLAIN>(g, xm, ep, st); break;
-    }
+    EPI_SWITCH(ep.mode, e = launch_thin_mode<MODE>(g, xm, ep, st));
     return e == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
@@ -1464,8 +1473,9 @@ static int launch_proj(syn_model* prof_m, int cls, int n_sm, int* status, const 
     g2.fix_part = fix_part; g2.fix_flag = fix_flag;
     const bool duo = kind == PAIR_DUO;
     const int smem = gemm_fixed_smem(g2.TN) + g2.n_stages * gemm2_stage_bytes(g2.TN, duo);
-    const cudaError_t le = duo ? launch_pdl_clusters(gemm2_kernel<true>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->duo, xm.box, g2, ep)
-                               : launch_pdl_clusters(gemm2_kernel<false>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->quad, xm.box, g2, ep);
+    cudaError_t le;
+    EPI_SWITCH(ep.mode, le = duo ? launch_pdl_clusters(gemm2_kernel<true, MODE>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->duo, xm.box, g2, ep)
+                                 : launch_pdl_clusters(gemm2_kernel<false, MODE>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->quad, xm.box, g2, ep));
     return le == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
