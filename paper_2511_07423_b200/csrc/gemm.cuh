@@ -124,12 +124,12 @@ struct EpiOperand {
     int slot;
 };
 
-template <int MODE>
-__device__ __forceinline__ void epi_load_rope(const EpiParams& p, EpiOperand<MODE>& o, int t0, int ncols, int quarter, int lane) {
+template <int MODE>   // passes i0 .. i0 + n - 1 of four, each four tokens
+__device__ __forceinline__ void epi_load_rope(const EpiParams& p, EpiOperand<MODE>& o, int t0, int ncols, int quarter, int lane, int i0 = 0, int n = 4) {
     const int tq = lane >> 3, c0 = (lane & 7) * 4;
     const int half = p.hd >> 1, dim = 16 * (quarter & ((half >> 4) - 1)) + (c0 & 15);   // lower dim of the pair
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = i0; i < i0 + n; ++i) {
         const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)(t0 + tq + 4 * i) * half + dim);   // 4 x (cos, sin)
         const bool tv = tq + 4 * i < ncols;
         o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)] = tv ? __ldg(cs) : make_float4(1.f, 0.f, 1.f, 0.f);
@@ -169,7 +169,7 @@ template <int MODE, bool LATE = false>
 __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float (&a)[EPI_COLS], float* scr, int m0,
                                          int t0, int ncols, int quarter, int lane) {
     if (MODE != EPI_SWIGLU && (MODE != EPI_LMHEAD || p.logits)) epi_stage(a, scr, lane);
-    if (LATE) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
+    if (LATE && MODE != EPI_QKV) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
     const int tq = lane >> 3, c0 = (lane & 7) * 4;   // token (+ 4 i) and first of four columns of this lane
     if (MODE == EPI_PLAIN) {
         const int f = m0 + quarter * 32 + c0;
@@ -218,7 +218,7 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
         const int region0 = which == 0 ? 0 : (which == 1 ? p.q_dim : p.q_dim + p.kv_dim);
         const int half = p.hd >> 1, hd_log = p.hd == 128 ? 7 : 6;   // head_dim is 64 or 128
         const size_t page_stride = (size_t)p.n_kv_heads * 2 * 16 * p.hd;
-        const int my_slot = o.slot;
+        const int my_slot = LATE ? ((which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0) : o.slot;
         if (which < 2) {
             // q and k tiles: columns 0..15 of the block are the dims [d0, d0 + 16) of one head, columns 16..31
             // the same dims + hd/2 (rope_tile_feature); a lane rotates its four columns with their partners
@@ -228,6 +228,7 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
             const int dim = 16 * (quarter & ((1 << g_log) - 1)) + (c0 & 15);            // lower dim of the pair
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+                if (LATE) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane, i, 1);
                 const float4 w0 = o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)], w1 = o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)];
                 const int t = tq + 4 * i;
                 const float4 mine = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
