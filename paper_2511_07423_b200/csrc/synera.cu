@@ -1338,10 +1338,61 @@ static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const 
 // Schedules of the CTA-pair kernel (gemm2.cuh).
 enum { PAIR_NONE = 0, PAIR_QUAD = 1, PAIR_DUO = 2 };
 
+// Estimated time, in SM cycles, of a projection on the one-CTA kernel (kind PAIR_NONE) or on CTA pairs: the work of its first
+// and of its last CTA or cluster, whichever is more.  An item costs its k-blocks times the larger of its tensor-core
+// cycles and of its operands at 57 bytes a cycle and SM from L2, its epilogue per output element, the accumulators it
+// stores and reads of others, and a fixed part; the coefficients are a least-squares fit to 540 event times (264 to 2 048 tokens,
+// all projections of the 1B, 8B and 32B shapes, three kernels; rms error 5, 5 and 9 %).
+static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int force, Gemm2Params& g, int& n_cl);
+static double proj_cost(int T, int packed_rows, int K, int n_sm, int mode, int kind) {
+    struct Fit { double main, epi[5], exch, item, fixed; };   // epi: PLAIN, QKV, RESID, SWIGLU, LMHEAD
+    static const Fit QUAD = {1.292, {0.07, 0.302, 0.190, 0.073, 0.283}, 0.302, -1650, 21300}, DUO = {1.152, {0.0, 0.302, 0.057, -0.093, 0.165}, 0.369, 5080, 20200},
+                     ONE = {1.138, {0.09, 0.362, 0.213, 0.086, 0.319}, 0.276, -2420, 20400};
+    const Fit& f = kind == PAIR_QUAD ? QUAD : (kind == PAIR_DUO ? DUO : ONE);
+    auto width = [&](int TN, int tt) { return (double)((std::min(TN, T - tt * TN) + 15) / 16 * 16); };
+    auto item = [&](int kb, int mt, double n, double mma, double bytes, double epi_share, double exch) {
+        return f.main * kb * std::max(mma, bytes / 57.0) + 128.0 * mt * n * (f.epi[mode] * epi_share + f.exch * exch) + f.item;
+    };
+    double worst = 0.0;
+    if (kind == PAIR_NONE) {
+        GemmParams g;
+        memset(&g, 0, sizeof(g));
+        int n_cta = 0;
+        if (gemm_plan(T, packed_rows, K, n_sm, mode, mode != EPI_RESID, g, n_cta)) return 1e30;
+        for (int cta : {0, n_cta - 1}) {
+            double sum = f.fixed;
+            GemmWork w;
+            for (int i = 0; g.ksplit > 1 ? gemm_work<true>(g, cta, n_cta, i, w) : gemm_work<false>(g, cta, n_cta, i, w); ++i) {
+                const int mt = w.mt_hi - w.mt_lo, S = g.splits;
+                const double n = width(g.TN, w.tt);
+                const double share = w.role == 1 ? 0.0 : 1.0 / S;
+                const double exch = w.role == 1 ? 1.0 : (w.role == 2 ? g.ksplit - 1.0 : 2.0 * (S - 1) / S);
+                sum += item(w.kb1 - w.kb0, mt, n, mt == 2 ? 4 * n : 576.0, 16384.0 * mt + 128 * n, share, exch);   // one accumulator: 144 cycles an MMA
+            }
+            worst = std::max(worst, sum);
+        }
+        return worst;
+    }
+    Gemm2Params g;
+    int n_cl = 0;
+    if (gemm2_plan(T, packed_rows, K, n_sm, mode, kind, g, n_cl) != kind) return 1e30;
+    const int mt = kind == PAIR_QUAD ? 2 : 1;
+    for (int cl : {0, n_cl - 1}) {
+        double sum = f.fixed;
+        Gemm2Work w;
+        for (int i = 0; gemm2_work(g, cl, n_cl, i, w); ++i) {
+            const double n = width(g.TN, w.tt);
+            sum += item(w.kb1 - w.kb0, mt, n, 2 * n * mt, 16384.0 * mt + 64 * n, 1.0 / w.nsplit, 2.0 * (w.nsplit - 1) / w.nsplit);
+        }
+        worst = std::max(worst, sum);
+    }
+    return worst;
+}
+
 // Launch shape of a projection on CTA pairs, or PAIR_NONE when the one-CTA kernel serves it better
 // (few tokens: the pair kernel's token tiles are the natural 256-token cut, it has no narrow tiles).
 // Host arithmetic only.  `force`: PAIR_QUAD / PAIR_DUO to take that item shape regardless (test hook).
-static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int force, Gemm2Params& g, int& n_cl) {
+static int gemm2_plan_by_rule(int T, int packed_rows, int K, int n_sm, int mode, int force, Gemm2Params& g, int& n_cl) {
     memset(&g, 0, sizeof(g));
     const int n_pairs = (packed_rows + 255) / 256, n_cl_max = n_sm / 2;
     g.num_kb = (K + 63) / 64;
@@ -1393,6 +1444,23 @@ static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int for
     g.n_stages = gemm2_stages(g.TN, kind == PAIR_DUO);
     if (g.n_stages < 2 || g.TN < 16 || g.TN > 256 || (g.n_tt - 1) * g.TN >= T) return PAIR_NONE;
     return kind;
+}
+
+// The rule above, unless another kernel is estimated at least 8 % faster.  Over the projections of a layer at the sizes the
+// estimate was fitted to, the choice costs 1.9 % more time than the best kernel everywhere would (at most 9.6 %; the rule alone
+// 5.1 and 30 %: it keeps gate/up of the 8B shape at 688 tokens on the one-CTA kernel, 153 us against 128, and those of the 1B
+// shape at 768 tokens on 512-feature items, 65 against 53).
+static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int force, Gemm2Params& g, int& n_cl) {
+    const int by_rule = gemm2_plan_by_rule(T, packed_rows, K, n_sm, mode, force, g, n_cl);
+    if (force != PAIR_NONE || T < 256 || n_sm < 2) return by_rule;
+    int best = by_rule;
+    double limit = proj_cost(T, packed_rows, K, n_sm, mode, by_rule) / 1.08;
+    for (int kind : {PAIR_NONE, PAIR_QUAD, PAIR_DUO}) {
+        const double c = kind == by_rule ? limit : proj_cost(T, packed_rows, K, n_sm, mode, kind);
+        if (c < limit) { best = kind; limit = c; }
+    }
+    if (best == by_rule || best == PAIR_NONE) return best;
+    return gemm2_plan_by_rule(T, packed_rows, K, n_sm, mode, best, g, n_cl);
 }
 
 constexpr int THIN_MAX_TOKENS = 512;
@@ -1453,21 +1521,33 @@ static int launch_thin(syn_model* prof_m, int cls, int n_sm, int* status, const 
 // What a caller may ask of launch_proj instead of the kernel the shape calls for (test hook).
 enum { PROJ_AUTO = 0, PROJ_QUAD = PAIR_QUAD, PROJ_DUO = PAIR_DUO, PROJ_THIN, PROJ_NOT_THIN };
 
-// One projection with the epilogue `ep` on whichever kernel its shape calls for.  `plan_mode` = the
-// epilogue the schedule is made for (the same, except in the test hook); `force`: test hook.
-static int launch_proj(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, const WMaps* wm, int packed_rows,
-                       int K, const XMaps& xm, const EpiParams& ep, cudaStream_t st, float* fix_part, int* fix_flag,
-                       int plan_mode = -1, int force = PROJ_AUTO) {
-    if (plan_mode < 0) plan_mode = ep.mode;
-    if (force == PROJ_THIN || (force == PROJ_AUTO && g_schedule != 1 && thin_takes(ep.T, packed_rows, K, n_sm, plan_mode)))
-        return launch_thin(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm, ep, st);
-    const int force_pair = force == PROJ_QUAD || force == PROJ_DUO ? force : PAIR_NONE;
+// Which kernel a projection takes and how, worked out once for the layers of a step.
+struct ProjPlan {
+    bool thin;
+    int kind;   // PAIR_NONE: the one-CTA kernel
     Gemm2Params g2;
-    int n_cl = 0;
-    const int kind = (wm && (g_schedule != 1 || force_pair != PAIR_NONE)) ? gemm2_plan(ep.T, packed_rows, K, n_sm, plan_mode, force_pair, g2, n_cl)
-                                                                            : PAIR_NONE;
-    if (kind == PAIR_NONE) return launch_gemm(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm.box, ep, st, fix_part, fix_flag, plan_mode);
+    int n_cl;
+};
+static ProjPlan proj_plan(int T, int packed_rows, int K, int n_sm, int plan_mode, int force = PROJ_AUTO) {
+    ProjPlan pl;
+    pl.thin = force == PROJ_THIN || (force == PROJ_AUTO && g_schedule != 1 && thin_takes(T, packed_rows, K, n_sm, plan_mode));
+    const int force_pair = force == PROJ_QUAD || force == PROJ_DUO ? force : PAIR_NONE;
+    pl.n_cl = 0;
+    pl.kind = !pl.thin && (g_schedule != 1 || force_pair != PAIR_NONE) ? gemm2_plan(T, packed_rows, K, n_sm, plan_mode, force_pair, pl.g2, pl.n_cl) : PAIR_NONE;
+    return pl;
+}
+
+// One projection with the epilogue `ep` on the kernel its plan says.  `plan_mode` = the epilogue the schedule is made for (the
+// same, except in the test hook).
+static int launch_proj(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, const WMaps* wm, int packed_rows,
+                       int K, const XMaps& xm, const EpiParams& ep, cudaStream_t st, float* fix_part, int* fix_flag, const ProjPlan& pl,
+                       int plan_mode = -1) {
+    if (plan_mode < 0) plan_mode = ep.mode;
+    if (pl.thin) return launch_thin(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm, ep, st);
+    if (pl.kind == PAIR_NONE) return launch_gemm(prof_m, cls, n_sm, status, w_packed, packed_rows, K, xm.box, ep, st, fix_part, fix_flag, plan_mode);
     if (!fix_part || !fix_flag) return SYN_E_INVALID_ARG;
+    Gemm2Params g2 = pl.g2;
+    const int n_cl = pl.n_cl, kind = pl.kind;
     ProfScope prof(cls >= 0 ? prof_m : nullptr, cls, st);
     g2.status = status; g2.spin_limit = g_spin_limit;
     g2.fix_part = fix_part; g2.fix_flag = fix_flag;
@@ -1597,6 +1677,8 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     // the writers of the residual stream: x += D, next operand bf16(x * gain), new partial sums
     EpiParams resid = base;
     resid.mode = EPI_RESID; resid.N = d; resid.d = d; resid.x = m->x; resid.xg = m->xn; resid.ssq_out = m->ssq;
+    // (the projections' plans, some 6 us each, are made in the first layer, while the kernels before run)
+    ProjPlan pl_qkv, pl_o, pl_gu, pl_d;
     int r;
     for (uint32_t l = 0; l < c.n_layers; ++l) {
         EpiParams e = scaled;
@@ -1604,26 +1686,31 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
         e.q = m->q; e.q_dim = q_dim; e.kv_dim = kv_dim; e.hd = c.head_dim; e.n_kv_heads = c.n_kv_heads;
         e.page_size = kv->page_size; e.rope = m->rope; e.pool = kv->pool + kv->layer_elems * l;
         e.slot = p->d<int>(p->o_slot);
-        if ((r = launch_proj(m, 1, m->n_sm, m->status_dev, m->wqkv[l], &m->tm_wqkv[l], m->qkv_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag)))
+        if (l == 0) pl_qkv = proj_plan(T, m->qkv_rows, d, m->n_sm, EPI_QKV);
+        if ((r = launch_proj(m, 1, m->n_sm, m->status_dev, m->wqkv[l], &m->tm_wqkv[l], m->qkv_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag, pl_qkv)))
             return r;
         if ((r = launch_attention(m, kv, p, l, m->tm_q, m->attn, st))) return r;
         e = resid;
         e.gain = m->norm2[l];
-        if ((r = launch_proj(m, 4, m->n_sm, m->status_dev, m->wo[l], &m->tm_wo[l], d, q_dim, m->tm_attn, e, st, m->fix_part, m->fix_flag)))
+        if (l == 0) pl_o = proj_plan(T, d, q_dim, m->n_sm, EPI_RESID);
+        if ((r = launch_proj(m, 4, m->n_sm, m->status_dev, m->wo[l], &m->tm_wo[l], d, q_dim, m->tm_attn, e, st, m->fix_part, m->fix_flag, pl_o)))
             return r;
         e = scaled;
         e.mode = EPI_SWIGLU; e.N = m->gu_rows; e.act = m->act; e.f_pad = m->f_pad;
-        if ((r = launch_proj(m, 5, m->n_sm, m->status_dev, m->wgu[l], &m->tm_wgu[l], m->gu_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag)))
+        if (l == 0) pl_gu = proj_plan(T, m->gu_rows, d, m->n_sm, EPI_SWIGLU);
+        if ((r = launch_proj(m, 5, m->n_sm, m->status_dev, m->wgu[l], &m->tm_wgu[l], m->gu_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag, pl_gu)))
             return r;
         e = resid;
         e.gain = l + 1 < c.n_layers ? m->norm1[l + 1] : m->final_norm;
-        if ((r = launch_proj(m, 6, m->n_sm, m->status_dev, m->wd[l], &m->tm_wd[l], d, m->f_pad, m->tm_act, e, st, m->fix_part, m->fix_flag)))
+        if (l == 0) pl_d = proj_plan(T, d, m->f_pad, m->n_sm, EPI_RESID);
+        if ((r = launch_proj(m, 6, m->n_sm, m->status_dev, m->wd[l], &m->tm_wd[l], d, m->f_pad, m->tm_act, e, st, m->fix_part, m->fix_flag, pl_d)))
             return r;
     }
     EpiParams e = scaled;
     e.mode = EPI_LMHEAD; e.N = m->v_rows; e.vocab = c.vocab; e.logits = logits_out; e.best = m->best;
     e.warp_max = warp_max; e.n_warp_max = m->v_rows / 32;
-    if ((r = launch_proj(m, 7, m->n_sm, m->status_dev, m->lm_head, &m->tm_lm_head, m->v_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag)))
+    const ProjPlan pl_lm = proj_plan(T, m->v_rows, d, m->n_sm, EPI_LMHEAD);
+    if ((r = launch_proj(m, 7, m->n_sm, m->status_dev, m->lm_head, &m->tm_lm_head, m->v_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag, pl_lm)))
         return r;
     {
         ProfScope prof(m, 8, st);
@@ -1974,7 +2061,7 @@ extern "C" int syn_op_linear_as(const void* x, const void* w, float* y, int32_t 
     const int force = schedule_as <= EPI_LMHEAD ? PROJ_NOT_THIN : (schedule_as == 9 ? PROJ_THIN : (schedule_as == 5 || schedule_as == 7 ? PROJ_QUAD : PROJ_DUO));
     const int plan_mode = schedule_as <= EPI_LMHEAD ? schedule_as : (schedule_as == 7 || schedule_as == 8 ? EPI_RESID : EPI_PLAIN);
     r = launch_proj(nullptr, -1, g_lin.n_sm, g_lin.status, g_lin.packed, &g_lin.wm, (N + 127) / 128 * 128, K, xm, e, st, g_lin.fix_part,
-                    g_lin.fix_flag, plan_mode, force);
+                    g_lin.fix_flag, proj_plan(T, (N + 127) / 128 * 128, K, g_lin.n_sm, plan_mode, force), plan_mode);
     if (r) return r;
     CU_OK(cudaStreamSynchronize(st));
     int sflag = 0;
