@@ -347,6 +347,7 @@ struct syn_plan {
     syn_step_stats stats;
     int n_req = 0, T = 0, max_pages = 0, n_items = 0, n_cta = 0, n_groups = 0, n_parts = 0;
     int attn = ATTN_WARP;   // which attention kernel the work list was made for
+    bool wrapped = false;   // how it was cut
     // one device buffer and its pinned host mirror
     uint8_t *dev = nullptr, *host = nullptr;
     size_t cap = 0, used = 0;
@@ -789,6 +790,7 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Host-side result of planning one batch (no device involved).
 struct HostPlan {
     int T = 0, n_cta = 0, n_parts = 0, kind = ATTN_WARP;
+    bool wrapped = false;   // units laid end to end over the CTAs, cut where a CTA is full
     std::vector<int> pos, slot, cta_begin;
     std::vector<AttnItem> items;          // sorted by CTA
     std::vector<MergeGroup> groups;
@@ -805,6 +807,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     const int G = c.n_q_heads / c.n_kv_heads, Hkv = c.n_kv_heads;
     if (chunk_offsets[0] != 0) return SYN_E_INVALID_ARG;
     int64_t ctx_sum = 0, keys_seen = 0, kv_units = 0;
+    int max_chunk = 0;
     for (int i = 0; i < n_req; ++i) {
         const int64_t n = (int64_t)chunk_offsets[i + 1] - chunk_offsets[i];
         if (n < 1 || n > SYN_MAX_CHUNK) return SYN_E_CHUNK_LEN;
@@ -818,6 +821,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         for (int k = 0; k < used; ++k) worst = std::max(worst, (uint32_t)row[k]);
         if (worst >= n_pages) return SYN_E_PAGE_OOB;
         ctx_sum += ctx_lens[i];
+        max_chunk = std::max(max_chunk, (int)n);
         kv_units += ctx_lens[i] + n;
         keys_seen += n * (int64_t)ctx_lens[i] + n * (n + 1) / 2;
     }
@@ -854,78 +858,163 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     }
     // Attention work list: (request, kv head, token group, key range).  Cost of an item, in SM cycles: its blocks of
     // 64 keys times a time per block that grows with the number of 16-row query tiles (more tensor work per key byte),
-    // plus a fixed overhead per item, plus one more if it covers only part of its unit's keys (an fp32 partial, a merge);
-    // least-squares fits to per-CTA durations measured on full batches.
-    // Three kernels.  Unless one is asked for: the tensor-memory one (row tiles of 128: the same time per block whatever
-    // the number of rows, a larger fixed cost per item; a chunk of more than 64 / G tokens is one item there and several
-    // items that each read the request's keys in the others) when it is cheaper by 3 %: it draws more power, and under the
-    // power cap a step that uses it runs its other kernels at a lower clock; at 544 tokens of the 8B shape the two are
-    // level and the step is not faster with it.  Otherwise the kernel of half-SM CTAs when there are no more units
-    // (request, token group, kv head) than SMs, so that keys have to be shared out in parts, the full-SM one else.
-    struct AttnCost { int block[5], item, part; };
-    static const AttnCost COST_WARP_128 = {{0, 1040, 1200, 1500, 1540}, 5500, 3000}, COST_WARP_64 = {{0, 765, 843, 967, 1062}, 3200, 3000},
-                          COST_TENSOR = {{0, 1450, 1450, 1450, 1450}, 8000, 4000}, COST_THIN_128 = {{0, 2300, 2400, 2600, 2900}, 3000, 4000},
-                          COST_THIN_64 = {{0, 1300, 1400, 1600, 1800}, 3000, 4000};
-    const AttnCost& cost_warp = c.head_dim == 128 ? COST_WARP_128 : COST_WARP_64;
-    auto group_of = [&](int kind) { return kind == ATTN_TENSOR ? std::min(SYN_MAX_CHUNK, 128 / G) : std::min(16, 64 / G); };
-    auto blocks_of = [](int L) { return (L + 63) / 64; };
-    auto total_of = [&](int kind, const AttnCost& ac, int64_t* units) {
-        const int tpg = group_of(kind);
-        int64_t sum = 0, n_units = 0;
+    // plus a fixed overhead per item, plus one more if it covers only part of its unit's keys (an fp32 partial); `fixed` is the
+    // kernel's own, `merge` and `merge_tile` (per part and query tile) what the CTA that ends a unit's last part has still to
+    // do.  Fitted to per-CTA durations of some twenty batches of the 1B, 8B and 32B shapes (rms error 7 to 10 %); the half-SM
+    // kernel's are 5 to 15 % above its fit, which was taken where HBM was not yet the bound.
+    struct AttnCost { int kind, block[5], item, part, fixed, merge, merge_tile; };
+    static const AttnCost COSTS[2][3] = {
+        {{ATTN_WARP, {0, 760, 820, 965, 1050}, 3400, 1600, 4000, 5000, 400}, {ATTN_TENSOR, {0, 1100, 1100, 1100, 1100}, 2800, 3900, 7100, 12000, 200},
+         {ATTN_THIN, {0, 1050, 1170, 2080, 2200}, 4700, 2800, 4500, 4000, 350}},
+        {{ATTN_WARP, {0, 1110, 1200, 1600, 1650}, 6500, 2400, 5600, 6000, 800}, {ATTN_TENSOR, {0, 1300, 1300, 1300, 1300}, 3400, 6500, 11400, 25000, 200},
+         {ATTN_THIN, {0, 2600, 2800, 4500, 4800}, 3700, 2200, 6500, 4500, 700}}};
+    const AttnCost* costs = COSTS[c.head_dim == 128 ? 1 : 0];
+    struct Unit { int req, j0, nj, L, nb; int64_t bc; };   // the same for every kv head
+    struct Layout {
+        const AttnCost* ac = nullptr;
+        std::vector<Unit> units;
+        int slots = 0;             // CTAs
+        int64_t n_units = 0, total = 0, longest = 0;
+        int64_t limit = 0;         // of an item in equal parts; wrapped: of a CTA
+        bool wrapped = false;
+        int64_t estimate = 0;
+    };
+    auto tiles = [&](const Unit& u) { return (u.nj * G + 15) / 16; };
+    // equal parts that end, with a merge of a few of them, by `limit`
+    auto parts_of = [&](const Layout& y, const Unit& u, int64_t limit) {
+        if (u.nb * u.bc + y.ac->item <= limit) return 1;
+        const int min_blocks = y.ac->kind == ATTN_THIN ? 1 : 4, max_parts = y.ac->kind == ATTN_THIN ? ATTN_THIN_MAX_PARTS : 64;
+        const int64_t most = std::max<int64_t>(min_blocks, (limit - y.ac->item - y.ac->part - y.ac->merge - 4 * tiles(u) * y.ac->merge_tile) / u.bc);   // blocks of a part
+        return (int)std::min<int64_t>(std::min<int64_t>(max_parts, std::max(1, u.nb / min_blocks)), (u.nb + most - 1) / most);
+    };
+    // The units one after the other, longest first, each CTA filled up to `limit`: what does not fit goes on in the next CTA
+    // (so at most two partials a CTA).  emit(unit, head, first block, one past the last, cta); false if the CTAs do not suffice.
+    auto wrap = [&](const Layout& y, int64_t limit, auto&& emit) {
+        const AttnCost& k = *y.ac;
+        const int min_blocks = 2, max_parts = k.kind == ATTN_THIN ? ATTN_THIN_MAX_PARTS : 64;
+        int cta = 0;
+        int64_t load = 0;
+        for (const Unit& u : y.units)
+            for (int h = 0; h < Hkv; ++h) {
+                int at = 0, np = 0;
+                while (at < u.nb) {
+                    const int64_t room = limit - load - k.item;
+                    const int left = u.nb - at;
+                    int take = left * u.bc + (at ? k.part : 0) <= room ? left : (int)std::min<int64_t>(left - 1, (room - k.part) / u.bc);
+                    if (take < left && (take < min_blocks || room < k.part)) take = 0;
+                    if (take == 0 && load == 0) return false;
+                    if (take) {
+                        emit(u, h, at, at + take, cta);
+                        load += take * u.bc + k.item + (take < u.nb ? k.part : 0);
+                        at += take;
+                        if (++np > max_parts) return false;
+                    }
+                    if (at < u.nb) {
+                        load = 0;
+                        if (++cta >= y.slots) return false;
+                    }
+                }
+            }
+        return true;
+    };
+    auto lay_out = [&](const AttnCost& k, int slots) {
+        Layout y;
+        y.ac = &k;
+        y.slots = slots;
+        const int tpg = k.kind == ATTN_TENSOR ? std::min(SYN_MAX_CHUNK, 128 / G) : std::min(16, 64 / G);
+        y.units.reserve(n_req);
         for (int i = 0; i < n_req; ++i) {
             const int n = chunk_offsets[i + 1] - chunk_offsets[i];
             for (int j0 = 0; j0 < n; j0 += tpg) {
-                const int nj = std::min(tpg, n - j0);
-                sum += ((int64_t)blocks_of(ctx_lens[i] + j0 + nj) * ac.block[std::min(4, (nj * G + 15) / 16)] + ac.item) * Hkv;
-                n_units += Hkv;
+                const int nj = std::min(tpg, n - j0), L = ctx_lens[i] + j0 + nj, nb = (L + 63) / 64;
+                y.units.push_back({i, j0, nj, L, nb, 0});
+                const int64_t bc = y.units.back().bc = k.block[std::min(4, tiles(y.units.back()))];
+                y.total += (nb * bc + k.item) * Hkv;
+                y.longest = std::max(y.longest, nb * bc + k.item);
             }
         }
-        if (units) *units = n_units;
-        return sum;
-    };
-    int64_t n_units = 0;
-    const int64_t total_warp = total_of(ATTN_WARP, cost_warp, &n_units);
-    const int kind = attention ? attention
-                               : (total_of(ATTN_TENSOR, COST_TENSOR, nullptr) * 103 < total_warp * 100 ? ATTN_TENSOR : (n_units <= n_sm ? ATTN_THIN : ATTN_WARP));
-    hp.kind = kind;
-    const AttnCost& ac = kind == ATTN_TENSOR ? COST_TENSOR : (kind == ATTN_THIN ? (c.head_dim == 128 ? COST_THIN_128 : COST_THIN_64) : cost_warp);
-    const int tok_per_group = group_of(kind);
-    const int n_cta_max = kind == ATTN_THIN ? thin_ctas : n_sm;
-    const int64_t total_cost = total_of(kind, ac, &n_units);
-    auto block_cost = [&](int nj) { return (int64_t)ac.block[std::min(4, (nj * G + 15) / 16)]; };
-    // Parts of a unit: as many as bring a part down to `limit`, each of at least min_blocks.
-    const int min_blocks = kind == ATTN_THIN ? 1 : 4, max_parts = kind == ATTN_THIN ? ATTN_THIN_MAX_PARTS : 64;
-    auto parts_of = [&](int L, int nj, int64_t limit) {
-        const int nb = blocks_of(L);
-        const int64_t bc = block_cost(nj);
-        if (nb * bc + ac.item <= limit) return 1;
-        const int64_t most = std::max<int64_t>(min_blocks, (limit - ac.item - ac.part) / bc);   // blocks of a part
-        return (int)std::min<int64_t>(std::min<int64_t>(max_parts, std::max(1, nb / min_blocks)), (nb + most - 1) / most);
-    };
-    // The limit.  Units that are many to a CTA need no parts, or only where one unit alone exceeds a CTA's fair share.  With
-    // few units to a CTA the longest parts decide: the smallest limit for which there is at most one part per CTA, if that is
-    // less than the fair share of whole units and their overheads would come to.
-    int64_t limit = std::max<int64_t>(8 * block_cost(64) + ac.item, (total_cost + n_cta_max - 1) / n_cta_max);
-    if (n_units <= n_cta_max) {
-        auto n_parts_at = [&](int64_t lim) {
-            int64_t n = 0;
-            for (int i = 0; i < n_req; ++i) {
-                const int nt = chunk_offsets[i + 1] - chunk_offsets[i];
-                for (int j0 = 0; j0 < nt; j0 += tok_per_group) {
-                    const int nj = std::min(tok_per_group, nt - j0);
-                    n += (int64_t)parts_of(ctx_lens[i] + j0 + nj, nj, lim) * Hkv;
-                }
+        y.n_units = (int64_t)y.units.size() * Hkv;
+        const int64_t mean = (y.total + slots - 1) / slots;
+        // many units to a CTA: whole, only one that alone exceeds a CTA's fair share is cut
+        y.limit = std::max(mean, 8 * (int64_t)k.block[4] + k.item);
+        y.estimate = std::max(mean, std::min(y.longest, y.limit)) + k.fixed;
+        if (y.n_units > 2 * slots) return y;
+        // Few: whole units (as good as their number divides), equal parts of which there are no more than CTAs, or wrapped; with
+        // two CTAs or more to a unit equal parts are as even and have fewer merges (64 units of the 8B shape on 296 CTAs: 29.5 us
+        // wrapped, 28.8 in equal parts).  Equal parts of more than 128 units: SYN_STATIC_MAX_PARTS of them if that is enough to cut
+        // some, else two to a unit.
+        int64_t best = y.n_units <= slots ? y.longest : std::max(y.longest, (y.n_units + slots - 1) / slots * (y.total / y.n_units));
+        y.limit = y.longest;
+        auto cut = [&](int64_t most) {
+            auto fits = [&](int64_t lim) {
+                int64_t n = 0;
+                for (const Unit& u : y.units) n += (int64_t)parts_of(y, u, lim) * Hkv;
+                return n <= most;
+            };
+            int64_t lo = k.item, hi = y.longest;
+            while (hi - lo > 256) {   // the number of parts falls with the limit; at `hi` nothing is cut
+                const int64_t mid = (lo + hi) / 2;
+                if (fits(mid)) hi = mid; else lo = mid;
             }
-            return n;
+            int64_t part = 0;
+            for (const Unit& u : y.units) {
+                const int np = parts_of(y, u, hi);
+                part = std::max(part, (u.nb + np - 1) / np * u.bc + k.item + (np > 1 ? k.part + k.merge + std::min(np, 8) * tiles(u) * k.merge_tile : 0));
+            }
+            if (part >= best) return false;
+            best = part;
+            y.limit = hi;
+            return true;
         };
-        int64_t lo = ac.item + ac.part + min_blocks * (int64_t)ac.block[1], hi = lo;
-        for (int i = 0; i < n_req; ++i) hi = std::max(hi, blocks_of(ctx_lens[i] + (chunk_offsets[i + 1] - chunk_offsets[i])) * (int64_t)ac.block[4] + ac.item);
-        while (hi - lo > 256) {   // n_parts_at falls with the limit; at `hi` nothing is cut
-            const int64_t mid = (lo + hi) / 2;
-            if (n_parts_at(mid) <= n_cta_max) hi = mid; else lo = mid;
+        if (y.n_units <= slots) {
+            const bool many = 2 * y.n_units > SYN_STATIC_MAX_PARTS;
+            if (!cut(many ? std::min(slots, SYN_STATIC_MAX_PARTS) : slots) && many) cut(std::min<int64_t>(slots, 2 * y.n_units));
         }
-        limit = hi;
+        if (2 * y.n_units > slots) {
+            std::sort(y.units.begin(), y.units.end(), [](const Unit& p, const Unit& q) {
+                return p.nb * p.bc != q.nb * q.bc ? p.nb * p.bc > q.nb * q.bc : (p.req != q.req ? p.req < q.req : p.j0 < q.j0);
+            });
+            auto nothing = [](const Unit&, int, int, int, int) {};
+            int64_t lo = mean, hi = mean + 2 * (k.item + k.part) + 2 * (int64_t)k.block[4];
+            int64_t merge = 0;   // a cut unit has two or three parts
+            for (const Unit& u : y.units) merge = std::max<int64_t>(merge, k.merge + 2 * tiles(u) * k.merge_tile);
+            if (lo + merge < best && wrap(y, hi, nothing)) {
+                while (hi - lo > 64 + mean / 64) {
+                    const int64_t mid = (lo + hi) / 2;
+                    if (wrap(y, mid, nothing)) hi = mid; else lo = mid;
+                }
+                if (hi + merge < best) { best = hi + merge; y.limit = hi; y.wrapped = true; }
+            }
+        }
+        y.estimate = best + k.fixed;
+        return y;
+    };
+    // Three kernels; the estimated time decides.  The tensor-memory one (row tiles of 128: the same time per block whatever the
+    // number of rows; a chunk of more than 64 / G tokens is one item there and several items that each read the request's keys
+    // in the others) is looked at if some chunk fills more than two row tiles of 16 (below, it was 2 to 12 us behind the better of
+    // the others in every batch tried), and has to be 3 % better, 12 % where there are more than two units (request, token group, kv head) to an SM:
+    // it draws more power, and under the power cap a step that uses it runs its other kernels at a lower clock (544 tokens of the
+    // 8B shape: 109 us against 112 a layer, and the step takes as long).
+    Layout lay;
+    if (attention) {
+        const int slots = attention == ATTN_THIN ? thin_ctas : n_sm;
+        lay = lay_out(costs[attention - 1], slots);
+    } else {
+        // Whole units, one to an SM at most: left to the half-SM kernel, whose parts let the next projection in as they end.
+        lay = lay_out(costs[0], n_sm);
+        if (lay.n_units <= n_sm && !lay.wrapped) lay.estimate = INT64_MAX / 256;
+        const int64_t lead = lay.n_units > 2 * n_sm ? 112 : 103;
+        Layout other = lay_out(costs[2], 2 * n_sm);
+        if (other.estimate < lay.estimate) lay = other;
+        if (max_chunk * G > 32) {
+            other = lay_out(costs[1], n_sm);
+            if (other.estimate * lead < lay.estimate * 100) lay = other;
+        }
+        if (lay.ac->kind == ATTN_THIN && thin_ctas != lay.slots) lay = lay_out(costs[2], thin_ctas);
     }
+    const int kind = lay.ac->kind;
+    hp.kind = kind;
+    hp.wrapped = lay.wrapped;
     // Positions that no chunk of the batch writes, for the kernel that requests keys before the chunks' are written: up
     // to the first page of the request that holds a written slot, of whichever request.
     std::vector<int> safe;
@@ -942,44 +1031,49 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         }
     }
     std::vector<AttnItem> items;
-    std::vector<int> item_cost;
+    std::vector<int> item_cost, owner;
     std::vector<MergeGroup>& groups = hp.groups;
     groups.clear();
     int n_parts = 0;
-    for (int i = 0; i < n_req; ++i) {
-        const int b = chunk_offsets[i], n = chunk_offsets[i + 1] - b;
-        for (int j0 = 0; j0 < n; j0 += tok_per_group) {
-            const int nj = std::min(tok_per_group, n - j0);
-            const int L = ctx_lens[i] + j0 + nj, nb = blocks_of(L);
-            const int np = parts_of(L, nj, limit);
-            for (int h = 0; h < Hkv; ++h) {
-                if (np > 1) {
-                    MergeGroup g = {b + j0, nj, h, n_parts, np, 0, 0, 0};
-                    groups.push_back(g);
-                }
-                for (int k = 0; k < np; ++k) {
-                    const int b0 = (int)((int64_t)k * nb / np), b1 = (int)((int64_t)(k + 1) * nb / np);
-                    AttnItem it = {b + j0, nj, h, i, b0 * 64, std::min(L, b1 * 64), ctx_lens[i] + j0,
-                                   np > 1 ? n_parts + k : -1, np > 1 ? (int)groups.size() - 1 : -1, kind == ATTN_THIN ? safe[i] : 0, 0, 0};
-                    items.push_back(it);
-                    item_cost.push_back((int)((b1 - b0) * block_cost(nj)) + ac.item + (np > 1 ? ac.part : 0));
-                }
-                if (np > 1) n_parts += np;
-            }
+    auto add_item = [&](const Unit& u, int h, int b0, int b1) {
+        const bool whole = b0 == 0 && b1 == u.nb;
+        const int q_tok = chunk_offsets[u.req] + u.j0;
+        if (!whole && b0 == 0) groups.push_back({q_tok, u.nj, h, n_parts, 0, 0, 0, 0});
+        if (!whole) groups.back().n_parts++;
+        items.push_back({q_tok, u.nj, h, u.req, b0 * 64, std::min(u.L, b1 * 64), ctx_lens[u.req] + u.j0, whole ? -1 : n_parts++,
+                         whole ? -1 : (int)groups.size() - 1, kind == ATTN_THIN ? safe[u.req] : 0, 0, 0});
+        item_cost.push_back((int)((b1 - b0) * u.bc) + lay.ac->item + (whole ? 0 : lay.ac->part));
+    };
+    if (lay.wrapped) {
+        wrap(lay, lay.limit, [&](const Unit& u, int h, int b0, int b1, int cta) {
+            add_item(u, h, b0, b1);
+            owner.push_back(cta);
+        });
+    } else {
+        for (const Unit& u : lay.units) {
+            const int np = parts_of(lay, u, lay.limit);
+            for (int h = 0; h < Hkv; ++h)
+                for (int k = 0; k < np; ++k) add_item(u, h, (int)((int64_t)k * u.nb / np), (int)((int64_t)(k + 1) * u.nb / np));
         }
     }
     const int n_items = (int)items.size();
-    const int n_cta = std::min(n_cta_max, n_items);
+    const int n_cta = lay.wrapped ? owner.back() + 1 : std::min(lay.slots, n_items);
+    std::vector<int> order(n_items);
+    for (int i = 0; i < n_items; ++i) order[i] = i;
+    std::vector<int>& count = hp.cta_begin;
+    count.assign(n_cta + 1, 0);
+    auto cost = [&](int i) { return item_cost[i]; };
+    if (lay.wrapped) {
+        for (int k : owner) count[k + 1]++;
+    } else {
     // longest first (equal costs: lower index first), each to the least loaded CTA (ties: lower CTA);
     // both orders are carried in one 64-bit key
-    std::vector<int> order(n_items), owner(n_items);
-    auto cost = [&](int i) { return item_cost[i]; };
+    owner.assign(n_items, 0);
     {
         // stable radix sort of the indices by decreasing cost, 11 bits a pass
         int top = 0;
         for (int i = 0; i < n_items; ++i) top = std::max(top, item_cost[i]);
         std::vector<int> tmp(n_items);
-        for (int i = 0; i < n_items; ++i) order[i] = i;
         int hist[2048];
         for (int shift = 0; shift < 32 && (top >> shift) != 0; shift += 11) {
             memset(hist, 0, sizeof(hist));
@@ -990,8 +1084,6 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
             order.swap(tmp);
         }
     }
-    std::vector<int>& count = hp.cta_begin;
-    count.assign(n_cta + 1, 0);
     {
         std::vector<uint64_t> heap(n_cta);   // (load << 16) | cta, smallest at the root
         for (int k = 0; k < n_cta; ++k) heap[k] = (uint64_t)k;   // all loads 0: already a heap
@@ -1015,9 +1107,9 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     }
     // Local search on the greedy result: relieve the most loaded CTA by moving one of its items to
     // another CTA, or by exchanging it for a cheaper one, as long as that lowers the larger of the
-    // two loads; partners are the least loaded CTAs.  Only when the greedy result is more than 1 %
-    // above the mean; stops within 0.3 % of it.
-    if (n_cta > 1) {
+    // two loads; partners are the least loaded CTAs.  Only when CTAs hold more than one item and the greedy result is more
+    // than 1 % above the mean; stops within 0.3 % of it.
+    if (n_cta < n_items) {
         std::vector<int64_t> load(n_cta, 0);
         int64_t sum = 0;
         for (int i = 0; i < n_items; ++i) {
@@ -1082,6 +1174,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
             std::fill(count.begin(), count.end(), 0);
             for (int i = 0; i < n_items; ++i) count[owner[i] + 1]++;
         }
+    }
     }
     for (int k = 0; k < n_cta; ++k) count[k + 1] += count[k];
     hp.items.assign(n_items, AttnItem());
@@ -1151,6 +1244,7 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     p->n_req = n_req; p->T = T; p->max_pages = max_pages; p->n_items = n_items; p->n_cta = n_cta;
     p->n_groups = (int)hp.groups.size(); p->n_parts = hp.n_parts;
     p->attn = hp.kind;
+    p->wrapped = hp.wrapped;
     p->stats = hp.stats;
     p->stats.h2d_bytes = (int64_t)off;
     p->kv = kv; p->kv_pool = kv->pool; p->kv_pages = kv->n_pages;
@@ -2122,12 +2216,14 @@ static int syn_op_attention_impl(syn_model* m, syn_kv* kv, const syn_plan* p, ui
 
 // Scratch of syn_op_attention_static: the fp32 partial outputs and (max, sum) pairs of attention
 // work items that cover only part of a request's keys, and the per-group completion counters.  File-scope device memory, so every GPU that
-// loads the library holds these ~8.5 MB from load to exit.  Host code may not pass these names to a
+// loads the library holds these ~19.7 MB from load to exit: two partials of 64 rows for each of 296 CTAs (work lists cut where a
+// CTA is full; half as many of 128 rows).  Host code may not pass these names to a
 // kernel (on the host they are stand-ins, not device addresses): static_scratch() asks the runtime
 // for the device addresses once per device.
-static __device__ __align__(256) float g_static_part_o[(size_t)SYN_STATIC_MAX_PARTS * 64 * 128];
-static __device__ __align__(256) float2 g_static_part_ml[(size_t)SYN_STATIC_MAX_PARTS * 64];
-static __device__ __align__(256) int g_static_group_count[SYN_STATIC_MAX_PARTS];
+constexpr int STATIC_PARTS = 2 * 2 * 148;
+static __device__ __align__(256) float g_static_part_o[(size_t)STATIC_PARTS * 64 * 128];
+static __device__ __align__(256) float2 g_static_part_ml[(size_t)STATIC_PARTS * 64];
+static __device__ __align__(256) int g_static_group_count[STATIC_PARTS];
 
 static int static_scratch(float** part_o, float2** part_ml, int** group_count) {
     constexpr int MAX_DEV = 64;
@@ -2162,7 +2258,8 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     const syn_model_desc& c = m->desc;
     const int q_dim = c.n_q_heads * c.head_dim;
     if (p->T > m->t_cap) return SYN_E_INVALID_ARG;
-    if ((int64_t)p->n_parts * attn_rows(p->attn) > (int64_t)SYN_STATIC_MAX_PARTS * 64) return SYN_E_CAPACITY;
+    if (p->n_parts > STATIC_PARTS * 64 / attn_rows(p->attn)) return SYN_E_CAPACITY;
+    if (!p->wrapped && p->n_parts > SYN_STATIC_MAX_PARTS && p->n_groups > SYN_STATIC_MAX_PARTS / 2) return SYN_E_CAPACITY;
     float* part_o = nullptr;
     float2* part_ml = nullptr;
     int* group_count = nullptr;
@@ -2171,7 +2268,7 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     CU_OK(cudaMemcpyAsync(m->q, q, (size_t)p->T * q_dim * 2, cudaMemcpyDeviceToDevice, st));
     // the group counters must start at zero; every partial row that is read is written first
-    CU_OK(cudaMemsetAsync(group_count, 0, (size_t)SYN_STATIC_MAX_PARTS * 4, st));
+    CU_OK(cudaMemsetAsync(group_count, 0, (size_t)STATIC_PARTS * 4, st));
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, (op16*)out, part_o, part_ml, group_count);
     return attention_kernel(m, kv, p, ap, m->tm_q, false, st) == cudaSuccess ? SYN_OK : SYN_E_CUDA;

@@ -1,0 +1,62 @@
+"""Work lists of batches with about one (request, kv head) unit to a CTA: units laid end to end over the CTAs and cut where
+one is full.  On the CPU the cover of every unit; on the device the attention of such lists against the oracle."""
+import random
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2511_07423_b200 as syn
+from workloads.configs import ModelShape
+
+import test_gpu_attention as base
+
+
+def _lengths(n, seed, hi):
+    r = random.Random(seed)
+    return [r.choice([0, 1, 63, 64, 65, r.randint(2, hi)]) for _ in range(n)], [r.randint(1, 8) for _ in range(n)]
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2, 3])
+@pytest.mark.parametrize("n_req,heads,hd,hi", [(10, 8, 128, 900), (19, 8, 128, 4000), (36, 8, 64, 2000), (7, 21, 128, 2000), (1, 1, 64, 20)])
+def test_cut_units_are_covered_exactly_once(kind, n_req, heads, hd, hi):
+    ctx, chunk = _lengths(n_req, n_req, hi)
+    off = np.concatenate([[0], np.cumsum(chunk)]).tolist()
+    pages = [(a + b + 15) // 16 for a, b in zip(ctx, chunk)]
+    table = torch.zeros(n_req, max(pages), dtype=torch.int32)
+    for i, first in enumerate(np.cumsum([0] + pages[:-1])):
+        table[i, :pages[i]] = torch.arange(first, first + pages[i], dtype=torch.int32)
+    syn.debug_set_attention(kind)
+    try:
+        p = syn.plan_host(ModelShape("cut", 1, 256, 4 * heads, heads, hd, 256, 512), sum(pages),
+                          torch.zeros(off[-1], dtype=torch.int32), off, table, ctx)
+    finally:
+        syn.debug_set_attention(0)
+    cb, n_cta = p["cta_begin"].numpy(), p["n_cta"]
+    items = p["items"].numpy()
+    assert cb[0] == 0 and cb[n_cta] == len(items) and (np.diff(cb[:n_cta + 1]) >= 1).all() and n_cta <= 148
+    units = {}
+    for q, nj, h, req, kb, ke, _, part, group in items:
+        assert kb % 64 == 0 and kb < ke and off[req] <= q and q + nj <= off[req + 1]
+        units.setdefault((req, q, nj, h), []).append((kb, ke, part, group))
+    assert len(units) == sum(-(-n // (16 if p["stats"].attn_rows == 64 else 32)) for n in chunk) * heads
+    for (req, q, nj, h), v in units.items():
+        v.sort()
+        assert v[0][0] == 0 and v[-1][1] == ctx[req] + q - off[req] + nj
+        assert (len(v) == 1) == (v[0][2] < 0)
+        for a, b in zip(v, v[1:]):
+            assert b[0] == a[1] and b[2] == a[2] + 1 and b[3] == a[3]   # one group, its partials side by side
+    parts = sorted(x[7] for x in items if x[7] >= 0)
+    assert parts == list(range(len(parts)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", [0, 1, 2, 3])
+@pytest.mark.parametrize("hd,Hkv,n_req", [(128, 8, 20), (64, 8, 20), (128, 8, 36)])
+def test_cut_units_match_the_oracle(hd, Hkv, n_req, kind):
+    ctx, chunk = _lengths(n_req, 5, 900)
+    syn.debug_set_attention(kind)
+    try:
+        base._run(hd, 4 * Hkv, Hkv, ctx, chunk)
+    finally:
+        syn.debug_set_attention(0)
