@@ -1,5 +1,5 @@
 // Ragged multi-query attention over the paged KV cache (paper Sec. 3.2 attention equation,
-// applied to a chunk of 1..16 query tokens per request appended to a cached prefix, Sec. 3.4).
+// applied to a chunk of 1..32 query tokens per request appended to a cached prefix, Sec. 3.4).
 //
 // One work item = (request, kv head, token sub-range of the chunk, key range).  The G query heads
 // that share the kv head and the chunk's tokens are packed into one tile of rows (row = j*G + g,

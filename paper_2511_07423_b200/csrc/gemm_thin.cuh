@@ -13,7 +13,7 @@
 //     global memory and no counters.
 //   - Same orientation, weight tiles and epilogues (epi_unit) as gemm.cuh.  Two accumulators take
 //     alternate k-steps (an MMA into the accumulator of its predecessor waits for it).
-// Measured, whole steps against the one-CTA kernel: 1B shape, 5 tokens 1 334 -> 866 us; 135 tokens 1 837 ->
+// Measured when it was written (the epilogues have since become shorter for all kernels), whole steps against the one-CTA kernel: 1B shape, 5 tokens 1 334 -> 866 us; 135 tokens 1 837 ->
 // 1 380 us; 8B shape, 40 tokens 5 353 -> 4 179 us (the weights alone take 2 325 us at the copy rate).  One launch of
 // the 8B o projection (33.5 MB) at 40 tokens: 8.8 us until its last MMA and 2.9 us more to its end.  What bounds it: HBM
 // while it streams (4.5 - 5 TB/s in a launch of its own), and about 3 us per launch that depend on the
