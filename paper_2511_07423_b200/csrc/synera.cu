@@ -1005,10 +1005,10 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         if (lay.n_units <= n_sm && !lay.wrapped) lay.estimate = INT64_MAX / 256;
         const int64_t lead = lay.n_units > 2 * n_sm ? 112 : 103;
         Layout other = lay_out(costs[2], 2 * n_sm);
-        if (other.estimate < lay.estimate) lay = other;
+        if (other.estimate < lay.estimate) lay = std::move(other);
         if (max_chunk * G > 32) {
             other = lay_out(costs[1], n_sm);
-            if (other.estimate * lead < lay.estimate * 100) lay = other;
+            if (other.estimate * lead < lay.estimate * 100) lay = std::move(other);
         }
         if (lay.ac->kind == ATTN_THIN && thin_ctas != lay.slots) lay = lay_out(costs[2], thin_ctas);
     }
@@ -1066,115 +1066,115 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     if (lay.wrapped) {
         for (int k : owner) count[k + 1]++;
     } else {
-    // longest first (equal costs: lower index first), each to the least loaded CTA (ties: lower CTA);
-    // both orders are carried in one 64-bit key
-    owner.assign(n_items, 0);
-    {
-        // stable radix sort of the indices by decreasing cost, 11 bits a pass
-        int top = 0;
-        for (int i = 0; i < n_items; ++i) top = std::max(top, item_cost[i]);
-        std::vector<int> tmp(n_items);
-        int hist[2048];
-        for (int shift = 0; shift < 32 && (top >> shift) != 0; shift += 11) {
-            memset(hist, 0, sizeof(hist));
-            for (int i = 0; i < n_items; ++i) hist[2047 - ((item_cost[order[i]] >> shift) & 2047)]++;
-            int run = 0;
-            for (int b = 0; b < 2048; ++b) { const int h = hist[b]; hist[b] = run; run += h; }
-            for (int i = 0; i < n_items; ++i) tmp[hist[2047 - ((item_cost[order[i]] >> shift) & 2047)]++] = order[i];
-            order.swap(tmp);
-        }
-    }
-    {
-        std::vector<uint64_t> heap(n_cta);   // (load << 16) | cta, smallest at the root
-        for (int k = 0; k < n_cta; ++k) heap[k] = (uint64_t)k;   // all loads 0: already a heap
-        for (int i : order) {
-            const uint64_t top = heap[0];
-            const int k = (int)(top & 0xFFFFu);
-            owner[i] = k;
-            count[k + 1]++;
-            const uint64_t v = (((top >> 16) + (uint64_t)cost(i)) << 16) | (uint64_t)k;
-            int at = 0;   // the root grows: sift it down
-            for (;;) {
-                int ch = 2 * at + 1;
-                if (ch >= n_cta) break;
-                if (ch + 1 < n_cta && heap[ch + 1] < heap[ch]) ++ch;
-                if (heap[ch] >= v) break;
-                heap[at] = heap[ch];
-                at = ch;
+        // longest first (equal costs: lower index first), each to the least loaded CTA (ties: lower CTA);
+        // both orders are carried in one 64-bit key
+        owner.assign(n_items, 0);
+        {
+            // stable radix sort of the indices by decreasing cost, 11 bits a pass
+            int top = 0;
+            for (int i = 0; i < n_items; ++i) top = std::max(top, item_cost[i]);
+            std::vector<int> tmp(n_items);
+            int hist[2048];
+            for (int shift = 0; shift < 32 && (top >> shift) != 0; shift += 11) {
+                memset(hist, 0, sizeof(hist));
+                for (int i = 0; i < n_items; ++i) hist[2047 - ((item_cost[order[i]] >> shift) & 2047)]++;
+                int run = 0;
+                for (int b = 0; b < 2048; ++b) { const int h = hist[b]; hist[b] = run; run += h; }
+                for (int i = 0; i < n_items; ++i) tmp[hist[2047 - ((item_cost[order[i]] >> shift) & 2047)]++] = order[i];
+                order.swap(tmp);
             }
-            heap[at] = v;
         }
-    }
-    // Local search on the greedy result: relieve the most loaded CTA by moving one of its items to
-    // another CTA, or by exchanging it for a cheaper one, as long as that lowers the larger of the
-    // two loads; partners are the least loaded CTAs.  Only when CTAs hold more than one item and the greedy result is more
-    // than 1 % above the mean; stops within 0.3 % of it.
-    if (n_cta < n_items) {
-        std::vector<int64_t> load(n_cta, 0);
-        int64_t sum = 0;
-        for (int i = 0; i < n_items; ++i) {
-            load[owner[i]] += cost(i);
-            sum += cost(i);
+        {
+            std::vector<uint64_t> heap(n_cta);   // (load << 16) | cta, smallest at the root
+            for (int k = 0; k < n_cta; ++k) heap[k] = (uint64_t)k;   // all loads 0: already a heap
+            for (int i : order) {
+                const uint64_t top = heap[0];
+                const int k = (int)(top & 0xFFFFu);
+                owner[i] = k;
+                count[k + 1]++;
+                const uint64_t v = (((top >> 16) + (uint64_t)cost(i)) << 16) | (uint64_t)k;
+                int at = 0;   // the root grows: sift it down
+                for (;;) {
+                    int ch = 2 * at + 1;
+                    if (ch >= n_cta) break;
+                    if (ch + 1 < n_cta && heap[ch + 1] < heap[ch]) ++ch;
+                    if (heap[ch] >= v) break;
+                    heap[at] = heap[ch];
+                    at = ch;
+                }
+                heap[at] = v;
+            }
         }
-        const int64_t mean = sum / n_cta;
-        if (*std::max_element(load.begin(), load.end()) > mean + mean / 100) {
-            std::vector<std::vector<int>> held(n_cta);
-            for (int i = 0; i < n_items; ++i) held[owner[i]].push_back(i);
-            std::vector<int> by_load(n_cta);   // CTAs by increasing load, kept sorted
-            for (int k = 0; k < n_cta; ++k) by_load[k] = k;
-            auto lighter = [&](int x, int y) { return load[x] != load[y] ? load[x] < load[y] : x < y; };
-            std::sort(by_load.begin(), by_load.end(), lighter);
-            auto resort = [&](int k) {   // k's load changed: move it to its place
-                int at = (int)(std::find(by_load.begin(), by_load.end(), k) - by_load.begin());
-                while (at + 1 < n_cta && lighter(by_load[at + 1], k)) { by_load[at] = by_load[at + 1]; ++at; }
-                while (at > 0 && lighter(k, by_load[at - 1])) { by_load[at] = by_load[at - 1]; --at; }
-                by_load[at] = k;
-            };
-            const int64_t good = mean + mean / 333;
-            const int n_cand = std::min(n_cta - 1, 16);
-            for (int round = 0; round < 128; ++round) {
-                const int hi = by_load[n_cta - 1];
-                if (load[hi] <= good) break;
-                int64_t best = load[hi];
-                int bi = -1, bk = -1, bj = -1;   // position in held[hi], the other CTA, position in held[bk] (-1: move)
-                for (int a = 0; a < (int)held[hi].size(); ++a) {
-                    const int64_t ca = cost(held[hi][a]);
-                    for (int q = 0; q < n_cand; ++q) {
-                        const int k = by_load[q];
-                        if (std::max(load[hi] - ca, load[k] + ca) < best) {
-                            best = std::max(load[hi] - ca, load[k] + ca);
-                            bi = a; bk = k; bj = -1;
-                        }
-                        for (int b2 = 0; b2 < (int)held[k].size(); ++b2) {
-                            const int64_t dlt = ca - cost(held[k][b2]);
-                            if (dlt > 0 && std::max(load[hi] - dlt, load[k] + dlt) < best) {
-                                best = std::max(load[hi] - dlt, load[k] + dlt);
-                                bi = a; bk = k; bj = b2;
+        // Local search on the greedy result: relieve the most loaded CTA by moving one of its items to
+        // another CTA, or by exchanging it for a cheaper one, as long as that lowers the larger of the
+        // two loads; partners are the least loaded CTAs.  Only when CTAs hold more than one item and the greedy result is more
+        // than 1 % above the mean; stops within 0.3 % of it.
+        if (n_cta < n_items) {
+            std::vector<int64_t> load(n_cta, 0);
+            int64_t sum = 0;
+            for (int i = 0; i < n_items; ++i) {
+                load[owner[i]] += cost(i);
+                sum += cost(i);
+            }
+            const int64_t mean = sum / n_cta;
+            if (*std::max_element(load.begin(), load.end()) > mean + mean / 100) {
+                std::vector<std::vector<int>> held(n_cta);
+                for (int i = 0; i < n_items; ++i) held[owner[i]].push_back(i);
+                std::vector<int> by_load(n_cta);   // CTAs by increasing load, kept sorted
+                for (int k = 0; k < n_cta; ++k) by_load[k] = k;
+                auto lighter = [&](int x, int y) { return load[x] != load[y] ? load[x] < load[y] : x < y; };
+                std::sort(by_load.begin(), by_load.end(), lighter);
+                auto resort = [&](int k) {   // k's load changed: move it to its place
+                    int at = (int)(std::find(by_load.begin(), by_load.end(), k) - by_load.begin());
+                    while (at + 1 < n_cta && lighter(by_load[at + 1], k)) { by_load[at] = by_load[at + 1]; ++at; }
+                    while (at > 0 && lighter(k, by_load[at - 1])) { by_load[at] = by_load[at - 1]; --at; }
+                    by_load[at] = k;
+                };
+                const int64_t good = mean + mean / 333;
+                const int n_cand = std::min(n_cta - 1, 16);
+                for (int round = 0; round < 128; ++round) {
+                    const int hi = by_load[n_cta - 1];
+                    if (load[hi] <= good) break;
+                    int64_t best = load[hi];
+                    int bi = -1, bk = -1, bj = -1;   // position in held[hi], the other CTA, position in held[bk] (-1: move)
+                    for (int a = 0; a < (int)held[hi].size(); ++a) {
+                        const int64_t ca = cost(held[hi][a]);
+                        for (int q = 0; q < n_cand; ++q) {
+                            const int k = by_load[q];
+                            if (std::max(load[hi] - ca, load[k] + ca) < best) {
+                                best = std::max(load[hi] - ca, load[k] + ca);
+                                bi = a; bk = k; bj = -1;
+                            }
+                            for (int b2 = 0; b2 < (int)held[k].size(); ++b2) {
+                                const int64_t dlt = ca - cost(held[k][b2]);
+                                if (dlt > 0 && std::max(load[hi] - dlt, load[k] + dlt) < best) {
+                                    best = std::max(load[hi] - dlt, load[k] + dlt);
+                                    bi = a; bk = k; bj = b2;
+                                }
                             }
                         }
                     }
+                    if (bi < 0 || load[hi] - best < mean / 1000) break;   // nothing, or next to nothing, to gain
+                    const int ia = held[hi][bi];
+                    if (bj < 0) {
+                        load[hi] -= cost(ia); load[bk] += cost(ia);
+                        owner[ia] = bk;
+                        held[bk].push_back(ia);
+                        held[hi].erase(held[hi].begin() + bi);
+                    } else {
+                        const int ib = held[bk][bj];
+                        const int64_t dlt = cost(ia) - cost(ib);
+                        load[hi] -= dlt; load[bk] += dlt;
+                        owner[ia] = bk; owner[ib] = hi;
+                        held[hi][bi] = ib; held[bk][bj] = ia;
+                    }
+                    resort(hi);
+                    resort(bk);
                 }
-                if (bi < 0 || load[hi] - best < mean / 1000) break;   // nothing, or next to nothing, to gain
-                const int ia = held[hi][bi];
-                if (bj < 0) {
-                    load[hi] -= cost(ia); load[bk] += cost(ia);
-                    owner[ia] = bk;
-                    held[bk].push_back(ia);
-                    held[hi].erase(held[hi].begin() + bi);
-                } else {
-                    const int ib = held[bk][bj];
-                    const int64_t dlt = cost(ia) - cost(ib);
-                    load[hi] -= dlt; load[bk] += dlt;
-                    owner[ia] = bk; owner[ib] = hi;
-                    held[hi][bi] = ib; held[bk][bj] = ia;
-                }
-                resort(hi);
-                resort(bk);
+                std::fill(count.begin(), count.end(), 0);
+                for (int i = 0; i < n_items; ++i) count[owner[i] + 1]++;
             }
-            std::fill(count.begin(), count.end(), 0);
-            for (int i = 0; i < n_items; ++i) count[owner[i] + 1]++;
         }
-    }
     }
     for (int k = 0; k < n_cta; ++k) count[k + 1] += count[k];
     hp.items.assign(n_items, AttnItem());
