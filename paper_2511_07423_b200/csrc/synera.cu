@@ -18,6 +18,7 @@
 #include "gemm.cuh"
 #include "gemm2.cuh"
 #include "gemm_thin.cuh"
+#include "pieces.h"
 #include "sampling.cuh"
 
 using namespace syn;
@@ -749,22 +750,22 @@ static int kv_copy(syn_kv* kv, uint32_t layer, const int32_t* page_table, int32_
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // launches of at most KV_COPY_PAGES pages; short transfers carry the smaller parameter
     const size_t kv_dim = (size_t)kv->model->desc.n_kv_heads * kv->model->desc.head_dim;
-    for (int64_t done = 0; done < n_pos;) {
-        const int at = (int)(pos0 + done), p0 = at / P;
-        const int n = (int)std::min<int64_t>(n_pos - done, (int64_t)KV_COPY_PAGES * P - at % P);
-        const int n_pg = (at % P + n + P - 1) / P;
-        bf16 *kk = (bf16*)k + (size_t)done * kv_dim, *vv = (bf16*)v + (size_t)done * kv_dim;
-        const bool vec = (((uintptr_t)kk | (uintptr_t)vv) & 15) == 0;
-        const int r = n_pg <= KV_COPY_PAGES_SMALL
-                          ? (vec ? kv_copy_launch<KV_COPY_PAGES_SMALL, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
-                                 : kv_copy_launch<KV_COPY_PAGES_SMALL, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool))
-                          : (vec ? kv_copy_launch<KV_COPY_PAGES, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
-                                 : kv_copy_launch<KV_COPY_PAGES, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool));
-        if (r) return r;
-        done += n;
-    }
-    CU_OK(cudaStreamSynchronize(st));
-    return SYN_OK;
+    return for_pieces(
+        pos0, n_pos, P, KV_COPY_PAGES,
+        [&](int at, int n, int64_t done) {
+            const int p0 = at / P, n_pg = (at % P + n + P - 1) / P;
+            bf16 *kk = (bf16*)k + (size_t)done * kv_dim, *vv = (bf16*)v + (size_t)done * kv_dim;
+            const bool vec = (((uintptr_t)kk | (uintptr_t)vv) & 15) == 0;
+            return n_pg <= KV_COPY_PAGES_SMALL
+                       ? (vec ? kv_copy_launch<KV_COPY_PAGES_SMALL, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
+                              : kv_copy_launch<KV_COPY_PAGES_SMALL, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool))
+                       : (vec ? kv_copy_launch<KV_COPY_PAGES, 8>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool)
+                              : kv_copy_launch<KV_COPY_PAGES, 1>(kv, layer, page_table + p0, n_pg, at, n, kk, vv, st, to_pool));
+        },
+        [&]() -> int {
+            CU_OK(cudaStreamSynchronize(st));
+            return SYN_OK;
+        });
 }
 
 static int syn_kv_import_impl(syn_kv* kv, uint32_t layer, const int32_t* page_table, int32_t pos0, int32_t n_pos,
