@@ -203,13 +203,27 @@ int syn_plan_stats(const syn_plan *p, syn_step_stats *out);
  * the first query token, index of its partial or -1, merge group or -1) (NULL to skip;
  * SYN_E_CAPACITY if items_cap is too small, *n_items then holds the count needed), cta_begin
  * [n_sm + 1] (CTA k owns items cta_begin[k] .. cta_begin[k+1]; NULL to skip), *n_cta, *stats (may be
- * NULL; h2d_bytes is left 0).  n_sm = number of CTAs to plan for (the device's SM count). */
+ * NULL; h2d_bytes is left 0).  n_sm = number of CTAs to plan for (the device's SM count).  Where the batch
+ * goes to the half-SM attention kernel, which a device runs with two CTAs to an SM, the work list is
+ * therefore not the step's: syn_plan_work_host returns that. */
 #define SYN_PLAN_ITEM_FIELDS 9
 int syn_plan_host(const syn_model_desc *desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req,
                   const int32_t *chunk_tokens, const int32_t *chunk_offsets, const int32_t *page_tables,
                   int32_t max_pages, const int32_t *ctx_lens, const int32_t *n_uncached, int32_t *pos, int32_t *slot,
                   int32_t *items, int32_t items_cap, int32_t *n_items, int32_t *cta_begin, int32_t *n_cta,
                   syn_step_stats *stats);
+
+/* The attention work list that a step on a device of n_sm SMs runs, whichever kernel takes it; arguments, validation and
+ * results as in syn_plan_host, except: items [items_cap][SYN_WORK_ITEM_FIELDS], the tenth field being the position up to
+ * which no chunk of the batch writes the request's keys (a multiple of 16; they may be read before the chunks' own are
+ * written; 0 in the lists of the other kernels); cta_begin [2 * n_sm + 1]; *attention (may be NULL) = the kernel, numbered as
+ * in syn_debug_set_attention.  n_sm at most 32767. */
+#define SYN_WORK_ITEM_FIELDS 10
+int syn_plan_work_host(const syn_model_desc *desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req,
+                       const int32_t *chunk_tokens, const int32_t *chunk_offsets, const int32_t *page_tables,
+                       int32_t max_pages, const int32_t *ctx_lens, const int32_t *n_uncached, int32_t *items,
+                       int32_t items_cap, int32_t *n_items, int32_t *cta_begin, int32_t *n_cta, int32_t *attention,
+                       syn_step_stats *stats);
 
 
 /* Per-kernel-class device timing.  With profiling on, syn_verify_run / syn_verify_batch bracket

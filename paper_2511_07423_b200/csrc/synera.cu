@@ -788,6 +788,9 @@ extern "C" void syn_plan_free(syn_plan* p) {
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// CTAs of the half-SM attention kernel that a device of n_sm SMs holds at a time.
+static int thin_attention_ctas(int n_sm) { return 2 * n_sm; }
+
 // Host-side result of planning one batch (no device involved).
 struct HostPlan {
     int T = 0, n_cta = 0, n_parts = 0, kind = ATTN_WARP;
@@ -1005,7 +1008,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         lay = lay_out(costs[0], n_sm);
         if (lay.n_units <= n_sm && !lay.wrapped) lay.estimate = INT64_MAX / 256;
         const int64_t lead = lay.n_units > 2 * n_sm ? 112 : 103;
-        Layout other = lay_out(costs[2], 2 * n_sm);
+        Layout other = lay_out(costs[2], thin_attention_ctas(n_sm));
         if (other.estimate < lay.estimate) lay = std::move(other);
         if (max_chunk * G > 32) {
             other = lay_out(costs[1], n_sm);
@@ -1208,7 +1211,7 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     if (!m || !kv || kv->model != m) return SYN_E_INVALID_ARG;
     HostPlan hp;
     int r = plan_compute(m->desc, (int)kv->page_size, kv->n_pages, m->n_sm, n_req, chunk_tokens, chunk_offsets, page_tables,
-                         max_pages, ctx_lens, n_uncached, g_attention, 2 * m->n_sm, hp);
+                         max_pages, ctx_lens, n_uncached, g_attention, thin_attention_ctas(m->n_sm), hp);
     if (r) return r;
     const int T = hp.T, n_items = (int)hp.items.size(), n_cta = hp.n_cta;
     size_t off = 0;
@@ -1252,34 +1255,61 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     return SYN_OK;
 }
 
-// The planner without a device: same validation and the same work list as syn_plan_create, returned
-// in caller-provided HOST arrays.
+// The planner without a device, for `thin_ctas` CTAs of the half-SM attention kernel; the work list goes to caller-provided HOST
+// arrays, `fields` ints an item.
+static int plan_host(const syn_model_desc* desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int thin_ctas, int32_t n_req,
+                     const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables, int32_t max_pages,
+                     const int32_t* ctx_lens, const int32_t* n_uncached, int32_t* items, int32_t items_cap, int fields,
+                     int32_t* n_items, int32_t* cta_begin, int32_t* n_cta, HostPlan& hp) {
+    if (!desc || page_size != 16 || !n_items || !n_cta) return SYN_E_INVALID_ARG;
+    if (desc->n_kv_heads == 0 || desc->n_q_heads % desc->n_kv_heads != 0 || desc->n_q_heads / desc->n_kv_heads > 8)
+        return SYN_E_INVALID_ARG;
+    int r = plan_compute(*desc, (int)page_size, n_pages, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages,
+                         ctx_lens, n_uncached, g_attention, thin_ctas, hp);
+    if (r) return r;
+    *n_items = (int)hp.items.size();
+    *n_cta = hp.n_cta;
+    if (items) {
+        if (items_cap < *n_items) return SYN_E_CAPACITY;
+        for (int i = 0; i < *n_items; ++i) {
+            const AttnItem& it = hp.items[i];
+            const int32_t row[SYN_WORK_ITEM_FIELDS] = {it.q_tok, it.nj, it.kvh, it.req, it.kv_begin, it.kv_end, it.q_pos0,
+                                                       it.part, it.grp, it.kv_safe};
+            memcpy(items + (size_t)i * fields, row, fields * sizeof(int32_t));
+        }
+    }
+    if (cta_begin) memcpy(cta_begin, hp.cta_begin.data(), (size_t)(hp.n_cta + 1) * 4);
+    return SYN_OK;
+}
+
 static int syn_plan_host_impl(const syn_model_desc* desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req,
                              const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables,
                              int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int32_t* pos,
                              int32_t* slot, int32_t* items, int32_t items_cap, int32_t* n_items, int32_t* cta_begin,
                              int32_t* n_cta, syn_step_stats* stats) {
-    if (!desc || page_size != 16 || !n_items || !n_cta) return SYN_E_INVALID_ARG;
-    if (desc->n_kv_heads == 0 || desc->n_q_heads % desc->n_kv_heads != 0 || desc->n_q_heads / desc->n_kv_heads > 8)
-        return SYN_E_INVALID_ARG;
     HostPlan hp;
-    int r = plan_compute(*desc, (int)page_size, n_pages, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages,
-                         ctx_lens, n_uncached, g_attention, n_sm, hp);   // n_sm CTAs whatever the kernel
+    // n_sm CTAs whatever the kernel: callers pass a cta_begin of that size
+    const int r = plan_host(desc, n_pages, page_size, n_sm, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages, ctx_lens,
+                            n_uncached, items, items_cap, SYN_PLAN_ITEM_FIELDS, n_items, cta_begin, n_cta, hp);
+    if (r && r != SYN_E_CAPACITY) return r;
+    if (pos) memcpy(pos, hp.pos.data(), hp.pos.size() * 4);
+    if (slot) memcpy(slot, hp.slot.data(), hp.slot.size() * 4);
     if (r) return r;
-    *n_items = (int)hp.items.size();
-    *n_cta = hp.n_cta;
-    if (pos) memcpy(pos, hp.pos.data(), (size_t)hp.T * 4);
-    if (slot) memcpy(slot, hp.slot.data(), (size_t)hp.T * 4);
-    if (items) {
-        if (items_cap < *n_items) return SYN_E_CAPACITY;
-        for (int i = 0; i < *n_items; ++i) {
-            const AttnItem& it = hp.items[i];
-            const int32_t row[SYN_PLAN_ITEM_FIELDS] = {it.q_tok, it.nj, it.kvh, it.req, it.kv_begin, it.kv_end, it.q_pos0,
-                                                       it.part, it.grp};
-            memcpy(items + (size_t)i * SYN_PLAN_ITEM_FIELDS, row, sizeof(row));
-        }
-    }
-    if (cta_begin) memcpy(cta_begin, hp.cta_begin.data(), (size_t)(hp.n_cta + 1) * 4);
+    if (stats) *stats = hp.stats;
+    return SYN_OK;
+}
+
+static int syn_plan_work_host_impl(const syn_model_desc* desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req,
+                                   const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables,
+                                   int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int32_t* items,
+                                   int32_t items_cap, int32_t* n_items, int32_t* cta_begin, int32_t* n_cta, int32_t* attention,
+                                   syn_step_stats* stats) {
+    if (n_sm <= 0 || n_sm > 32767) return SYN_E_INVALID_ARG;
+    HostPlan hp;
+    const int r = plan_host(desc, n_pages, page_size, n_sm, thin_attention_ctas(n_sm), n_req, chunk_tokens, chunk_offsets, page_tables,
+                            max_pages, ctx_lens, n_uncached, items, items_cap, SYN_WORK_ITEM_FIELDS, n_items, cta_begin, n_cta, hp);
+    if (r) return r;
+    if (attention) *attention = hp.kind;
     if (stats) *stats = hp.stats;
     return SYN_OK;
 }
@@ -2333,6 +2363,10 @@ extern "C" int syn_kv_export(syn_kv* kv, uint32_t layer, const int32_t* page_tab
 
 extern "C" int syn_plan_host(const syn_model_desc* desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req, const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables, int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int32_t* pos, int32_t* slot, int32_t* items, int32_t items_cap, int32_t* n_items, int32_t* cta_begin, int32_t* n_cta, syn_step_stats* stats) {
     SYN_GUARD(syn_plan_host_impl(desc, n_pages, page_size, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages, ctx_lens, n_uncached, pos, slot, items, items_cap, n_items, cta_begin, n_cta, stats));
+}
+
+extern "C" int syn_plan_work_host(const syn_model_desc* desc, uint32_t n_pages, uint32_t page_size, int32_t n_sm, int32_t n_req, const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables, int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, int32_t* items, int32_t items_cap, int32_t* n_items, int32_t* cta_begin, int32_t* n_cta, int32_t* attention, syn_step_stats* stats) {
+    SYN_GUARD(syn_plan_work_host_impl(desc, n_pages, page_size, n_sm, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages, ctx_lens, n_uncached, items, items_cap, n_items, cta_begin, n_cta, attention, stats));
 }
 
 extern "C" int syn_plan_create(syn_model* m, syn_kv* kv, int32_t n_req, const int32_t* chunk_tokens, const int32_t* chunk_offsets, const int32_t* page_tables, int32_t max_pages, const int32_t* ctx_lens, const int32_t* n_uncached, syn_plan** out) {
