@@ -53,6 +53,25 @@ def test_cut_units_are_covered_exactly_once(kind, n_req, heads, hd, hi, export):
     assert parts == list(range(len(parts)))
 
 
+def test_keys_that_may_be_read_before_the_chunks_are_written():
+    """Up to the first page of a request that any request of the batch writes, over shared pages too; nothing in the lists of the
+    kernels that wait for the projection first."""
+    table = torch.tensor([[5, 1, 7, 2, 0, 4, 9], [5, 1, 7, 2, 0, 4, 8], [3, 6, 10, -1, -1, -1, -1], [5, 1, 7, 2, 11, -1, -1],
+                          [12, -1, -1, -1, -1, -1, -1]], dtype=torch.int32)
+    # request 0 writes 48..79 (pages 2 and 0), request 1 reads up to 95 through the same pages and writes page 8, request 2
+    # ends on a page boundary, request 3 shares pages 5, 1, 7 and writes 64.. in a page of its own, request 4 has three keys
+    ctx, chunk = [48, 96, 32, 64, 3], [32, 4, 16, 2, 1]
+    off = [0] + np.cumsum(chunk).tolist()
+    for kind, want in ((3, {0: 48, 1: 48, 2: 32, 3: 48, 4: 0}), (1, dict.fromkeys(range(5), 0)), (2, dict.fromkeys(range(5), 0))):
+        syn.debug_set_attention(kind)
+        try:
+            p = syn.plan_work_host(ModelShape("safe", 1, 256, 8, 2, 64, 256, 512), 13, torch.zeros(off[-1], dtype=torch.int32), off, table, ctx)
+        finally:
+            syn.debug_set_attention(0)
+        assert p["attention"] == kind
+        assert {(int(r[3]), int(r[9])) for r in p["items"]} == set(want.items())
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("kind", [0, 1, 2, 3])
 @pytest.mark.parametrize("hd,Hkv,n_req", [(128, 8, 20), (64, 8, 20), (128, 8, 36)])

@@ -37,21 +37,30 @@ def test_scores_that_keep_growing(hd):
 
 def test_a_context_written_by_another_request_of_the_batch():
     """Two requests over one page table, the second one's context ending with the first one's chunk (a long run of
-    uncached tokens in one step): its keys must not be read before they are written."""
+    uncached tokens in one step): its keys must not be read before they are written.  The first request writes whole pages
+    of the second one's first stage of 64 keys, which without a look at the other requests' chunks would be read early."""
     import paper_2511_07423_b200 as syn
     shape, seed = TINY, 31
     glob, layers = cpu_model(shape, seed)
     model = syn.Model(shape, *to_cuda(glob, layers))
-    toks = gen.gen_context_tokens(Workload("w", shape, seed, 1, None, None, 0.5), 0, 70)
-    table = torch.tensor([[5, 1, 7, 2, 0]], dtype=torch.int32)
-    kv = syn.KVCache(model, 8)
-    for at, n in ((0, 32), (32, 16)):
-        kv.verify_batch(toks[at:at + n], [0, n], table, [at], [n])
-    # the pieces one after the other ...
-    kv.verify_batch(toks[48:60], [0, 12], table, [48], [12])
-    _, _, want = kv.verify_batch(toks[60:70], [0, 10], table, [60], [10], want_logits=True)
-    # ... and as two requests of one batch, over slots that hold something else before
-    for _ in range(3):
-        kv.verify_batch(toks[:22].flip(0), [0, 22], table, [48], [22])
-        _, _, got = kv.verify_batch(toks[48:70], [0, 12, 22], table.repeat(2, 1), [48, 60], [12, 10], want_logits=True)
-        assert torch.equal(got[12:], want)
+    toks = gen.gen_context_tokens(Workload("w", shape, seed, 1, None, None, 0.5), 0, 90)
+    table = torch.tensor([[5, 1, 7, 2, 0, 4]], dtype=torch.int32)
+    two = dict(chunk_tokens=toks[48:90], chunk_offsets=[0, 32, 42], page_tables=table.repeat(2, 1), ctx_lens=[48, 80])
+    syn.debug_set_attention(3)
+    try:
+        safe = {int(r[3]): int(r[9]) for r in syn.plan_work_host(shape, 8, **two)["items"]}
+        assert safe == {0: 48, 1: 48}
+        kv = syn.KVCache(model, 8)
+        for at, n in ((0, 32), (32, 16)):
+            kv.verify_batch(toks[at:at + n], [0, n], table, [at], [n])
+        # the pieces one after the other ...
+        kv.verify_batch(toks[48:80], [0, 32], table, [48], [32])
+        _, _, want = kv.verify_batch(toks[80:90], [0, 10], table, [80], [10], want_logits=True)
+        # ... and as two requests of one batch, over slots that hold something else before
+        for _ in range(3):
+            kv.verify_batch(toks[:32].flip(0), [0, 32], table, [48], [32])
+            kv.verify_batch(toks[:10].flip(0), [0, 10], table, [80], [10])
+            _, _, got = kv.verify_batch(*two.values(), [32, 10], want_logits=True)
+            assert torch.equal(got[32:], want)
+    finally:
+        syn.debug_set_attention(0)
