@@ -880,15 +880,17 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         int slots = 0;             // CTAs
         int64_t n_units = 0, total = 0, longest = 0;
         int64_t limit = 0;         // of an item in equal parts; wrapped: of a CTA
+        bool merge_counts = true;  // the merge of a unit's parts has to end by `limit` too
         bool wrapped = false;
         int64_t estimate = 0;
     };
     auto tiles = [&](const Unit& u) { return (u.nj * G + 15) / 16; };
-    // equal parts that end, with a merge of a few of them, by `limit`
+    // equal parts that end by `limit`, where it counts with a merge of a few of them
     auto parts_of = [&](const Layout& y, const Unit& u, int64_t limit) {
         if (u.nb * u.bc + y.ac->item <= limit) return 1;
         const int min_blocks = y.ac->kind == ATTN_THIN ? 1 : 4, max_parts = y.ac->kind == ATTN_THIN ? ATTN_THIN_MAX_PARTS : 64;
-        const int64_t most = std::max<int64_t>(min_blocks, (limit - y.ac->item - y.ac->part - y.ac->merge - 4 * tiles(u) * y.ac->merge_tile) / u.bc);   // blocks of a part
+        const int64_t tail = y.merge_counts ? y.ac->part + y.ac->merge + 4 * tiles(u) * y.ac->merge_tile : 0;
+        const int64_t most = std::max<int64_t>(min_blocks, (limit - y.ac->item - tail) / u.bc);   // blocks of a part
         return (int)std::min<int64_t>(std::min<int64_t>(max_parts, std::max(1, u.nb / min_blocks)), (u.nb + most - 1) / most);
     };
     // The units one after the other, longest first, each CTA filled up to `limit`: what does not fit goes on in the next CTA
@@ -939,10 +941,27 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         }
         y.n_units = (int64_t)y.units.size() * Hkv;
         const int64_t mean = (y.total + slots - 1) / slots;
-        // many units to a CTA: whole, only one that alone exceeds a CTA's fair share is cut
-        y.limit = std::max(mean, 8 * (int64_t)k.block[4] + k.item);
-        y.estimate = std::max(mean, std::min(y.longest, y.limit)) + k.fixed;
-        if (y.n_units > 2 * slots) return y;
+        if (y.n_units > 2 * slots) {
+            // Many units to a CTA: whole, unless one alone exceeds a CTA's fair share by so much that parts of it pay for
+            // themselves.  The merge of a unit's parts runs beside other items and counts as work, not as time that a part has to
+            // leave free (with the merge inside the share, three requests of 6 000 keys among 58 of the 8B shape were cut into
+            // parts of 4 blocks: 528 parts and 520 us a layer; 96 and 60 with this).
+            y.merge_counts = false;
+            y.estimate = INT64_MAX;
+            for (int64_t limit = std::max(mean, 8 * (int64_t)k.block[4] + k.item);; limit += limit / 4) {
+                int64_t total = 0, longest = 0;
+                for (const Unit& u : y.units) {
+                    const int np = parts_of(y, u, limit);
+                    total += u.nb * u.bc + k.item;
+                    if (np > 1) total += (int64_t)np * (k.item + k.part) - k.item + k.merge + std::min(np, 8) * tiles(u) * k.merge_tile;
+                    longest = std::max(longest, (u.nb + np - 1) / np * u.bc + k.item + (np > 1 ? k.part : 0));
+                }
+                const int64_t estimate = std::max((total * Hkv + slots - 1) / slots, longest) + k.fixed;
+                if (estimate < y.estimate) { y.estimate = estimate; y.limit = limit; }
+                if (limit >= y.longest) break;   // nothing is cut
+            }
+            return y;
+        }
         // Few: whole units (as good as their number divides), equal parts of which there are no more than CTAs, or wrapped; with
         // two CTAs or more to a unit equal parts are as even and have fewer merges (64 units of the 8B shape on 296 CTAs: 29.5 us
         // wrapped, 28.8 in equal parts).  Equal parts of more than 128 units: SYN_STATIC_MAX_PARTS of them if that is enough to cut

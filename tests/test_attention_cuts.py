@@ -53,6 +53,29 @@ def test_cut_units_are_covered_exactly_once(kind, n_req, heads, hd, hi, export):
     assert parts == list(range(len(parts)))
 
 
+@pytest.mark.parametrize("kind", [0, 1, 2, 3])
+@pytest.mark.parametrize("heads,hd", [(8, 128), (8, 64)])
+def test_few_long_requests_among_many_short_ones_are_not_cut_small(kind, heads, hd):
+    """More than two units to a CTA: a long one is cut into parts of about a CTA's fair share, no smaller, so there are no more
+    parts than CTAs."""
+    ctx, chunk = [5953] * 3 + [100] * 80, [32] * 3 + [4] * 80
+    off = np.concatenate([[0], np.cumsum(chunk)]).tolist()
+    pages = [(a + b + 15) // 16 for a, b in zip(ctx, chunk)]
+    table = torch.zeros(len(ctx), max(pages), dtype=torch.int32)
+    for i, first in enumerate(np.cumsum([0] + pages[:-1])):
+        table[i, :pages[i]] = torch.arange(first, first + pages[i], dtype=torch.int32)
+    syn.debug_set_attention(kind)
+    try:
+        p = syn.plan_work_host(ModelShape("cut", 1, 256, 4 * heads, heads, hd, 256, 512), sum(pages),
+                               torch.zeros(off[-1], dtype=torch.int32), off, table, ctx)
+    finally:
+        syn.debug_set_attention(0)
+    cb, items = p["cta_begin"].numpy(), p["items"].numpy()
+    keys = [int((items[a:b, 5] - items[a:b, 4]).sum()) for a, b in zip(cb, cb[1:])]
+    assert 0 < p["stats"].attn_split_items <= p["n_cta"], p["stats"].attn_split_items
+    assert max(keys) <= 1.5 * sum(keys) / len(keys)
+
+
 def test_keys_that_may_be_read_before_the_chunks_are_written():
     """Up to the first page of a request that any request of the batch writes, over shared pages too; nothing in the lists of the
     kernels that wait for the projection first."""
