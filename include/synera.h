@@ -294,19 +294,19 @@ int syn_op_attention(syn_model *m, syn_kv *kv, const syn_plan *p, uint32_t layer
  * no counterpart; this is a service of the library.)  Same arguments, same result and same
  * asynchronous behaviour as syn_op_attention, but the partial results of work items that cover
  * only part of a request's keys live in a fixed array inside the library instead of a workspace
- * that grows on demand (about 19.7 MB of every GPU that loads the library, from load to exit).  It takes
- * two partials for each CTA of a plan that lays requests end to end over the CTAs and cuts where one is
- * full; of a plan that cuts them evenly, SYN_STATIC_MAX_PARTS partials or those of half as many
- * (request, kv head) units.  The call itself allocates and frees nothing; the
- * model, cache and plan it is given were of course allocated earlier by their own calls.
- *   - A plan with more (attn_split_items of syn_plan_stats()) is refused with SYN_E_CAPACITY before anything is launched.
+ * that grows on demand.  The array holds SYN_STATIC_MAX_PARTS partials of 64 rows, or half as many of
+ * the 128-row kind of a plan made for the tcgen05 kernel: two for each CTA of a plan for the 148 SMs of a
+ * B200, which is more than any such plan has (about 19.7 MB of every GPU that loads the library, from load
+ * to exit).  The call itself allocates and frees nothing; the model, cache and plan it is given were of course allocated earlier by their own calls.
+ *   - A plan with more partial work items than that (attn_split_items x attn_rows of syn_plan_stats()
+ *     above SYN_STATIC_MAX_PARTS x 64) is refused with SYN_E_CAPACITY before anything is launched.
  *   - The first call on each device looks up the array's device address (with that device
  *     current); make that first call outside any stream capture.
  *   - All calls on a device share the one array.  It keeps the previous call's contents; nothing
  *     in it needs clearing, because every partial that is read is written earlier in the same
  *     call.  Two calls that overlap on the GPU (different streams) race on it: serialise them.
  * Errors: SYN_E_INVALID_ARG, SYN_E_CAPACITY, SYN_E_CUDA. */
-#define SYN_STATIC_MAX_PARTS 256
+#define SYN_STATIC_MAX_PARTS 592
 int syn_op_attention_static(syn_model *m, syn_kv *kv, const syn_plan *p, uint32_t layer, const void *q, void *out,
                             void *cuda_stream);
 

@@ -348,7 +348,6 @@ struct syn_plan {
     syn_step_stats stats;
     int n_req = 0, T = 0, max_pages = 0, n_items = 0, n_cta = 0, n_groups = 0, n_parts = 0;
     int attn = ATTN_WARP;   // which attention kernel the work list was made for
-    bool wrapped = false;   // how it was cut
     // one device buffer and its pinned host mirror
     uint8_t *dev = nullptr, *host = nullptr;
     size_t cap = 0, used = 0;
@@ -794,7 +793,6 @@ static int thin_attention_ctas(int n_sm) { return 2 * n_sm; }
 // Host-side result of planning one batch (no device involved).
 struct HostPlan {
     int T = 0, n_cta = 0, n_parts = 0, kind = ATTN_WARP;
-    bool wrapped = false;   // units laid end to end over the CTAs, cut where a CTA is full
     std::vector<int> pos, slot, cta_begin;
     std::vector<AttnItem> items;          // sorted by CTA
     std::vector<MergeGroup> groups;
@@ -964,7 +962,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         }
         // Few: whole units (as good as their number divides), equal parts of which there are no more than CTAs, or wrapped; with
         // two CTAs or more to a unit equal parts are as even and have fewer merges (64 units of the 8B shape on 296 CTAs: 29.5 us
-        // wrapped, 28.8 in equal parts).  Equal parts of more than 128 units: SYN_STATIC_MAX_PARTS of them if that is enough to cut
+        // wrapped, 28.8 in equal parts).  Equal parts of more than 128 units: 256 of them if that is enough to cut
         // some, else two to a unit.
         int64_t best = y.n_units <= slots ? y.longest : std::max(y.longest, (y.n_units + slots - 1) / slots * (y.total / y.n_units));
         y.limit = y.longest;
@@ -990,8 +988,9 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
             return true;
         };
         if (y.n_units <= slots) {
-            const bool many = 2 * y.n_units > SYN_STATIC_MAX_PARTS;
-            if (!cut(many ? std::min(slots, SYN_STATIC_MAX_PARTS) : slots) && many) cut(std::min<int64_t>(slots, 2 * y.n_units));
+            const int even_parts = 256;
+            const bool many = 2 * y.n_units > even_parts;
+            if (!cut(many ? std::min(slots, even_parts) : slots) && many) cut(std::min<int64_t>(slots, 2 * y.n_units));
         }
         if (2 * y.n_units > slots) {
             std::sort(y.units.begin(), y.units.end(), [](const Unit& p, const Unit& q) {
@@ -1037,7 +1036,6 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
     }
     const int kind = lay.ac->kind;
     hp.kind = kind;
-    hp.wrapped = lay.wrapped;
     // Positions that no chunk of the batch writes, for the kernel that requests keys before the chunks' are written: up
     // to the first page of the request that holds a written slot, of whichever request.
     std::vector<int> safe;
@@ -1267,7 +1265,6 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     p->n_req = n_req; p->T = T; p->max_pages = max_pages; p->n_items = n_items; p->n_cta = n_cta;
     p->n_groups = (int)hp.groups.size(); p->n_parts = hp.n_parts;
     p->attn = hp.kind;
-    p->wrapped = hp.wrapped;
     p->stats = hp.stats;
     p->stats.h2d_bytes = (int64_t)off;
     p->kv = kv; p->kv_pool = kv->pool; p->kv_pages = kv->n_pages;
@@ -2270,10 +2267,9 @@ static int syn_op_attention_impl(syn_model* m, syn_kv* kv, const syn_plan* p, ui
 // CTA is full; half as many of 128 rows).  Host code may not pass these names to a
 // kernel (on the host they are stand-ins, not device addresses): static_scratch() asks the runtime
 // for the device addresses once per device.
-constexpr int STATIC_PARTS = 2 * 2 * 148;
-static __device__ __align__(256) float g_static_part_o[(size_t)STATIC_PARTS * 64 * 128];
-static __device__ __align__(256) float2 g_static_part_ml[(size_t)STATIC_PARTS * 64];
-static __device__ __align__(256) int g_static_group_count[STATIC_PARTS];
+static __device__ __align__(256) float g_static_part_o[(size_t)SYN_STATIC_MAX_PARTS * 64 * 128];
+static __device__ __align__(256) float2 g_static_part_ml[(size_t)SYN_STATIC_MAX_PARTS * 64];
+static __device__ __align__(256) int g_static_group_count[SYN_STATIC_MAX_PARTS];
 
 static int static_scratch(float** part_o, float2** part_ml, int** group_count) {
     constexpr int MAX_DEV = 64;
@@ -2308,8 +2304,7 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     const syn_model_desc& c = m->desc;
     const int q_dim = c.n_q_heads * c.head_dim;
     if (p->T > m->t_cap) return SYN_E_INVALID_ARG;
-    if (p->n_parts > STATIC_PARTS * 64 / attn_rows(p->attn)) return SYN_E_CAPACITY;
-    if (!p->wrapped && p->n_parts > SYN_STATIC_MAX_PARTS && p->n_groups > SYN_STATIC_MAX_PARTS / 2) return SYN_E_CAPACITY;
+    if ((int64_t)p->n_parts * attn_rows(p->attn) > (int64_t)SYN_STATIC_MAX_PARTS * 64) return SYN_E_CAPACITY;
     float* part_o = nullptr;
     float2* part_ml = nullptr;
     int* group_count = nullptr;
@@ -2318,7 +2313,7 @@ static int syn_op_attention_static_impl(syn_model* m, syn_kv* kv, const syn_plan
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     CU_OK(cudaMemcpyAsync(m->q, q, (size_t)p->T * q_dim * 2, cudaMemcpyDeviceToDevice, st));
     // the group counters must start at zero; every partial row that is read is written first
-    CU_OK(cudaMemsetAsync(group_count, 0, (size_t)STATIC_PARTS * 4, st));
+    CU_OK(cudaMemsetAsync(group_count, 0, (size_t)SYN_STATIC_MAX_PARTS * 4, st));
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, (op16*)out, part_o, part_ml, group_count);
     return attention_kernel(m, kv, p, ap, m->tm_q, false, st) == cudaSuccess ? SYN_OK : SYN_E_CUDA;

@@ -76,6 +76,31 @@ def test_few_long_requests_among_many_short_ones_are_not_cut_small(kind, heads, 
     assert max(keys) <= 1.5 * sum(keys) / len(keys)
 
 
+@pytest.mark.parametrize("kind", [0, 1, 2, 3])
+@pytest.mark.parametrize("heads,hd,group", [(8, 128, 4), (8, 64, 4), (21, 128, 1), (2, 64, 5)])
+def test_no_plan_has_more_partials_than_the_static_array_holds(kind, heads, hd, group):
+    """syn_op_attention_static: 592 partials of 64 rows, 296 of 128.  Lists end to end have two a CTA at most, equal parts no
+    more than CTAs, and where a CTA has several units fewer than one a CTA and one more for each unit that is cut."""
+    r = random.Random(heads * hd + kind)
+    syn.debug_set_attention(kind)
+    try:
+        for _ in range(60):
+            n_long, n_short = r.randint(1, max(1, 320 // heads)), r.choice([0, r.randint(0, 620 // heads)])
+            hi = r.randint(300, 6000)
+            ctx = [hi + r.randint(0, hi // r.choice([1, 4, 1000])) for _ in range(n_long)] + [r.randint(1, 60) for _ in range(n_short)]
+            chunk = [r.choice([1, 5, 32])] * n_long + [r.choice([1, 4])] * n_short
+            off = np.concatenate([[0], np.cumsum(chunk)]).tolist()
+            pages = [(a + b + 15) // 16 for a, b in zip(ctx, chunk)]
+            table = torch.zeros(len(ctx), max(pages), dtype=torch.int32)
+            for i, first in enumerate(np.cumsum([0] + pages[:-1])):
+                table[i, :pages[i]] = torch.arange(first, first + pages[i], dtype=torch.int32)
+            s = syn.plan_work_host(ModelShape("cut", 1, 256, group * heads, heads, hd, 256, 512), sum(pages),
+                                   torch.zeros(off[-1], dtype=torch.int32), off, table, ctx)["stats"]
+            assert s.attn_split_items * s.attn_rows <= 592 * 64, (ctx, chunk)
+    finally:
+        syn.debug_set_attention(0)
+
+
 def test_keys_that_may_be_read_before_the_chunks_are_written():
     """Up to the first page of a request that any request of the batch writes, over shared pages too; nothing in the lists of the
     kernels that wait for the projection first."""
