@@ -962,15 +962,14 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
         }
         // Few: whole units (as good as their number divides), equal parts of which there are no more than CTAs, or wrapped; with
         // two CTAs or more to a unit equal parts are as even and have fewer merges (64 units of the 8B shape on 296 CTAs: 29.5 us
-        // wrapped, 28.8 in equal parts).  Equal parts of more than 128 units: 256 of them if that is enough to cut
-        // some, else two to a unit.
+        // wrapped, 28.8 in equal parts).
         int64_t best = y.n_units <= slots ? y.longest : std::max(y.longest, (y.n_units + slots - 1) / slots * (y.total / y.n_units));
         y.limit = y.longest;
-        auto cut = [&](int64_t most) {
+        if (y.n_units <= slots) {
             auto fits = [&](int64_t lim) {
                 int64_t n = 0;
                 for (const Unit& u : y.units) n += (int64_t)parts_of(y, u, lim) * Hkv;
-                return n <= most;
+                return n <= slots;
             };
             int64_t lo = k.item, hi = y.longest;
             while (hi - lo > 256) {   // the number of parts falls with the limit; at `hi` nothing is cut
@@ -982,15 +981,10 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
                 const int np = parts_of(y, u, hi);
                 part = std::max(part, (u.nb + np - 1) / np * u.bc + k.item + (np > 1 ? k.part + k.merge + std::min(np, 8) * tiles(u) * k.merge_tile : 0));
             }
-            if (part >= best) return false;
-            best = part;
-            y.limit = hi;
-            return true;
-        };
-        if (y.n_units <= slots) {
-            const int even_parts = 256;
-            const bool many = 2 * y.n_units > even_parts;
-            if (!cut(many ? std::min(slots, even_parts) : slots) && many) cut(std::min<int64_t>(slots, 2 * y.n_units));
+            if (part < best) {
+                best = part;
+                y.limit = hi;
+            }
         }
         if (2 * y.n_units > slots) {
             std::sort(y.units.begin(), y.units.end(), [](const Unit& p, const Unit& q) {

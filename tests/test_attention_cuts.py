@@ -76,6 +76,27 @@ def test_few_long_requests_among_many_short_ones_are_not_cut_small(kind, heads, 
     assert max(keys) <= 1.5 * sum(keys) / len(keys)
 
 
+@pytest.mark.parametrize("n_req", range(15, 21))
+def test_a_little_less_than_one_or_one_unit_to_an_sm_is_shared_out_over_all_ctas(n_req):
+    """120 to 160 units of unequal lengths on the 296 CTAs of the half-SM kernel."""
+    syn.debug_set_attention(3)
+    try:
+        for seed in range(8):
+            r = random.Random(seed)
+            ctx = [r.randint(256, 2048) for _ in range(n_req)]
+            pages = [(n + 20) // 16 for n in ctx]
+            table = torch.zeros(n_req, max(pages), dtype=torch.int32)
+            for i, first in enumerate(np.cumsum([0] + pages[:-1])):
+                table[i, :pages[i]] = torch.arange(first, first + pages[i], dtype=torch.int32)
+            p = syn.plan_work_host(ModelShape("cut", 1, 256, 32, 8, 128, 256, 512), sum(pages),
+                                   torch.zeros(5 * n_req, dtype=torch.int32), list(range(0, 5 * n_req + 1, 5)), table, ctx)
+            cb, items = p["cta_begin"].numpy(), p["items"].numpy()
+            keys = [int((items[a:b, 5] - items[a:b, 4]).sum()) for a, b in zip(cb, cb[1:])]
+            assert len(keys) > 256 and max(keys) <= 1.95 * sum(keys) / 296, (seed, len(keys), max(keys))
+    finally:
+        syn.debug_set_attention(0)
+
+
 @pytest.mark.parametrize("kind", [0, 1, 2, 3])
 @pytest.mark.parametrize("heads,hd,group", [(8, 128, 4), (8, 64, 4), (21, 128, 1), (2, 64, 5)])
 def test_no_plan_has_more_partials_than_the_static_array_holds(kind, heads, hd, group):
