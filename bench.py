@@ -32,8 +32,11 @@ UNIT = "tokens/s"
 # workload (mean over all launches of the kernel function), with the hash of the kernel's source files at capture
 # time: the figure is reported only while those sources are unchanged.  Summaries of the captures: profiles/.
 KERNEL_SOURCES = {"attn_kernel": ("attention.cuh", "ptx.cuh"), "attn2_kernel": ("attention2.cuh", "attention.cuh", "ptx.cuh"),
+                  "attn_thin_kernel": ("attention_thin.cuh", "attention.cuh", "ptx.cuh"),
                   "gemm_kernel": ("gemm.cuh", "ptx.cuh"),
-                  "gemm2_kernel": ("gemm2.cuh", "gemm.cuh", "ptx.cuh")}
+                  "gemm2_kernel": ("gemm2.cuh", "gemm.cuh", "ptx.cuh"),
+                  "thin_kernel": ("gemm_thin.cuh", "gemm.cuh", "ptx.cuh")}
+ATTENTION_KERNELS = {1: "attn_kernel", 2: "attn2_kernel", 3: "attn_thin_kernel"}
 NCU_TRAFFIC = {
     # workload: {kernel function: (bytes per launch, sha256 of its source files, concatenated in KERNEL_SOURCES order)}
     "cfg3-8b": {
@@ -46,6 +49,17 @@ NCU_TRAFFIC = {
         "attn2_kernel": (645360384, "7fa04845d77dfc4a75ca49139f07f2f0889eaeb7f399609f71523e9aeed52efd"),
     },
 }
+
+
+def projection_kernel(T: int, N: int, K: int, epilogue: str, schedule: str = "auto") -> str:
+    """The kernel function that serves a projection: the library's launch rule, asked of its schedule exports."""
+    import paper_2511_07423_b200 as syn
+    if schedule == "auto":
+        if syn.thin_plan_host(T, N, K, epilogue)["takes_it"]:
+            return "thin_kernel"
+        if syn.gemm2_plan_host(T, N, K, epilogue)["kind"] != 0:
+            return "gemm2_kernel"
+    return "gemm_kernel"
 
 
 def _source_hash(kernel: str) -> str:
@@ -208,7 +222,7 @@ def run_ours(args):
     shape = wl.shape
     peaks = _peaks()
     syn.debug_set_schedule({"auto": 0, "one-cta": 1}[args.schedule])
-    syn.debug_set_attention({"auto": 0, "warp-mma": 1, "tcgen05": 2}[args.attention])
+    syn.debug_set_attention({"auto": 0, "warp-mma": 1, "tcgen05": 2, "half-sm": 3}[args.attention])
 
     via_host = shape.dense_params() * 2 > 40e9
     model = synthetic.load_model(shape, wl.seed, via_host=via_host)
@@ -296,19 +310,17 @@ def run_ours(args):
         if name == "attention":
             k["kv_gbs"] = kv_bytes_layer / (avg * 1e-3) / 1e9
         kernels[name] = k
-    # The projection classes are launches of two kernel functions: gemm2_kernel (CTA pairs, from 256 tokens on) and
-    # gemm_kernel (one CTA per item); which one a class takes is the library's launch rule, asked of its schedule export.
+    # The projection classes are launches of three kernel functions: thin_kernel (batches of few tokens), gemm2_kernel (CTA
+    # pairs) and gemm_kernel (one CTA per item).
     shapes = {"qkv_gemm": (qd + 2 * kd, d, "qkv"), "o_gemm": (d, qd, "resid"), "gate_up_gemm": (2 * ((f + 63) // 64 * 64), d, "swiglu"),
               "down_gemm": (d, (f + 63) // 64 * 64, "resid"), "lm_head_gemm": (V, d, "lmhead")}
     func_of = {}
     for name, (N_, K_, epi) in shapes.items():
-        pair = args.schedule == "auto" and syn.gemm2_plan_host(T, N_, K_, epi)["kind"] != 0
-        func_of[name] = "gemm2_kernel" if pair else "gemm_kernel"
+        func_of[name] = projection_kernel(T, N_, K_, epi, args.schedule)
         if name in kernels:
             kernels[name]["kernel"] = func_of[name]
     ridge = peaks["tf_sustained"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
-    # the attention kernel the planner chose for this batch: row tiles of 64 (warp-level MMAs) or 128 (tcgen05)
-    attn_func = "attn2_kernel" if st.attn_rows == 128 else "attn_kernel"
+    attn_func = ATTENTION_KERNELS[plan.attention_kernel()]   # the planner's choice for this batch
     kernels["attention"]["kernel"] = attn_func
 
     def func_roof(func):
@@ -333,7 +345,7 @@ def run_ours(args):
             out.update({"bound": "hbm", "achieved": wb / (ms_step * 1e-3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s"})
         return out
 
-    roofs = [r_ for r_ in (func_roof(fn) for fn in ("gemm2_kernel", "gemm_kernel", attn_func)) if r_]
+    roofs = [r_ for r_ in (func_roof(fn) for fn in ("gemm2_kernel", "gemm_kernel", "thin_kernel", attn_func)) if r_]
     for r_ in roofs:
         r_["frac"] = r_["achieved"] / r_["peak"]
         r_["peak_source"] = peaks["source"] + (" sustained" if r_["bound"] == "tensor" else "")
@@ -464,10 +476,10 @@ def main():
     ap.add_argument("--config", type=int, default=3, help="1..6; 3 = the 8B-shape step the metric is quoted on; 6 = 32-token chunked partial prefill")
     ap.add_argument("--pool-tokens", type=int, default=None)
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--attention", default="auto", choices=["auto", "warp-mma", "tcgen05"],
+    ap.add_argument("--attention", default="auto", choices=["auto", "warp-mma", "tcgen05", "half-sm"],
                     help="auto: the planner's cost model picks the attention kernel for the batch")
     ap.add_argument("--schedule", default="auto", choices=["auto", "one-cta"],
-                    help="auto: every projection takes the kernel its shape calls for; one-cta: none takes the CTA-pair kernel")
+                    help="auto: every projection takes the kernel its shape calls for; one-cta: none takes the CTA-pair or the half-SM kernel")
     args = ap.parse_args()
     if args.impl == "reference":
         run_reference(args)

@@ -183,7 +183,7 @@ typedef struct {
     double attn_flops;             /* 4 * Hq*hd * n_layers * sum over tokens of keys seen    */
     int32_t attn_items, attn_split_items; /* attention work items per layer / those that are partial */
     int32_t kernel_launches;       /* kernels launched by one syn_verify_run                */
-    int32_t attn_rows;             /* row tile of the attention kernel the batch was planned for: 64 (warp-level MMAs) or 128 (tcgen05) */
+    int32_t attn_rows;             /* row tile of the attention kernel the batch was planned for: 64 (warp-level MMAs) or 128 (tcgen05); the kernel: syn_plan_attention */
     int64_t h2d_bytes;             /* batch description uploaded per step by syn_verify_batch */
     double t_gpu_ms;               /* device time of the step, first kernel to last (CUDA events); 0 unless profiling is on */
     double t_wall_ms;              /* host wall time of the blocking call that ran it; 0 unless profiling is on  */
@@ -194,6 +194,9 @@ typedef struct {
  * t_wall_ms.  SYN_E_INVALID_ARG before the first step.  syn_plan_stats: the counters of a plan. */
 int syn_last_step_stats(syn_model *m, syn_step_stats *out);
 int syn_plan_stats(const syn_plan *p, syn_step_stats *out);
+/* The attention kernel a plan was laid out for, numbered as in syn_debug_set_attention: 1, 2 or 3 (attn_rows is 64 for 1
+ * and 3).  Which kernel a projection takes: syn_thin_plan_host, then syn_gemm2_plan_host.  Errors: SYN_E_INVALID_ARG. */
+int syn_plan_attention(const syn_plan *p);
 
 /* The host planner of syn_plan_create / syn_verify_batch on its own, without a device: the same
  * validation (same error codes, same order) and the same outputs, written to caller-provided HOST

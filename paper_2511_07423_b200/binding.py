@@ -57,7 +57,7 @@ _LIB: Optional[C.CDLL] = None
 
 EXPORTS = ["syn_model_load", "syn_model_free", "syn_kv_alloc", "syn_kv_free", "syn_kv_import", "syn_kv_export",
            "syn_verify_batch", "syn_plan_create", "syn_plan_free", "syn_verify_run", "syn_model_status",
-           "syn_last_step_stats", "syn_plan_stats", "syn_plan_host", "syn_plan_work_host", "syn_strerror", "syn_last_cuda_error", "syn_op_linear",
+           "syn_last_step_stats", "syn_plan_stats", "syn_plan_attention", "syn_plan_host", "syn_plan_work_host", "syn_strerror", "syn_last_cuda_error", "syn_op_linear",
            "syn_op_linear_as", "syn_op_linear_reset", "syn_debug_set_spin_limit", "syn_debug_linear_counter", "syn_debug_set_schedule",
            "syn_debug_set_attention",
            "syn_op_attention", "syn_op_attention_static",
@@ -320,6 +320,13 @@ class Plan:
                                           C.c_void_p(q.data_ptr()), C.c_void_p(out.data_ptr()), _stream_ptr(stream)),
                "syn_op_attention")
         return out
+
+    def attention_kernel(self) -> int:
+        """syn_plan_attention: the attention kernel the plan was laid out for, numbered as in debug_set_attention."""
+        r = self._lib.syn_plan_attention(self._h)
+        if r < 0:
+            _check(r, "syn_plan_attention")
+        return r
 
     def attention_static(self, layer: int, q: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         """syn_op_attention_static: the attention of the step for callers that cannot allocate while

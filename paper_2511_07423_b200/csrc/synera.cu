@@ -1344,6 +1344,8 @@ static int syn_plan_create_impl(syn_model* m, syn_kv* kv, int32_t n_req, const i
     return SYN_OK;
 }
 
+extern "C" int syn_plan_attention(const syn_plan* p) { return p ? p->attn : SYN_E_INVALID_ARG; }
+
 extern "C" int syn_plan_stats(const syn_plan* p, syn_step_stats* out) {
     if (!p || !out) return SYN_E_INVALID_ARG;
     *out = p->stats;
