@@ -447,11 +447,21 @@ static cudaError_t kernel_smem(K kernel, int bytes) {
     if (e == cudaSuccess && bytes > 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
+// Which variants of the one-CTA projection kernel an epilogue meets (gemm_plan): leftover tiles of a residual projection are
+// not cut along K, only qkv and residual projections share K.
+constexpr bool gemm_variant_used(int variant, int mode) {
+    return variant == GEMM_KSPLIT ? mode != EPI_RESID : (variant == GEMM_RSPLIT ? mode != EPI_SWIGLU && mode != EPI_LMHEAD : true);
+}
+template <int VARIANT, int MODE>
+static cudaError_t gemm_kernel_smem() {
+    if constexpr (gemm_variant_used(VARIANT, MODE)) return kernel_smem(gemm_kernel<VARIANT, MODE>, GEMM_SMEM_MAX);
+    else return cudaSuccess;
+}
 template <int MODE>
 static cudaError_t projection_smem() {   // the projection kernels with one epilogue
-    const cudaError_t all[] = {kernel_smem(gemm_kernel<GEMM_WAVES, MODE>, GEMM_SMEM_MAX), kernel_smem(gemm_kernel<GEMM_KSPLIT, MODE>, GEMM_SMEM_MAX),
-                               kernel_smem(gemm_kernel<GEMM_RSPLIT, MODE>, GEMM_SMEM_MAX), kernel_smem(gemm2_kernel<false, MODE>, GEMM_SMEM_MAX),
-                               kernel_smem(gemm2_kernel<true, MODE>, GEMM_SMEM_MAX), kernel_smem(thin_kernel<MODE>, THIN_SMEM_MAX)};
+    const cudaError_t all[] = {gemm_kernel_smem<GEMM_WAVES, MODE>(), gemm_kernel_smem<GEMM_KSPLIT, MODE>(), gemm_kernel_smem<GEMM_RSPLIT, MODE>(),
+                               kernel_smem(gemm2_kernel<false, MODE>, GEMM_SMEM_MAX), kernel_smem(gemm2_kernel<true, MODE>, GEMM_SMEM_MAX),
+                               kernel_smem(thin_kernel<MODE>, THIN_SMEM_MAX)};
     for (cudaError_t e : all)
         if (e != cudaSuccess) return e;
     return cudaSuccess;
@@ -1448,6 +1458,19 @@ static int gemm_plan(int T, int packed_rows, int K, int n_sm, int mode, bool may
         default: { constexpr int MODE = EPI_PLAIN; call; break; }          \
     }
 
+template <int VARIANT, int MODE>
+static cudaError_t launch_gemm_variant(const GemmParams& g, int n_cta, const CUtensorMap& tmB, const EpiParams& ep, cudaStream_t st) {
+    const int smem = gemm_fixed_smem(g.TN) + g.n_stages * gemm_stage_bytes(g.TN);
+    if constexpr (gemm_variant_used(VARIANT, MODE)) return launch_pdl(gemm_kernel<VARIANT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep);
+    else return note_cuda(cudaErrorInvalidDeviceFunction);
+}
+template <int MODE>
+static cudaError_t launch_gemm_mode(const GemmParams& g, int n_cta, const CUtensorMap& tmB, const EpiParams& ep, cudaStream_t st) {
+    return g.splits > 1 ? launch_gemm_variant<GEMM_RSPLIT, MODE>(g, n_cta, tmB, ep, st)
+           : g.ksplit > 1 ? launch_gemm_variant<GEMM_KSPLIT, MODE>(g, n_cta, tmB, ep, st)
+                          : launch_gemm_variant<GEMM_WAVES, MODE>(g, n_cta, tmB, ep, st);
+}
+
 // One projection with the epilogue `ep`; `plan_mode` = the epilogue its schedule is made for (the
 // same, except in the test hook, which runs any schedule with the plain store epilogue).
 static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const op16* w_packed, int packed_rows, int K,
@@ -1464,11 +1487,8 @@ static int launch_gemm(syn_model* prof_m, int cls, int n_sm, int* status, const 
     g.status = status;
     g.fix_part = fix_part; g.fix_flag = fix_flag;
     g.spin_limit = g_spin_limit;
-    const int smem = gemm_fixed_smem(g.TN) + g.n_stages * gemm_stage_bytes(g.TN);
     cudaError_t le;
-    EPI_SWITCH(ep.mode, le = g.splits > 1 ? launch_pdl(gemm_kernel<GEMM_RSPLIT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep)
-                        : g.ksplit > 1 ? launch_pdl(gemm_kernel<GEMM_KSPLIT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep)
-                                       : launch_pdl(gemm_kernel<GEMM_WAVES, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep));
+    EPI_SWITCH(ep.mode, le = launch_gemm_mode<MODE>(g, n_cta, tmB, ep, st));
     return le == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 

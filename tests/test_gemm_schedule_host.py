@@ -179,3 +179,13 @@ def test_pair_schedule_sweep(force):
             _check2(T, N, K, epi, force)
     for n_sm in (2, 7, 132, 148, 160):
         _check2(544, 28672, 4096, "swiglu", force, n_sm)
+
+
+def test_variants_that_are_not_built_are_never_asked_for():
+    """The one-CTA kernel has no K-shared form of the SwiGLU and lm_head epilogues and no leftover tiles cut along K for the
+    residual one."""
+    for N, K, epi in [(16384, 2048, "swiglu"), (28672, 4096, "swiglu"), (1408, 256, "swiglu"), (32000, 2048, "lmhead"),
+                      (128256, 4096, "lmhead"), (1024, 256, "lmhead"), (2048, 8192, "resid"), (5120, 27648, "resid"), (256, 704, "resid")]:
+        for T in range(1, 2400, 13):
+            p = syn.gemm_plan_host(T, N, K, epi)
+            assert p["ksplit"] == 1 if epi == "resid" else p["splits"] == 1, (T, N, K, epi)
