@@ -271,11 +271,11 @@ int syn_op_linear_reset(void);
  * that a wait for a count that can no longer be reached runs out; the counters are cleared again when
  * the timeout is reported.  A wait that runs out unwinds normally: the kernel ends, the results of
  * that call are invalid, the next call works.
- * syn_debug_set_schedule: 0 (default) lets every projection take the kernel its shape calls for (CTA
- * pairs from 256 tokens on); 1 keeps all of them on the one-CTA kernel, so that both can be measured
- * and checked on the same batch.  Process-wide.
+ * syn_debug_set_schedule: 0 (default) lets every projection take the kernel its shape calls for (half-SM
+ * CTAs for few tokens, CTA pairs from 256 tokens on); 1 keeps all of them on the one-CTA kernel, so that they
+ * can be measured and checked on the same batch.  Process-wide.
  * syn_debug_set_attention: which attention kernel the plans made AFTERWARDS are laid out for (a plan
- * keeps its kernel): 0 (default) the cheaper of the two for the batch by the planner's cost model, 1 the
+ * keeps its kernel): 0 (default) the cheapest for the batch by the planner's cost model, 1 the
  * warp-level-MMA kernel (row tiles of 64), 2 the tcgen05 kernel (row tiles of 128: a whole chunk of up to
  * 128 / G tokens is one work item per kv head), 3 the warp-level-MMA kernel in CTAs of half an SM (row tiles of
  * 64; few requests).  Process-wide. */
@@ -300,7 +300,8 @@ int syn_op_attention(syn_model *m, syn_kv *kv, const syn_plan *p, uint32_t layer
  * that grows on demand.  The array holds SYN_STATIC_MAX_PARTS partials of 64 rows, or half as many of
  * the 128-row kind of a plan made for the tcgen05 kernel: two for each CTA of a plan for the 148 SMs of a
  * B200, which is more than any such plan has (about 19.7 MB of every GPU that loads the library, from load
- * to exit).  The call itself allocates and frees nothing; the model, cache and plan it is given were of course allocated earlier by their own calls.
+ * to exit).  The call itself allocates and frees nothing; the model, cache and plan it is given were of
+ * course allocated earlier by their own calls.
  *   - A plan with more partial work items than that (attn_split_items x attn_rows of syn_plan_stats()
  *     above SYN_STATIC_MAX_PARTS x 64) is refused with SYN_E_CAPACITY before anything is launched.
  *   - The first call on each device looks up the array's device address (with that device

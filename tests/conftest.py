@@ -26,7 +26,7 @@ def pytest_collection_modifyitems(config, items):
             it.add_marker(skip)
 
 
-@pytest.fixture(params=[1, 2], ids=["warp_mma_attention", "tcgen05_attention"])
+@pytest.fixture(params=[1, 2, 3], ids=["warp_mma_attention", "tcgen05_attention", "half_sm_attention"])
 def attention_kind(request):
     """Plans made inside the test are laid out for the named attention kernel (the default leaves the
     choice to the planner's cost model)."""

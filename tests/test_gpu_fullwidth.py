@@ -49,7 +49,7 @@ def test_two_layers_at_full_width_meet_a_third_of_the_stated_tolerance(cfg, n_ju
 
 
 def test_wide_batch_at_the_1b_width_puts_64_wide_heads_through_the_pair_kernels():
-    """Configuration 2's own batch (129 tokens) stays on the one-CTA kernel.  A wider mix at the same width
+    """Configuration 2's own batch (129 tokens) goes to the half-SM kernel, its lm_head to the one-CTA kernel.  A wider mix at the same width
     (64 requests, chunks of 9-16 tokens: about 800 tokens) sends the qkv projection (64-wide heads, two per
     128-feature tile), gate/up, down (K shared between clusters) and the lm_head through the CTA-pair kernel."""
     import paper_2511_07423_b200 as syn

@@ -86,18 +86,37 @@ def test_config1_tiny_real_prefill():
     print("config 1:", res)
 
 
-@pytest.mark.parametrize("shape,ctx,chunk", [
+MINI_BATCHES = [
     (MINI_1B, [0, 33, 48, 200, 515, 1030], [1, 8, 16, 5, 3, 11]),     # head_dim 64, G = 4
     (MINI_8B, [17, 64, 300, 1200], [16, 2, 9, 13]),                    # head_dim 128, G = 4
     (ModelShape("g5", 2, 640, 10, 2, 128, 1376, 3000), [100, 40], [16, 13]),   # G = 5, ffn and vocab with ragged tails
-])
-def test_mini_shapes_synthetic_cache(shape, ctx, chunk, attention_kind):
+]
+
+
+def _mini_batch(shape, ctx, chunk):
     wl = Workload("mini", shape, 11, len(ctx), ("list", tuple(ctx)), ("list", tuple(chunk)), 0.7)
     batch = gen.gen_batch(wl)
     glob, layers, model, kv, orc, pools = _setup(shape, wl.seed, batch)
     fill_synthetic_kv(shape, wl.seed, batch, range(batch.n_req), kv=kv, orc=orc, pools=pools)
     res = _run_and_judge(wl, shape, batch, glob, layers, kv, orc, pools)
     print(shape.name, res)
+
+
+@pytest.mark.parametrize("shape,ctx,chunk", MINI_BATCHES)
+def test_mini_shapes_synthetic_cache(shape, ctx, chunk, attention_kind):
+    _mini_batch(shape, ctx, chunk)
+
+
+@pytest.mark.parametrize("shape,ctx,chunk", MINI_BATCHES)
+def test_mini_shapes_on_the_one_cta_projection_kernel(shape, ctx, chunk):
+    """Its narrow token tiles under the real epilogues; left to itself a batch this small goes to the half-SM kernel."""
+    import paper_2511_07423_b200 as syn
+    assert syn.thin_plan_host(sum(chunk), shape.q_dim + 2 * shape.kv_dim, shape.d_model, "qkv")["takes_it"]
+    syn.debug_set_schedule(1)
+    try:
+        _mini_batch(shape, ctx, chunk)
+    finally:
+        syn.debug_set_schedule(0)
 
 
 @pytest.mark.parametrize("shape,ctx,chunk,unc", [
