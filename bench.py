@@ -39,14 +39,19 @@ KERNEL_SOURCES = {"attn_kernel": ("attention.cuh", "ptx.cuh"), "attn2_kernel": (
 ATTENTION_KERNELS = {1: "attn_kernel", 2: "attn2_kernel", 3: "attn_thin_kernel"}
 NCU_TRAFFIC = {
     # workload: {kernel function: (bytes per launch, sha256 of its source files, concatenated in KERNEL_SOURCES order)}
+    "cfg2-1b": {
+        "thin_kernel": (32196796, "2e01dbe3661164617189274d7da000de05012eaeeb668e0e0b285f040c9db72e"),
+        "attn_thin_kernel": (101482616, "c15f438fe67f82a42070b50b1a589e21cdee7de006bae23d6701a98435f29729"),
+        "gemm_kernel": (132080128, "01423ee77c3e6e9cd2a0b3d7cfacb36cd74633fc48409c049d7b319f7a9bf44c"),
+    },
     "cfg3-8b": {
-        "attn_kernel": (616005760, "e7eab610c1c0e32bcd8a2b1b08bccefa5523b7c068fd3c6ca6349d9a5a0c9722"),
-        "gemm_kernel": (284994688, "415a44815d425fce6e0ffc40b6e9788e53f3b2c3d4b3acc83ceb62134c7a078c"),
-        "gemm2_kernel": (99183492, "61a52084542c4d41ffc56e91dceb9efb0846429310e9840952db0981acfd97ec"),
+        "attn_kernel": (615962556, "8cd80ea1f2e28708eabb2221a023e64c167ce5dcbad16aaaf965c0f1dcf61f05"),
+        "gemm_kernel": (284728176, "01423ee77c3e6e9cd2a0b3d7cfacb36cd74633fc48409c049d7b319f7a9bf44c"),
+        "gemm2_kernel": (99020461, "b9b3fd16ffeb2cdbca861d0fbafeb9d9f2d15003e4c3f3fbccade3fc4e2a0c48"),
     },
     # one layer's launch of the same work list, captured through `opbench attention --config 6 --kind 2`
     "cfg6-8b-chunk32": {
-        "attn2_kernel": (645360384, "7fa04845d77dfc4a75ca49139f07f2f0889eaeb7f399609f71523e9aeed52efd"),
+        "attn2_kernel": (644797184, "2dd11156593b20096e42310454f2fbdb28bacb67a59033656c84df11431cc558"),
     },
 }
 

@@ -10,9 +10,10 @@
 //   - queries go straight from L2 to registers: no Q tile, no barrier for it;
 //   - K and V that no chunk of the batch writes (AttnItem::kv_safe) are requested before the projection that
 //     writes the chunks' K and V has finished.
-// What bounds it: with 64-dim heads the arithmetic of a stage on one warp and the last CTA's merge (1B shape, 40 requests 43.8 us a
-// layer against 49.3 of the full-SM kernel, 150 requests 60 against 72; 26 and 39 are the bytes at the copy rate); with
-// 128-dim heads and many units the warps' arithmetic (8B shape, 64 requests 146 us against 113), so those keep the full-SM kernel.
+// What bounds it: with 64-dim heads the arithmetic of a stage on one warp and the last CTA's merge (1B shape, contexts
+// 256-2048, chunks 1-8: 150 requests 71 us a layer against 88 of the full-SM kernel, 40 requests 33.0 against 33.4 and a step of 4
+// layers 385 us against 395); with 128-dim heads and many units the warps' arithmetic (8B shape, 64 requests of 512-4096,
+// chunks 1-16: 174 us against 137), so those keep the full-SM kernel.
 #pragma once
 #include "attention.cuh"
 

@@ -25,13 +25,13 @@
 // 16-byte pieces of token-major rows:
 //   EPI_QKV    : RMSNorm scale, RoPE on q and k (the partner dimension sits 16 lanes away), q store,
 //                paged-KV append
-//   EPI_RESID  : x += D (the residual stream, fp32), the next projection's operand bf16(x * gain) and
+//   EPI_RESID  : x += D (the residual stream, fp32), the next projection's operand half(x * gain) and
 //                the sums of x^2 over each group of 32 features that the next RMSNorm needs
 //   EPI_SWIGLU : RMSNorm scale, silu(gate) * up (a gate feature and its up feature sit 16 lanes apart)
 //   EPI_LMHEAD : RMSNorm scale, optional logits, vocabulary argmax (warp reduction, packed 64-bit atomicMax)
 //   EPI_PLAIN  : fp32 store (test hook)
 // RMSNorm is split between producer and consumer: the kernel that writes the residual stream
-// (EPI_RESID, or prep_kernel for the first layer) stores bf16(x * gain) and partial sums of x^2; the
+// (EPI_RESID, or prep_kernel for the first layer) stores half(x * gain) and partial sums of x^2; the
 // projection that consumes it multiplies its accumulators by the token's 1/sqrt(mean(x^2) + eps),
 // a per-column scalar in this orientation, which its epilogue warps work out from the partial sums
 // while the main loop runs.
@@ -190,7 +190,7 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
             }
         }
     } else if (MODE == EPI_RESID) {
-        // x += D; operand of the next projection bf16(x * gain); sum of x^2 over this warp's 32 features
+        // x += D; operand of the next projection half(x * gain); sum of x^2 over this warp's 32 features
         const int f = m0 + quarter * 32 + c0;
         const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.x);
         const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.y);
@@ -426,7 +426,7 @@ __global__ void pack_weight_kernel(PackSrc src, op16* __restrict__ out, int num_
 // (four groups of four; a group covers the four TMEM lane quarters; draining TMEM is limited per
 // warp, so many warps share it).
 // ------------------------------------------------------------------------------------------
-constexpr int GEMM_BK = 64;                        // bf16 elements per k-block = one 128-byte swizzle row
+constexpr int GEMM_BK = 64;                        // 16-bit elements per k-block = one 128-byte swizzle row
 constexpr int GEMM_TILE_BYTES = 128 * GEMM_BK * 2; // 16 KB: one 128-feature tile of one k-block
 constexpr int GEMM_A_BYTES = 2 * GEMM_TILE_BYTES;  // stage room for a pair
 constexpr int GEMM_BOX_ROWS = 32;                  // token rows per B box
@@ -691,7 +691,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     // consecutive MMAs alternate between the two accumulators: back-to-back MMAs into
                     // one accumulator wait for each other
 #pragma unroll
-                    for (int k = 0; k < GEMM_BK / 16; ++k)  // 16 bf16 = 32 bytes = 2 descriptor address units
+                    for (int k = 0; k < GEMM_BK / 16; ++k)  // 16 halves = 32 bytes = 2 descriptor address units
                         for (int mt = w.mt_lo; mt < w.mt_hi; ++mt) {
                             const uint64_t da = umma_desc_k128(a_addr + mt * GEMM_TILE_BYTES);
                             umma_bf16(tmem_base + mt * acc_stride, da + 2 * k, db + 2 * k, idesc, j > 0 || k > 0);

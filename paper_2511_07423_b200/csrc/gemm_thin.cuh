@@ -4,8 +4,9 @@
 //   - A CTA takes HALF an SM (at most 113 KB of shared memory, 256 TMEM columns, 320 threads of at most
 //     102 registers), so that the CTAs of two consecutive kernels are resident together: while a
 //     kernel drains, its successor has set up its barriers and filled its operand ring with weights
-//     (they depend on nothing).  A kernel lets its successor start once its own predecessor is
-//     complete, so at most two kernels of the chain are ever unfinished.
+//     (they depend on nothing).  This kernel lets its successor start once its own predecessor is
+//     complete, so that of a chain of such kernels at most two are unfinished (the full-SM kernels
+//     let theirs start before they wait; it cannot become resident beside them anyway).
 //   - Work item = 128 output features x one token tile (all tokens up to 128, else equal tiles) x one of
 //     S parts of K.  The S CTAs of an item are a cluster: they hand each other fp32 accumulators
 //     through distributed shared memory (a reduce-scatter over units of 32 features x 16 tokens, added in
@@ -13,12 +14,12 @@
 //     global memory and no counters.
 //   - Same orientation, weight tiles and epilogues (epi_unit) as gemm.cuh.  Two accumulators take
 //     alternate k-steps (an MMA into the accumulator of its predecessor waits for it).
-// Measured when it was written (the epilogues have since become shorter for all kernels), whole steps against the one-CTA kernel: 1B shape, 5 tokens 1 334 -> 866 us; 135 tokens 1 837 ->
-// 1 380 us; 8B shape, 40 tokens 5 353 -> 4 179 us (the weights alone take 2 325 us at the copy rate).  One launch of
-// the 8B o projection (33.5 MB) at 40 tokens: 8.8 us until its last MMA and 2.9 us more to its end.  What bounds it: HBM
-// while it streams (4.5 - 5 TB/s in a launch of its own), and about 3 us per launch that depend on the
+// Whole steps, every projection on the one-CTA kernel -> with this one: 1B shape, 5 tokens 1 187 -> 821 us; 135 tokens
+// 1 611 -> 1 340 us; 8B shape, 40 tokens 4 600 -> 3 820 us (the weights alone take 2 325 us at the copy rate), 119 tokens
+// 6 100 -> 5 760 us.  The 8B o projection (33.5 MB) at 40 tokens: 26.1 -> 15.5 us between events in the step.  What bounds
+// it: HBM while it streams (4.5 - 5 TB/s in a launch of its own), and about 3 us per launch that depend on the
 // predecessor (its results visible, token operand, exchange, epilogue).  Tried and dropped: 256 CTAs instead of
-// 148 and fewer (8B shape 4 775 us), asking L2 for the next projection's weights (1 to 5 % slower: the
+// 148 and fewer (14 % slower at the 8B shape), asking L2 for the next projection's weights (1 to 5 % slower: the
 // requests compete with the loads that the step waits for), two cluster barriers around plain remote
 // stores instead of the counted asynchronous ones.
 #pragma once

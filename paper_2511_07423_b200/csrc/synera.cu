@@ -94,7 +94,7 @@ static cudaError_t launch_pdl_clusters(void (*kernel)(KArgs...), dim3 grid, dim3
 // ------------------------------------------------------------------------------------------ small kernels
 
 // Token embedding (paper Sec. 4.5: the flattened batch enters the transformer), the first layer's
-// GEMM operand bf16(x * gain) with the sums of x^2 per 32 features its RMSNorm scale is made of,
+// GEMM operand half(x * gain) with the sums of x^2 per 32 features its RMSNorm scale is made of,
 // RoPE table, argmax reset.
 __global__ void __launch_bounds__(256)
 prep_kernel(const bf16* __restrict__ embed, const int* __restrict__ tokens, const int* __restrict__ pos,
@@ -1831,7 +1831,7 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     // the consumers of a normalised operand: RMSNorm scale from the partial sums of x^2
     EpiParams scaled = base;
     scaled.ssq_in = m->ssq; scaled.n_ssq = d / 32; scaled.inv_d = inv_d; scaled.eps = c.rms_eps;
-    // the writers of the residual stream: x += D, next operand bf16(x * gain), new partial sums
+    // the writers of the residual stream: x += D, next operand half(x * gain), new partial sums
     EpiParams resid = base;
     resid.mode = EPI_RESID; resid.N = d; resid.d = d; resid.x = m->x; resid.xg = m->xn; resid.ssq_out = m->ssq;
     // (the projections' plans, some 6 us each, are made in the first layer, while the kernels before run)

@@ -220,12 +220,12 @@ def main():
     l.add_argument("--N", type=int, default=28672)
     l.add_argument("--K", type=int, default=4096)
     l.add_argument("--iters", type=int, default=10)
-    l.add_argument("--sched", default="plain", help="schedule: plain, qkv, resid, swiglu, lmhead, pair_quad, pair_duo, pair_quad_resid, pair_duo_resid")
+    l.add_argument("--sched", default="plain", help="schedule: plain, qkv, resid, swiglu, lmhead, pair_quad, pair_duo, pair_quad_resid, pair_duo_resid, thin")
     l.add_argument("--one-cta", action="store_true", help="keep the projection on the one-CTA kernel whatever its shape")
     t = sub.add_parser("attention")
     t.add_argument("--config", type=int, default=3)
     t.add_argument("--pool-tokens", type=int, default=None)
-    t.add_argument("--kind", type=int, default=0, help="attention kernel: 0 default, 1 warp-level MMAs, 2 tcgen05")
+    t.add_argument("--kind", type=int, default=0, help="attention kernel: 0 default, 1 warp-level MMAs, 2 tcgen05, 3 half-SM CTAs")
     t.add_argument("--iters", type=int, default=10)
     m = sub.add_parser("sample")
     m.add_argument("--config", type=int, default=3)
