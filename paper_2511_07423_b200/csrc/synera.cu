@@ -1543,7 +1543,9 @@ static double proj_cost(int T, int packed_rows, int K, int n_sm, int mode, int k
         }
         worst = std::max(worst, sum);
     }
-    return worst;
+    // 256-feature items left after the full waves and cut along K: 84 of them between 264 and 2 040 tokens took 1.09 times the
+    // estimate, up to 1.25 (qkv of the 32B shape at 544 tokens: 61 us estimated, 71 measured, 62 on the one-CTA kernel)
+    return kind == PAIR_DUO && g.rem_base > 1 ? 1.15 * worst : worst;
 }
 
 // Launch shape of a projection on CTA pairs, or PAIR_NONE when the one-CTA kernel serves it better
@@ -1603,10 +1605,12 @@ static int gemm2_plan_by_rule(int T, int packed_rows, int K, int n_sm, int mode,
     return kind;
 }
 
-// The rule above, unless another kernel is estimated at least 8 % faster.  Over the projections of a layer at the sizes the
-// estimate was fitted to, the choice costs 1.9 % more time than the best kernel everywhere would (at most 9.6 %; the rule alone
-// 5.1 and 30 %: it keeps gate/up of the 8B shape at 688 tokens on the one-CTA kernel, 153 us against 128, and those of the 1B
-// shape at 768 tokens on 512-feature items, 65 against 53).
+// The rule above, unless another kernel is estimated at least 8 % faster.  Measured at 28 sizes of 264 to 2 040 tokens, the
+// projections of a layer of the three shapes, all three kernels (316 points): the choice costs 1.4 % more time than the best
+// kernel everywhere would, the rule alone 4.3 %; at worst 29 and 92 % (the 32B o at 1 536 tokens, 88 us on the rule's 512-feature
+// items against 69 on the one-CTA kernel; the 32B down at 2 040, 849 us on the one-CTA kernel against 442).  It is never more
+// than 3 % behind the rule.  Gate/up of the 8B shape at 688 to 768 tokens stays on the one-CTA kernel by the 8 % (158 us
+// against 130).
 static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int force, Gemm2Params& g, int& n_cl) {
     const int by_rule = gemm2_plan_by_rule(T, packed_rows, K, n_sm, mode, force, g, n_cl);
     if (force != PAIR_NONE || T < 256 || n_sm < 2) return by_rule;

@@ -189,3 +189,10 @@ def test_variants_that_are_not_built_are_never_asked_for():
         for T in range(1, 2400, 13):
             p = syn.gemm_plan_host(T, N, K, epi)
             assert p["ksplit"] == 1 if epi == "resid" else p["splits"] == 1, (T, N, K, epi)
+
+
+@pytest.mark.parametrize("T", [513, 520, 544, 576, 608, 640])
+def test_leftover_items_of_256_features_are_not_taken_for_cheaper_than_they_are(T):
+    """qkv of the 32B shape: 84 items on 74 clusters, the last ten cut along K (71 - 80 us), against 61 - 70 us on the one-CTA
+    kernel or in one wave of 512-feature items."""
+    assert syn.gemm2_plan_host(T, 7168, 5120, "qkv")["kind"] != 2
