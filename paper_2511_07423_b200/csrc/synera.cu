@@ -953,7 +953,7 @@ static int plan_compute(const syn_model_desc& c, int P, uint32_t n_pages, int n_
             // Many units to a CTA: whole, unless one alone exceeds a CTA's fair share by so much that parts of it pay for
             // themselves.  The merge of a unit's parts runs beside other items and counts as work, not as time that a part has to
             // leave free (with the merge inside the share, three requests of 6 000 keys among 58 of the 8B shape were cut into
-            // parts of 4 blocks: 528 parts and 520 us a layer; 96 and 60 with this).
+            // parts of 4 blocks: 528 parts and 520 us a layer; 96 and 58 with this).
             y.merge_counts = false;
             y.estimate = INT64_MAX;
             for (int64_t limit = std::max(mean, 8 * (int64_t)k.block[4] + k.item);; limit += limit / 4) {
