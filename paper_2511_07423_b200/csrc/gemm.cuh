@@ -98,7 +98,7 @@ __host__ __device__ __forceinline__ int rope_tile_feature(int l, int hd) {   // 
     return (q / groups) * hd + 16 * (q % groups) + (ll & 15) + ((ll & 16) ? half : 0);
 }
 
-constexpr int GEMM_EPI_WARPS = 16;               // four groups of four (one warp per TMEM lane quarter)
+constexpr int GEMM_EPI_WARPS = 16;               // at most: four groups of four (one warp per TMEM lane quarter)
 
 // Epilogue of one 16-token chunk of one warp: a[j] = D[feature of this lane][token t0 + j] (tokens
 // j >= ncols are padding), already summed and scaled.  In this orientation a lane holds ONE output
@@ -124,16 +124,35 @@ struct EpiOperand {
     int slot;
 };
 
-template <int MODE>   // passes i0 .. i0 + n - 1 of four, each four tokens
-__device__ __forceinline__ void epi_load_rope(const EpiParams& p, EpiOperand<MODE>& o, int t0, int ncols, int quarter, int lane, int i0 = 0, int n = 4) {
+// Loads of data that no kernel beside this one writes, issued where they stand: the compiler moves a plain __ldg down to its
+// use, behind the barriers whose wait is to hide it (the o projection of the 1B shape, 5 tokens: a gain that came from HBM held
+// the last 1 400 cycles of the kernel).
+__device__ __forceinline__ float4 ldg_here(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ldg_here(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ldg_here(const int* p) {
+    int v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+template <int MODE>
+__device__ __forceinline__ void epi_load_rope(const EpiParams& p, EpiOperand<MODE>& o, int t0, int ncols, int quarter, int lane) {
     const int tq = lane >> 3, c0 = (lane & 7) * 4;
     const int half = p.hd >> 1, dim = 16 * (quarter & ((half >> 4) - 1)) + (c0 & 15);   // lower dim of the pair
 #pragma unroll
-    for (int i = i0; i < i0 + n; ++i) {
+    for (int i = 0; i < 4; ++i) {
         const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)(t0 + tq + 4 * i) * half + dim);   // 4 x (cos, sin)
         const bool tv = tq + 4 * i < ncols;
-        o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)] = tv ? __ldg(cs) : make_float4(1.f, 0.f, 1.f, 0.f);
-        o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)] = tv ? __ldg(cs + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
+        o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)] = tv ? ldg_here(cs) : make_float4(1.f, 0.f, 1.f, 0.f);
+        o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)] = tv ? ldg_here(cs + 1) : make_float4(1.f, 0.f, 1.f, 0.f);
     }
 }
 
@@ -142,7 +161,7 @@ __device__ __forceinline__ void epi_load(const EpiParams& p, EpiOperand<MODE>& o
     const int tq = lane >> 3, c0 = (lane & 7) * 4;
     if (MODE == EPI_RESID) {
         const int f = m0 + quarter * 32 + c0;
-        o.gain = __ldg(reinterpret_cast<const uint2*>(p.gain + f));
+        o.gain = ldg_here(reinterpret_cast<const uint2*>(p.gain + f));
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             o.v[i & (MODE == EPI_RESID ? 3 : 0)] = tq + 4 * i < ncols ? *reinterpret_cast<const float4*>(p.x + (size_t)(t0 + tq + 4 * i) * p.d + f)
@@ -150,7 +169,7 @@ __device__ __forceinline__ void epi_load(const EpiParams& p, EpiOperand<MODE>& o
     } else if (MODE == EPI_QKV) {
         const int which = m0 < p.q_dim ? 0 : (m0 < p.q_dim + p.kv_dim ? 1 : 2);
         // KV slot (page * 16 + row) of token lane & 15, handed round by shuffles
-        o.slot = (which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0;
+        o.slot = (which > 0 && (lane & 15) < ncols) ? ldg_here(p.slot + t0 + (lane & 15)) : 0;
         if (which < 2) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane);
     }
 }
@@ -163,13 +182,26 @@ __device__ __forceinline__ void epi_stage(const float (&a)[EPI_COLS], float* scr
     __syncwarp();
 }
 
-// ... and out of it row by row; `o` holds what epi_load brought (LATE: it is loaded here, once the chunk's own registers are
-// free).  SWIGLU and LMHEAD have ways of their own (below).
-template <int MODE, bool LATE = false>
+// ... and out of it: the lane's four columns of the four tokens tq, tq + 4, ...  All loads stand before the first store (to the
+// compiler a store may change the scratch, and a token at a time the four round trips follow one another: 1 000 cycles of a
+// residual unit, 350 together).
+__device__ __forceinline__ void epi_rows(const float* scr, float4 (&rows)[4], int tq, int c0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) rows[i] = *reinterpret_cast<const float4*>(scr + (tq + 4 * i) * EPI_SCR_STRIDE + c0);
+}
+
+// The chunk that a warp finishes next: what it reads is requested as soon as the operand's registers are free, and arrives while
+// the present chunk is stored and the next one staged.
+struct EpiNext {
+    bool any;
+    int m0, t0, ncols;
+};
+
+// ... `o` holds what epi_load brought.  SWIGLU and LMHEAD have ways of their own (below).
+template <int MODE>
 __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float (&a)[EPI_COLS], float* scr, int m0,
-                                         int t0, int ncols, int quarter, int lane) {
+                                         int t0, int ncols, int quarter, int lane, const EpiNext& next) {
     if (MODE != EPI_SWIGLU && (MODE != EPI_LMHEAD || p.logits)) epi_stage(a, scr, lane);
-    if (LATE && MODE != EPI_QKV) epi_load<MODE>(p, o, m0, t0, ncols, quarter, lane);
     const int tq = lane >> 3, c0 = (lane & 7) * 4;   // token (+ 4 i) and first of four columns of this lane
     if (MODE == EPI_PLAIN) {
         const int f = m0 + quarter * 32 + c0;
@@ -192,33 +224,40 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
     } else if (MODE == EPI_RESID) {
         // x += D; operand of the next projection half(x * gain); sum of x^2 over this warp's 32 features
         const int f = m0 + quarter * 32 + c0;
-        const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.x);
-        const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&o.gain.y);
+        const uint2 gain = o.gain;
+        const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162*>(&gain.x);
+        const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162*>(&gain.y);
+        float4 nx[4];
+        float ss[4];
+        epi_rows(scr, nx, tq, c0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 xv = o.v[i & (MODE == EPI_RESID ? 3 : 0)];
+            nx[i] = make_float4(xv.x + nx[i].x, xv.y + nx[i].y, xv.z + nx[i].z, xv.w + nx[i].w);
+            ss[i] = tq + 4 * i < ncols ? (nx[i].x * nx[i].x + nx[i].y * nx[i].y) + (nx[i].z * nx[i].z + nx[i].w * nx[i].w) : 0.f;
+        }
+        if (next.any) epi_load<MODE>(p, o, next.m0, next.t0, next.ncols, quarter, lane);
+#pragma unroll
+        for (int k = 1; k < 8; k <<= 1)   // the eight lanes of the token, a fixed order
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ss[i] += __shfl_xor_sync(0xFFFFFFFFu, ss[i], k);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = tq + 4 * i;
-            const bool tv = t < ncols;
-            const float4 row = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
-            const float4 xv = o.v[i & (MODE == EPI_RESID ? 3 : 0)];
-            const float4 nx = make_float4(xv.x + row.x, xv.y + row.y, xv.z + row.z, xv.w + row.w);
-            float ss = tv ? (nx.x * nx.x + nx.y * nx.y) + (nx.z * nx.z + nx.w * nx.w) : 0.f;
-            if (tv) {
+            if (t < ncols) {
                 const size_t at = (size_t)(t0 + t) * p.d + f;
-                *reinterpret_cast<float4*>(p.x + at) = nx;
-                *reinterpret_cast<uint2*>(p.xg + at) = pack4_op(nx.x * __low2float(g01), nx.y * __high2float(g01),
-                                                                  nx.z * __low2float(g23), nx.w * __high2float(g23));
+                *reinterpret_cast<float4*>(p.x + at) = nx[i];
+                *reinterpret_cast<uint2*>(p.xg + at) = pack4_op(nx[i].x * __low2float(g01), nx[i].y * __high2float(g01),
+                                                                  nx[i].z * __low2float(g23), nx[i].w * __high2float(g23));
+                if ((lane & 7) == 0) p.ssq_out[(size_t)(t0 + t) * (p.d >> 5) + ((m0 >> 5) + quarter)] = ss[i];
             }
-            ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1);   // the eight lanes of the token, a fixed order
-            ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 2);
-            ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 4);
-            if (tv && (lane & 7) == 0) p.ssq_out[(size_t)(t0 + t) * (p.d >> 5) + ((m0 >> 5) + quarter)] = ss;
         }
     } else if (MODE == EPI_QKV) {
         const int which = m0 < p.q_dim ? 0 : (m0 < p.q_dim + p.kv_dim ? 1 : 2);
         const int region0 = which == 0 ? 0 : (which == 1 ? p.q_dim : p.q_dim + p.kv_dim);
         const int half = p.hd >> 1, hd_log = p.hd == 128 ? 7 : 6;   // head_dim is 64 or 128
         const size_t page_stride = (size_t)p.n_kv_heads * 2 * 16 * p.hd;
-        const int my_slot = LATE ? ((which > 0 && (lane & 15) < ncols) ? __ldg(p.slot + t0 + (lane & 15)) : 0) : o.slot;
+        const int my_slot = o.slot;
         if (which < 2) {
             // q and k tiles: columns 0..15 of the block are the dims [d0, d0 + 16) of one head, columns 16..31
             // the same dims + hd/2 (rope_tile_feature); a lane rotates its four columns with their partners
@@ -226,33 +265,39 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
             const int fhead = (m0 - region0) + ((quarter >> g_log) << hd_log);   // first feature of the head, inside q or k
             const bool hi = c0 >= 16;
             const int dim = 16 * (quarter & ((1 << g_log) - 1)) + (c0 & 15);            // lower dim of the pair
+            const float sg = hi ? 1.f : -1.f;   // dim i: x cos - y sin; dim i + hd/2: y cos + x sin
+            float4 mine[4], part[4];
+            uint2 rot[4];
+            epi_rows(scr, mine, tq, c0);
+            epi_rows(scr, part, tq, c0 ^ 16);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (LATE) epi_load_rope<MODE>(p, o, t0, ncols, quarter, lane, i, 1);
                 const float4 w0 = o.v[(2 * i) & (MODE == EPI_QKV ? 7 : 0)], w1 = o.v[(2 * i + 1) & (MODE == EPI_QKV ? 7 : 0)];
+                rot[i] = pack4_op(mine[i].x * w0.x + sg * part[i].x * w0.y, mine[i].y * w0.z + sg * part[i].y * w0.w,
+                                  mine[i].z * w1.x + sg * part[i].z * w1.y, mine[i].w * w1.z + sg * part[i].w * w1.w);
+            }
+            if (next.any) epi_load<MODE>(p, o, next.m0, next.t0, next.ncols, quarter, lane);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
                 const int t = tq + 4 * i;
-                const float4 mine = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
-                const float4 part = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + (c0 ^ 16));
-                const float sg = hi ? 1.f : -1.f;   // dim i: x cos - y sin; dim i + hd/2: y cos + x sin
-                const float r0 = mine.x * w0.x + sg * part.x * w0.y;
-                const float r1 = mine.y * w0.z + sg * part.y * w0.w;
-                const float r2 = mine.z * w1.x + sg * part.z * w1.y;
-                const float r3 = mine.w * w1.z + sg * part.w * w1.w;
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
                     op16* dst;
                     if (which == 0) dst = p.q + (size_t)(t0 + t) * p.q_dim + fhead;
                     else dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fhead >> hd_log) * 2) * 16 * p.hd + (size_t)(sl & 15) * p.hd;
-                    *reinterpret_cast<uint2*>(dst + dim + (hi ? half : 0)) = pack4_op(r0, r1, r2, r3);
+                    *reinterpret_cast<uint2*>(dst + dim + (hi ? half : 0)) = rot[i];
                 }
             }
         } else {
             // v tiles: features in natural order
             const int fr = (m0 - region0) + quarter * 32 + c0;
+            float4 rows[4];
+            epi_rows(scr, rows, tq, c0);
+            if (next.any) epi_load<MODE>(p, o, next.m0, next.t0, next.ncols, quarter, lane);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int t = tq + 4 * i;
-                const float4 row = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
+                const float4 row = rows[i];
                 const int sl = __shfl_sync(0xFFFFFFFFu, my_slot, t);
                 if (t < ncols) {
                     op16* dst = p.pool + (size_t)(sl >> 4) * page_stride + ((size_t)(fr >> hd_log) * 2 + 1) * 16 * p.hd +
@@ -307,10 +352,12 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
         }
         if (p.logits) {
             const int f = fl + c0;
+            float4 rows[4];
+            epi_rows(scr, rows, tq, c0);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int t = tq + 4 * i;
-                const float4 v = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
+                const float4 v = rows[i];
                 if (t < ncols) {
                     float* dst = p.logits + (size_t)(t0 + t) * p.vocab + f;
                     if ((p.vocab & 3) == 0 && f + 4 <= p.vocab) {
@@ -330,14 +377,15 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
 // Whether an epilogue multiplies by the RMSNorm scale of its tokens.
 __host__ __device__ constexpr bool epi_scaled(int mode) { return mode == EPI_QKV || mode == EPI_SWIGLU || mode == EPI_LMHEAD; }
 
-// The kernels of 576 threads have no registers to hold a chunk beside the rows it meets (loaded early, the residual rows are
-// spilled and the epilogue of a 256 x 256 tile takes 50 k cycles instead of 31 k).
-__host__ __device__ constexpr bool epi_late(int mode) { return mode == EPI_QKV || mode == EPI_RESID; }
+// Epilogue warps of the kernels that take a whole SM: 16 (four groups of four warps, one to a TMEM lane quarter) with 96 registers
+// each; qkv 12 with 128, because a chunk with its RoPE rows does not fit into 96.
+__host__ __device__ constexpr int gemm_epi_warps(int mode) { return mode == EPI_QKV ? 12 : GEMM_EPI_WARPS; }
+__host__ __device__ constexpr int gemm_threads(int mode) { return (2 + gemm_epi_warps(mode)) * 32; }
 
 // A chunk's accumulators, summed, through the epilogue.
 template <int MODE>
 __device__ __forceinline__ void epi_chunk(const EpiParams& p, EpiOperand<MODE>& o, const uint32_t (&r)[EPI_COLS], const float* rs, float* scr,
-                                          int m0, int t0, int ncols, int quarter, int lane) {
+                                          int m0, int t0, int ncols, int quarter, int lane, const EpiNext& next) {
     float a[EPI_COLS];
 #pragma unroll
     for (int j = 0; j < EPI_COLS; j += 4) {
@@ -345,15 +393,30 @@ __device__ __forceinline__ void epi_chunk(const EpiParams& p, EpiOperand<MODE>& 
         a[j] = __uint_as_float(r[j]); a[j + 1] = __uint_as_float(r[j + 1]); a[j + 2] = __uint_as_float(r[j + 2]); a[j + 3] = __uint_as_float(r[j + 3]);
         if (epi_scaled(MODE)) { a[j] *= k.x; a[j + 1] *= k.y; a[j + 2] *= k.z; a[j + 3] *= k.w; }
     }
-    epi_unit<MODE, epi_late(MODE)>(p, o, a, scr, m0, t0, ncols, quarter, lane);
+    epi_unit<MODE>(p, o, a, scr, m0, t0, ncols, quarter, lane, next);
+}
+
+// Accumulators of another part of K that its CTA left in global memory, added to (or, `first`, put into) a chunk.
+__device__ __forceinline__ void epi_add_part(uint32_t (&r)[EPI_COLS], const float4* src, bool first) {
+    float4 q[EPI_COLS / 4];
+#pragma unroll
+    for (int v = 0; v < EPI_COLS / 4; ++v) q[v] = __ldcg(src + v * 32);
+#pragma unroll
+    for (int v = 0; v < EPI_COLS / 4; ++v) {
+        r[4 * v] = first ? __float_as_uint(q[v].x) : __float_as_uint(__uint_as_float(r[4 * v]) + q[v].x);
+        r[4 * v + 1] = first ? __float_as_uint(q[v].y) : __float_as_uint(__uint_as_float(r[4 * v + 1]) + q[v].y);
+        r[4 * v + 2] = first ? __float_as_uint(q[v].z) : __float_as_uint(__uint_as_float(r[4 * v + 2]) + q[v].z);
+        r[4 * v + 3] = first ? __float_as_uint(q[v].w) : __float_as_uint(__uint_as_float(r[4 * v + 3]) + q[v].w);
+    }
 }
 
 // RMSNorm scales of the tokens n0 .. n0 + n_valid - 1 from the partial sums of x^2 their source rows
-// carry: one warp per token (warp `e` of GEMM_EPI_WARPS takes every sixteenth), a fixed reduction
+// carry: one warp per token (warp `e` of NW takes every NW-th), a fixed reduction
 // order, so every CTA that needs a token's scale gets the same bits.
+template <int NW>
 __device__ __forceinline__ void epi_rms_scales(const EpiParams& p, float* dst, int n0, int n_valid, int e, int lane) {
     const int nq = p.n_ssq >> 2;
-    for (int t = e; t < n_valid; t += GEMM_EPI_WARPS) {
+    for (int t = e; t < n_valid; t += NW) {
         const float4* row = reinterpret_cast<const float4*>(p.ssq_in + (size_t)(n0 + t) * p.n_ssq);
         float sum = 0.f;
         for (int i = lane; i < nq; i += 32) {
@@ -421,7 +484,7 @@ __global__ void pack_weight_kernel(PackSrc src, op16* __restrict__ out, int num_
 }
 
 // ------------------------------------------------------------------------------------------
-// The kernel.  One persistent CTA per SM, 576 threads: warp 0 = producer (bulk copy of the weight
+// The kernel.  One persistent CTA per SM, 576 threads (qkv: 448): warp 0 = producer (bulk copy of the weight
 // tiles + TMA boxes of the token tile), warp 1 = TMEM owner and MMA issuer, warps 2..17 = epilogue
 // (four groups of four; a group covers the four TMEM lane quarters; draining TMEM is limited per
 // warp, so many warps share it).
@@ -432,7 +495,6 @@ constexpr int GEMM_A_BYTES = 2 * GEMM_TILE_BYTES;  // stage room for a pair
 constexpr int GEMM_BOX_ROWS = 32;                  // token rows per B box
 constexpr int GEMM_BOX_BYTES = GEMM_BOX_ROWS * GEMM_BK * 2;
 constexpr int GEMM_MAX_STAGES = 8;
-constexpr int GEMM_THREADS = (2 + GEMM_EPI_WARPS) * 32;
 constexpr int GEMM_SMEM_MAX = 232448;
 constexpr int GEMM_BAR_BYTES = 256;                // mbarriers and the TMEM address word
 
@@ -576,10 +638,11 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 }
 
 template <int VARIANT, int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+__global__ void __launch_bounds__(gemm_threads(MODE), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) {
     constexpr bool KSPLIT = VARIANT == GEMM_KSPLIT;
     constexpr bool RSPLIT = VARIANT == GEMM_RSPLIT;
+    constexpr int EW = gemm_epi_warps(MODE);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int stage_bytes = gemm_stage_bytes(g.TN);
@@ -607,8 +670,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             mbar_init(&empty_bar[s], 1);
         }
         mbar_init(accf_bar, 1);
-        mbar_init(acce_bar, GEMM_EPI_WARPS);
-        mbar_init(rs_bar, GEMM_EPI_WARPS);
+        mbar_init(acce_bar, EW);
+        mbar_init(rs_bar, EW);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -707,7 +770,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
         // ------------------------------------------------------------ epilogue
         const int e = warp - 2;
         const int grp = e >> 2;               // the groups take the 16-token chunks round robin
-        constexpr int NGRP = GEMM_EPI_WARPS / 4;
+        constexpr int NGRP = EW / 4;
         const int quarter = warp & 3;         // TMEM lane quarter this warp may read
         constexpr bool scaled = epi_scaled(MODE);
         float* const scr = scr_s + e * EPI_SCR_FLOATS;
@@ -720,30 +783,44 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             const int nchunks = (n_valid + EPI_COLS - 1) / EPI_COLS;
             float* const rsi = rs_s + (i & 1) * gemm_rs_stride(g.TN);
             if (scaled) {   // while the main loop runs: the scales of this item's tokens
-                epi_rms_scales(p, rsi, n0, n_valid, e, lane);
+                epi_rms_scales<EW>(p, rsi, n0, n_valid, e, lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(rs_bar);
             }
+            // The chunks [c_lo, c_hi) of this CTA's tiles are finished here, the warp's group takes every NGRP-th of them.
+            const int S = RSPLIT ? g.splits : 1, sp = RSPLIT ? w.split : 0;
+            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S, nc = max(c_hi - c_lo, 1);
+            const int total_chunks = (w.mt_hi - w.mt_lo) * (c_hi - c_lo);
+            auto unit_at = [&](int ci) {
+                EpiNext u;
+                u.m0 = w.pair * 256 + (w.mt_lo + ci / nc) * 128;
+                const int c = c_lo + ci % nc;
+                u.t0 = n0 + c * EPI_COLS;
+                u.ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                u.any = ci < total_chunks && u.m0 < p.N;
+                return u;
+            };
+            EpiOperand<MODE> opnd;   // of the warp's first chunk: in flight while the main loop runs
+            EpiNext unit = unit_at(grp);
+            if (unit.any && (!KSPLIT || w.role != 1)) epi_load<MODE>(p, opnd, unit.m0, unit.t0, unit.ncols, quarter, lane);
             ok = mbar_wait(accf_bar, i & 1, g.status, limit);
             if (ok && scaled) ok = mbar_wait(rs_bar, i & 1, g.status, limit);
             if (!ok) break;
             tc_fence_after();
-            const int total_chunks = (w.mt_hi - w.mt_lo) * nchunks;
             if (RSPLIT) {
                 // ---- reduce-scatter over the S CTAs that share this tile.  CTA `split` keeps the
                 // chunks [c_lo, c_hi) of both 128-feature tiles.  Exchange slot of a CTA:
                 // [tile of the pair][chunk][lane quarter][4][lane][4 floats], so that one 16-byte access
                 // per lane covers 512 contiguous bytes per warp.
-                const int S = g.splits, sp = w.split, tile = cta / S;
+                const int tile = cta / S;
                 const int cpt = g.TN / EPI_COLS;
                 const size_t slot_elems = (size_t)2 * cpt * 128 * EPI_COLS;
-                const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S;
                 float* const mine = g.fix_part + (size_t)cta * slot_elems;
                 int nth = 0;
                 for (int mt = 0; mt < 2; ++mt)
                     for (int c = 0; c < nchunks; ++c) {
                         if (c >= c_lo && c < c_hi) continue;
-                        if ((nth++ & (NGRP - 1)) != grp) continue;
+                        if (nth++ % NGRP != grp) continue;
                         uint32_t r[EPI_COLS];
                         tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                         tmem_ld_wait();
@@ -757,7 +834,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                 // all warps of all S CTAs must have stored before anyone reads; the CTAs of a tile are
                 // neighbours in the grid and the grid is at most one CTA per SM, so they run together
                 if (lane == 0) {
-                    const int want = S * GEMM_EPI_WARPS;
+                    const int want = S * EW;
                     const long long t_end = clock64() + limit;
                     while (ld_acquire_gpu(g.fix_flag + tile) < want) {
                         if (clock64() > t_end) {
@@ -767,45 +844,28 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     }
                 }
                 __syncwarp();
-                nth = 0;
-                for (int mt = 0; mt < 2; ++mt)
-                    for (int c = c_lo; c < c_hi; ++c) {
-                        if ((nth++ & (NGRP - 1)) != grp) continue;
-                        const int m0 = w.pair * 256 + mt * 128;
-                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                        EpiOperand<MODE> opnd;
-                        if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
-                        uint32_t own[EPI_COLS], r[EPI_COLS];
-                        tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
-                        tmem_ld_wait();
-                        const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
-                        for (int q = 0; q < S; ++q) {   // fixed order: the parts in split order
-                            if (q == sp) {
+                for (int ci = grp; ci < total_chunks; ci += NGRP) {
+                    const int mt = ci / nc, c = c_lo + ci % nc;
+                    uint32_t own[EPI_COLS], r[EPI_COLS];
+                    tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
+                    tmem_ld_wait();
+                    const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
+                    for (int q = 0; q < S; ++q) {   // fixed order: the parts in split order
+                        if (q == sp) {
 #pragma unroll
-                                for (int v = 0; v < EPI_COLS; ++v)
-                                    r[v] = q == 0 ? own[v] : __float_as_uint(__uint_as_float(r[v]) + __uint_as_float(own[v]));
-                            } else {
-                                const float4* src = reinterpret_cast<const float4*>(g.fix_part + (size_t)(tile * S + q) * slot_elems + at) + lane;
-#pragma unroll
-                                for (int v = 0; v < EPI_COLS / 4; ++v) {
-                                    const float4 q4 = __ldcg(src + v * 32);
-                                    if (q == 0) {
-                                        r[4 * v] = __float_as_uint(q4.x); r[4 * v + 1] = __float_as_uint(q4.y);
-                                        r[4 * v + 2] = __float_as_uint(q4.z); r[4 * v + 3] = __float_as_uint(q4.w);
-                                    } else {
-                                        r[4 * v] = __float_as_uint(__uint_as_float(r[4 * v]) + q4.x);
-                                        r[4 * v + 1] = __float_as_uint(__uint_as_float(r[4 * v + 1]) + q4.y);
-                                        r[4 * v + 2] = __float_as_uint(__uint_as_float(r[4 * v + 2]) + q4.z);
-                                        r[4 * v + 3] = __float_as_uint(__uint_as_float(r[4 * v + 3]) + q4.w);
-                                    }
-                                }
-                            }
+                            for (int v = 0; v < EPI_COLS; ++v)
+                                r[v] = q == 0 ? own[v] : __float_as_uint(__uint_as_float(r[v]) + __uint_as_float(own[v]));
+                        } else {
+                            epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + (size_t)(tile * S + q) * slot_elems + at) + lane, q == 0);
                         }
-                        if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
                     }
+                    const EpiNext next = unit_at(ci + NGRP);
+                    if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
+                    unit = next;
+                }
                 // the last warp of the tile's CTAs to finish reading clears the counters for the next launch
                 __syncwarp();
-                if (lane == 0 && atomicAdd(g.fix_flag + g.n_sm + tile, 1) == S * GEMM_EPI_WARPS - 1) {
+                if (lane == 0 && atomicAdd(g.fix_flag + g.n_sm + tile, 1) == S * EW - 1) {
                     g.fix_flag[tile] = 0;
                     g.fix_flag[g.n_sm + tile] = 0;
                 }
@@ -813,11 +873,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             }
             if (!KSPLIT || w.role == 0) {
                 for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = w.mt_lo + ci / nchunks, c = ci % nchunks;
-                    const int m0 = w.pair * 256 + mt * 128;
-                    const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                    EpiOperand<MODE> opnd;
-                    if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
+                    const int mt = w.mt_lo + ci / nc, c = ci % nc;
                     uint32_t r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                     tmem_ld_wait();
@@ -825,7 +881,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(acce_bar);
                     }
-                    if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
+                    const EpiNext next = unit_at(ci + NGRP);
+                    if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
+                    unit = next;
                 }
                 if (grp >= total_chunks) {   // a group without any chunk still releases the accumulators
                     tc_fence_before();
@@ -841,7 +899,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             if (w.role == 1) {
                 float* mine = g.fix_part + (size_t)(w.rtile * H + w.hpart) * part_elems;
                 for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = w.mt_lo + ci / nchunks, c = ci % nchunks;
+                    const int mt = w.mt_lo + ci / nc, c = ci % nc;
                     uint32_t r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                     tmem_ld_wait();
@@ -864,7 +922,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             }
             // owner: the helpers ran first; the wait is bounded all the same
             if (lane == 0) {
-                const int want = H * GEMM_EPI_WARPS;
+                const int want = H * EW;
                 const long long t_end = clock64() + limit;
                 while (ld_acquire_gpu(g.fix_flag + w.rtile) < want) {
                     if (clock64() > t_end) {
@@ -875,8 +933,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             }
             __syncwarp();
             for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                const int mt = w.mt_lo + ci / nchunks, c = ci % nchunks;
-                const int m0 = w.pair * 256 + mt * 128;
+                const int mt = w.mt_lo + ci / nc, c = ci % nc;
                 uint32_t r[EPI_COLS];
                 tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                 tmem_ld_wait();
@@ -885,23 +942,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     if (lane == 0) mbar_arrive(acce_bar);
                 }
                 const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
-                for (int h = 0; h < H; ++h) {   // fixed order: own k range, then the helpers' in part order
-                    const float4* src = reinterpret_cast<const float4*>(g.fix_part + (size_t)(w.rtile * H + h) * part_elems + at) + lane;
-#pragma unroll
-                    for (int v = 0; v < EPI_COLS / 4; ++v) {
-                        const float4 q4 = __ldcg(src + v * 32);
-                        r[4 * v] = __float_as_uint(__uint_as_float(r[4 * v]) + q4.x);
-                        r[4 * v + 1] = __float_as_uint(__uint_as_float(r[4 * v + 1]) + q4.y);
-                        r[4 * v + 2] = __float_as_uint(__uint_as_float(r[4 * v + 2]) + q4.z);
-                        r[4 * v + 3] = __float_as_uint(__uint_as_float(r[4 * v + 3]) + q4.w);
-                    }
-                }
-                const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                EpiOperand<MODE> opnd;
-                if (m0 < p.N) {
-                    if (!epi_late(MODE)) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
-                    epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
-                }
+                for (int h = 0; h < H; ++h)   // fixed order: own k range, then the helpers' in part order
+                    epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + (size_t)(w.rtile * H + h) * part_elems + at) + lane, false);
+                const EpiNext next = unit_at(ci + NGRP);
+                if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
+                unit = next;
             }
             if (grp >= total_chunks) {
                 tc_fence_before();
@@ -909,7 +954,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             }
             // the last warp to finish reading clears the tile's counters for the next launch
             __syncwarp();
-            if (lane == 0 && atomicAdd(g.fix_flag + g.n_sm + w.rtile, 1) == GEMM_EPI_WARPS - 1) {
+            if (lane == 0 && atomicAdd(g.fix_flag + g.n_sm + w.rtile, 1) == EW - 1) {
                 g.fix_flag[w.rtile] = 0;
                 g.fix_flag[g.n_sm + w.rtile] = 0;
             }

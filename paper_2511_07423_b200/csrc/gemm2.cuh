@@ -93,11 +93,12 @@ __host__ __device__ __forceinline__ bool gemm2_work(const Gemm2Params& g, int cl
 }
 
 template <bool DUO, int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+__global__ void __launch_bounds__(gemm_threads(MODE), 1)
 gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Gemm2Params g, EpiParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int stage_bytes = gemm2_stage_bytes(g.TN, DUO);
+    constexpr int EW = gemm_epi_warps(MODE);
     constexpr int A_BYTES = DUO ? GEMM_TILE_BYTES : GEMM_A_BYTES;
     uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + g.n_stages * stage_bytes);   // used in the rank-0 CTA
     uint64_t* empty_bar = full_bar + GEMM_MAX_STAGES;   // own: the stage's MMAs are done (commit arrives in both CTAs)
@@ -123,8 +124,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             mbar_init(&empty_bar[s], 1);
         }
         mbar_init(accf_bar, 1);
-        mbar_init(acce_bar, 2 * GEMM_EPI_WARPS);
-        mbar_init(rs_bar, GEMM_EPI_WARPS);
+        mbar_init(acce_bar, 2 * EW);
+        mbar_init(rs_bar, EW);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -232,7 +233,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         // ------------------------------------------------------------ epilogue (both CTAs)
         const int e = warp - 2;
         const int grp = e >> 2;               // the groups take the 16-token chunks round robin
-        constexpr int NGRP = GEMM_EPI_WARPS / 4;
+        constexpr int NGRP = EW / 4;
         const int quarter = warp & 3;         // TMEM lane quarter this warp may read
         constexpr bool scaled = epi_scaled(MODE);
         const uint32_t acce_c = mapa_rank(smem_u32(acce_bar), 0);
@@ -246,31 +247,45 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             const int nchunks = (n_valid + EPI_COLS - 1) / EPI_COLS;
             float* const rsi = rs_s + (i & 1) * gemm_rs_stride(g.TN);
             if (scaled) {   // while the main loop runs: the scales of this item's tokens
-                epi_rms_scales(p, rsi, n0, n_valid, e, lane);
+                epi_rms_scales<EW>(p, rsi, n0, n_valid, e, lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(rs_bar);
             }
+            // this CTA's features: QUAD both tiles of pair 2 grp + rank, DUO tile `rank` of pair grp; of their chunks it finishes
+            // [c_lo, c_hi), the warp's group every NGRP-th of them
+            const int n_mt = DUO ? 1 : 2;
+            const int row0 = DUO ? w.grp * 256 + (int)rank * 128 : (2 * w.grp + (int)rank) * 256;
+            const int S = w.nsplit, sp = w.split;
+            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S, nc = max(c_hi - c_lo, 1);
+            const int total_chunks = n_mt * (c_hi - c_lo);
+            auto unit_at = [&](int ci) {
+                EpiNext u;
+                u.m0 = row0 + ci / nc * 128;
+                const int c = c_lo + ci % nc;
+                u.t0 = n0 + c * EPI_COLS;
+                u.ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
+                u.any = ci < total_chunks && u.m0 < p.N;
+                return u;
+            };
+            EpiOperand<MODE> opnd;   // of the warp's first chunk: in flight while the main loop runs
+            EpiNext unit = unit_at(grp);
+            if (unit.any) epi_load<MODE>(p, opnd, unit.m0, unit.t0, unit.ncols, quarter, lane);
             ok = mbar_wait(accf_bar, i & 1, g.status, limit);
             if (ok && scaled) ok = mbar_wait(rs_bar, i & 1, g.status, limit);
             if (!ok) break;
             tc_fence_after();
-            // this CTA's features: QUAD both tiles of pair 2 grp + rank, DUO tile `rank` of pair grp
-            const int n_mt = DUO ? 1 : 2;
-            const int row0 = DUO ? w.grp * 256 + (int)rank * 128 : (2 * w.grp + (int)rank) * 256;
-            const int total_chunks = n_mt * nchunks;
             if (w.nsplit > 1) {
                 // ---- reduce-scatter between the S clusters that share this tile, CTAs of equal rank
                 // (see gemm.cuh): this CTA keeps the chunks [c_lo, c_hi) and hands the others over.
-                const int S = w.nsplit, sp = w.split, cnt = w.counter * 2 + (int)rank;   // counter pair of (tile, rank)
+                const int cnt = w.counter * 2 + (int)rank;   // counter pair of (tile, rank)
                 const int cpt = g.TN / EPI_COLS;
                 const size_t slot_elems = (size_t)2 * cpt * 128 * EPI_COLS;
-                const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S;
                 float* const mine = g.fix_part + (size_t)blockIdx.x * slot_elems;
                 int nth = 0;
                 for (int mt = 0; mt < n_mt; ++mt)
                     for (int c = 0; c < nchunks; ++c) {
                         if (c >= c_lo && c < c_hi) continue;
-                        if ((nth++ & (NGRP - 1)) != grp) continue;
+                        if (nth++ % NGRP != grp) continue;
                         uint32_t r[EPI_COLS];
                         tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                         if (DUO) {
@@ -290,7 +305,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 __syncwarp();
                 if (lane == 0) atomicAdd(g.fix_flag + cnt, 1);
                 if (lane == 0) {
-                    const int want = S * GEMM_EPI_WARPS;
+                    const int want = S * EW;
                     const long long t_end = clock64() + limit;
                     while (ld_acquire_gpu(g.fix_flag + cnt) < want) {
                         if (clock64() > t_end) {
@@ -300,63 +315,42 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     }
                 }
                 __syncwarp();
-                nth = 0;
-                for (int mt = 0; mt < n_mt; ++mt)
-                    for (int c = c_lo; c < c_hi; ++c) {
-                        if ((nth++ & (NGRP - 1)) != grp) continue;
-                        const int m0 = row0 + mt * 128;
-                        const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                        EpiOperand<MODE> opnd;
-                        if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
-                        uint32_t own[EPI_COLS], r[EPI_COLS];
-                        tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
-                        if (DUO) {
-                            tmem_ld16(tmem_base + acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
-                            tmem_ld_wait();
+                for (int ci = grp; ci < total_chunks; ci += NGRP) {
+                    const int mt = ci / nc, c = c_lo + ci % nc;
+                    uint32_t own[EPI_COLS], r[EPI_COLS];
+                    tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
+                    if (DUO) {
+                        tmem_ld16(tmem_base + acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
+                        tmem_ld_wait();
 #pragma unroll
-                            for (int v = 0; v < EPI_COLS; ++v) own[v] = __float_as_uint(__uint_as_float(own[v]) + __uint_as_float(r[v]));
-                        } else {
-                            tmem_ld_wait();
-                        }
-                        const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
-                        for (int q = 0; q < S; ++q) {   // fixed order: the parts in split order
-                            if (q == sp) {
-#pragma unroll
-                                for (int v = 0; v < EPI_COLS; ++v)
-                                    r[v] = q == 0 ? own[v] : __float_as_uint(__uint_as_float(r[v]) + __uint_as_float(own[v]));
-                            } else {
-                                const size_t peer = (size_t)((w.first_cl + q) * 2 + (int)rank);   // the CTA of the same rank in the cluster of part q
-                                const float4* src = reinterpret_cast<const float4*>(g.fix_part + peer * slot_elems + at) + lane;
-#pragma unroll
-                                for (int v = 0; v < EPI_COLS / 4; ++v) {
-                                    const float4 q4 = __ldcg(src + v * 32);
-                                    if (q == 0) {
-                                        r[4 * v] = __float_as_uint(q4.x); r[4 * v + 1] = __float_as_uint(q4.y);
-                                        r[4 * v + 2] = __float_as_uint(q4.z); r[4 * v + 3] = __float_as_uint(q4.w);
-                                    } else {
-                                        r[4 * v] = __float_as_uint(__uint_as_float(r[4 * v]) + q4.x);
-                                        r[4 * v + 1] = __float_as_uint(__uint_as_float(r[4 * v + 1]) + q4.y);
-                                        r[4 * v + 2] = __float_as_uint(__uint_as_float(r[4 * v + 2]) + q4.z);
-                                        r[4 * v + 3] = __float_as_uint(__uint_as_float(r[4 * v + 3]) + q4.w);
-                                    }
-                                }
-                            }
-                        }
-                        if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
+                        for (int v = 0; v < EPI_COLS; ++v) own[v] = __float_as_uint(__uint_as_float(own[v]) + __uint_as_float(r[v]));
+                    } else {
+                        tmem_ld_wait();
                     }
+                    const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
+                    for (int q = 0; q < S; ++q) {   // fixed order: the parts in split order
+                        if (q == sp) {
+#pragma unroll
+                            for (int v = 0; v < EPI_COLS; ++v)
+                                r[v] = q == 0 ? own[v] : __float_as_uint(__uint_as_float(r[v]) + __uint_as_float(own[v]));
+                        } else {
+                            const size_t peer = (size_t)((w.first_cl + q) * 2 + (int)rank);   // the CTA of the same rank in the cluster of part q
+                            epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + peer * slot_elems + at) + lane, q == 0);
+                        }
+                    }
+                    const EpiNext next = unit_at(ci + NGRP);
+                    if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
+                    unit = next;
+                }
                 __syncwarp();
-                if (lane == 0 && atomicAdd(g.fix_flag + 2 * g.n_sm + cnt, 1) == S * GEMM_EPI_WARPS - 1) {
+                if (lane == 0 && atomicAdd(g.fix_flag + 2 * g.n_sm + cnt, 1) == S * EW - 1) {
                     g.fix_flag[cnt] = 0;
                     g.fix_flag[2 * g.n_sm + cnt] = 0;
                 }
                 continue;
             }
             for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                const int mt = ci / nchunks, c = ci % nchunks;
-                const int m0 = row0 + mt * 128;
-                const int tc0 = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                EpiOperand<MODE> opnd;
-                if (!epi_late(MODE) && m0 < p.N) epi_load<MODE>(p, opnd, m0, tc0, ncols, quarter, lane);
+                const int mt = ci / nc, c = ci % nc;
                 uint32_t r[EPI_COLS];
                 tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                 if (DUO) {
@@ -372,7 +366,9 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     tc_fence_before();
                     if (lane == 0) mbar_arrive_cluster(acce_c);
                 }
-                if (m0 < p.N) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, m0, tc0, ncols, quarter, lane);
+                const EpiNext next = unit_at(ci + NGRP);
+                if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
+                unit = next;
             }
             if (grp >= total_chunks) {   // a group without any chunk still releases the accumulators
                 tc_fence_before();

@@ -283,20 +283,25 @@ thin_kernel(const __grid_constant__ CUtensorMap tmB, ThinParams g, EpiParams p) 
                 read_acc(c, a);
             } else {   // the parts in split order
                 const uint32_t src = smem_u32(recv + (size_t)(4 * c + quarter - u_lo) * S * (THIN_UNIT_FLOATS * 4)) + lane * 16;
+                // (the next part's four loads in flight while one is added)
+                float4 f[2][EPI_COLS / 4];
 #pragma unroll
                 for (int v = 0; v < EPI_COLS / 4; ++v) {
-                    float4 t = lds_v4(src + v * 512);
+                    f[0][v] = lds_v4(src + v * 512);
+                    a[4 * v] = a[4 * v + 1] = a[4 * v + 2] = a[4 * v + 3] = 0.f;
+                }
 #pragma unroll
-                    for (int q0 = 1; q0 < THIN_MAX_SPLITS; q0 += 4) {   // four loads in flight
-                        float4 f[4];
+                for (int q = 0; q < THIN_MAX_SPLITS; ++q) {
+                    if (q >= S) break;
+                    if (q + 1 < S) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (q0 + q < S) f[q] = lds_v4(src + (q0 + q) * (THIN_UNIT_FLOATS * 4) + v * 512);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (q0 + q < S) { t.x += f[q].x; t.y += f[q].y; t.z += f[q].z; t.w += f[q].w; }
+                        for (int v = 0; v < EPI_COLS / 4; ++v) f[(q + 1) & 1][v] = lds_v4(src + (q + 1) * (THIN_UNIT_FLOATS * 4) + v * 512);
                     }
-                    a[4 * v] = t.x; a[4 * v + 1] = t.y; a[4 * v + 2] = t.z; a[4 * v + 3] = t.w;
+#pragma unroll
+                    for (int v = 0; v < EPI_COLS / 4; ++v) {
+                        const float4 t = f[q & 1][v];
+                        a[4 * v] += t.x; a[4 * v + 1] += t.y; a[4 * v + 2] += t.z; a[4 * v + 3] += t.w;
+                    }
                 }
             }
             if (scaled) {
@@ -304,8 +309,8 @@ thin_kernel(const __grid_constant__ CUtensorMap tmB, ThinParams g, EpiParams p) 
                 for (int v = 0; v < EPI_COLS; ++v) a[v] *= rs_s[c * EPI_COLS + v];
             }
             const int tc = n0 + c * EPI_COLS, ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-            if (c != c_first) epi_load<MODE>(p, opnd, m0, tc, ncols, quarter, lane);
-            epi_unit<MODE>(p, opnd, a, scr, m0, tc, ncols, quarter, lane);
+            const EpiNext next = {4 * (c + 2) + quarter < u_hi, m0, tc + 2 * EPI_COLS, min(EPI_COLS, n_valid - (c + 2) * EPI_COLS)};
+            epi_unit<MODE>(p, opnd, a, scr, m0, tc, ncols, quarter, lane, next);
         }
     }
     if (S > 1) cluster_wait();   // nobody leaves while another part may still send to it

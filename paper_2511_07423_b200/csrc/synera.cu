@@ -1461,7 +1461,7 @@ static int gemm_plan(int T, int packed_rows, int K, int n_sm, int mode, bool may
 template <int VARIANT, int MODE>
 static cudaError_t launch_gemm_variant(const GemmParams& g, int n_cta, const CUtensorMap& tmB, const EpiParams& ep, cudaStream_t st) {
     const int smem = gemm_fixed_smem(g.TN) + g.n_stages * gemm_stage_bytes(g.TN);
-    if constexpr (gemm_variant_used(VARIANT, MODE)) return launch_pdl(gemm_kernel<VARIANT, MODE>, dim3(n_cta), dim3(GEMM_THREADS), smem, st, tmB, g, ep);
+    if constexpr (gemm_variant_used(VARIANT, MODE)) return launch_pdl(gemm_kernel<VARIANT, MODE>, dim3(n_cta), dim3(gemm_threads(MODE)), smem, st, tmB, g, ep);
     else return note_cuda(cudaErrorInvalidDeviceFunction);
 }
 template <int MODE>
@@ -1715,8 +1715,8 @@ static int launch_proj(syn_model* prof_m, int cls, int n_sm, int* status, const 
     const bool duo = kind == PAIR_DUO;
     const int smem = gemm_fixed_smem(g2.TN) + g2.n_stages * gemm2_stage_bytes(g2.TN, duo);
     cudaError_t le;
-    EPI_SWITCH(ep.mode, le = duo ? launch_pdl_clusters(gemm2_kernel<true, MODE>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->duo, xm.box, g2, ep)
-                                 : launch_pdl_clusters(gemm2_kernel<false, MODE>, dim3(2 * n_cl), dim3(GEMM_THREADS), smem, st, 2, wm->quad, xm.box, g2, ep));
+    EPI_SWITCH(ep.mode, le = duo ? launch_pdl_clusters(gemm2_kernel<true, MODE>, dim3(2 * n_cl), dim3(gemm_threads(MODE)), smem, st, 2, wm->duo, xm.box, g2, ep)
+                                 : launch_pdl_clusters(gemm2_kernel<false, MODE>, dim3(2 * n_cl), dim3(gemm_threads(MODE)), smem, st, 2, wm->quad, xm.box, g2, ep));
     return le == cudaSuccess ? SYN_OK : SYN_E_CUDA;
 }
 
