@@ -197,6 +197,18 @@ struct EpiNext {
     int m0, t0, ncols;
 };
 
+// The chunks of an item that a warp finishes, in turn: every NGRP-th of the chunks [c_lo, c_hi) of its tiles, from the grp-th on
+// (carried along: a division a chunk costs as much as a quarter of its stores).
+template <int NGRP>
+struct EpiCursor {
+    int mt, c, left, c_lo, c_hi;   // left: chunks from this one on, over all groups (<= 0: none for this warp)
+    __device__ __forceinline__ EpiCursor(int grp, int mt_lo, int lo, int hi, int total) : mt(mt_lo), c(lo + grp), left(total - grp), c_lo(lo), c_hi(hi) { wrap(); }
+    __device__ __forceinline__ void advance() { c += NGRP; left -= NGRP; wrap(); }
+    __device__ __forceinline__ void wrap() {
+        while (left > 0 && c >= c_hi) { c -= c_hi - c_lo; ++mt; }
+    }
+};
+
 // ... `o` holds what epi_load brought.  SWIGLU and LMHEAD have ways of their own (below).
 template <int MODE>
 __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o, const float (&a)[EPI_COLS], float* scr, int m0,
@@ -352,12 +364,10 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
         }
         if (p.logits) {
             const int f = fl + c0;
-            float4 rows[4];
-            epi_rows(scr, rows, tq, c0);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 4; ++i) {   // (a token at a time: with all four rows first an item's epilogue took 23.5 k cycles against 19.5 k)
                 const int t = tq + 4 * i;
-                const float4 v = rows[i];
+                const float4 v = *reinterpret_cast<const float4*>(scr + t * EPI_SCR_STRIDE + c0);
                 if (t < ncols) {
                     float* dst = p.logits + (size_t)(t0 + t) * p.vocab + f;
                     if ((p.vocab & 3) == 0 && f + 4 <= p.vocab) {
@@ -378,8 +388,9 @@ __device__ __forceinline__ void epi_unit(const EpiParams& p, EpiOperand<MODE>& o
 __host__ __device__ constexpr bool epi_scaled(int mode) { return mode == EPI_QKV || mode == EPI_SWIGLU || mode == EPI_LMHEAD; }
 
 // Epilogue warps of the kernels that take a whole SM: 16 (four groups of four warps, one to a TMEM lane quarter) with 96 registers
-// each; qkv 12 with 128, because a chunk with its RoPE rows does not fit into 96.
-__host__ __device__ constexpr int gemm_epi_warps(int mode) { return mode == EPI_QKV ? 12 : GEMM_EPI_WARPS; }
+// each; 12 with 128 where a chunk's operand is in flight beside it, which does not fit into 96 (8B shape, cycles from the last MMA
+// to the end with 12 and 16 warps: o 27.4 and 30.9 k, down 27.1 and 30.4 k at 2 048 tokens, down 20.2 and 24.9 k at 544).
+__host__ __device__ constexpr int gemm_epi_warps(int mode) { return mode == EPI_QKV || mode == EPI_RESID ? 12 : GEMM_EPI_WARPS; }
 __host__ __device__ constexpr int gemm_threads(int mode) { return (2 + gemm_epi_warps(mode)) * 32; }
 
 // A chunk's accumulators, summed, through the epilogue.
@@ -484,7 +495,7 @@ __global__ void pack_weight_kernel(PackSrc src, op16* __restrict__ out, int num_
 }
 
 // ------------------------------------------------------------------------------------------
-// The kernel.  One persistent CTA per SM, 576 threads (qkv: 448): warp 0 = producer (bulk copy of the weight
+// The kernel.  One persistent CTA per SM, 576 threads (448 with 12 epilogue warps): warp 0 = producer (bulk copy of the weight
 // tiles + TMA boxes of the token tile), warp 1 = TMEM owner and MMA issuer, warps 2..17 = epilogue
 // (four groups of four; a group covers the four TMEM lane quarters; draining TMEM is limited per
 // warp, so many warps share it).
@@ -789,19 +800,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             }
             // The chunks [c_lo, c_hi) of this CTA's tiles are finished here, the warp's group takes every NGRP-th of them.
             const int S = RSPLIT ? g.splits : 1, sp = RSPLIT ? w.split : 0;
-            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S, nc = max(c_hi - c_lo, 1);
+            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S;
             const int total_chunks = (w.mt_hi - w.mt_lo) * (c_hi - c_lo);
-            auto unit_at = [&](int ci) {
+            EpiCursor<NGRP> cur(grp, w.mt_lo, c_lo, c_hi, total_chunks);
+            auto unit_here = [&]() {
                 EpiNext u;
-                u.m0 = w.pair * 256 + (w.mt_lo + ci / nc) * 128;
-                const int c = c_lo + ci % nc;
-                u.t0 = n0 + c * EPI_COLS;
-                u.ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                u.any = ci < total_chunks && u.m0 < p.N;
+                u.m0 = w.pair * 256 + cur.mt * 128;
+                u.t0 = n0 + cur.c * EPI_COLS;
+                u.ncols = min(EPI_COLS, n_valid - cur.c * EPI_COLS);
+                u.any = cur.left > 0 && u.m0 < p.N;
                 return u;
             };
             EpiOperand<MODE> opnd;   // of the warp's first chunk: in flight while the main loop runs
-            EpiNext unit = unit_at(grp);
+            EpiNext unit = unit_here();
             if (unit.any && (!KSPLIT || w.role != 1)) epi_load<MODE>(p, opnd, unit.m0, unit.t0, unit.ncols, quarter, lane);
             ok = mbar_wait(accf_bar, i & 1, g.status, limit);
             if (ok && scaled) ok = mbar_wait(rs_bar, i & 1, g.status, limit);
@@ -844,8 +855,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                     }
                 }
                 __syncwarp();
-                for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = ci / nc, c = c_lo + ci % nc;
+                while (cur.left > 0) {
+                    const int mt = cur.mt, c = cur.c;
                     uint32_t own[EPI_COLS], r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
                     tmem_ld_wait();
@@ -859,7 +870,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                             epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + (size_t)(tile * S + q) * slot_elems + at) + lane, q == 0);
                         }
                     }
-                    const EpiNext next = unit_at(ci + NGRP);
+                    cur.advance();
+                    const EpiNext next = unit_here();
                     if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
                     unit = next;
                 }
@@ -872,16 +884,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                 continue;
             }
             if (!KSPLIT || w.role == 0) {
-                for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = w.mt_lo + ci / nc, c = ci % nc;
+                while (cur.left > 0) {
+                    const int mt = cur.mt, c = cur.c;
                     uint32_t r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                     tmem_ld_wait();
-                    if (ci + NGRP >= total_chunks) {   // last TMEM read of this warp for this item
+                    if (cur.left <= NGRP) {   // last TMEM read of this warp for this item
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(acce_bar);
                     }
-                    const EpiNext next = unit_at(ci + NGRP);
+                    cur.advance();
+                    const EpiNext next = unit_here();
                     if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
                     unit = next;
                 }
@@ -898,18 +911,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
             const size_t part_elems = (size_t)2 * cpt * 128 * EPI_COLS;
             if (w.role == 1) {
                 float* mine = g.fix_part + (size_t)(w.rtile * H + w.hpart) * part_elems;
-                for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = w.mt_lo + ci / nc, c = ci % nc;
+                while (cur.left > 0) {
+                    const int mt = cur.mt, c = cur.c;
                     uint32_t r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                     tmem_ld_wait();
-                    if (ci + NGRP >= total_chunks) {
+                    if (cur.left <= NGRP) {
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(acce_bar);
                     }
                     uint4* dst = reinterpret_cast<uint4*>(mine + (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS) + lane;
 #pragma unroll
                     for (int v = 0; v < EPI_COLS / 4; ++v) dst[v * 32] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+                    cur.advance();
                 }
                 if (grp >= total_chunks) {
                     tc_fence_before();
@@ -932,19 +946,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmB, GemmParams g, EpiParams p) 
                 }
             }
             __syncwarp();
-            for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                const int mt = w.mt_lo + ci / nc, c = ci % nc;
+            while (cur.left > 0) {
+                const int mt = cur.mt, c = cur.c;
                 uint32_t r[EPI_COLS];
                 tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                 tmem_ld_wait();
-                if (ci + NGRP >= total_chunks) {
+                if (cur.left <= NGRP) {
                     tc_fence_before();
                     if (lane == 0) mbar_arrive(acce_bar);
                 }
                 const size_t at = (((size_t)mt * cpt + c) * 4 + quarter) * 32 * EPI_COLS;
                 for (int h = 0; h < H; ++h)   // fixed order: own k range, then the helpers' in part order
                     epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + (size_t)(w.rtile * H + h) * part_elems + at) + lane, false);
-                const EpiNext next = unit_at(ci + NGRP);
+                cur.advance();
+                const EpiNext next = unit_here();
                 if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
                 unit = next;
             }

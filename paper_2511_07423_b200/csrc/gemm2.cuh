@@ -256,19 +256,19 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             const int n_mt = DUO ? 1 : 2;
             const int row0 = DUO ? w.grp * 256 + (int)rank * 128 : (2 * w.grp + (int)rank) * 256;
             const int S = w.nsplit, sp = w.split;
-            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S, nc = max(c_hi - c_lo, 1);
+            const int c_lo = sp * nchunks / S, c_hi = (sp + 1) * nchunks / S;
             const int total_chunks = n_mt * (c_hi - c_lo);
-            auto unit_at = [&](int ci) {
+            EpiCursor<NGRP> cur(grp, 0, c_lo, c_hi, total_chunks);
+            auto unit_here = [&]() {
                 EpiNext u;
-                u.m0 = row0 + ci / nc * 128;
-                const int c = c_lo + ci % nc;
-                u.t0 = n0 + c * EPI_COLS;
-                u.ncols = min(EPI_COLS, n_valid - c * EPI_COLS);
-                u.any = ci < total_chunks && u.m0 < p.N;
+                u.m0 = row0 + cur.mt * 128;
+                u.t0 = n0 + cur.c * EPI_COLS;
+                u.ncols = min(EPI_COLS, n_valid - cur.c * EPI_COLS);
+                u.any = cur.left > 0 && u.m0 < p.N;
                 return u;
             };
             EpiOperand<MODE> opnd;   // of the warp's first chunk: in flight while the main loop runs
-            EpiNext unit = unit_at(grp);
+            EpiNext unit = unit_here();
             if (unit.any) epi_load<MODE>(p, opnd, unit.m0, unit.t0, unit.ncols, quarter, lane);
             ok = mbar_wait(accf_bar, i & 1, g.status, limit);
             if (ok && scaled) ok = mbar_wait(rs_bar, i & 1, g.status, limit);
@@ -315,8 +315,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     }
                 }
                 __syncwarp();
-                for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                    const int mt = ci / nc, c = c_lo + ci % nc;
+                while (cur.left > 0) {
+                    const int mt = cur.mt, c = cur.c;
                     uint32_t own[EPI_COLS], r[EPI_COLS];
                     tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), own);
                     if (DUO) {
@@ -338,7 +338,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                             epi_add_part(r, reinterpret_cast<const float4*>(g.fix_part + peer * slot_elems + at) + lane, q == 0);
                         }
                     }
-                    const EpiNext next = unit_at(ci + NGRP);
+                    cur.advance();
+                    const EpiNext next = unit_here();
                     if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
                     unit = next;
                 }
@@ -349,8 +350,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 }
                 continue;
             }
-            for (int ci = grp; ci < total_chunks; ci += NGRP) {
-                const int mt = ci / nc, c = ci % nc;
+            while (cur.left > 0) {
+                const int mt = cur.mt, c = cur.c;
                 uint32_t r[EPI_COLS];
                 tmem_ld16(tmem_base + mt * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * EPI_COLS), r);
                 if (DUO) {
@@ -362,11 +363,12 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 } else {
                     tmem_ld_wait();
                 }
-                if (ci + NGRP >= total_chunks) {   // last TMEM read of this warp for this item
+                if (cur.left <= NGRP) {   // last TMEM read of this warp for this item
                     tc_fence_before();
                     if (lane == 0) mbar_arrive_cluster(acce_c);
                 }
-                const EpiNext next = unit_at(ci + NGRP);
+                cur.advance();
+                const EpiNext next = unit_here();
                 if (unit.any) epi_chunk<MODE>(p, opnd, r, rsi + c * EPI_COLS, scr, unit.m0, unit.t0, unit.ncols, quarter, lane, next);
                 unit = next;
             }
