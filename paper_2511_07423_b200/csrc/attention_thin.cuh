@@ -29,9 +29,9 @@ struct AttnThinSmem {
     static constexpr int PAGES = HD == 128 ? 2 : 4;                // per stage
     static constexpr int PAGE_BYTES = 2 * 16 * HD * 2;             // K and V of one page, one head
     static constexpr int STAGE_BYTES = PAGES * PAGE_BYTES;         // 16 KB
-    // two slots of O[16][HD] + (m, l)[16], or (m, l) and weights of every part of the 64 rows
-    static constexpr int MERGE_BYTES = ATTN_THIN_MAX_PARTS * 64 * 8 > 2 * 16 * (HD + 4) * 4 ? ATTN_THIN_MAX_PARTS * 64 * 8
-                                                                                            : 2 * 16 * (HD + 4) * 4;
+    // two slots of O[16][HD] + (m, l)[16], or a weight for every part of the 64 rows and one over their sums
+    static constexpr int WEIGHT_BYTES = (ATTN_THIN_MAX_PARTS + 1) * 64 * 4, SLOT_BYTES = 2 * 16 * (HD + 4) * 4;
+    static constexpr int MERGE_BYTES = WEIGHT_BYTES > SLOT_BYTES ? WEIGHT_BYTES : SLOT_BYTES;
     static constexpr int TOTAL = 1024 + ATTN_THIN_STAGES * STAGE_BYTES + MERGE_BYTES + 512;
     static_assert(2 * (TOTAL + 1024) <= 233472, "two CTAs per SM");
 };
@@ -42,6 +42,7 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
 __device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(src)), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void l1_prefetch(const void* src) { asm volatile("prefetch.global.L1 [%0];" ::"l"(src)); }
 __device__ __forceinline__ void attn_thin_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 template <int HD>
@@ -138,6 +139,7 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
     // ---------------------------------------------------------------- consumers (warps 0..3)
     // A wait that runs out sets `ok` = false; the warp then skips all further waits and arithmetic but still walks the
     // items and takes part in every named barrier, so no other warp is left waiting for it.
+    if (list_ok && it_begin < it_end && lane < 2) l1_prefetch(reinterpret_cast<const uint8_t*>(p.items + it_begin) + lane * (sizeof(AttnItem) - 4));
     pdl_wait();   // Q and the chunk's K/V come from the preceding projection kernel
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int g = lane >> 2, c = lane & 3;
@@ -199,6 +201,8 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
             l[r] += __shfl_xor_sync(0xFFFFFFFFu, l[r], 1);
             l[r] += __shfl_xor_sync(0xFFFFFFFFu, l[r], 2);
         }
+        int part0 = 0, n_parts = 0;   // of the item's merge group
+        if (item.part >= 0) { part0 = p.groups[item.grp].part0; n_parts = p.groups[item.grp].n_parts; }
         // the warps of a row tile, in a fixed order: (0 + 2) + (1 + 3), or 0 + 1
         if (nph > 1) {
             attn_thin_bar();   // slots free: the previous item's readers are done
@@ -238,61 +242,61 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
         }
         // a partial item: count it; the CTA that completes the group combines the partials in part order
         if (item.part >= 0) {
-            __threadfence();
             attn_thin_bar();
-            const MergeGroup gr = p.groups[item.grp];
-            if (threadIdx.x == 0) {
-                const int done = atomicAdd(p.group_count + item.grp, 1);
-                const int last = done == gr.n_parts - 1;
-                if (last) p.group_count[item.grp] = 0;   // ready for the next launch
-                *last_flag = last;
-            }
+            // (one thread's release covers what the barrier ordered before it, its acquire what the barrier orders behind it)
+            if (threadIdx.x == 0) *last_flag = atomic_add_acq_rel(p.group_count + item.grp, 1) == n_parts - 1;
             attn_thin_bar();
             if (*last_flag) {
-                __threadfence();
-                // What this costs is the round trips to L2, on the step's critical path: a thread has fifteen float4 of
-                // the partial outputs in flight (NU places of the rows x UK parts), the first of them together with the
-                // (m, l) pairs.  (8B shape, 9 parts of 20 rows: 8.8 k cycles with two parts at a time after the pairs.)
-                const int np = min(gr.n_parts, ATTN_THIN_MAX_PARTS);
-                float2* ml_s = reinterpret_cast<float2*>(merge);   // [part][64]
-                constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5;
-                const int n_vec = rows * VR;
-                const float4* src = reinterpret_cast<const float4*>(p.part_o + (size_t)gr.part0 * p.row_cap * HD);
+                // What this costs is round trips, on the step's critical path: the (m, l) pairs and the first UK parts of the
+                // outputs (NU places of the rows each) are in flight together, and the weights wait for the pairs alone.  (Loads
+                // past the last part repeat it: left out under a condition they cost 600 bytes of spills in the stage loop.)
+                if (threadIdx.x == 0) p.group_count[item.grp] = 0;   // ready for the next launch
+                const int np = min(n_parts, ATTN_THIN_MAX_PARTS);
+                float* w_s = merge;                                   // [part][64]
+                float* inv_s = merge + ATTN_THIN_MAX_PARTS * 64;      // [64]
+                constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5, CAP = 64;   // CAP: rows of a part
+                const int n_vec = rows * VR, by_g = 4096 / G + 1;   // row / G = row * by_g >> 12 for rows up to 64
+                const float4* src = reinterpret_cast<const float4*>(p.part_o) + (size_t)part0 * (CAP * VR);
                 float4 v[UK][NU];
                 auto fetch = [&](int u0, int k0) {
 #pragma unroll
                     for (int k = 0; k < UK; ++k)
 #pragma unroll
-                        for (int i = 0; i < NU; ++i)
-                            v[k][i] = __ldcg(src + (size_t)min(k0 + k, np - 1) * p.row_cap * VR + min(u0 + i * 128, n_vec - 1));
+                        for (int i = 0; i < NU; ++i) v[k][i] = __ldcg(src + min(k0 + k, np - 1) * (CAP * VR) + min(u0 + i * 128, n_vec - 1));
                 };
-                fetch(threadIdx.x, 0);
-                {
-                    const int row = threadIdx.x & 63;
-                    const float2* ml = p.part_ml + (size_t)gr.part0 * p.row_cap + min(row, rows - 1);
-                    for (int k0 = threadIdx.x >> 6; k0 < np; k0 += 16) {
-                        float2 t[8];
+                {   // lanes 2 r and 2 r + 1 take the even and the odd parts of row r, eight of them at a time
+                    const int row = threadIdx.x >> 1, odd = threadIdx.x & 1;
+                    const float2* ml = p.part_ml + (size_t)part0 * CAP + min(row, rows - 1);
+                    float2 t[8];
+                    auto pairs = [&](int k0) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) t[k] = __ldcg(ml + (size_t)min(k0 + 2 * k, np - 1) * p.row_cap);
-#pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            if (k0 + 2 * k < np) ml_s[(k0 + 2 * k) * 64 + row] = t[k];
-                    }
-                }
-                attn_thin_bar();
-                if (threadIdx.x < rows) {   // weight of every part of a row, already divided by the row's sum
-                    float2* col = ml_s + threadIdx.x;
+                        for (int k = 0; k < 8; ++k) t[k] = k0 + odd + 2 * k < np ? __ldcg(ml + (k0 + odd + 2 * k) * CAP) : make_float2(-INFINITY, 0.f);
+                    };
+                    pairs(0);
+                    fetch(threadIdx.x, 0);
                     float mx = -INFINITY, lsum = 0.f;
-#pragma unroll 4
-                    for (int k = 0; k < np; ++k) mx = fmaxf(mx, col[k * 64].x);
+                    for (int k0 = 0; k0 < np; k0 += 16) {
+                        if (k0) pairs(k0);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) mx = fmaxf(mx, t[k].x);
+                    }
+                    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
                     const float bs = mx == -INFINITY ? 0.f : mx;
-#pragma unroll 4
-                    for (int k = 0; k < np; ++k) lsum += col[k * 64].y * ex2_approx(col[k * 64].x - bs);
-                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-#pragma unroll 4
-                    for (int k = 0; k < np; ++k) col[k * 64].x = ex2_approx(col[k * 64].x - bs) * inv;
+                    for (int k0 = 0; k0 < np; k0 += 16) {
+                        if (np > 16) pairs(k0);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            if (k0 + 2 * k >= np) break;
+                            const float w = ex2_approx(t[k].x - bs);
+                            lsum += t[k].y * w;
+                            w_s[(k0 + odd + 2 * k) * 64 + row] = w;
+                        }
+                    }
+                    lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, 1);
+                    if (!odd) inv_s[row] = lsum > 0.f ? 1.f / lsum : 0.f;
                 }
                 attn_thin_bar();
+                op16* const out0 = p.out + (size_t)item.q_tok * p.q_dim + item.kvh * G * HD;
                 for (int u0 = threadIdx.x; u0 < n_vec; u0 += NU * 128) {
                     float4 acc[NU];
 #pragma unroll
@@ -300,19 +304,23 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                     for (int k0 = 0; k0 < np; k0 += UK) {
                         if (k0 > 0 || u0 != (int)threadIdx.x) fetch(u0, k0);
 #pragma unroll
-                        for (int k = 0; k < UK; ++k)
+                        for (int k = 0; k < UK; ++k) {
+                            if (k0 + k >= np) break;
 #pragma unroll
                             for (int i = 0; i < NU; ++i) {
-                                const float w = k0 + k < np ? ml_s[(k0 + k) * 64 + min(u0 + i * 128, n_vec - 1) / VR].x : 0.f;
+                                const float w = w_s[(k0 + k) * 64 + min(u0 + i * 128, n_vec - 1) / VR];
                                 acc[i].x += v[k][i].x * w; acc[i].y += v[k][i].y * w; acc[i].z += v[k][i].z * w; acc[i].w += v[k][i].w * w;
                             }
+                        }
                     }
 #pragma unroll
                     for (int i = 0; i < NU; ++i) {
-                        const int u = u0 + i * 128, row = u / VR, j = row / G, gq = row - j * G;
-                        if (u < n_vec)
-                            *reinterpret_cast<uint2*>(p.out + (size_t)(gr.q_tok + j) * p.q_dim + (gr.kvh * G + gq) * HD + 4 * (u % VR)) =
-                                make_uint2(pack_op(acc[i].x, acc[i].y), pack_op(acc[i].z, acc[i].w));
+                        const int u = u0 + i * 128, row = u / VR, j = row * by_g >> 12, gq = row - j * G;
+                        if (u < n_vec) {
+                            const float inv = inv_s[row];
+                            *reinterpret_cast<uint2*>(out0 + (size_t)j * p.q_dim + gq * HD + 4 * (u % VR)) =
+                                make_uint2(pack_op(acc[i].x * inv, acc[i].y * inv), pack_op(acc[i].z * inv, acc[i].w * inv));
+                        }
                     }
                 }
                 attn_thin_bar();   // the weights' area is the next item's merge slots
