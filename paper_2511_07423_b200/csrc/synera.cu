@@ -1752,6 +1752,10 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
 // one request 840 / 830 / - / 883 (104 CTAs), 1B shape, two requests 878 / 870 / 863 / 844, 8B shape, eight requests
 // 4 048 / 3 956 / 3 939 / 3 922, 16 requests 2 414 / 2 400 / 2 403 / 2 440 (16 layers).  Where a layer has more than 16 MB of
 // keys a CTA waits for its own first (8B shape, eight requests, without that: 3 974).
+// Only where most items are parts: while those are merged HBM idles, whereas whole units of unequal length keep some CTAs loading
+// to the end, and these the requests delay (1B shape, with and without: 32 requests of 256 - 2 048 keys 1 300 and 1 268 us a step,
+// 26 of 380 - 474 keys 894 and 863, 4 of 78 - 125 keys 787 and 755; one request in 104 parts 774 and 788; 8B shape, eight requests in
+// 288 parts 3 764 and 3 818).
 constexpr int64_t ATTN_AHEAD_BYTES = 24 << 20, ATTN_AHEAD_TILES = 10, ATTN_AHEAD_LATE_BYTES = 16 << 20;
 
 // What the attention may ask of L2 ahead: `budget` bytes (taken off) of a projection's weights beyond what the operand rings
@@ -1792,7 +1796,7 @@ static int launch_attention(syn_model* m, syn_kv* kv, const syn_plan* p, uint32_
                             op16* out, cudaStream_t st) {
     AttnParams ap;
     attn_params(ap, m, kv, p, layer, out, m->part_o, m->part_ml, m->group_count);
-    if (p->attn == ATTN_THIN) {
+    if (p->attn == ATTN_THIN && 2 * p->n_parts > p->n_items) {
         const syn_model_desc& c = m->desc;
         const int d = c.d_model, q_dim = c.n_q_heads * c.head_dim;
         int64_t budget = std::min(ATTN_AHEAD_BYTES, (int64_t)p->n_cta * ATTN_AHEAD_TILES * GEMM_TILE_BYTES);
