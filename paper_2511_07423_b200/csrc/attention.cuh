@@ -493,35 +493,29 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         }
         // a partial item: count it; the CTA that completes the group combines the partials
         if (item.part >= 0) {
-            __threadfence();
+            const int part0 = p.groups[item.grp].part0, n_parts = p.groups[item.grp].n_parts;
             consumer_bar();
-            if (threadIdx.x == 0) {
-                const MergeGroup gr = p.groups[item.grp];
-                const int done = atomicAdd(p.group_count + item.grp, 1);
-                const int last = done == gr.n_parts - 1;
-                if (last) p.group_count[item.grp] = 0;   // ready for the next launch
-                *last_flag = last;
-            }
+            // (one thread's release covers what the barrier ordered before it, its acquire what the barrier orders behind it)
+            if (threadIdx.x == 0) *last_flag = atomic_add_acq_rel(p.group_count + item.grp, 1) == n_parts - 1;
             consumer_bar();
             if (*last_flag) {
-                __threadfence();
+                if (threadIdx.x == 0) p.group_count[item.grp] = 0;   // ready for the next launch
                 // 4 threads per row, each 1/4 of the row's columns; all loads of a thread are independent
-                const MergeGroup gr = p.groups[item.grp];
                 constexpr int CW = HD / 4;   // columns per thread
                 const int row = threadIdx.x >> 2, c0 = (threadIdx.x & 3) * CW;
                 if (row < rows) {
                     float mx = -INFINITY;
-                    for (int k = 0; k < gr.n_parts; ++k) mx = fmaxf(mx, __ldcg(&p.part_ml[(size_t)(gr.part0 + k) * p.row_cap + row]).x);
+                    for (int k = 0; k < n_parts; ++k) mx = fmaxf(mx, __ldcg(&p.part_ml[(size_t)(part0 + k) * p.row_cap + row]).x);
                     const float bs = mx == -INFINITY ? 0.f : mx;
                     float lsum = 0.f;
                     float4 acc[CW / 4];
 #pragma unroll
                     for (int i = 0; i < CW / 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int k = 0; k < gr.n_parts; ++k) {
-                        const float2 ml = __ldcg(&p.part_ml[(size_t)(gr.part0 + k) * p.row_cap + row]);
+                    for (int k = 0; k < n_parts; ++k) {
+                        const float2 ml = __ldcg(&p.part_ml[(size_t)(part0 + k) * p.row_cap + row]);
                         const float w = ex2_approx(ml.x - bs);
                         lsum += ml.y * w;
-                        const float4* src = reinterpret_cast<const float4*>(p.part_o + ((size_t)(gr.part0 + k) * p.row_cap + row) * HD + c0);
+                        const float4* src = reinterpret_cast<const float4*>(p.part_o + ((size_t)(part0 + k) * p.row_cap + row) * HD + c0);
 #pragma unroll
                         for (int i = 0; i < CW / 4; ++i) {
                             const float4 v = __ldcg(src + i);
@@ -530,7 +524,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     }
                     const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
                     const int j = row / G, gq = row - j * G;
-                    uint2* dst = reinterpret_cast<uint2*>(p.out + (size_t)(gr.q_tok + j) * p.q_dim + (gr.kvh * G + gq) * HD + c0);
+                    uint2* dst = reinterpret_cast<uint2*>(p.out + (size_t)(item.q_tok + j) * p.q_dim + (item.kvh * G + gq) * HD + c0);
 #pragma unroll
                     for (int i = 0; i < CW / 4; ++i)
                         dst[i] = make_uint2(pack_op(acc[i].x * inv, acc[i].y * inv), pack_op(acc[i].z * inv, acc[i].w * inv));
