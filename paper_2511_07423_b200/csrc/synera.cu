@@ -1624,7 +1624,7 @@ static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int for
     return gemm2_plan_by_rule(T, packed_rows, K, n_sm, mode, best, g, n_cl);
 }
 
-constexpr int THIN_MAX_TOKENS = 512;
+constexpr int THIN_MAX_TOKENS = 512, THIN_MAX_TOKENS_QKV = 1024;
 
 // Launch shape of a projection on the thin kernel (gemm_thin.cuh): at most one CTA per SM where K is shared, so that the
 // other half of every SM is free for the next kernel; at least two k-blocks each.
@@ -1635,7 +1635,13 @@ static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
     g.n_tt = (T + THIN_MAX_TN - 1) / THIN_MAX_TN;
     g.TN = ((T + g.n_tt - 1) / g.n_tt + 15) / 16 * 16;
     g.n_tt = (T + g.TN - 1) / g.TN;
-    g.splits = std::max(1, std::min(std::min(THIN_MAX_SPLITS, n_sm / (g.n_tiles * g.n_tt)), g.num_kb / 2));
+    const int items = g.n_tiles * g.n_tt;
+    g.splits = std::max(1, std::min(std::min(THIN_MAX_SPLITS, n_sm / items), g.num_kb / 2));
+    // Two CTAs to an SM where several token tiles make L2 -> SM traffic the bound (the operands in flight of one CTA, 96 KB, bring
+    // 36 bytes a cycle of the 63 that an SM can take), K leaves every part 16 k-blocks, and clusters of four fill the slots
+    // (larger clusters and those of three or six do not all fit at a time: 1B down at 320 tokens 29.5 < 35.5 us with six).  Event
+    // times, one CTA to an SM and two: 1B down at 448 tokens 33.3 > 29.2 us, at 512 34.6 > 31.4; 8B o at 160 tokens 23.0 > 21.0.
+    if (g.n_tt >= 2 && 4 * items <= 2 * n_sm && 4 * items >= 3 * n_sm / 2 && g.num_kb >= 64) g.splits = 4;
     const int recv = g.splits > 1 ? thin_recv_bytes(g.TN, g.splits) : 0;
     g.recv_own = recv > 0 && recv <= THIN_RECV_OWN_MAX;
     g.n_stages = thin_stages(g.TN, g.recv_own ? recv : 0);
@@ -1649,11 +1655,14 @@ static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
 //   several token tiles read the weights once each, which only pays while every CTA has little work: 1B shape at 256 tokens
 //   qkv 31.1 > 20.9 (16 k-blocks a CTA), gate/up 29.1 > 28.1 (32), down 36.9 > 25.0 (32), 8B shape o 35.1 > 27.0 (32); but
 //   8B shape qkv 31.1 < 36.3 (176 tokens, 64 k-blocks), down 46 < 54 (112), 1B gate/up 35 < 41 at 320 tokens (384 CTAs).
+//   Beyond 512 tokens qkv of a narrow model (32 k-blocks, two CTAs to an SM): 1B 30.5 > 23.0 at 576 tokens, 33.1 > 23.2 at 640,
+//   29.0 > 24.5 at 768, 29.0 = 28.8 at 1 024; its o gains little (24.4 > 22.8 at 576).
 static bool thin_takes(int T, int packed_rows, int K, int n_sm, int mode) {
-    if (T > THIN_MAX_TOKENS) return false;
+    if (T > (mode == EPI_QKV ? THIN_MAX_TOKENS_QKV : THIN_MAX_TOKENS)) return false;
     ThinParams g;
     thin_plan(T, packed_rows, K, n_sm, g);
-    const int ctas = g.n_tiles * g.n_tt * g.splits, nk = (g.num_kb + g.splits - 1) / g.splits;
+    const int items = g.n_tiles * g.n_tt, S = std::min(g.splits, std::max(1, n_sm / items));   // (one CTA to an SM)
+    const int ctas = items * S, nk = (g.num_kb + S - 1) / S;
     if (g.n_tt == 1) return T <= 64 || ctas <= 3 * n_sm;
     return mode == EPI_RESID ? ctas <= n_sm && nk <= 64 : ctas <= 2 * n_sm && nk <= 32;
 }

@@ -68,3 +68,24 @@ def test_product_matches_oracle(T, N, K):
     scale = np.abs(ref).max()
     err = np.abs(y.cpu().double().numpy() - ref).max()
     assert err <= 2e-5 * scale * max(1.0, (K / 256) ** 0.5), (err, scale)   # fp32 sums, as for the other kernels
+
+
+def test_two_ctas_to_an_sm():
+    """Several token tiles, 38 to 74 items and a K of 64 k-blocks and more: parts in clusters of four, 16 k-blocks or more each."""
+    for T, N, K, splits in ((448, 2048, 8192, 4), (512, 2048, 8192, 4), (160, 4096, 4096, 4), (256, 4096, 4096, 4),
+                            (320, 2048, 8192, 3), (448, 2048, 2048, 2), (128, 4096, 4096, 4), (160, 6144, 4096, 1), (1024, 3072, 2048, 1)):
+        p = syn.thin_plan_host(T, N, K)
+        assert p["splits"] == splits, (T, N, K, p)
+    assert syn.thin_plan_host(1024, 3072, 2048, "qkv")["takes_it"] and not syn.thin_plan_host(1025, 3072, 2048, "qkv")["takes_it"]
+    assert not syn.thin_plan_host(576, 6144, 4096, "qkv")["takes_it"]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,N,K", [
+    (385, 2048, 4096),    # four token tiles, the last of one token; 64 items in clusters of four
+    (449, 2048, 8192),    # 113 tokens in the last tile
+    (160, 4096, 4160),    # two token tiles of 80, 65 k-blocks in parts of 16 and 17
+    (1024, 384, 2048),    # eight token tiles
+])
+def test_products_of_several_token_tiles_match_the_oracle(T, N, K):
+    test_product_matches_oracle(T, N, K)
