@@ -123,12 +123,15 @@ prep_kernel(const bf16* __restrict__ embed, const int* __restrict__ tokens, cons
     }
 }
 
-// Greedy verification (paper Sec. 3.1 "draft & verify", Sec. 4.5): one thread per request.
+// Greedy verification (paper Sec. 3.1 "draft & verify", Sec. 4.5): one thread per request.  The blocking calls have the results and
+// the kernels' status written straight to pinned host memory (three copies behind the kernel took 5 us).
 __global__ void verify_kernel(const unsigned long long* __restrict__ best, const int* __restrict__ tokens,
                               const int* __restrict__ offsets, const int* __restrict__ n_uncached, int n_req,
-                              int* __restrict__ accept_len, int* __restrict__ correction, int* __restrict__ top1_out) {
+                              int* __restrict__ accept_len, int* __restrict__ correction, int* __restrict__ top1_out,
+                              const int* status, int* status_out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
+    if (i == 0 && status_out) *status_out = *status;
     if (i >= n_req) return;
     const int b = offsets[i], n = offsets[i + 1] - b, u = n_uncached[i];
     if (top1_out)
@@ -280,8 +283,6 @@ struct syn_model {
          *q = nullptr, *attn = nullptr, *act = nullptr;
     float2* rope = nullptr;
     unsigned long long* best = nullptr;
-    int *acc_dev = nullptr, *corr_dev = nullptr;
-    int b_cap = 0;
     XMaps tm_xn, tm_attn, tm_act;
     CUtensorMap tm_q, tm_q4;
     float* fix_part = nullptr;      // stored accumulators of K-split remainder tiles (one slot per SM)
@@ -368,7 +369,7 @@ static void free_workspace(syn_model* m) {
     m->t_cap = 0;
 }
 
-static int ensure_workspace(syn_model* m, int T, int B, int n_parts) {
+static int ensure_workspace(syn_model* m, int T, int n_parts) {
     const syn_model_desc& c = m->desc;
     const int q_dim = c.n_q_heads * c.head_dim;
     if (T > m->t_cap) {
@@ -417,14 +418,6 @@ static int ensure_workspace(syn_model* m, int T, int B, int n_parts) {
         CU_OK(cudaMalloc(&m->fix_part, (size_t)m->n_sm * GEMM_FIX_SLOT_BYTES));
         CU_OK(cudaMalloc(&m->fix_flag, (size_t)GEMM_FLAG_INTS * m->n_sm * 4));
         CU_OK(cudaMemset(m->fix_flag, 0, (size_t)GEMM_FLAG_INTS * m->n_sm * 4));
-    }
-    if (B > m->b_cap) {
-        cudaFree(m->acc_dev); cudaFree(m->corr_dev);
-        m->acc_dev = m->corr_dev = nullptr; m->b_cap = 0;
-        const int cap = (B + 255) / 256 * 256;
-        CU_OK(cudaMalloc(&m->acc_dev, (size_t)cap * 4));
-        CU_OK(cudaMalloc(&m->corr_dev, (size_t)cap * 4));
-        m->b_cap = cap;
     }
     if (n_parts > m->part_cap) {
         cudaFree(m->part_o); cudaFree(m->part_ml); cudaFree(m->group_count);
@@ -488,7 +481,7 @@ extern "C" void syn_model_free(syn_model* m) {
         for (bf16* p : *v) cudaFree(p);
     cudaFree(m->embed); cudaFree(m->lm_head); cudaFree(m->final_norm); cudaFree(m->inv_freq); cudaFree(m->status_dev);
     free_workspace(m);
-    cudaFree(m->acc_dev); cudaFree(m->corr_dev); cudaFree(m->part_o); cudaFree(m->part_ml); cudaFree(m->group_count);
+    cudaFree(m->part_o); cudaFree(m->part_ml); cudaFree(m->group_count);
     cudaFree(m->fix_part); cudaFree(m->fix_flag);
     if (m->pinned_out) cudaFreeHost(m->pinned_out);
     cudaFree(m->sw.logits); cudaFree(m->sw.topk_logit); cudaFree(m->sw.topk_id); cudaFree(m->sw.slm_id);
@@ -1345,7 +1338,7 @@ static int syn_plan_create_impl(syn_model* m, syn_kv* kv, int32_t n_req, const i
         cudaError_t e = cudaMemcpy(p->dev, p->host, p->used, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) r = SYN_E_CUDA;
     }
-    if (r == SYN_OK) r = ensure_workspace(m, p->T, p->n_req, p->n_parts);
+    if (r == SYN_OK) r = ensure_workspace(m, p->T, p->n_parts);
     if (r != SYN_OK) {
         syn_plan_free(p);
         return r;
@@ -1821,10 +1814,10 @@ static int launch_attention(syn_model* m, syn_kv* kv, const syn_plan* p, uint32_
 }
 
 static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, int* corr_dev, int* top1_dev,
-                    float* logits_out, cudaStream_t st, uint32_t* warp_max = nullptr) {
+                    float* logits_out, cudaStream_t st, uint32_t* warp_max = nullptr, int* status_out = nullptr) {
     const syn_model_desc& c = m->desc;
     const int T = p->T, d = c.d_model, q_dim = c.n_q_heads * c.head_dim, kv_dim = c.n_kv_heads * c.head_dim;
-    if (T > m->t_cap || p->n_req > m->b_cap || p->n_parts > m->part_cap) return SYN_E_INVALID_ARG;
+    if (T > m->t_cap || p->n_parts > m->part_cap) return SYN_E_INVALID_ARG;
     const int* tokens = p->d<int>(p->o_tokens);
     const float inv_d = 1.0f / (float)d;
     m->last_stats = p->stats;
@@ -1889,7 +1882,7 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     {
         ProfScope prof(m, 8, st);
         if (launch_pdl(verify_kernel, dim3((p->n_req + 127) / 128), dim3(128), 0, st, m->best, tokens, p->d<int>(p->o_offsets),
-                       p->d<int>(p->o_uncached), p->n_req, acc_dev, corr_dev, top1_dev) != cudaSuccess)
+                       p->d<int>(p->o_uncached), p->n_req, acc_dev, corr_dev, top1_dev, m->status_dev, status_out) != cudaSuccess)
             return SYN_E_CUDA;
     }
     if (m->profile) {
@@ -1953,7 +1946,7 @@ static int syn_verify_batch_impl(syn_model* m, syn_kv* kv, int32_t n_req, const 
     syn_plan* p = m->scratch_plan;
     int r = plan_build(p, m, kv, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages, ctx_lens, n_uncached);
     if (r) return r;
-    if ((r = ensure_workspace(m, p->T, p->n_req, p->n_parts))) return r;
+    if ((r = ensure_workspace(m, p->T, p->n_parts))) return r;
     if (n_req > m->pinned_out_cap) {
         if (m->pinned_out) cudaFreeHost(m->pinned_out);
         m->pinned_out = nullptr; m->pinned_out_cap = 0;
@@ -1963,20 +1956,17 @@ static int syn_verify_batch_impl(syn_model* m, syn_kv* kv, int32_t n_req, const 
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     CU_OK(cudaMemcpyAsync(p->dev, p->host, p->used, cudaMemcpyHostToDevice, st));
-    if ((r = run_step(m, kv, p, m->acc_dev, m->corr_dev, nullptr, logits_out, st))) return r;
-    int* po = m->pinned_out;
-    CU_OK(cudaMemcpyAsync(po, m->acc_dev, (size_t)n_req * 4, cudaMemcpyDeviceToHost, st));
-    CU_OK(cudaMemcpyAsync(po + m->pinned_out_cap, m->corr_dev, (size_t)n_req * 4, cudaMemcpyDeviceToHost, st));
-    CU_OK(cudaMemcpyAsync(po + 2 * m->pinned_out_cap, m->status_dev, 4, cudaMemcpyDeviceToHost, st));
+    int *const po = m->pinned_out, *const po_corr = po + m->pinned_out_cap, *const po_status = po + 2 * m->pinned_out_cap;
+    if ((r = run_step(m, kv, p, po, po_corr, nullptr, logits_out, st, nullptr, po_status))) return r;
     CU_OK(cudaStreamSynchronize(st));
-    if (po[2 * m->pinned_out_cap]) {
+    if (*po_status) {
         cudaMemset(m->status_dev, 0, 4);
         if (m->group_count) cudaMemset(m->group_count, 0, (size_t)m->part_cap * 4);
         if (m->fix_flag) cudaMemset(m->fix_flag, 0, (size_t)GEMM_FLAG_INTS * m->n_sm * 4);
         return SYN_E_DEVICE_TIMEOUT;
     }
     memcpy(accept_len, po, (size_t)n_req * 4);
-    memcpy(correction_token, po + m->pinned_out_cap, (size_t)n_req * 4);
+    memcpy(correction_token, po_corr, (size_t)n_req * 4);
     return SYN_OK;
 }
 
@@ -2070,7 +2060,7 @@ static int syn_verify_batch_sampled_impl(syn_model* m, syn_kv* kv, int32_t n_req
     int r = plan_build(p, m, kv, n_req, chunk_tokens, chunk_offsets, page_tables, max_pages, ctx_lens, n_uncached);
     if (r) return r;
     if ((r = check_sampling(cfg, (int)m->desc.vocab, p->T, n_req, slm_ids, slm_probs, rand_accept, rand_sample))) return r;
-    if ((r = ensure_workspace(m, p->T, p->n_req, p->n_parts))) return r;
+    if ((r = ensure_workspace(m, p->T, p->n_parts))) return r;
     if ((r = ensure_sample_ws(m, p->T, n_req, cfg->slm_k, logits_out == nullptr))) return r;
     if (n_req > m->pinned_out_cap) {
         if (m->pinned_out) cudaFreeHost(m->pinned_out);
@@ -2087,25 +2077,22 @@ static int syn_verify_batch_sampled_impl(syn_model* m, syn_kv* kv, int32_t n_req
     CU_OK(cudaMemcpyAsync(w.slm_prob, slm_probs, (size_t)p->T * cfg->slm_k * 4, cudaMemcpyHostToDevice, st));
     CU_OK(cudaMemcpyAsync(w.rand_accept, rand_accept, (size_t)p->T * 4, cudaMemcpyHostToDevice, st));
     CU_OK(cudaMemcpyAsync(w.rand_sample, rand_sample, (size_t)n_req * 4, cudaMemcpyHostToDevice, st));
-    if ((r = run_step(m, kv, p, m->acc_dev, m->corr_dev, nullptr, logits, st, w.warp_max))) return r;
+    int *const po = m->pinned_out, *const po_corr = po + m->pinned_out_cap, *const po_status = po + 2 * m->pinned_out_cap;
+    if ((r = run_step(m, kv, p, po, po_corr, nullptr, logits, st, w.warp_max, po_status))) return r;
     // the greedy results of the step are replaced by the sampled ones
     if ((r = sample_stage(m, st, logits, p->T, (int)m->desc.vocab, n_req, p->d<int>(p->o_tokens), p->d<int>(p->o_offsets),
                           p->d<int>(p->o_uncached), *cfg, w.topk_id, w.topk_logit, w.slm_id, w.slm_prob, w.rand_accept,
-                          w.rand_sample, m->acc_dev, m->corr_dev, w.warp_max, m->v_rows / 32)))
+                          w.rand_sample, po, po_corr, w.warp_max, m->v_rows / 32)))
         return r;
-    int* po = m->pinned_out;
-    CU_OK(cudaMemcpyAsync(po, m->acc_dev, (size_t)n_req * 4, cudaMemcpyDeviceToHost, st));
-    CU_OK(cudaMemcpyAsync(po + m->pinned_out_cap, m->corr_dev, (size_t)n_req * 4, cudaMemcpyDeviceToHost, st));
-    CU_OK(cudaMemcpyAsync(po + 2 * m->pinned_out_cap, m->status_dev, 4, cudaMemcpyDeviceToHost, st));
     CU_OK(cudaStreamSynchronize(st));
-    if (po[2 * m->pinned_out_cap]) {
+    if (*po_status) {
         cudaMemset(m->status_dev, 0, 4);
         if (m->group_count) cudaMemset(m->group_count, 0, (size_t)m->part_cap * 4);
         if (m->fix_flag) cudaMemset(m->fix_flag, 0, (size_t)GEMM_FLAG_INTS * m->n_sm * 4);
         return SYN_E_DEVICE_TIMEOUT;
     }
     memcpy(accept_len, po, (size_t)n_req * 4);
-    memcpy(correction_token, po + m->pinned_out_cap, (size_t)n_req * 4);
+    memcpy(correction_token, po_corr, (size_t)n_req * 4);
     return SYN_OK;
 }
 
