@@ -123,12 +123,22 @@ prep_kernel(const bf16* __restrict__ embed, const int* __restrict__ tokens, cons
     }
 }
 
+// The lm_head's operand of the rows that verification looks at, side by side (one block a row).
+__global__ void __launch_bounds__(256)
+judging_rows_kernel(const op16* xg, const float* ssq, const int* __restrict__ rows, op16* xj, float* ssqj, int d) {
+    pdl_launch_dependents();
+    const size_t from = (size_t)rows[blockIdx.x], to = blockIdx.x;   // (the plan is older than the step)
+    pdl_wait();
+    for (int i = threadIdx.x * 8; i < d; i += blockDim.x * 8) *reinterpret_cast<uint4*>(xj + to * d + i) = *reinterpret_cast<const uint4*>(xg + from * d + i);
+    for (int i = threadIdx.x; i < d >> 5; i += blockDim.x) ssqj[to * (d >> 5) + i] = ssq[from * (d >> 5) + i];
+}
+
 // Greedy verification (paper Sec. 3.1 "draft & verify", Sec. 4.5): one thread per request.  The blocking calls have the results and
 // the kernels' status written straight to pinned host memory (three copies behind the kernel took 5 us).
 __global__ void verify_kernel(const unsigned long long* __restrict__ best, const int* __restrict__ tokens,
                               const int* __restrict__ offsets, const int* __restrict__ n_uncached, int n_req,
                               int* __restrict__ accept_len, int* __restrict__ correction, int* __restrict__ top1_out,
-                              const int* status, int* status_out) {
+                              const int* __restrict__ first_row, const int* status, int* status_out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (i == 0 && status_out) *status_out = *status;
@@ -136,10 +146,11 @@ __global__ void verify_kernel(const unsigned long long* __restrict__ best, const
     const int b = offsets[i], n = offsets[i + 1] - b, u = n_uncached[i];
     if (top1_out)
         for (int j = 0; j < n; ++j) top1_out[b + j] = (int)(0xFFFFFFFFu - (uint32_t)(best[b + j] & 0xFFFFFFFFull));
+    const unsigned long long* mine = best + (first_row ? first_row[i] : b + u - 1);   // the row that judges the first draft
     int a = 0;
-    while (a < n - u && (int)(0xFFFFFFFFu - (uint32_t)(best[b + u - 1 + a] & 0xFFFFFFFFull)) == tokens[b + u + a]) ++a;
+    while (a < n - u && (int)(0xFFFFFFFFu - (uint32_t)(mine[a] & 0xFFFFFFFFull)) == tokens[b + u + a]) ++a;
     accept_len[i] = a;
-    correction[i] = (int)(0xFFFFFFFFu - (uint32_t)(best[b + u - 1 + a] & 0xFFFFFFFFull));
+    correction[i] = (int)(0xFFFFFFFFu - (uint32_t)(mine[a] & 0xFFFFFFFFull));
 }
 
 // Copy K/V of logical positions between a dense bf16 [n_pos][Hkv][hd] buffer and the paged pool (half precision).  The
@@ -283,7 +294,9 @@ struct syn_model {
          *q = nullptr, *attn = nullptr, *act = nullptr;
     float2* rope = nullptr;
     unsigned long long* best = nullptr;
-    XMaps tm_xn, tm_attn, tm_act;
+    op16* xj = nullptr;      // operand and sums of the rows that verification looks at, where the lm_head runs over those alone
+    float* ssqj = nullptr;
+    XMaps tm_xn, tm_attn, tm_act, tm_xj;
     CUtensorMap tm_q, tm_q4;
     float* fix_part = nullptr;      // stored accumulators of K-split remainder tiles (one slot per SM)
     int* fix_flag = nullptr;        // their arrival / release counters, [GEMM_FLAG_INTS * n_sm], zero between launches
@@ -354,6 +367,8 @@ struct syn_plan {
     size_t cap = 0, used = 0;
     // offsets into the buffer
     size_t o_tokens, o_pos, o_slot, o_offsets, o_uncached, o_tables, o_items, o_cta, o_groups;
+    size_t o_row, o_first;   // the judging rows, and where a request's begin among them
+    int n_judging = 0;       // rows whose argmax verification looks at: a request's from its last uncached token on
     // the cache the page ids and slots were validated against
     const syn_kv* kv = nullptr;
     const void* kv_pool = nullptr;
@@ -364,7 +379,8 @@ struct syn_plan {
 
 static void free_workspace(syn_model* m) {
     cudaFree(m->x); cudaFree(m->ssq); cudaFree(m->xn); cudaFree(m->q); cudaFree(m->attn); cudaFree(m->act);
-    cudaFree(m->rope); cudaFree(m->best);
+    cudaFree(m->rope); cudaFree(m->best); cudaFree(m->xj); cudaFree(m->ssqj);
+    m->xj = nullptr; m->ssqj = nullptr;
     m->x = m->ssq = nullptr; m->xn = m->q = m->attn = m->act = nullptr; m->rope = nullptr; m->best = nullptr;
     m->t_cap = 0;
 }
@@ -383,6 +399,9 @@ static int ensure_workspace(syn_model* m, int T, int n_parts) {
         CU_OK(cudaMalloc(&m->act, (size_t)cap * m->f_pad * 2));
         CU_OK(cudaMalloc(&m->rope, (size_t)cap * (c.head_dim / 2) * 8));
         CU_OK(cudaMalloc(&m->best, (size_t)cap * 8));
+        CU_OK(cudaMalloc(&m->xj, (size_t)(cap / 2) * c.d_model * 2));
+        CU_OK(cudaMalloc(&m->ssqj, (size_t)(cap / 2) * (c.d_model / 32) * 4));
+        CU_OK(cudaMemset(m->xj, 0, (size_t)(cap / 2) * c.d_model * 2));
         CU_OK(cudaMemset(m->xn, 0, (size_t)cap * c.d_model * 2));
         CU_OK(cudaMemset(m->q, 0, (size_t)cap * q_dim * 2));
         CU_OK(cudaMemset(m->attn, 0, (size_t)cap * q_dim * 2));
@@ -390,6 +409,7 @@ static int ensure_workspace(syn_model* m, int T, int n_parts) {
         m->t_cap = cap;
         int r;
         if ((r = make_xmaps(&m->tm_xn, m->xn, cap, c.d_model))) return r;
+        if ((r = make_xmaps(&m->tm_xj, m->xj, cap / 2, c.d_model))) return r;
         if ((r = make_xmaps(&m->tm_attn, m->attn, cap, q_dim))) return r;
         if ((r = make_xmaps(&m->tm_act, m->act, cap, m->f_pad))) return r;
         // Q tile of the attention kernel: [token][128-byte line][64]; box = min(16, 64/G) tokens x (G * hd/64) lines
@@ -465,7 +485,7 @@ static cudaError_t set_kernel_attributes() {
         kernel_smem(attn_kernel<128>, AttnSmem<128>::TOTAL), kernel_smem(attn_kernel<64>, AttnSmem<64>::TOTAL),
         kernel_smem(attn2_kernel<128>, Attn2Smem<128>::TOTAL), kernel_smem(attn2_kernel<64>, Attn2Smem<64>::TOTAL),
         kernel_smem(attn_thin_kernel<128>, AttnThinSmem<128>::TOTAL), kernel_smem(attn_thin_kernel<64>, AttnThinSmem<64>::TOTAL),
-        kernel_smem(prep_kernel, 0), kernel_smem(verify_kernel, 0), kernel_smem(topk_rows_kernel, 0), kernel_smem(sample_verify_kernel, 0)};
+        kernel_smem(prep_kernel, 0), kernel_smem(verify_kernel, 0), kernel_smem(judging_rows_kernel, 0), kernel_smem(topk_rows_kernel, 0), kernel_smem(sample_verify_kernel, 0)};
     for (cudaError_t e : all)
         if (e != cudaSuccess) return e;
     return cudaSuccess;
@@ -1236,6 +1256,8 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     p->o_offsets = take((size_t)(n_req + 1) * 4);
     p->o_uncached = take((size_t)n_req * 4);
     p->o_tables = take((size_t)n_req * max_pages * 4);
+    p->o_row = take((size_t)T * 4);
+    p->o_first = take((size_t)n_req * 4);
     p->o_items = take((size_t)n_items * sizeof(AttnItem));
     p->o_cta = take((size_t)(n_cta + 1) * 4);
     p->o_groups = take(std::max<size_t>(1, hp.groups.size()) * sizeof(MergeGroup));
@@ -1254,7 +1276,13 @@ static int plan_build(syn_plan* p, syn_model* m, syn_kv* kv, int32_t n_req, cons
     memcpy(p->h<int>(p->o_pos), hp.pos.data(), (size_t)T * 4);
     memcpy(p->h<int>(p->o_slot), hp.slot.data(), (size_t)T * 4);
     memcpy(p->h<int>(p->o_offsets), chunk_offsets, (size_t)(n_req + 1) * 4);
-    for (int i = 0; i < n_req; ++i) p->h<int>(p->o_uncached)[i] = n_uncached ? n_uncached[i] : 1;
+    p->n_judging = 0;
+    for (int i = 0; i < n_req; ++i) {
+        const int u = n_uncached ? n_uncached[i] : 1;
+        p->h<int>(p->o_uncached)[i] = u;
+        p->h<int>(p->o_first)[i] = p->n_judging;
+        for (int t = chunk_offsets[i] + u - 1; t < chunk_offsets[i + 1]; ++t) p->h<int>(p->o_row)[p->n_judging++] = t;
+    }
     memcpy(p->h<int>(p->o_tables), page_tables, (size_t)n_req * max_pages * 4);
     memcpy(p->h<AttnItem>(p->o_items), hp.items.data(), (size_t)n_items * sizeof(AttnItem));
     memcpy(p->h<int>(p->o_cta), hp.cta_begin.data(), (size_t)(n_cta + 1) * 4);
@@ -1847,6 +1875,10 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     // (the projections' plans, some 6 us each, are made in the first layer, while the kernels before run)
     ProjPlan pl_qkv, pl_o, pl_gu, pl_d;
     int r;
+    // Where nobody asked for logits or argmaxes, the lm_head runs over the rows that verification looks at, if they are at most
+    // half of more than 128 (up to there its time is that of its weights: 1B shape 37 us at 128 tokens, 105 at 768; a
+    // prefill iteration of 768 tokens of 24 requests needs 24 rows).
+    const bool judging_only = !logits_out && !top1_dev && T > 128 && 2 * p->n_judging <= T;
     for (uint32_t l = 0; l < c.n_layers; ++l) {
         EpiParams e = scaled;
         e.mode = EPI_QKV; e.N = m->qkv_rows;
@@ -1873,16 +1905,25 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
         if ((r = launch_proj(m, 6, m->n_sm, m->status_dev, m->wd[l], &m->tm_wd[l], d, m->f_pad, m->tm_act, e, st, m->fix_part, m->fix_flag, pl_d)))
             return r;
     }
+    const int T_lm = judging_only ? p->n_judging : T;
     EpiParams e = scaled;
+    if (judging_only) {
+        ProfScope prof(m, 8, st);
+        if (launch_pdl(judging_rows_kernel, dim3(T_lm), dim3(256), 0, st, m->xn, m->ssq, p->d<int>(p->o_row), m->xj, m->ssqj, d) != cudaSuccess)
+            return SYN_E_CUDA;
+        e.T = T_lm;
+        e.ssq_in = m->ssqj;
+    }
     e.mode = EPI_LMHEAD; e.N = m->v_rows; e.vocab = c.vocab; e.logits = logits_out; e.best = m->best;
     e.warp_max = warp_max; e.n_warp_max = m->v_rows / 32;
-    const ProjPlan pl_lm = proj_plan(T, m->v_rows, d, m->n_sm, EPI_LMHEAD);
-    if ((r = launch_proj(m, 7, m->n_sm, m->status_dev, m->lm_head, &m->tm_lm_head, m->v_rows, d, m->tm_xn, e, st, m->fix_part, m->fix_flag, pl_lm)))
+    const ProjPlan pl_lm = proj_plan(T_lm, m->v_rows, d, m->n_sm, EPI_LMHEAD);
+    if ((r = launch_proj(m, 7, m->n_sm, m->status_dev, m->lm_head, &m->tm_lm_head, m->v_rows, d, judging_only ? m->tm_xj : m->tm_xn, e, st, m->fix_part, m->fix_flag, pl_lm)))
         return r;
     {
         ProfScope prof(m, 8, st);
         if (launch_pdl(verify_kernel, dim3((p->n_req + 127) / 128), dim3(128), 0, st, m->best, tokens, p->d<int>(p->o_offsets),
-                       p->d<int>(p->o_uncached), p->n_req, acc_dev, corr_dev, top1_dev, m->status_dev, status_out) != cudaSuccess)
+                       p->d<int>(p->o_uncached), p->n_req, acc_dev, corr_dev, top1_dev, judging_only ? p->d<int>(p->o_first) : nullptr,
+                       m->status_dev, status_out) != cudaSuccess)
             return SYN_E_CUDA;
     }
     if (m->profile) {
