@@ -18,8 +18,9 @@
 // 1 611 -> 1 340 us; 8B shape, 40 tokens 4 600 -> 3 820 us (the weights alone take 2 325 us at the copy rate), 119 tokens
 // 6 100 -> 5 760 us.  The 8B o projection (33.5 MB) at 40 tokens: 26.1 -> 15.5 us between events in the step.  What bounds
 // it: HBM while it streams (4.5 - 5 TB/s in a launch of its own), and about 3 us per launch that depend on the
-// predecessor (its results visible, token operand, exchange, epilogue).  Tried and dropped: 256 CTAs instead of
-// 148 and fewer (14 % slower at the 8B shape), asking L2 for the next projection's weights (1 to 5 % slower: the
+// predecessor (its results visible, token operand, exchange, epilogue).  With the epilogues that load ahead and the shorter
+// attention merges those steps take 759, 1 240, 3 740 and 5 770 us.  Tried and dropped: 256 CTAs instead of 148 and fewer with one
+// token tile (14 % slower at the 8B shape), asking L2 for the next projection's weights (1 to 5 % slower: the
 // requests compete with the loads that the step waits for), two cluster barriers around plain remote
 // stores instead of the counted asynchronous ones.
 #pragma once
