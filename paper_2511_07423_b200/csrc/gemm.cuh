@@ -20,7 +20,7 @@
 //                 its own columns: a reduce-scatter, after which all S CTAs share the epilogue.
 // Every CTA starts its k loop at a different k-block, so the CTAs that share a token tile do not
 // ask L2 for the same lines at the same moment.  Accumulation is tcgen05.mma into TMEM, read back
-// with tcgen05.ld by sixteen epilogue warps; a thread then holds one output feature for sixteen
+// with tcgen05.ld by twelve or sixteen epilogue warps; a thread then holds one output feature for sixteen
 // tokens; a warp turns its 32 x 16 block round in shared memory, so that every lane reads and writes
 // 16-byte pieces of token-major rows:
 //   EPI_QKV    : RMSNorm scale, RoPE on q and k (the partner dimension sits 16 lanes away), q store,
