@@ -29,8 +29,8 @@ struct AttnThinSmem {
     static constexpr int PAGES = HD == 128 ? 2 : 4;                // per stage
     static constexpr int PAGE_BYTES = 2 * 16 * HD * 2;             // K and V of one page, one head
     static constexpr int STAGE_BYTES = PAGES * PAGE_BYTES;         // 16 KB
-    // two slots of O[16][HD] + (m, l)[16], or a weight for every part of the 64 rows and one over their sums
-    static constexpr int WEIGHT_BYTES = (ATTN_THIN_MAX_PARTS + 1) * 64 * 4, SLOT_BYTES = 2 * 16 * (HD + 4) * 4;
+    // two slots of O[16][HD] + (m, l)[16], or a weight for every part of the 64 rows
+    static constexpr int WEIGHT_BYTES = ATTN_THIN_MAX_PARTS * 64 * 4, SLOT_BYTES = 2 * 16 * (HD + 4) * 4;
     static constexpr int MERGE_BYTES = WEIGHT_BYTES > SLOT_BYTES ? WEIGHT_BYTES : SLOT_BYTES;
     static constexpr int TOTAL = 1024 + ATTN_THIN_STAGES * STAGE_BYTES + MERGE_BYTES + 512;
     static_assert(2 * (TOTAL + 1024) <= 233472, "two CTAs per SM");
@@ -252,8 +252,7 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                 // past the last part repeat it: left out under a condition they cost 600 bytes of spills in the stage loop.)
                 if (threadIdx.x == 0) p.group_count[item.grp] = 0;   // ready for the next launch
                 const int np = min(n_parts, ATTN_THIN_MAX_PARTS);
-                float* w_s = merge;                                   // [part][64]
-                float* inv_s = merge + ATTN_THIN_MAX_PARTS * 64;      // [64]
+                float* w_s = merge;   // [part][64]
                 constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5, CAP = 64;   // CAP: rows of a part
                 const int n_vec = rows * VR, by_g = 4096 / G + 1;   // row / G = row * by_g >> 12 for rows up to 64
                 const float4* src = reinterpret_cast<const float4*>(p.part_o) + (size_t)part0 * (CAP * VR);
@@ -282,18 +281,29 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                     }
                     mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
                     const float bs = mx == -INFINITY ? 0.f : mx;
+                    // the sum goes through the parts in their order, whoever holds them (a part past the last adds zero), and the
+                    // weights are divided by it before they meet the outputs: both are part of what a step's logits are, bit for bit
                     for (int k0 = 0; k0 < np; k0 += 16) {
                         if (np > 16) pairs(k0);
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             if (k0 + 2 * k >= np) break;
-                            const float w = ex2_approx(t[k].x - bs);
-                            lsum += t[k].y * w;
+                            const float w = ex2_approx(t[k].x - bs), w_of = __shfl_xor_sync(0xFFFFFFFFu, w, 1);
+                            const float l_of = __shfl_xor_sync(0xFFFFFFFFu, t[k].y, 1);
+                            lsum += (odd ? l_of : t[k].y) * (odd ? w_of : w);
+                            lsum += (odd ? t[k].y : l_of) * (odd ? w : w_of);
                             w_s[(k0 + odd + 2 * k) * 64 + row] = w;
                         }
                     }
-                    lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, 1);
-                    if (!odd) inv_s[row] = lsum > 0.f ? 1.f / lsum : 0.f;
+                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+                    for (int k0 = odd; k0 < np; k0 += 8) {   // (its own entries)
+                        float w[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) w[k] = w_s[min(k0 + 2 * k, ATTN_THIN_MAX_PARTS - 1) * 64 + row] * inv;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (k0 + 2 * k < np) w_s[(k0 + 2 * k) * 64 + row] = w[k];
+                    }
                 }
                 attn_thin_bar();
                 op16* const out0 = p.out + (size_t)item.q_tok * p.q_dim + item.kvh * G * HD;
@@ -316,11 +326,9 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
 #pragma unroll
                     for (int i = 0; i < NU; ++i) {
                         const int u = u0 + i * 128, row = u / VR, j = row * by_g >> 12, gq = row - j * G;
-                        if (u < n_vec) {
-                            const float inv = inv_s[row];
+                        if (u < n_vec)
                             *reinterpret_cast<uint2*>(out0 + (size_t)j * p.q_dim + gq * HD + 4 * (u % VR)) =
-                                make_uint2(pack_op(acc[i].x * inv, acc[i].y * inv), pack_op(acc[i].z * inv, acc[i].w * inv));
-                        }
+                                make_uint2(pack_op(acc[i].x, acc[i].y), pack_op(acc[i].z, acc[i].w));
                     }
                 }
                 attn_thin_bar();   // the weights' area is the next item's merge slots

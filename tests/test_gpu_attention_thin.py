@@ -64,3 +64,56 @@ def test_a_context_written_by_another_request_of_the_batch():
             assert torch.equal(got[32:], want)
     finally:
         syn.debug_set_attention(0)
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv,ctx,chunk", [
+    (128, 8, 4, [2500], [16]),          # 32 parts and fewer of 32 rows
+    (64, 32, 8, [3000], [16]),          # 64 rows
+    (128, 16, 8, [1400, 700], [9, 5]),  # fewer than 17 parts
+])
+def test_parts_are_merged_in_their_order(hd, Hq, Hkv, ctx, chunk):
+    """Keys of zero make every weight 1 and every sum of a part a whole number, so the merge alone decides the last bits: the
+    weight of a part is divided by the row's sum, then the parts are added in order with fused multiply-adds."""
+    import numpy as np
+    import paper_2511_07423_b200 as syn
+    from workloads.configs import ModelShape
+    shape, seed = ModelShape("merge", 1, 256, Hq, Hkv, hd, 256, 512), 5
+    batch = base._batch(ctx, chunk, seed=seed)
+    model = syn.Model(shape, *to_cuda(*cpu_model(shape, seed)))
+    kv = syn.KVCache(model, batch.n_pages)
+    g = torch.Generator().manual_seed(seed)
+    values = []
+    for r in range(batch.n_req):
+        n = ctx[r] + chunk[r]
+        v = torch.randint(-27, 28, (n, Hkv, hd), generator=g) + torch.where(torch.arange(n) < n // 2, 100, -100).view(n, 1, 1)
+        kv.import_kv(0, batch.page_tables[r], 0, torch.zeros(n, Hkv, hd, dtype=torch.bfloat16, device="cuda"), v.to(torch.bfloat16).cuda())
+        values.append(v.numpy().astype(np.float64).cumsum(0))
+    T = batch.n_tokens
+    q = torch.randn(T, shape.q_dim, generator=g).to(torch.float16)
+    args = (torch.zeros(T, dtype=torch.int32), batch.chunk_offsets, batch.page_tables, batch.ctx_lens)
+    syn.debug_set_attention(3)
+    try:
+        out = syn.Plan(kv, *args).attention(0, q.cuda())
+        work = syn.plan_work_host(shape, batch.n_pages, *args, n_sm=torch.cuda.get_device_properties(0).multi_processor_count)
+    finally:
+        syn.debug_set_attention(0)
+    torch.cuda.synchronize()
+    assert model.status() == 0 and work["attention"] == 3
+    groups = {}
+    for q_tok, nj, kvh, req, k0, k1, pos0, part, grp, _ in work["items"].tolist():
+        if part >= 0:
+            groups.setdefault(grp, []).append((part, q_tok, nj, kvh, req, k0, k1, pos0))
+    assert max(map(len, groups.values())) > 2
+    got = out.cpu().view(T, Hkv, Hq // Hkv, hd)
+    for items in groups.values():
+        for j in range(items[0][2]):
+            _, q_tok, _, kvh, req, _, _, pos0 = items[0]
+            seen = [(k0, min(k1, pos0 + j + 1)) for _, _, _, _, _, k0, k1, _ in sorted(items)]
+            inv = np.float32(1) / np.float32(pos0 + j + 1)
+            acc = np.zeros(hd, dtype=np.float32)
+            for k0, k1 in seen:
+                if k1 > k0:   # (in 64 bits the product is exact, so this rounds once, like a fused multiply-add)
+                    s = values[req][k1 - 1, kvh] - (values[req][k0 - 1, kvh] if k0 else 0)
+                    acc = (s * np.float64(inv) + acc).astype(np.float32)
+            want = torch.from_numpy(acc).to(torch.float16).expand(Hq // Hkv, hd)
+            assert torch.equal(got[q_tok + j, kvh], want), (req, kvh, j)
