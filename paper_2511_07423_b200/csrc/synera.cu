@@ -1648,7 +1648,7 @@ static int gemm2_plan(int T, int packed_rows, int K, int n_sm, int mode, int for
 constexpr int THIN_MAX_TOKENS = 512, THIN_MAX_TOKENS_QKV = 1024;
 
 // Launch shape of a projection on the thin kernel (gemm_thin.cuh): at most one CTA per SM where K is shared, so that the
-// other half of every SM is free for the next kernel; at least two k-blocks each.
+// other half of every SM is free for the next kernel, but for the case below; at least two k-blocks each.
 static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
     memset(&g, 0, sizeof(g));
     g.num_kb = (K + 63) / 64;
@@ -1662,7 +1662,11 @@ static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
     // 36 bytes a cycle of the 63 that an SM can take), K leaves every part 16 k-blocks, and clusters of four fill the slots
     // (larger clusters and those of three or six do not all fit at a time: 1B down at 320 tokens 29.5 < 35.5 us with six).  Event
     // times, one CTA to an SM and two: 1B down at 448 tokens 33.3 > 29.2 us, at 512 34.6 > 31.4; 8B o at 160 tokens 23.0 > 21.0.
-    if (g.n_tt >= 2 && 4 * items <= 2 * n_sm && 4 * items >= 3 * n_sm / 2 && g.num_kb >= 64) g.splits = 4;
+    // By items, o and down (128 k-blocks) of models of that many tiles, 144 to 256 tokens (three or four token tiles: 384 and 512):
+    // 56 items 25.0 > 23.5 and 37.3 > 31.5, 60 36.5 > 31.4 (down), 68 24.8 > 22.9 and 37.3 > 29.1; from 72 on a last cluster of
+    // four waits for a whole round of the others: 72 29.2 < 34.2 and 38.6 < 44.6, 74 27.1 < 36.2 and 39.4 < 46.2; steps of 69 and 70
+    // items are 1.04 to 1.14 times as fast, so the line is at 70 of the 74 that two CTAs to an SM would make.
+    if (g.n_tt >= 2 && 4 * items <= 2 * n_sm - 16 && 4 * items >= 3 * n_sm / 2 && g.num_kb >= 64) g.splits = 4;
     const int recv = g.splits > 1 ? thin_recv_bytes(g.TN, g.splits) : 0;
     g.recv_own = recv > 0 && recv <= THIN_RECV_OWN_MAX;
     g.n_stages = thin_stages(g.TN, g.recv_own ? recv : 0);

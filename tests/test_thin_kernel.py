@@ -71,8 +71,11 @@ def test_product_matches_oracle(T, N, K):
 
 
 def test_two_ctas_to_an_sm():
-    """Several token tiles, 38 to 74 items and a K of 64 k-blocks and more: parts in clusters of four, 16 k-blocks or more each."""
-    for T, N, K, splits in ((448, 2048, 8192, 4), (512, 2048, 8192, 4), (160, 4096, 4096, 4), (256, 4096, 4096, 4),
+    """Several token tiles, 56 to 70 items and a K of 64 k-blocks and more: parts in clusters of four, 16 k-blocks or more each.
+    Clusters of four beyond 70 do not all run at a time."""
+    for T, N, K, splits in ((600, 1408, 4096, 2), (160, 3584, 4096, 4), (272, 2944, 4096, 4), (160, 4480, 4096, 4), (160, 4608, 4096, 2),   # 55, 56, 69, 70, 72
+                            (400, 2304, 8192, 2), (256, 4736, 8192, 2), (320, 3200, 4096, 1), (160, 3584, 4032, 2),   # 72, 74, 75; 63 k-blocks
+                            (448, 2048, 8192, 4), (512, 2048, 8192, 4), (160, 4096, 4096, 4), (256, 4096, 4096, 4),
                             (320, 2048, 8192, 3), (448, 2048, 2048, 2), (128, 4096, 4096, 4), (160, 6144, 4096, 1), (1024, 3072, 2048, 1)):
         p = syn.thin_plan_host(T, N, K)
         assert p["splits"] == splits, (T, N, K, p)
