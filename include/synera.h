@@ -179,10 +179,10 @@ typedef struct {
     int64_t weight_bytes;          /* bf16 bytes of all projections streamed once per step  */
     int64_t kv_read_bytes;         /* sum over requests of (ctx+n) * 2*Hkv*hd*2 * n_layers   */
     int64_t kv_write_bytes;        /* T * 2*Hkv*hd*2 * n_layers                             */
-    double dense_flops;            /* 2 * T * projection parameters                         */
+    double dense_flops;            /* 2 * rows * parameters of every projection: T rows, in the lm_head of a step without logits and argmaxes perhaps fewer (syn_verify_run) */
     double attn_flops;             /* 4 * Hq*hd * n_layers * sum over tokens of keys seen    */
     int32_t attn_items, attn_split_items; /* attention work items per layer / those that are partial */
-    int32_t kernel_launches;       /* kernels launched by one syn_verify_run                */
+    int32_t kernel_launches;       /* kernels launched by one syn_verify_run: 1 + 5 n_layers + 2, one more where the lm_head runs over fewer rows */
     int32_t attn_rows;             /* row tile of the attention kernel the batch was planned for: 64 (warp-level MMAs) or 128 (tcgen05); the kernel: syn_plan_attention */
     int64_t h2d_bytes;             /* batch description uploaded per step by syn_verify_batch */
     double t_gpu_ms;               /* device time of the step, first kernel to last (CUDA events); 0 unless profiling is on */
@@ -191,7 +191,8 @@ typedef struct {
 /* The last step launched on this model by syn_verify_batch, syn_verify_batch_sampled or syn_verify_run
  * (the paper's cloud runtime reports per-iteration execution time, Sec. 6.7).  With syn_set_profile on,
  * t_gpu_ms is filled (the call then waits for that step to finish) and, for the blocking calls,
- * t_wall_ms.  SYN_E_INVALID_ARG before the first step.  syn_plan_stats: the counters of a plan. */
+ * t_wall_ms.  SYN_E_INVALID_ARG before the first step.  syn_plan_stats: the counters of a plan, that is of its step with
+ * logits or argmaxes asked for. */
 int syn_last_step_stats(syn_model *m, syn_step_stats *out);
 int syn_plan_stats(const syn_plan *p, syn_step_stats *out);
 /* The attention kernel a plan was laid out for, numbered as in syn_debug_set_attention: 1, 2 or 3 (attn_rows is 64 for 1
@@ -234,8 +235,8 @@ int syn_plan_work_host(const syn_model_desc *desc, uint32_t n_pages, uint32_t pa
  * adds up the elapsed time and launch count of each class since the last call, and clears them.
  * Classes: 0 prep, 1 qkv GEMM, 2 attention, 3 attention merge, 4 o GEMM, 5 gate/up GEMM,
  * 6 down GEMM, 7 lm_head GEMM, 8 verify (greedy compare, and the sampling stage of
- * syn_verify_batch_sampled), 9 unused (the residual update and the norm statistic are part of the
- * o and down GEMMs).  ms, launches: HOST arrays of SYN_N_KERNEL_CLASSES. */
+ * syn_verify_batch_sampled), 9 the gather of the rows that the lm_head runs over where those are not all (the residual update
+ * and the norm statistic are part of the o and down GEMMs).  ms, launches: HOST arrays of SYN_N_KERNEL_CLASSES. */
 #define SYN_N_KERNEL_CLASSES 10
 int syn_set_profile(syn_model *m, int on);
 int syn_get_profile(syn_model *m, double *ms, int32_t *launches);

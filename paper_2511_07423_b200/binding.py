@@ -50,7 +50,7 @@ class StepStats(C.Structure):
                 ("t_gpu_ms", C.c_double), ("t_wall_ms", C.c_double)]
 
 KERNEL_CLASSES = ("prep", "qkv_gemm", "attention", "attention_merge", "o_gemm", "gate_up_gemm", "down_gemm",
-                  "lm_head_gemm", "verify", "unused")
+                  "lm_head_gemm", "verify", "judging_rows")
 
 
 _LIB: Optional[C.CDLL] = None

@@ -1852,7 +1852,14 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     if (T > m->t_cap || p->n_parts > m->part_cap) return SYN_E_INVALID_ARG;
     const int* tokens = p->d<int>(p->o_tokens);
     const float inv_d = 1.0f / (float)d;
+    // Where nobody asked for logits or argmaxes, the lm_head runs over the rows that verification looks at, if they are at most
+    // half of more than 128 (up to there its time is that of its weights: 1B shape 37 us at 128 tokens, 105 at 768; a
+    // prefill iteration of 768 tokens of 24 requests needs 24 rows).
+    const bool judging_only = !logits_out && !top1_dev && T > 128 && 2 * p->n_judging <= T;
+    const int T_lm = judging_only ? p->n_judging : T;
     m->last_stats = p->stats;
+    m->last_stats.dense_flops -= 2.0 * (T - T_lm) * (double)d * c.vocab;
+    m->last_stats.kernel_launches += judging_only;
     m->have_last = true;
     m->step_timed = false;
     m->last_wall_ms = 0.0;
@@ -1879,10 +1886,6 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     // (the projections' plans, some 6 us each, are made in the first layer, while the kernels before run)
     ProjPlan pl_qkv, pl_o, pl_gu, pl_d;
     int r;
-    // Where nobody asked for logits or argmaxes, the lm_head runs over the rows that verification looks at, if they are at most
-    // half of more than 128 (up to there its time is that of its weights: 1B shape 37 us at 128 tokens, 105 at 768; a
-    // prefill iteration of 768 tokens of 24 requests needs 24 rows).
-    const bool judging_only = !logits_out && !top1_dev && T > 128 && 2 * p->n_judging <= T;
     for (uint32_t l = 0; l < c.n_layers; ++l) {
         EpiParams e = scaled;
         e.mode = EPI_QKV; e.N = m->qkv_rows;
@@ -1909,10 +1912,9 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
         if ((r = launch_proj(m, 6, m->n_sm, m->status_dev, m->wd[l], &m->tm_wd[l], d, m->f_pad, m->tm_act, e, st, m->fix_part, m->fix_flag, pl_d)))
             return r;
     }
-    const int T_lm = judging_only ? p->n_judging : T;
     EpiParams e = scaled;
     if (judging_only) {
-        ProfScope prof(m, 8, st);
+        ProfScope prof(m, 9, st);
         if (launch_pdl(judging_rows_kernel, dim3(T_lm), dim3(256), 0, st, m->xn, m->ssq, p->d<int>(p->o_row), m->xj, m->ssqj, d) != cudaSuccess)
             return SYN_E_CUDA;
         e.T = T_lm;
