@@ -160,6 +160,10 @@ int syn_verify_batch(syn_model *m, syn_kv *kv, int32_t n_req, const int64_t *req
  * top1_dev is NULL or DEVICE int32 [T] (argmax per chunk position).  It does not synchronise:
  * call syn_model_status after synchronising the stream to learn of a device-side timeout.
  * A plan may be run any number of times (each run rewrites the same KV slots).
+ * With neither top1_dev nor logits_out, and more than 128 tokens of which verification looks at the argmax of at most half
+ * (a request's from its last uncached token on), the lm_head runs over those rows alone; likewise in syn_verify_batch without
+ * logits_out.  The other number of rows may take another kernel or another split of K, whose fp32 sums differ in their last
+ * bits: two tokens whose logits differ by less than that may then be decided the other way than in a call that asks for logits.
  * A plan belongs to the cache it was created with: its page ids and KV slots were checked against
  * that cache's size, so syn_verify_run, syn_op_attention and syn_op_attention_static return
  * SYN_E_INVALID_ARG, before any launch, when they are given another cache (or that cache freed and

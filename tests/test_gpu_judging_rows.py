@@ -1,10 +1,12 @@
 """Calls that ask for no logits run the lm_head over the rows that verification looks at only: the same results as greedy
 verification of the logits that the same batch gives where they are asked for."""
+import dataclasses
+
 import pytest
 import torch
 
 from workloads import gen
-from workloads.configs import MINI_1B, MINI_8B, Workload
+from workloads.configs import MINI_1B, MINI_8B, SHAPE_1B, Workload
 
 import test_gpu_verify as base
 
@@ -70,3 +72,40 @@ def test_the_step_counts_what_it_ran(chunk, unc, fewer):
         assert st.dense_flops == of_plan.dense_flops - 2.0 * (T - n) * shape.d_model * shape.vocab
         assert bench.lm_head_rows(of_plan, st, shape.d_model, shape.vocab) == n
     assert model.status() == 0
+
+
+@pytest.mark.parametrize("n_req,unc", [(5, 28), (20, 31)])
+def test_full_width_tokens_differ_at_rounding_level_ties_only(n_req, unc):
+    """The widths of the 1B shape: the lm_head over 25 of 160 and 40 of 640 rows against the logits of the same batch.  A row's
+    sums may be taken in another order, so a token whose logit is within the bound of fp32 sums of the largest is as good."""
+    import paper_2511_07423_b200 as syn
+    from paper_2511_07423_b200 import synthetic
+    shape = dataclasses.replace(SHAPE_1B, n_layers=2)
+    chunk = [32] * n_req
+    batch = gen.gen_batch(Workload("judging", shape, 3, n_req, ("list", (24,) * n_req), ("list", tuple(chunk)), 0.7))
+    model = synthetic.load_model(shape, 3)
+    kv = syn.KVCache(model, batch.n_pages)
+    synthetic.fill_cache(kv, shape, 3, batch)
+    # |error| of a sum of d exact products in any order <= d 2^-24 sum |x w| <= d 2^-24 |x| |w|, |x| = sqrt(d) after the norm; two
+    # sums of each of two logits
+    glob = gen.gen_globals(shape, 3, device="cuda")
+    d = shape.d_model
+    x_norm = d ** 0.5 * float(glob["final_norm"].float().abs().max())
+    bound = 4 * d * 2.0 ** -24 * x_norm * float(glob["lm_head"].float().norm(dim=1).max())
+    tokens = torch.randint(0, shape.vocab, (sum(chunk),), generator=torch.Generator().manual_seed(n_req), dtype=torch.int32)
+    args, unc_t = (batch.chunk_offsets, batch.page_tables, batch.ctx_lens), torch.full((n_req,), unc, dtype=torch.int32)
+    accepted = 0
+    for _ in range(4):   # with drafts that are nobody's, then with more and more of the model's own
+        _, _, logits = kv.verify_batch(tokens, *args, n_uncached=unc_t, want_logits=True)
+        acc, cor = kv.verify_batch(tokens, *args, n_uncached=unc_t)[:2]
+        assert model.status() == 0
+        for i, n in enumerate(chunk):
+            b, rows = 32 * i, logits[32 * i + unc - 1:32 * i + n]
+            near = [set(torch.nonzero(r >= r.max() - bound).flatten().tolist()) for r in rows]
+            a = int(acc[i])
+            accepted += a
+            assert all(int(tokens[b + unc + j]) in near[j] for j in range(a)) and int(cor[i]) in near[a]
+            if a < n - unc:   # the draft that was turned down is not the only token that the row allows
+                assert near[a] != {int(tokens[b + unc + a])}
+                tokens[b + unc + a] = int(cor[i])
+    assert accepted >= n_req
