@@ -23,14 +23,15 @@ constexpr int ATTN_THIN_WARPS = 4;
 constexpr int ATTN_THIN_THREADS = (ATTN_THIN_WARPS + 1) * 32;
 constexpr int ATTN_THIN_STAGES = 5;
 constexpr int ATTN_THIN_MAX_PARTS = 32;   // of one row group
+constexpr int ATTN_THIN_ROWS = 64;        // of an item's tile (AttnParams::row_cap): row stride of the parts
 
 template <int HD>
 struct AttnThinSmem {
     static constexpr int PAGES = HD == 128 ? 2 : 4;                // per stage
     static constexpr int PAGE_BYTES = 2 * 16 * HD * 2;             // K and V of one page, one head
     static constexpr int STAGE_BYTES = PAGES * PAGE_BYTES;         // 16 KB
-    // two slots of O[16][HD] + (m, l)[16], or a weight for every part of the 64 rows
-    static constexpr int WEIGHT_BYTES = ATTN_THIN_MAX_PARTS * 64 * 4, SLOT_BYTES = 2 * 16 * (HD + 4) * 4;
+    // two slots of O[16][HD] + (m, l)[16], or a weight for every part of the rows
+    static constexpr int WEIGHT_BYTES = ATTN_THIN_MAX_PARTS * ATTN_THIN_ROWS * 4, SLOT_BYTES = 2 * 16 * (HD + 4) * 4;
     static constexpr int MERGE_BYTES = WEIGHT_BYTES > SLOT_BYTES ? WEIGHT_BYTES : SLOT_BYTES;
     static constexpr int TOTAL = 1024 + ATTN_THIN_STAGES * STAGE_BYTES + MERGE_BYTES + 512;
     static_assert(2 * (TOTAL + 1024) <= 233472, "two CTAs per SM");
@@ -231,11 +232,11 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                         for (int nt = 0; nt < HD / 8; ++nt)
                             *reinterpret_cast<uint32_t*>(dst + nt * 8 + 2 * c) = pack_op(o[nt][2 * r] * inv, o[nt][2 * r + 1] * inv);
                     } else {
-                        float* dst = p.part_o + ((size_t)item.part * p.row_cap + row) * HD;
+                        float* dst = p.part_o + ((size_t)item.part * ATTN_THIN_ROWS + row) * HD;
 #pragma unroll
                         for (int nt = 0; nt < HD / 8; ++nt)
                             *reinterpret_cast<float2*>(dst + nt * 8 + 2 * c) = make_float2(o[nt][2 * r], o[nt][2 * r + 1]);
-                        if (c == 0) p.part_ml[(size_t)item.part * p.row_cap + row] = make_float2(m[r], l[r]);
+                        if (c == 0) p.part_ml[(size_t)item.part * ATTN_THIN_ROWS + row] = make_float2(m[r], l[r]);
                     }
                 }
             }
@@ -252,8 +253,9 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                 // past the last part repeat it: left out under a condition they cost 600 bytes of spills in the stage loop.)
                 if (threadIdx.x == 0) p.group_count[item.grp] = 0;   // ready for the next launch
                 const int np = min(n_parts, ATTN_THIN_MAX_PARTS);
-                float* w_s = merge;   // [part][64]
-                constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5, CAP = 64;   // CAP: rows of a part
+                float* w_s = merge;   // [part][row]
+                constexpr int VR = HD / 4, NU = HD == 128 ? 5 : 3, UK = HD == 128 ? 3 : 5, CAP = ATTN_THIN_ROWS;
+                static_assert(CAP == 64, "two lanes of 128 threads take a row; row / G below");
                 const int n_vec = rows * VR, by_g = 4096 / G + 1;   // row / G = row * by_g >> 12 for rows up to 64
                 const float4* src = reinterpret_cast<const float4*>(p.part_o) + (size_t)part0 * (CAP * VR);
                 float4 v[UK][NU];
@@ -292,17 +294,17 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                             const float l_of = __shfl_xor_sync(0xFFFFFFFFu, t[k].y, 1);
                             lsum += (odd ? l_of : t[k].y) * (odd ? w_of : w);
                             lsum += (odd ? t[k].y : l_of) * (odd ? w : w_of);
-                            w_s[(k0 + odd + 2 * k) * 64 + row] = w;
+                            w_s[(k0 + odd + 2 * k) * CAP + row] = w;
                         }
                     }
                     const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
                     for (int k0 = odd; k0 < np; k0 += 8) {   // (its own entries)
                         float w[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) w[k] = w_s[min(k0 + 2 * k, ATTN_THIN_MAX_PARTS - 1) * 64 + row] * inv;
+                        for (int k = 0; k < 4; ++k) w[k] = w_s[min(k0 + 2 * k, ATTN_THIN_MAX_PARTS - 1) * CAP + row] * inv;
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if (k0 + 2 * k < np) w_s[(k0 + 2 * k) * 64 + row] = w[k];
+                            if (k0 + 2 * k < np) w_s[(k0 + 2 * k) * CAP + row] = w[k];
                     }
                 }
                 attn_thin_bar();
@@ -318,7 +320,7 @@ attn_thin_kernel(const __grid_constant__ CUtensorMap tmKV, AttnParams p) {
                             if (k0 + k >= np) break;
 #pragma unroll
                             for (int i = 0; i < NU; ++i) {
-                                const float w = w_s[(k0 + k) * 64 + min(u0 + i * 128, n_vec - 1) / VR];
+                                const float w = w_s[(k0 + k) * CAP + min(u0 + i * 128, n_vec - 1) / VR];
                                 acc[i].x += v[k][i].x * w; acc[i].y += v[k][i].y * w; acc[i].z += v[k][i].z * w; acc[i].w += v[k][i].w * w;
                             }
                         }

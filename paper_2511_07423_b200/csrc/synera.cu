@@ -356,7 +356,7 @@ struct syn_kv {
 
 // The attention kernels a work list can be made for.
 enum { ATTN_WARP = 1, ATTN_TENSOR = 2, ATTN_THIN = 3 };
-static int attn_rows(int kind) { return kind == ATTN_TENSOR ? 128 : 64; }
+static int attn_rows(int kind) { return kind == ATTN_TENSOR ? 128 : kind == ATTN_THIN ? ATTN_THIN_ROWS : 64; }
 
 struct syn_plan {
     syn_step_stats stats;
