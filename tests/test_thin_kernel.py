@@ -13,7 +13,7 @@ SHAPES = [(3072, 2048), (2048, 2048), (16384, 2048), (2048, 8192), (32000, 2048)
 
 
 def test_launch_shapes():
-    for T in list(range(1, 260)) + [300, 512]:
+    for T in list(range(1, 260)) + [300, 512, 513, 640, 769, 897, 1024]:
         for N, K in SHAPES:
             p = syn.thin_plan_host(T, N, K)
             S, nkb, U = p["splits"], p["num_kb"], p["TN"] // 16 * 4
@@ -85,10 +85,11 @@ def test_two_ctas_to_an_sm():
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("T,N,K", [
-    (385, 2048, 4096),    # four token tiles, the last of one token; 64 items in clusters of four
-    (449, 2048, 8192),    # 113 tokens in the last tile
+    (385, 2048, 4096),    # four token tiles of 112, 49 tokens in the last; 64 items in clusters of four
+    (449, 2048, 8192),    # four token tiles of 128, 65 tokens in the last
     (160, 4096, 4160),    # two token tiles of 80, 65 k-blocks in parts of 16 and 17
     (1024, 384, 2048),    # eight token tiles
+    (897, 384, 2048),     # the last of eight token tiles has one token: four units for six parts of K, two of which finish nothing
 ])
 def test_products_of_several_token_tiles_match_the_oracle(T, N, K):
     test_product_matches_oracle(T, N, K)
