@@ -198,7 +198,7 @@ struct EpiNext {
 };
 
 // The chunks of an item that a warp finishes, in turn: every NGRP-th of the chunks [c_lo, c_hi) of its tiles, from the grp-th on
-// (carried along: a division a chunk costs as much as a quarter of its stores).
+// (carried along instead of divided out for every chunk).
 template <int NGRP>
 struct EpiCursor {
     int mt, c, left, c_lo, c_hi;   // left: chunks from this one on, over all groups (<= 0: none for this warp)
@@ -389,7 +389,9 @@ __host__ __device__ constexpr bool epi_scaled(int mode) { return mode == EPI_QKV
 
 // Epilogue warps of the kernels that take a whole SM: 16 (four groups of four warps, one to a TMEM lane quarter) with 96 registers
 // each; 12 with 128 where a chunk's operand is in flight beside it, which does not fit into 96 (8B shape, cycles from the last MMA
-// to the end with 12 and 16 warps: o 27.4 and 30.9 k, down 27.1 and 30.4 k at 2 048 tokens, down 20.2 and 24.9 k at 544).
+// to the end with 12 and 16 warps: o 27.4 and 30.9 k, down 27.1 and 30.4 k at 2 048 tokens, down 20.2 and 24.9 k at 544).  Where a
+// CTA finishes few chunks a warp's share is rounded up more often with three groups: o of the 8B shape at 320 to 512 tokens, K in
+// parts, 33.1 < 35.0 us between events; the steps of those sizes are 1.02 to 1.04 times as fast all the same.
 __host__ __device__ constexpr int gemm_epi_warps(int mode) { return mode == EPI_QKV || mode == EPI_RESID ? 12 : GEMM_EPI_WARPS; }
 __host__ __device__ constexpr int gemm_threads(int mode) { return (2 + gemm_epi_warps(mode)) * 32; }
 
@@ -496,8 +498,8 @@ __global__ void pack_weight_kernel(PackSrc src, op16* __restrict__ out, int num_
 
 // ------------------------------------------------------------------------------------------
 // The kernel.  One persistent CTA per SM, 576 threads (448 with 12 epilogue warps): warp 0 = producer (bulk copy of the weight
-// tiles + TMA boxes of the token tile), warp 1 = TMEM owner and MMA issuer, warps 2..17 = epilogue
-// (four groups of four; a group covers the four TMEM lane quarters; draining TMEM is limited per
+// tiles + TMA boxes of the token tile), warp 1 = TMEM owner and MMA issuer, warps 2..17 (2..13) = epilogue
+// (four or three groups of four; a group covers the four TMEM lane quarters; draining TMEM is limited per
 // warp, so many warps share it).
 // ------------------------------------------------------------------------------------------
 constexpr int GEMM_BK = 64;                        // 16-bit elements per k-block = one 128-byte swizzle row

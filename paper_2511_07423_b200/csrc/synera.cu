@@ -134,7 +134,8 @@ judging_rows_kernel(const op16* xg, const float* ssq, const int* __restrict__ ro
 }
 
 // Greedy verification (paper Sec. 3.1 "draft & verify", Sec. 4.5): one thread per request.  The blocking calls have the results and
-// the kernels' status written straight to pinned host memory (three copies behind the kernel took 5 us).
+// the kernels' status written straight to pinned host memory (with three copies behind the kernel a call of four requests of
+// the two-layer shape took 84.6 us and takes 69.7; one on four layers of the 1B shape 243.7 and 230.0).
 __global__ void verify_kernel(const unsigned long long* __restrict__ best, const int* __restrict__ tokens,
                               const int* __restrict__ offsets, const int* __restrict__ n_uncached, int n_req,
                               int* __restrict__ accept_len, int* __restrict__ correction, int* __restrict__ top1_out,
@@ -1681,7 +1682,7 @@ static void thin_plan(int T, int packed_rows, int K, int n_sm, ThinParams& g) {
 //   qkv 31.1 > 20.9 (16 k-blocks a CTA), gate/up 29.1 > 28.1 (32), down 36.9 > 25.0 (32), 8B shape o 35.1 > 27.0 (32); but
 //   8B shape qkv 31.1 < 36.3 (176 tokens, 64 k-blocks), down 46 < 54 (112), 1B gate/up 35 < 41 at 320 tokens (384 CTAs).
 //   Beyond 512 tokens qkv of a narrow model (32 k-blocks, two CTAs to an SM): 1B 30.5 > 23.0 at 576 tokens, 33.1 > 23.2 at 640,
-//   29.0 > 24.5 at 768, 29.0 = 28.8 at 1 024; its o gains little (24.4 > 22.8 at 576).
+//   29.0 > 24.5 at 768, 29.0 = 28.8 at 1 024; its o would gain little (24.4 > 22.8 at 576) and is left to the other kernels.
 static bool thin_takes(int T, int packed_rows, int K, int n_sm, int mode) {
     if (T > (mode == EPI_QKV ? THIN_MAX_TOKENS_QKV : THIN_MAX_TOKENS)) return false;
     ThinParams g;
@@ -1789,7 +1790,9 @@ static void attn_params(AttnParams& ap, const syn_model* m, const syn_kv* kv, co
 // Only where most items are parts: while those are merged HBM idles, whereas whole units of unequal length keep some CTAs loading
 // to the end, and these the requests delay (1B shape, with and without: 32 requests of 256 - 2 048 keys 1 300 and 1 268 us a step,
 // 26 of 380 - 474 keys 894 and 863, 4 of 78 - 125 keys 787 and 755; one request in 104 parts 774 and 788; 8B shape, eight requests in
-// 288 parts 3 764 and 3 818).
+// 288 parts 3 764 and 3 818).  Where the line lies, over 176 batches of 3 to 32 requests, steps with the requests over those without:
+// no item a part 1B 1.02 - 1.08 and 8B 1.01 - 1.02; up to half of them 1B 1.02 - 1.04, 8B 1.00 - 1.01; half to 0.8 1B 0.99 - 1.03,
+// 8B 0.99 - 1.01; above that 1B 0.98 - 1.03, 8B 0.98 - 1.01.
 constexpr int64_t ATTN_AHEAD_BYTES = 24 << 20, ATTN_AHEAD_TILES = 10, ATTN_AHEAD_LATE_BYTES = 16 << 20;
 
 // What the attention may ask of L2 ahead: `budget` bytes (taken off) of a projection's weights beyond what the operand rings
@@ -1854,7 +1857,10 @@ static int run_step(syn_model* m, syn_kv* kv, const syn_plan* p, int* acc_dev, i
     const float inv_d = 1.0f / (float)d;
     // Where nobody asked for logits or argmaxes, the lm_head runs over the rows that verification looks at, if they are at most
     // half of more than 128 (up to there its time is that of its weights: 1B shape 37 us at 128 tokens, 105 at 768; a
-    // prefill iteration of 768 tokens of 24 requests needs 24 rows).
+    // prefill iteration of 768 tokens of 24 requests needs 24 rows).  At the edge, steps of two layers with all rows and with
+    // those: 1B shape 129 tokens, 64 rows 162.7 > 158.7 us, 160 and 80 163.0 = 162.9, 192 and 96 177.2 = 177.1, 256 and 128
+    // 205.8 > 197.6; 8B shape 129 and 64 449 > 431, 160 and 80 462 > 437, 256 and 128 578 > 521; 32B width, one layer, 129 and 64
+    // 545 > 511, 256 and 128 664 > 593.
     const bool judging_only = !logits_out && !top1_dev && T > 128 && 2 * p->n_judging <= T;
     const int T_lm = judging_only ? p->n_judging : T;
     m->last_stats = p->stats;
