@@ -40,18 +40,19 @@ ATTENTION_KERNELS = {1: "attn_kernel", 2: "attn2_kernel", 3: "attn_thin_kernel"}
 NCU_TRAFFIC = {
     # workload: {kernel function: (bytes per launch, sha256 of its source files, concatenated in KERNEL_SOURCES order)}
     "cfg2-1b": {
-        "thin_kernel": (32196796, "2e01dbe3661164617189274d7da000de05012eaeeb668e0e0b285f040c9db72e"),
-        "attn_thin_kernel": (101482616, "c15f438fe67f82a42070b50b1a589e21cdee7de006bae23d6701a98435f29729"),
-        "gemm_kernel": (132080128, "01423ee77c3e6e9cd2a0b3d7cfacb36cd74633fc48409c049d7b319f7a9bf44c"),
+        "thin_kernel": (32195190, "fa5f683e6a5c7abe0be3488893c027d08bd9a7ed5c75a0720623dad00594554c"),
+        "attn_thin_kernel": (76128496, "1d468a7e86d98543e36893f4f4a5fbb6df584938f417c20fac8394f28a1b26d3"),
+        "gemm_kernel": (132276480, "26fe9944f9b4a16b70456ccee3a5f3d29f0b3e4fa1c5edbb926a18c4e04824ae"),
     },
     "cfg3-8b": {
-        "attn_kernel": (615962556, "8cd80ea1f2e28708eabb2221a023e64c167ce5dcbad16aaaf965c0f1dcf61f05"),
-        "gemm_kernel": (284728176, "01423ee77c3e6e9cd2a0b3d7cfacb36cd74633fc48409c049d7b319f7a9bf44c"),
-        "gemm2_kernel": (99020461, "b9b3fd16ffeb2cdbca861d0fbafeb9d9f2d15003e4c3f3fbccade3fc4e2a0c48"),
+        "attn_kernel": (615884072, "dc1e7f9baeabaec514957be006cac65f38481a5bbb4c01e1c91e0ef264885c29"),
+        "gemm_kernel": (285624824, "26fe9944f9b4a16b70456ccee3a5f3d29f0b3e4fa1c5edbb926a18c4e04824ae"),
+        "gemm2_kernel": (98209944, "1719247565d956cd473cd3daeb0e2214bb3831e61722d3cff4ba2fdcfcbc9486"),
     },
-    # one layer's launch of the same work list, captured through `opbench attention --config 6 --kind 2`
     "cfg6-8b-chunk32": {
-        "attn2_kernel": (644797184, "2dd11156593b20096e42310454f2fbdb28bacb67a59033656c84df11431cc558"),
+        "attn2_kernel": (641542920, "7f910f2dcbcbdf97bc7afea4eccec9d73ffedbb8abd3a89133c7be29deb8f33e"),
+        "gemm_kernel": (106176088, "26fe9944f9b4a16b70456ccee3a5f3d29f0b3e4fa1c5edbb926a18c4e04824ae"),
+        "gemm2_kernel": (270231394, "1719247565d956cd473cd3daeb0e2214bb3831e61722d3cff4ba2fdcfcbc9486"),
     },
 }
 
