@@ -1,5 +1,7 @@
 """Calls that ask for no logits run the lm_head over the rows that verification looks at only: the same results as greedy
-verification of the logits that the same batch gives where they are asked for."""
+verification of the logits that the same batch gives where they are asked for.  The small models are compared token for token,
+on seeds whose closest pair of logits is decided alike (0.001 apart, below what fp32 sums could move it in the worst case); the
+full widths allow for ties at rounding level."""
 import dataclasses
 
 import pytest
